@@ -185,16 +185,16 @@ dssd_status dssd_device_resample(const float *p_row, const float *draft_q,
  * nothing.
  *
  * Same inputs, outputs and results as dssd_device_resample (the two share the kernel).
- *   - Sizes whose scratch need (dssd_device_resample_workspace_bytes: 256 bytes of counters plus
- *     8 bytes per 4096 vocabulary entries per sequence) exceeds DSSD_STATIC_SCRATCH_BYTES, i.e.
- *     B * ceil(V / 4096) > 131 040, are refused with DSSD_ERR_UNSUPPORTED before anything is
+ *   - Sizes whose scratch need (dssd_device_resample_workspace_bytes: at least 8 bytes per 4096
+ *     vocabulary entries per sequence) exceeds DSSD_STATIC_SCRATCH_BYTES, i.e.
+ *     B * ceil(V / 4096) > 131 072, are refused with DSSD_ERR_UNSUPPORTED before anything is
  *     enqueued; use dssd_device_resample for those.
  *   - The first call made with a given device current looks up the array's device address (once
  *     per device ordinal, for the context current at that moment: a process that creates a second
  *     context on the same device must not use this entry point from it).  Make that first call
  *     during set-up, before any stream capture is begun.
- *   - Every call on a device uses the same array.  Each call clears the counters it needs and
- *     overwrites the rest before reading it, so calls that follow one another on a stream are
+ *   - Every call on a device uses the same array.  Each call
+ *     overwrites what it reads, so calls that follow one another on a stream are
  *     independent; two calls that run on the GPU at the same time (different streams, or
  *     different host threads without ordering) race on the array and give undefined results.
  */

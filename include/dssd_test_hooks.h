@@ -39,8 +39,8 @@ dssd_status dssd_test_edge_verify_wait_runs_out(const void *target_logits, dssd_
 
 /*
  * dssd_device_resample in which the chunk sums of sequence `drop_seq` (0 <= drop_seq < B) are
- * computed but never stored, and a draw polls at most `poll_limit` times for a missing chunk sum.
- * That sequence ends with token = -1 and DSSD_RS_FLAG_TIMEOUT | DSSD_RS_FLAG_INVALID; every other
+ * computed but never stored.  (The sums are read after the kernel that forms them has ended, so a
+ * missing one is seen at the first look; `poll_limit` is not used.)  That sequence ends with token = -1 and DSSD_RS_FLAG_TIMEOUT | DSSD_RS_FLAG_INVALID; every other
  * sequence is drawn for as usual.  Arguments otherwise as dssd_device_resample.
  */
 dssd_status dssd_test_device_resample_wait_runs_out(const float *p_row, const float *draft_q,

@@ -158,7 +158,7 @@ namespace {
 dssd_status device_resample_any(const void *p_row, int p_half, const float *draft_q, const int32_t *accept_len,
                                 const float *uniforms, int B, int gamma, int V, int32_t *token, uint32_t *flags,
                                 void *workspace, size_t workspace_bytes, void *cuda_stream, int select = 0,
-                                int drop_seq_plus1 = 0, unsigned poll_limit = 0)
+                                int drop_seq_plus1 = 0)
 {
     t_last_cuda_error = 0;
     dssd_status st = check_sizes(B, gamma, V);
@@ -184,7 +184,6 @@ dssd_status device_resample_any(const void *p_row, int p_half, const float *draf
     P.token = token;
     P.flags = flags;
     P.test_drop_seq_plus1 = drop_seq_plus1;
-    P.test_poll_limit = poll_limit;
     cudaError_t e = dssd::resample_launch(P, workspace, static_cast<cudaStream_t>(cuda_stream));
     return e == cudaSuccess ? DSSD_OK : cuda_fail(e);
 }
@@ -198,9 +197,10 @@ dssd_status dssd_test_device_resample_wait_runs_out(const float *p_row, const fl
                                                     int drop_seq, unsigned poll_limit,
                                                     void *cuda_stream)
 {
+    (void)poll_limit;  // a withheld sum is seen at the first look
     if (B >= 1 && (drop_seq < 0 || drop_seq >= B)) return DSSD_ERR_INVALID_ARG;
     return device_resample_any(p_row, 0, draft_q, accept_len, uniforms, B, gamma, V, token, flags, workspace,
-                               workspace_bytes, cuda_stream, 0, drop_seq + 1, poll_limit);
+                               workspace_bytes, cuda_stream, 0, drop_seq + 1);
 }
 
 dssd_status dssd_device_resample(const float *p_row, const float *draft_q,

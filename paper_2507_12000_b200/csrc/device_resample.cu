@@ -1,41 +1,44 @@
-// Device half of the verification round: residual (or bonus) inverse-CDF draw.
+// Device half of the verification round: residual (or bonus) inverse-CDF draw, as two kernels.
 //
-// Pass A, ticket (b, c): stream chunk c of p_row[b] and of Q_n[b], form r = max(0, p - q) (or
-// r = p for the bonus draw) and add it up in float64 -> one or two chunk sums, 8-byte slots that are
-// valid once they differ from the all-ones pattern that the kernel itself clears its scratch to
-// (a cooperative launch; one grid-wide barrier, split around the first ticket's loads, separates
-// the clearing from the first use).  A ticket costs one barrier and waits for no round trip.
-// Pass B, ticket b, taken by a CTA once no chunk is left for it: a block-wide float64 prefix over
-// the sequence's chunk sums gives Z and the chunk holding u' * Z; every thread fetches its run of
-// that chunk (from L2 or HBM), a second prefix finds the thread, and the thread walks its run.
-// The draws run after the streams because their dependent round trips are several times longer
-// while the memory system is saturated.
+//   resample_mass_kernel  one CTA per (sequence, one to four tiles of kTile entries): streams its part of
+//                         p_row[b] and of Q_n[b], forms r = max(0, p - q) (or r = p for the bonus draw)
+//                         and adds it up in float64: one sum per chunk of kResampleSub entries.
+//   resample_draw_kernel  one CTA per sequence: a float64 prefix over the sequence's chunk sums gives Z
+//                         and the chunk that holds u' * Z; every thread fetches its run of that chunk, a
+//                         second prefix finds the thread and its run gives the token.
+//
+// Plain stores and the order of the two launches (launch.h) connect them: no ticket, no wait, nothing
+// in the scratch that has to be cleared.
 // All sums are float64, so the token differs from an index-order float64 scan only when u' * Z
 // lies within rounding (about 1e-13 relative) of a CDF step.
 #include "device_resample.h"
 #include "edge_verify.h"
 
-#include <atomic>
 #include <mutex>
 
-#include <limits.h>
 #include <math.h>
 
-#include <utility>
-
-#include <cooperative_groups.h>
-
 #include "dssd_device.cuh"
+#include "launch.h"
 
 namespace dssd {
 
 namespace {
 
-constexpr bool kWideTickets = true;  // whole tickets request all their loads at once (ticket_mass2)
-constexpr int kResampleCtas = 4;      // resident CTAs per SM aimed at
-constexpr int kSub = kResampleSub;         // entries per chunk sum: a ticket covers P.subs of them
-constexpr int kRun = kSub / kThreads;      // contiguous entries per thread in pass B
-static_assert(kRun == 16, "pass B fetches a run as one group of 16 entries");
+constexpr int kSub = kResampleSub;      // entries per chunk sum
+constexpr int kRows = 4;                 // chunks per tile: quad number u * kThreads + t of a tile is thread t's u-th
+constexpr int kTile = kRows * kSub;      // entries that a CTA streams at a time
+static_assert(kSub == 4 * kThreads, "a chunk is one quad per thread of the mass kernel");
+// Tiles per CTA of the mass kernel.  Few tiles: one each, so that all SMs share them.  More than about
+// one and a half waves of 740 resident CTAs: two, more than six waves: four, which pays for a CTA's
+// start and its reduction less often.  Measured (us, mass kernel with the draw behind it; 1 / 2 / 4 tiles):
+// B = 256 V = 151936 (9728 tiles) 45.7 / 45.0 / 41.7, B = 64 V = 128256 (2048) 21.4 / 21.4 / 32.1,
+// B = 8 V = 32000 (64) 7.9 / 8.7 / 10.2.
+constexpr unsigned long long kTwoTiles = 1200, kFourTiles = 4800;
+constexpr int kDrawThreads = 128;        // threads that draw for a sequence
+constexpr int kDrawWarps = kDrawThreads / 32;
+constexpr int kRun = kSub / kDrawThreads;  // entries of a chunk per thread
+constexpr int kKeep = 8;                 // chunk sums that a lane keeps: enough for 256 chunks without a second look
 
 __device__ __forceinline__ double res(float p, float q) { return fmax(0.0, (double)p - (double)q); }
 
@@ -56,10 +59,30 @@ __device__ __forceinline__ float4 half_quad(uint2 v)
     const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
     return make_float4(a.x, a.y, b.x, b.y);
 }
-__device__ __forceinline__ uint2 ld_stream8(const void *p)
+// Loads of a row that an earlier kernel of the chain may have written: they stay behind pdl_wait()
+// and do not go through the read-only path.  Vectors are read once and not kept in L1.
+__device__ __forceinline__ uint4 ld_row16(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_row8(const void *p)
 {
     uint2 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_row(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned short ld_row(const uint16_t *p)
+{
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -73,16 +96,12 @@ struct RowF32 {  // p_row as float32
         return r;
     }
     __device__ __forceinline__ bool aligned(int e) const { return (reinterpret_cast<uintptr_t>(p + e) & 15u) == 0; }
-    __device__ __forceinline__ float ld(int64_t e) const { return __ldg(p + e); }
+    __device__ __forceinline__ float ld(int64_t e) const { return ld_row(p + e); }
     __device__ __forceinline__ Raw ld_quad_stream(int e0, int64_t quad) const
     {
-        return ld_stream16(reinterpret_cast<const uint4 *>(p + e0) + quad);
+        return ld_row16(p + e0 + 4 * quad);
     }
     __device__ __forceinline__ float4 quad(const Raw &v) const { return as_f4(v); }
-    __device__ __forceinline__ float4 ld_quad(int e0, int64_t quad) const
-    {
-        return __ldg(reinterpret_cast<const float4 *>(p + e0) + quad);
-    }
 };
 
 struct RowF16 {  // p_row as binary16 bit patterns
@@ -95,16 +114,12 @@ struct RowF16 {  // p_row as binary16 bit patterns
         return r;
     }
     __device__ __forceinline__ bool aligned(int e) const { return (reinterpret_cast<uintptr_t>(p + e) & 7u) == 0; }
-    __device__ __forceinline__ float ld(int64_t e) const { return half_bits_to_float(__ldg(p + e)); }
+    __device__ __forceinline__ float ld(int64_t e) const { return half_bits_to_float(ld_row(p + e)); }
     __device__ __forceinline__ Raw ld_quad_stream(int e0, int64_t quad) const
     {
-        return ld_stream8(reinterpret_cast<const uint2 *>(p + e0) + quad);
+        return ld_row8(p + e0 + 4 * quad);
     }
     __device__ __forceinline__ float4 quad(const Raw &v) const { return half_quad(v); }
-    __device__ __forceinline__ float4 ld_quad(int e0, int64_t quad) const
-    {
-        return half_quad(__ldg(reinterpret_cast<const uint2 *>(p + e0) + quad));
-    }
 };
 
 // four consecutive logits: how they are loaded and widened
@@ -136,10 +151,10 @@ struct RowLogits {  // row n of the target logits, turned into probabilities on 
         RowLogits r;
         r.row = reinterpret_cast<const char *>(P.logits) +
                 ((size_t)b * (size_t)(P.gamma + 1) + (size_t)n) * (size_t)P.row_stride * Elem<DT>::kBytes;
-        const ReadySlot s = reinterpret_cast<const ReadySlot *>(P.ready)[b];
+        const ReadySlot *s = reinterpret_cast<const ReadySlot *>(P.ready) + b;
         r.c1 = P.c1;
-        r.nref = -s.ref2;
-        r.invS = s.invS;
+        r.nref = -ld_after(&s->ref2);
+        r.invS = ld_after(&s->invS);
         return r;
     }
     __device__ __forceinline__ float prob(float l) const { return ex2(fmaf(l, c1, nref)) * invS; }
@@ -157,121 +172,121 @@ struct RowLogits {  // row n of the target logits, turned into probabilities on 
         const float4 l = LogitQuad<DT>::widen(v);
         return make_float4(prob(l.x), prob(l.y), prob(l.z), prob(l.w));
     }
-    __device__ __forceinline__ float4 ld_quad(int e0, int64_t quad) const { return this->quad(ld_quad_stream(e0, quad)); }
 };
 
-// per-thread part of sum_{e in [e0,e1)} r_e ; q == nullptr means r = p
-template <typename RV>
-__device__ __forceinline__ double chunk_mass(const RV &row, const float *q, int e0, int e1)
+// This thread's part of the four chunk sums of the tile that starts at entry e0 (entries up to e1 only).
+// All loads are requested before the first is used.  Where the rows are not aligned, or the tile is
+// not a full one, entries are loaded one by one, neighbouring threads on neighbouring entries of the
+// same chunk.  q is not read without kHasQ (then r = p); with kPlain the sums of p go to `plain`.
+template <bool kHasQ, bool kPlain, typename RV>
+__device__ __forceinline__ void tile_mass(const RV &row, const float *q, int e0, int e1, double (&acc)[kRows], double *plain = nullptr)
 {
     const int tid = threadIdx.x;
-    double acc = 0.0;
-    int done = e0;
-    const bool aligned = row.aligned(e0) && (!q || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0);
-    if (aligned) {
-        const int nvec = (e1 - e0) / 4;
-        if (q) {
-            const uint4 *q4 = reinterpret_cast<const uint4 *>(q + e0);
-            int i = tid;
-            for (; i + 3 * kThreads < nvec; i += 4 * kThreads) {
-                typename RV::Raw a[4];
-                uint4 b[4];
+    if (e1 - e0 == kTile && row.aligned(e0) && (!kHasQ || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0)) {
+        typename RV::Raw a[kRows];
+        uint4 b[kRows];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    a[u] = row.ld_quad_stream(e0, i + u * kThreads);
-                    b[u] = ld_stream16(q4 + i + u * kThreads);
-                }
+        for (int u = 0; u < kRows; ++u) a[u] = row.ld_quad_stream(e0, tid + u * kThreads);
+        if (kHasQ) {
+            const float *qp = q + e0 + 4 * tid;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float4 x = row.quad(a[u]), y = as_f4(b[u]);
-                    acc += (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
-                }
-            }
-            for (; i < nvec; i += kThreads) {
-                const float4 x = row.quad(row.ld_quad_stream(e0, i)), y = as_f4(ld_stream16(q4 + i));
-                acc += (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
-            }
-        } else {
-            int i = tid;
-            for (; i + 3 * kThreads < nvec; i += 4 * kThreads) {
-                typename RV::Raw a[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) a[u] = row.ld_quad_stream(e0, i + u * kThreads);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float4 x = row.quad(a[u]);
-                    acc += ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-                }
-            }
-            for (; i < nvec; i += kThreads) {
-                const float4 x = row.quad(row.ld_quad_stream(e0, i));
-                acc += ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-            }
+            for (int u = 0; u < kRows; ++u) b[u] = ld_row16(qp + u * kSub);
         }
-        done = e0 + nvec * 4;
-    }
-    for (int e = done + tid; e < e1; e += kThreads) acc += q ? res(row.ld(e), __ldg(q + e)) : (double)row.ld(e);
-    return acc;
-}
-
-// A whole ticket of two full chunk sums whose rows are 16-byte aligned: all of a thread's loads
-// (eight quads of p and of q) are requested before the first is used.  Quads u < 4 of a thread
-// belong to the first chunk sum, the others to the second; the order of addition within each is
-// the one chunk_mass uses, so both give the same bits.
-template <typename RV>
-__device__ __forceinline__ void ticket_mass2(const RV &row, const float *q, int e0, double &acc0, double &acc1)
-{
-    const int tid = threadIdx.x;
-    typename RV::Raw a[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) a[u] = row.ld_quad_stream(e0, tid + u * kThreads);
-    if (q) {
-        const uint4 *q4 = reinterpret_cast<const uint4 *>(q + e0);
-        uint4 b[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) b[u] = ld_stream16(q4 + tid + u * kThreads);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float4 x = row.quad(a[u]), y = as_f4(b[u]);
-            const double t = (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
-            if (u < 4) acc0 += t;
-            else acc1 += t;
+        for (int u = 0; u < kRows; ++u) {
+            const float4 x = row.quad(a[u]);
+            if (kHasQ) {
+                const float4 y = as_f4(b[u]);
+                acc[u] = (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
+            }
+            if (!kHasQ || kPlain) {
+                const double s = ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
+                if (kPlain) plain[u] = s;
+                if (!kHasQ) acc[u] = s;
+            }
         }
     } else {
+        const int first = e0 + tid, left = e1 - first;
+        float x[4 * kRows], y[4 * kRows];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float4 x = row.quad(a[u]);
-            const double t = ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-            if (u < 4) acc0 += t;
-            else acc1 += t;
+        for (int j = 0; j < 4 * kRows; ++j) {
+            x[j] = y[j] = 0.f;
+            if (j * kThreads < left) x[j] = row.ld((int64_t)first + j * kThreads);
+        }
+        if (kHasQ) {
+            const float *qp = q + first;
+#pragma unroll
+            for (int j = 0; j < 4 * kRows; ++j)
+                if (j * kThreads < left) y[j] = ld_row(qp + j * kThreads);
+        }
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            double r[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                r[j] = (4 * u + j) * kThreads < left ? (kHasQ ? res(x[4 * u + j], y[4 * u + j]) : (double)x[4 * u + j]) : 0.0;
+            acc[u] = (r[0] + r[1]) + (r[2] + r[3]);
+            if (kPlain)
+                plain[u] = ((double)x[4 * u] + (double)x[4 * u + 1]) + ((double)x[4 * u + 2] + (double)x[4 * u + 3]);
         }
     }
 }
 
-// CTA-wide sum in a fixed order; result valid in thread 0
-__device__ __forceinline__ double block_sum(double x, double *s_w)
+// Four sums over the warp at the price of six shuffled doubles: the lane ends up with sum number
+// (bit 4 of the lane) * 2 + (bit 3 of the lane).
+__device__ __forceinline__ double warp_sum4(const double (&x)[4])
 {
-    x = warp_sum(x);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = x;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0) {
+    const bool hi = threadIdx.x & 16, lo = threadIdx.x & 8;
+    double a = hi ? x[2] : x[0], b = hi ? x[3] : x[1];
+    a += __shfl_xor_sync(0xffffffffu, hi ? x[0] : x[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, hi ? x[1] : x[3], 16);
+    double c = lo ? b : a;
+    c += __shfl_xor_sync(0xffffffffu, lo ? a : b, 8);
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) t += s_w[w];
-    }
-    return t;
+    for (int o = 4; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    return c;
 }
 
-struct Pick {  // what thread 0 hands to the CTA for pass B
-    int ok;        // Z > 0 and finite
-    int chunk;     // chunk holding the target
-    int beyond;    // no chunk prefix exceeds the target: take the last positive entry
-    double base;   // mass before that chunk
-    double target; // u' * Z
-};
+// r for thread t's run of the chunk [e0, e0 + kSub), entries e0 + kRun * t + j in r[j]; 0 from entry e1
+// on.  All loads are requested before the first is used.
+template <bool kHasQ, typename RV>
+__device__ __forceinline__ void load_run(const RV &row, const float *q, int e0, int e1, double (&r)[kRun])
+{
+    const int first = e0 + kRun * (int)threadIdx.x, left = e1 - first;
+    float y[kRun];
+    if (e1 - e0 == kSub && row.aligned(e0) && (!kHasQ || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0)) {
+        typename RV::Raw a[kRun / 4];
+#pragma unroll
+        for (int u = 0; u < kRun / 4; ++u) a[u] = row.ld_quad_stream(first, u);
+        if (kHasQ) {
+#pragma unroll
+            for (int u = 0; u < kRun / 4; ++u) {
+                const float4 v = as_f4(ld_row16(q + first + 4 * u));
+                y[4 * u] = v.x, y[4 * u + 1] = v.y, y[4 * u + 2] = v.z, y[4 * u + 3] = v.w;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kRun / 4; ++u) {
+            const float4 x = row.quad(a[u]);
+            r[4 * u] = kHasQ ? res(x.x, y[4 * u]) : (double)x.x;
+            r[4 * u + 1] = kHasQ ? res(x.y, y[4 * u + 1]) : (double)x.y;
+            r[4 * u + 2] = kHasQ ? res(x.z, y[4 * u + 2]) : (double)x.z;
+            r[4 * u + 3] = kHasQ ? res(x.w, y[4 * u + 3]) : (double)x.w;
+        }
+    } else {
+        float x[kRun];
+#pragma unroll
+        for (int j = 0; j < kRun; ++j) {
+            x[j] = y[j] = 0.f;
+            if (j < left) x[j] = row.ld((int64_t)first + j);
+            if (kHasQ && j < left) y[j] = ld_row(q + first + j);
+        }
+#pragma unroll
+        for (int j = 0; j < kRun; ++j) r[j] = j < left ? (kHasQ ? res(x[j], y[j]) : (double)x[j]) : 0.0;
+    }
+}
 
-constexpr unsigned long long kFill64 = ~0ull;
+constexpr unsigned long long kNoSum = ~0ull;  // stored in place of a withheld chunk sum (a sum is never this NaN)
 
 // is a sequence with accepted length n (0 <= n <= gamma) one this launch draws for?
 __device__ __forceinline__ bool selected(const ResampleParams &P, int n)
@@ -279,409 +294,293 @@ __device__ __forceinline__ bool selected(const ResampleParams &P, int n)
     return P.select == 0 || (P.select == 1 ? n == P.gamma : n < P.gamma);
 }
 
-__device__ __forceinline__ unsigned long long logical(unsigned long long raw) { return raw + 1ull; }
+__device__ __forceinline__ bool missing(double m) { return (unsigned long long)__double_as_longlong(m) == kNoSum; }
 
-// chunk sum (b, c); a sum whose store has not landed yet still shows the fill pattern and is
-// polled for (bounded); when the wait runs out the fill pattern itself comes back (see timed_out)
-__device__ __forceinline__ double load_chunk_sum(const ResampleParams &P, const unsigned long long *cs, int c, unsigned polls)
+// Where in a row the draw falls.
+struct Pick {
+    bool ok;        // the row's mass Z is positive and finite
+    bool late;      // a chunk sum is missing
+    bool beyond;    // no chunk prefix exceeds the target: take the last positive entry
+    int chunk;
+    double base;    // mass before that chunk
+    double target;  // the running mass that the token's must exceed
+};
+
+__device__ __forceinline__ double warp_scan(double x)  // inclusive, in lane order
 {
-    unsigned long long w = ld_relaxed_u64(cs + c);
-    for (unsigned it = 0; w == kFill64 && it < polls; ++it) {
-        __nanosleep(32);
-        w = ld_relaxed_u64(cs + c);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double up = __shfl_up_sync(0xffffffffu, x, o);
+        if ((int)(threadIdx.x & 31) >= o) x += up;
     }
-    return __longlong_as_double((long long)w);
+    return x;
 }
 
-__device__ __forceinline__ bool timed_out(double m) { return (unsigned long long)__double_as_longlong(m) == kFill64; }
+__device__ __forceinline__ double shfl_f64(double x, int src) { return __shfl_sync(0xffffffffu, x, src); }
 
-// every thread's verdict on its chunk sums; on a timeout the sequence gets no token
-__device__ __forceinline__ bool give_up(const ResampleParams &P, int64_t b, bool mine, unsigned fl)
+// The chunk sums that lane l of a warp looks at: a contiguous share of the n_sub, the first kKeep of
+// them in registers.  sum(c) loads chunk sum c.
+struct LaneSums {
+    int c0, c1;
+    double m[kKeep];
+};
+template <class Sum>
+__device__ __forceinline__ void load_sums(LaneSums &L, int n_sub, Sum sum)
 {
-    if (!__syncthreads_or(mine)) return false;
-    if (threadIdx.x == 0) {
-        P.token[b] = -1;
-        if (P.flags) P.flags[b] = fl | DSSD_RS_FLAG_INVALID | DSSD_RS_FLAG_TIMEOUT;
-    }
-    return true;
+    const int per = (n_sub + 31) / 32;
+    L.c0 = min(n_sub, (int)(threadIdx.x & 31) * per);
+    L.c1 = min(n_sub, L.c0 + per);
+#pragma unroll
+    for (int k = 0; k < kKeep; ++k) L.m[k] = L.c0 + k < L.c1 ? sum(L.c0 + k) : 0.0;
 }
 
-// CTA-wide inclusive prefix sum in index order of the threads; `total` is the sum over the CTA
-__device__ __forceinline__ double block_scan(double x, double *s_scan, double &total)
+// Every warp does the same, so nothing is exchanged: a prefix over the lanes' shares gives Z, and the
+// first chunk whose inclusive prefix exceeds target(Z) - the last one with mass when there is none - is
+// the pick.  `beyond` set by the caller means that no prefix is known to exceed the target.  The
+// float64 additions that depend on one another are what this costs: the prefix within a lane's share is
+// formed once and compared in parallel.
+template <class Sum, class Target>
+__device__ __forceinline__ Pick pick_chunk(const LaneSums &L, Sum sum, bool beyond, Target target)
+{
+    const int lane = threadIdx.x & 31;
+    double pre[kKeep];
+    double s = 0.0;
+    bool late = false;
+    unsigned positive = 0;
+#pragma unroll
+    for (int k = 0; k < kKeep; ++k) {
+        s += L.m[k];
+        pre[k] = s;
+        late |= missing(L.m[k]);
+        positive |= L.m[k] > 0.0 ? 1u << k : 0u;
+    }
+    for (int c = L.c0 + kKeep; c < L.c1; ++c) {
+        const double x = sum(c);
+        s += x;
+        late |= missing(x);
+    }
+    const double incl = warp_scan(s);
+    const double up = __shfl_up_sync(0xffffffffu, incl, 1);
+    const double excl = lane ? up : 0.0;
+    Pick pk;
+    const double Z = shfl_f64(incl, 31);
+    pk.late = __any_sync(0xffffffffu, late);
+    pk.ok = (Z > 0.0) && (Z < INFINITY);
+    pk.target = target(Z);
+    const unsigned cross = beyond ? 0u : __ballot_sync(0xffffffffu, s > 0.0 && incl > pk.target);
+    const unsigned mass = __ballot_sync(0xffffffffu, s > 0.0);
+    pk.beyond = cross == 0;
+    const int owner = cross ? __ffs(cross) - 1 : mass ? 31 - __clz(mass) : 0;
+    // the lane's own chunks: the first that crosses, else the last with mass
+    int k = 0;
+    unsigned over = 0;
+#pragma unroll
+    for (int j = 0; j < kKeep; ++j) over |= cross && excl + pre[j] > pk.target ? 1u << j : 0u;
+    over &= positive;
+    bool hit = over != 0;
+    if (hit) k = __ffs(over) - 1;
+    else if (positive) k = 31 - __clz(positive);
+    double base = excl;
+#pragma unroll
+    for (int j = 1; j < kKeep; ++j)
+        if (j == k) base = excl + pre[j - 1];
+    if (lane == owner && !hit) {  // (beyond kKeep chunks per lane only)
+        double C = excl + pre[kKeep - 1];
+        for (int c = L.c0 + kKeep; c < L.c1 && !hit; ++c) {
+            const double x = sum(c);
+            if (x > 0.0) {
+                k = c - L.c0;
+                base = C;
+                hit = cross != 0 && C + x > pk.target;
+            }
+            C += x;
+        }
+    }
+    pk.chunk = __shfl_sync(0xffffffffu, L.c0 + k, owner);
+    pk.base = shfl_f64(base, owner);
+    return pk;
+}
+
+// The draw inside the picked chunk, entries [e0, e1), by the whole CTA: the token is the first entry whose
+// running mass exceeds the target, else (rounding, or pk.beyond) the last one with mass; -1 when
+// the chunk has none.  `base` moves on by the chunk's mass; `hit`: the target was exceeded.  The result is
+// the same in all threads.  q == nullptr means r = p.
+struct WalkShared {
+    double sum[kDrawWarps];
+    int tok[kDrawWarps];   // the warp's token; hit in bit 30
+};
+template <typename RV>
+__device__ __forceinline__ int walk_chunk(const Pick &pk, const RV &row, const float *q, int e0, int e1, double &base, bool &hit,
+                                          WalkShared &sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
-    }
-    __syncthreads();
-    if (lane == 31) s_scan[warp] = incl;
-    __syncthreads();
-    double before = 0.0, all = 0.0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const double v = s_scan[w];
-        if (w < warp) before += v;
-        all += v;
-    }
-    total = all;
-    return before + incl;
-}
-
-// The draw inside the chunk that `pk` names: every thread fetches its run of the chunk, a prefix over
-// the CTA finds the thread whose run holds the target, and that thread walks its run.  The token
-// (its index in the row plus tok_base, or -1 when the chunk has no positive entry) and the flags
-// go to *token_out / *flags_out.  q == nullptr means r = p.
-template <typename RV>
-__device__ __forceinline__ void walk_chunk(const Pick &pk, int V, const RV &row, const float *q, unsigned fl, int tok_base,
-                                           int32_t *token_out, uint32_t *flags_out, double *s_w, int *s_i)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int e0 = pk.chunk * kSub, e1 = min(V, e0 + kSub);
-    const int r0 = min(e1, e0 + tid * kRun), r1 = min(e1, r0 + kRun);
+    double r[kRun], pre[kRun];
+    if (q) load_run<true>(row, q, e0, e1, r);
+    else load_run<false>(row, q, e0, e1, r);
+    unsigned positive = 0;
     double mine = 0.0;
-    int last_pos = -1;
-    // The run's 16 entries are all requested before the first is used (one round trip for the
-    // run, not one per entry); entries past the row's end read as 0.
-    const bool vec = (r1 - r0 == kRun) && row.aligned(r0) && (!q || (reinterpret_cast<uintptr_t>(q + r0) & 15u) == 0);
 #pragma unroll
-    for (int g = 0; g < kRun; g += 16) {
-        float pv[16], qv[16];
-        if (vec) {
+    for (int j = 0; j < kRun; ++j) {
+        mine += r[j];
+        pre[j] = mine;
+        positive |= r[j] > 0.0 ? 1u << j : 0u;
+    }
+    const double incl = warp_scan(mine);
+    __syncthreads();  // (an earlier chunk's results have been read)
+    if (lane == 31) sh.sum[warp] = incl;
+    __syncthreads();
+    double before = base;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 a = row.ld_quad(r0 + g, j);
-                pv[4 * j] = a.x, pv[4 * j + 1] = a.y, pv[4 * j + 2] = a.z, pv[4 * j + 3] = a.w;
-                float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (q) c = __ldg(reinterpret_cast<const float4 *>(q + r0 + g) + j);
-                qv[4 * j] = c.x, qv[4 * j + 1] = c.y, qv[4 * j + 2] = c.z, qv[4 * j + 3] = c.w;
-            }
-        } else {
+    for (int w = 0; w < kDrawWarps; ++w) {
+        if (w == warp) before = base;
+        base += sh.sum[w];
+    }
+    const double up = __shfl_up_sync(0xffffffffu, incl, 1);
+    const double C = before + (lane ? up : 0.0);
+    unsigned over = 0;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int e = r0 + g + j;
-                pv[j] = e < r1 ? row.ld(e) : 0.f;
-                qv[j] = (q && e < r1) ? __ldg(q + e) : 0.f;
-            }
-        }
+    for (int j = 0; j < kRun; ++j) over |= !pk.beyond && C + pre[j] > pk.target ? 1u << j : 0u;
+    over &= positive;
+    const unsigned cross = __ballot_sync(0xffffffffu, over != 0), mass = __ballot_sync(0xffffffffu, positive != 0);
+    const int owner = cross ? __ffs(cross) - 1 : mass ? 31 - __clz(mass) : 0;
+    int t = -1;
+    if (positive) t = e0 + kRun * (int)threadIdx.x + (over ? __ffs(over) - 1 : 31 - __clz(positive));
+    if (lane == owner) sh.tok[warp] = t < 0 ? -1 : cross ? t | (1 << 30) : t;
+    __syncthreads();
+    // the first warp that crosses, else the last with mass
+    int tok = -1;
+    hit = false;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const double r = q ? res(pv[j], qv[j]) : (double)pv[j];
-            mine += r;
-            if (r > 0.0) last_pos = r0 + g + j;
+    for (int w = 0; w < kDrawWarps; ++w) {
+        const int x = sh.tok[w];
+        if (x >= 0 && !hit) {
+            tok = x & ~(1 << 30);
+            hit = (x >> 30) & 1;
         }
     }
-    // exclusive prefix of the per-thread run sums across the CTA
-    double incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
-    }
-    __syncthreads();
-    if (lane == 31) s_w[warp] = incl;
-    __syncthreads();
-    double before = pk.base;
-    for (int w = 0; w < warp; ++w) before += s_w[w];
-    before += incl - mine;
-    const bool crosses = !pk.beyond && (before + mine > pk.target);
-    const unsigned bal = __ballot_sync(0xffffffffu, crosses);
-    if (tid == 0) { s_i[0] = 0x7fffffff; s_i[1] = -1; }
-    __syncthreads();
-    if (lane == 0 && bal) atomicMin(&s_i[0], warp * 32 + __ffs(bal) - 1);
-    if (last_pos >= 0) atomicMax(&s_i[1], last_pos);
-    __syncthreads();
-    const int first = s_i[0];
-    if (first == 0x7fffffff) {
-        if (tid == 0) {
-            *token_out = s_i[1] < 0 ? -1 : tok_base + s_i[1];
-            if (flags_out) *flags_out = fl | (s_i[1] < 0 ? DSSD_RS_FLAG_INVALID : 0u);
-        }
-    } else if (tid == first) {
-        double C = before;
-        int tok = last_pos;
-        for (int e = r0; e < r1; ++e) {
-            C += q ? res(row.ld(e), __ldg(q + e)) : (double)row.ld(e);
-            if (C > pk.target) { tok = e; break; }
-        }
-        tok = tok >= 0 ? tok : s_i[1];
-        *token_out = tok < 0 ? -1 : tok_base + tok;
-        if (flags_out) *flags_out = fl;
-    }
+    return tok;
 }
 
-// pass B for sequence b; q == nullptr means r = p
+// The draw for sequence b by one CTA; q == nullptr means r = p.
 template <typename RV>
-__device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const float *q, unsigned fl, float u,
-                     double *s_w, Pick *s_pick, int *s_i)
+__device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const float *q, unsigned fl, float u, LaneSums &L,
+                     WalkShared &sh)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned long long *cs = reinterpret_cast<unsigned long long *>(P.chunk_sum) + (size_t)b * P.n_sub;
-    const unsigned polls = b + 1 == (int64_t)P.test_drop_seq_plus1 ? P.test_poll_limit : P.spin_limit;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        bool ok;
-        if (P.n_sub <= kThreads) {
-            // one chunk per thread: a single scan gives Z and every inclusive prefix
-            const double m = tid < P.n_sub ? load_chunk_sum(P, cs, tid, polls) : 0.0;
-            if (give_up(P, b, timed_out(m), fl)) return;
-            double Z;
-            const double incl = block_scan(m, s_w, Z);
-            ok = (Z > 0.0) && (Z < INFINITY);
-            if (ok) {
-                const double target = (double)u * Z;
-                if (tid == 0) {
-                    s_i[0] = 0x7fffffff;
-                    s_i[1] = -1;
-                }
-                __syncthreads();
-                const bool crosses = tid < P.n_sub && incl > target;
-                const unsigned bal = __ballot_sync(0xffffffffu, crosses);
-                if (lane == 0 && bal) atomicMin(&s_i[0], warp * 32 + __ffs(bal) - 1);
-                const unsigned pos = __ballot_sync(0xffffffffu, tid < P.n_sub && m > 0.0);
-                if (lane == 0 && pos) atomicMax(&s_i[1], warp * 32 + 31 - __clz(pos));
-                __syncthreads();
-                const int first = s_i[0], last = s_i[1];
-                if (tid == (first != 0x7fffffff ? first : last)) {
-                    Pick pk;
-                    pk.ok = 1;
-                    pk.beyond = first == 0x7fffffff;
-                    pk.chunk = tid;
-                    pk.base = incl - m;
-                    pk.target = target;
-                    *s_pick = pk;
-                }
-                __syncthreads();
-                break;
-            }
-        } else {
-        // Z = sum of the chunk sums, in groups of one chunk per thread
-        double Z = 0.0;
-        bool late = false;
-        for (int base = 0; base < P.n_sub; base += kThreads) {
-            const int c = base + tid;
-            const double m = c < P.n_sub ? load_chunk_sum(P, cs, c, polls) : 0.0;
-            late |= timed_out(m);
-            double tot;
-            block_scan(m, s_w, tot);
-            Z += tot;
-            __syncthreads();
-        }
-        if (give_up(P, b, late, fl)) return;
-        ok = (Z > 0.0) && (Z < INFINITY);
-        if (ok) {
-            // the first chunk whose inclusive prefix exceeds the target, else the last chunk with mass
-            const double target = (double)u * Z;
-            if (tid == 0) {
-                s_i[0] = 0x7fffffff;
-                s_i[1] = -1;
-            }
-            __syncthreads();
-            double carry = 0.0;
-            double my_base_first = 0.0, my_base_last = 0.0;
-            int my_first = 0x7fffffff, my_last = -1;
-            for (int base = 0; base < P.n_sub; base += kThreads) {
-                const int c = base + tid;
-                const double m = c < P.n_sub ? load_chunk_sum(P, cs, c, polls) : 0.0;
-                double tot;
-                const double incl = carry + block_scan(m, s_w, tot);
-                if (c < P.n_sub && incl > target && my_first == 0x7fffffff) {
-                    my_first = c;
-                    my_base_first = incl - m;
-                }
-                if (c < P.n_sub && m > 0.0) {
-                    my_last = c;
-                    my_base_last = incl - m;
-                }
-                carry += tot;
-                __syncthreads();
-            }
-            if (my_first != 0x7fffffff) atomicMin(&s_i[0], my_first);
-            if (my_last >= 0) atomicMax(&s_i[1], my_last);
-            __syncthreads();
-            const int first = s_i[0], last = s_i[1];
-            if (first != 0x7fffffff ? (my_first == first) : (my_last == last && last >= 0)) {
-                Pick pk;
-                pk.ok = 1;
-                pk.beyond = first == 0x7fffffff;
-                pk.chunk = pk.beyond ? last : first;
-                pk.base = pk.beyond ? my_base_last : my_base_first;
-                pk.target = target;
-                *s_pick = pk;
-            }
-            __syncthreads();
-            break;
-        }
-        }
-        if (q == nullptr) {  // already drawing from p: the row has no usable mass
-            if (tid == 0) {
-                P.token[b] = -1;
-                if (P.flags) P.flags[b] = fl | DSSD_RS_FLAG_INVALID;
-            }
-            return;
-        }
-        // residual has no mass (p == q): draw from p instead
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int width = P.rows_per_sum * kSub;  // entries per stored sum
+    double *cs = P.chunk_sum + (size_t)b * P.n_sub;
+    auto sum = [&](int c) { return ld_after(cs + c); };
+    auto target = [&](double Z) { return (double)u * Z; };
+    Pick pk = pick_chunk(L, sum, false, target);
+    if (!pk.ok && !pk.late && q) {
+        // The residual has no mass (p == q): draw from p instead.  Rare, so its sums are formed here, a warp
+        // at each, where the others were.
         q = nullptr;
         fl |= DSSD_RS_FLAG_FALLBACK;
-        for (int c = 0; c < P.n_sub; ++c) {
-            const int e0 = c * kSub, e1 = min(P.V, e0 + kSub);
-            const double tot = block_sum(chunk_mass(row, nullptr, e0, e1), s_w);
-            if (tid == 0) st_relaxed_u64(cs + c, (unsigned long long)__double_as_longlong(tot));
+        __syncthreads();  // every warp has read the sums that are replaced now
+        for (int c = tid >> 5; c < P.n_sub; c += kDrawWarps) {
+            double tot = 0.0;
+            const int end = (int)min((long long)P.V, (long long)(c + 1) * width);
+            for (int e = c * width + lane; e < end; e += 32) tot += (double)row.ld(e);
+            tot = warp_sum(tot);
+            if (lane == 0) cs[c] = tot;
         }
         __syncthreads();
+        load_sums(L, P.n_sub, sum);
+        pk = pick_chunk(L, sum, false, target);
     }
-    const Pick pk = *s_pick;
-    walk_chunk<RV>(pk, P.V, row, q, fl, 0, P.token + b, P.flags ? P.flags + b : nullptr, s_w, s_i);
+    int tok = -1;
+    if (pk.ok && !pk.late) {
+        double base = pk.base;
+        bool hit = false;
+        for (int k = 0; k < P.rows_per_sum && !hit; ++k) {
+            const long long e0 = (long long)pk.chunk * width + k * kSub;
+            if (e0 >= P.V) break;
+            const int t = walk_chunk<RV>(pk, row, q, (int)e0, (int)min((long long)P.V, e0 + kSub), base, hit, sh);
+            if (t >= 0) tok = t;
+        }
+    }
+    if (tid == 0) {
+        P.token[b] = tok;
+        if (P.flags) P.flags[b] = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u) | (pk.late ? DSSD_RS_FLAG_TIMEOUT : 0u);
+    }
 }
 
+// Bound by HBM and L2: 231 MB of rows at B = 256 V = 151936 in 32 us (a quarter of p_row from L2), where the
+// persistent kernel it replaces, with tickets, a cleared scratch and the draws at its end, took 41 us
+// with them; B = 1 V = 50272: 6.5 us for both kernels against 8.9.  48 registers, so five CTAs share an SM
+// and one CTA's reduction lies under the others' loads (four: 36.1 us).
 template <typename RV>
-__global__ void __launch_bounds__(kThreads, kResampleCtas) resample_kernel(const __grid_constant__ ResampleParams P)
+__global__ void __launch_bounds__(kThreads, 5) resample_mass_kernel(const __grid_constant__ ResampleParams P)
 {
-    __shared__ double s_w[2][kWarps][2];
-    __shared__ double s_scan[kWarps];
-    __shared__ Pick s_pick;
-    __shared__ int s_i[2];
-    __shared__ unsigned long long s_ticket[2];
-    __shared__ float s_first_u;
-    __shared__ int s_first_n;
+    __shared__ double s_w[kResampleMaxTiles * kRows][kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-    // ---- the scratch is cleared here, by the kernel itself: every chunk sum to the all-ones pattern,
-    // the ticket counter to twice the number of CTAs (every CTA's first two tickets are its own
-    // number and that plus the number of CTAs), the draw counter to the number of CTAs when every
-    // sequence has a CTA of its own.  One grid-wide barrier (a cooperative launch: all CTAs are
-    // resident) separates the clearing from the first use; it is split around the first ticket's
-    // loads, which need nothing of the scratch. ----
-    namespace cg = cooperative_groups;
-    cg::grid_group grid = cg::this_grid();
-    const bool early = (unsigned long long)P.B <= (unsigned long long)gridDim.x;
-    {
-        uint4 *w = reinterpret_cast<uint4 *>(P.ticket);  // the scratch starts with the counters
-        const size_t nw = P.fill_bytes / 16;
-        for (size_t i = (size_t)blockIdx.x * kThreads + tid; i < nw; i += (size_t)gridDim.x * kThreads) {
-            uint4 v = make_uint4(~0u, ~0u, ~0u, ~0u);
-            if (i == 0) {  // raw value of a 64-bit counter: logical value - 1
-                const unsigned long long raw = 2ull * gridDim.x - 1ull;
-                v.x = (unsigned)raw;
-                v.y = (unsigned)(raw >> 32);
-            }
-            if (i == 8 && early) {  // the draw counter, 128 bytes on
-                v.x = gridDim.x - 1u;
-                v.y = 0u;
-            }
-            w[i] = v;
-        }
+    // from the last sequence backwards: when the rows were written by a kernel just before this one, the
+    // end of the array is the part most likely still in L2
+    const unsigned t = gridDim.x - 1u - blockIdx.x;
+    const int64_t b = t / (unsigned)P.n_ctas;
+    const int first = (int)(t - (unsigned)b * (unsigned)P.n_ctas) * P.tiles;  // the CTA's first tile
+    pdl_wait();
+    pdl_trigger();
+    const int n = ld_after(P.accept_len + b);
+    if (n < 0 || n > P.gamma || !selected(P, n)) return;  // the draw does not read this sequence's sums
+    const RV row = RV::make(P, b, n);
+    const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
+    const int tiles = min(P.tiles, (P.V + kTile - 1) / kTile - first);
+    for (int k = 0; k < tiles; ++k) {
+        const int e0 = (first + k) * kTile, e1 = min(P.V, e0 + kTile);
+        double acc[kRows];
+        if (q) tile_mass<true, false>(row, q, e0, e1, acc);
+        else tile_mass<false, false>(row, q, e0, e1, acc);
+        const double x = warp_sum4(acc);
+        if ((lane & 7) == 0) s_w[k * kRows + (lane >> 3)][warp] = x;
     }
-    auto arrived = grid.barrier_arrive();
-    bool waited = false;
-
-    // ---- pass A: chunk sums.  One barrier per ticket, no round trip waited for. ----
-    unsigned long long next_raw = 0;  // thread 0: the ticket after the next one, drawn early
-    // when there is at most one draw per CTA, a CTA's draw is the sequence of its own number, so
-    // that neither a ticket nor the sequence's accepted length and uniform are waited for when the
-    // draws begin (with more draws than CTAs the first ticket is taken when the draws begin, by
-    // whoever gets there first)
-    const unsigned long long my_draw = blockIdx.x;
-    int first_n = INT_MIN;  // not loaded
-    float first_u = 0.f;
-    unsigned long long t = blockIdx.x;
-    for (int it = 0; t < P.total_tickets; ++it) {
-        const int buf = it & 1;
-        // tickets run from the last sequence's last chunk backwards: when the rows were written by a
-        // kernel just before this one, the end of the array is the part most likely still in L2
-        const unsigned long long tr = P.total_tickets - 1ull - t;
-        const int64_t b = (int64_t)(tr / (unsigned)P.n_chunks);
-        const int c = (int)(tr - (unsigned long long)b * (unsigned)P.n_chunks);
-        const int n = __ldg(P.accept_len + b);
-        double acc0 = 0.0, acc1 = 0.0;  // the ticket's chunk sums
-        if (n >= 0 && n <= P.gamma && selected(P, n)) {
-            const RV row = RV::make(P, b, n);
-            const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
-            const int e0 = c * P.subs * kSub, e1 = min(P.V, e0 + kSub), e2 = min(P.V, e0 + P.subs * kSub);
-            static_assert(kSub == 4 * 4 * kThreads, "a thread's four quads per chunk sum");
-            if (kWideTickets && e2 - e0 == 2 * kSub && row.aligned(e0) && (!q || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0)) {
-                ticket_mass2(row, q, e0, acc0, acc1);
-            } else {
-                acc0 = chunk_mass(row, q, e0, e1);
-                if (e2 > e1) acc1 = chunk_mass(row, q, e1, e2);
-            }
-        }
-        acc0 = warp_sum(acc0);
-        acc1 = warp_sum(acc1);
-        if (lane == 0) {
-            s_w[buf][warp][0] = acc0;
-            s_w[buf][warp][1] = acc1;
-        }
-        if (it == 0) {  // the first ticket's loads are done: from here on the scratch is used
-            grid.barrier_wait(std::move(arrived));
-            waited = true;
-        }
-        if (tid == 0) {
-            s_ticket[buf] = it == 0 ? t + gridDim.x : logical(next_raw);
-            next_raw = atomicAdd(P.ticket, 1ull);
-            if (it == 0 && early && my_draw < (unsigned long long)P.B) {
-                first_n = __ldg(P.accept_len + ((unsigned long long)P.B - 1ull - my_draw));
-                first_u = __ldg(P.uniforms + ((unsigned long long)P.B - 1ull - my_draw));
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double tot0 = 0.0, tot1 = 0.0;
+    __syncthreads();
+    const int sums = tiles * kRows / P.rows_per_sum;
+    if (tid < sums) {
+        const int c = first * kRows / P.rows_per_sum + tid;
+        double tot = 0.0;
+        for (int k = 0; k < P.rows_per_sum; ++k) {
+            double x = 0.0;
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                tot0 += s_w[buf][w][0];
-                tot1 += s_w[buf][w][1];
-            }
-            unsigned long long *cs = reinterpret_cast<unsigned long long *>(P.chunk_sum) + (size_t)b * P.n_sub + P.subs * c;
-            if (b + 1 != (int64_t)P.test_drop_seq_plus1) {  // (the test hook withholds these stores)
-                st_relaxed_u64(cs, (unsigned long long)__double_as_longlong(tot0));
-                if (P.subs == 2 && 2 * c + 1 < P.n_sub) st_relaxed_u64(cs + 1, (unsigned long long)__double_as_longlong(tot1));
-            }
+            for (int w = 0; w < kWarps; ++w) x += s_w[tid * P.rows_per_sum + k][w];
+            tot += x;
         }
-        t = s_ticket[buf];
+        if (b + 1 == (int64_t)P.test_drop_seq_plus1) tot = __longlong_as_double((long long)kNoSum);
+        if (c < P.n_sub) P.chunk_sum[(size_t)b * P.n_sub + c] = tot;
     }
+}
 
-    // ---- pass B: the draws, one sequence per ticket, once this CTA has no chunk left.  By then
-    // the memory system is no longer saturated by the streams, so a draw's two round trips are
-    // short; a chunk sum that has not landed yet is polled for (its CTA is still running). ----
-    if (!waited) grid.barrier_wait(std::move(arrived));
-    __syncthreads();
-    if (tid == 0) {
-        s_ticket[0] = early ? my_draw : logical(atomicAdd(P.draw_ticket, 1ull));
-        s_first_n = first_n;
-        s_first_u = first_u;
-        next_raw = atomicAdd(P.draw_ticket, 1ull);
-    }
-    __syncthreads();
-    unsigned long long d = s_ticket[0];
-    const bool prefetched = s_first_n != INT_MIN;
-    for (int it = 1; d < (unsigned long long)P.B; ++it) {
-        const int buf = it & 1;
-        if (tid == 0) {
-            s_ticket[buf] = logical(next_raw);
-            next_raw = atomicAdd(P.draw_ticket, 1ull);
+// One CTA per sequence.  Bound by latency: one round trip for the sums, one for the chunk, and the float64
+// additions that depend on one another (4 us at B = 256; a chunk of 4096 entries instead of 1024 took 5.9,
+// one warp per sequence with 32 entries per lane 6.0).
+template <typename RV>
+__global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __grid_constant__ ResampleParams P)
+{
+    __shared__ WalkShared sh;
+    const int64_t b = blockIdx.x;
+    const double *cs = P.chunk_sum + (size_t)b * P.n_sub;
+    pdl_wait();
+    pdl_trigger();
+    // one round trip for all that decides where to look
+    const int n = ld_after(P.accept_len + b);
+    const float u = ld_after(P.uniforms + b);
+    LaneSums L;
+    load_sums(L, P.n_sub, [&](int c) { return ld_after(cs + c); });
+    if (n < 0 || n > P.gamma) {
+        if (threadIdx.x == 0) {
+            P.token[b] = -1;
+            if (P.flags) P.flags[b] = DSSD_RS_FLAG_INVALID;
         }
-        const int64_t b = (int64_t)P.B - 1 - (int64_t)d;  // in the order in which pass A completes the sequences
-        const int n = (it == 1 && prefetched) ? s_first_n : __ldg(P.accept_len + b);
-        const float u = (it == 1 && prefetched) ? s_first_u : __ldg(P.uniforms + b);
-        if (n < 0 || n > P.gamma) {
-            if (tid == 0) {
-                P.token[b] = -1;
-                if (P.flags) P.flags[b] = DSSD_RS_FLAG_INVALID;
-            }
-        } else if (!selected(P, n)) {
-            if (P.select == 1 && tid == 0) {  // a rejected sequence: its token comes from the device half
-                P.token[b] = -1;
-                if (P.flags) P.flags[b] = 0u;
-            }
-        } else {
-            const RV row = RV::make(P, b, n);
-            const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
-            draw<RV>(P, b, row, q, q ? 0u : DSSD_RS_FLAG_BONUS, u, s_scan, &s_pick, s_i);
+    } else if (!selected(P, n)) {
+        if (P.select == 1 && threadIdx.x == 0) {  // a rejected sequence: its token comes from the device half
+            P.token[b] = -1;
+            if (P.flags) P.flags[b] = 0u;
         }
-        __syncthreads();
-        d = s_ticket[buf];
+    } else {
+        const RV row = RV::make(P, b, n);
+        const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
+        draw<RV>(P, b, row, q, q ? 0u : DSSD_RS_FLAG_BONUS, u, L, sh);
     }
 }
 
@@ -697,42 +596,6 @@ __global__ void __launch_bounds__(kThreads, kResampleCtas) resample_kernel(const
 // dense kernel walks a row.  Plain stores and stream order connect the launches: no slot is read
 // before the launch that wrote it has ended, so the scratch needs no fill.
 
-template <typename RV>
-__device__ __forceinline__ void chunk_mass2(const RV &row, const float *q, int e0, int e1, double &acc_r, double &acc_p)
-{
-    const int tid = threadIdx.x;
-    int done = e0;
-    const bool aligned = row.aligned(e0) && (!q || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0);
-    if (aligned) {
-        const int nvec = (e1 - e0) / 4;
-        const uint4 *q4 = reinterpret_cast<const uint4 *>(q + e0);
-        for (int i = tid; i < nvec; i += 4 * kThreads) {
-            typename RV::Raw a[4];
-            uint4 c[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool in = i + u * kThreads < nvec;
-                a[u] = in ? row.ld_quad_stream(e0, i + u * kThreads) : typename RV::Raw();
-                c[u] = (in && q) ? ld_stream16(q4 + i + u * kThreads) : make_uint4(0u, 0u, 0u, 0u);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (i + u * kThreads >= nvec) continue;
-                const float4 x = row.quad(a[u]), y = as_f4(c[u]);
-                acc_p += ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-                if (q) acc_r += (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
-            }
-        }
-        done = e0 + nvec * 4;
-    }
-    for (int e = done + tid; e < e1; e += kThreads) {
-        const float pv = row.ld(e);
-        acc_p += (double)pv;
-        if (q) acc_r += res(pv, __ldg(q + e));
-    }
-    if (!q) acc_r = acc_p;
-}
-
 __device__ __forceinline__ RowF32 shard_row(const ShardResampleParams &P, int64_t b)
 {
     RowF32 r;
@@ -740,43 +603,38 @@ __device__ __forceinline__ RowF32 shard_row(const ShardResampleParams &P, int64_
     return r;
 }
 
-__global__ void __launch_bounds__(kThreads, kResampleCtas) shard_mass_kernel(const __grid_constant__ ShardResampleParams P)
+__global__ void __launch_bounds__(kThreads, 4) shard_mass_kernel(const __grid_constant__ ShardResampleParams P)
 {
-    __shared__ double s_w[kWarps][2];
+    __shared__ double s_w[2 * kRows][kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long total = (long long)P.B * P.n_sub;
-    for (long long t = blockIdx.x; t < total; t += gridDim.x) {
-        const int64_t b = t / P.n_sub;
-        const int c = (int)(t - b * P.n_sub);
-        const int n = __ldg(P.accept_len + b);
-        double acc_r = 0.0, acc_p = 0.0;
-        const bool valid = n >= 0 && n <= P.gamma;
-        if (valid) {
-            const RowF32 row = shard_row(P, b);
-            const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
-            const int e0 = c * kSub, e1 = min(P.V, e0 + kSub);
-            chunk_mass2(row, q, e0, e1, acc_r, acc_p);
-        }
-        acc_r = warp_sum(acc_r);
-        acc_p = warp_sum(acc_p);
-        __syncthreads();  // the previous ticket's sums have been read
-        if (lane == 0) {
-            s_w[warp][0] = acc_r;
-            s_w[warp][1] = acc_p;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double tr = 0.0, tp = 0.0;
+    const unsigned n_tiles = (unsigned)((P.V + kTile - 1) / kTile);
+    const int64_t b = blockIdx.x / n_tiles;
+    const int tile = (int)(blockIdx.x - (unsigned)b * n_tiles);
+    pdl_wait();
+    pdl_trigger();
+    const int n = ld_after(P.accept_len + b);
+    const bool valid = n >= 0 && n <= P.gamma;
+    double acc_r[kRows] = {}, acc_p[kRows] = {};
+    if (valid) {
+        const RowF32 row = shard_row(P, b);
+        const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
+        const int e0 = tile * kTile, e1 = min(P.V, e0 + kTile);
+        if (q) tile_mass<true, true>(row, q, e0, e1, acc_r, acc_p);
+        else tile_mass<false, true>(row, q, e0, e1, acc_r, acc_p);
+    }
+    const double r = warp_sum4(acc_r), p = warp_sum4(acc_p);
+    if ((lane & 7) == 0) {
+        s_w[2 * (lane >> 3)][warp] = r;
+        s_w[2 * (lane >> 3) + 1][warp] = p;
+    }
+    __syncthreads();
+    if (tid < 2 * kRows) {
+        const int c = tile * kRows + tid / 2;
+        double tot = 0.0;
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                tr += s_w[w][0];
-                tp += s_w[w][1];
-            }
-            const double nan = __longlong_as_double(0x7ff8000000000000ll);
-            double *cs = P.chunk_sum + ((size_t)b * P.n_sub + c) * 2;
-            cs[0] = valid ? tr : nan;
-            cs[1] = valid ? tp : nan;
-        }
+        for (int w = 0; w < kWarps; ++w) tot += s_w[tid][w];
+        if (!valid) tot = __longlong_as_double(0x7ff8000000000000ll);
+        if (c < P.n_sub) P.chunk_sum[((size_t)b * P.n_sub + c) * 2 + (tid & 1)] = tot;
     }
 }
 
@@ -785,12 +643,14 @@ __global__ void __launch_bounds__(kThreads) shard_total_kernel(const __grid_cons
 {
     const int lane = threadIdx.x & 31;
     const long long b = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    pdl_wait();
+    pdl_trigger();
     if (b >= P.B) return;
     const double *cs = P.chunk_sum + (size_t)b * P.n_sub * 2;
     double r = 0.0, p = 0.0;
     for (int c = lane; c < P.n_sub; c += 32) {
-        r += cs[2 * c];
-        p += cs[2 * c + 1];
+        r += ld_after(cs + 2 * c);
+        p += ld_after(cs + 2 * c + 1);
     }
     r = warp_sum(r);
     p = warp_sum(p);
@@ -800,226 +660,137 @@ __global__ void __launch_bounds__(kThreads) shard_total_kernel(const __grid_cons
     }
 }
 
-__global__ void __launch_bounds__(kThreads) shard_draw_kernel(const __grid_constant__ ShardResampleParams P)
+// one CTA per sequence
+__global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_constant__ ShardResampleParams P)
 {
-    __shared__ double s_scan[kWarps];
-    __shared__ Pick s_pick;
-    __shared__ int s_i[2];
-    const int tid = threadIdx.x;
+    __shared__ WalkShared sh;
     const int64_t b = blockIdx.x;
-    const int n = __ldg(P.accept_len + b);
-    int32_t *token_out = P.token + b;
-    uint32_t *flags_out = P.flags ? P.flags + b : nullptr;
-    if (n < 0 || n > P.gamma) {
-        if (tid == 0) {
-            *token_out = -1;
-            if (flags_out) *flags_out = DSSD_RS_FLAG_INVALID;
+    pdl_wait();
+    pdl_trigger();
+    const int n = ld_after(P.accept_len + b);
+    const float u = ld_after(P.uniforms + b);
+    int tok = -1;
+    unsigned fl = DSSD_RS_FLAG_INVALID;
+    if (n >= 0 && n <= P.gamma) {
+        // The verdict on the sequence, from all shards' masses: every thread of every shard takes the
+        // same steps in the same order.
+        fl = n == P.gamma ? DSSD_RS_FLAG_BONUS : 0u;
+        const double *masses = P.masses + 2 * b;
+        const size_t step = 2 * (size_t)P.B;  // between shards
+        int col = 0;
+        double Z = 0.0;
+        for (int h = 0; h < P.G; ++h) Z += ld_after(masses + h * step);
+        bool ok = (Z > 0.0) && (Z < INFINITY);
+        if (!ok && n < P.gamma) {  // no residual mass anywhere: draw from p instead
+            fl |= DSSD_RS_FLAG_FALLBACK;
+            col = 1;
+            Z = 0.0;
+            for (int h = 0; h < P.G; ++h) Z += ld_after(masses + h * step + 1);
+            ok = (Z > 0.0) && (Z < INFINITY);
         }
-        return;
-    }
-    // The verdict on the sequence, from all shards' masses: every thread of every shard takes the
-    // same steps in the same order.
-    unsigned fl = n == P.gamma ? DSSD_RS_FLAG_BONUS : 0u;
-    int col = 0;
-    double Z = 0.0;
-    for (int h = 0; h < P.G; ++h) Z += __ldg(P.masses + ((size_t)h * P.B + b) * 2);
-    bool ok = (Z > 0.0) && (Z < INFINITY);
-    if (!ok && n < P.gamma) {  // no residual mass anywhere: draw from p instead
-        fl |= DSSD_RS_FLAG_FALLBACK;
-        col = 1;
-        Z = 0.0;
-        for (int h = 0; h < P.G; ++h) Z += __ldg(P.masses + ((size_t)h * P.B + b) * 2 + 1);
-        ok = (Z > 0.0) && (Z < INFINITY);
-    }
-    if (!ok) {
-        if (tid == 0) {
-            *token_out = -1;
-            if (flags_out) *flags_out = fl | DSSD_RS_FLAG_INVALID;
+        const double t = (double)u * Z;
+        double C = 0.0, before = 0.0;
+        int owner = -1, last_mass = -1;
+        for (int h = 0; h < P.G; ++h) {
+            const double m = ld_after(masses + h * step + col);
+            if (m > 0.0) last_mass = h;
+            if (owner < 0 && C + m > t) {
+                owner = h;
+                before = C;
+            }
+            C += m;
         }
-        return;
-    }
-    const double t = (double)__ldg(P.uniforms + b) * Z;
-    double C = 0.0, before = 0.0;
-    int owner = -1, last_mass = -1;
-    for (int h = 0; h < P.G; ++h) {
-        const double m = __ldg(P.masses + ((size_t)h * P.B + b) * 2 + col);
-        if (m > 0.0) last_mass = h;
-        if (owner < 0 && C + m > t) {
-            owner = h;
-            before = C;
+        const bool beyond = owner < 0;  // rounding left no shard above t: the last shard with mass, its last positive entry
+        if (beyond) owner = last_mass;
+        if (!ok) {
+            fl |= DSSD_RS_FLAG_INVALID;
+        } else if (owner == P.g) {
+            // this shard holds the target: the chunk first, then the walk inside it
+            const double *cs = P.chunk_sum + (size_t)b * P.n_sub * 2 + col;
+            auto sum = [&](int c) { return ld_after(cs + 2 * c); };
+            LaneSums L;
+            load_sums(L, P.n_sub, sum);
+            const Pick pk = pick_chunk(L, sum, beyond, [&](double) { return t - before; });
+            const RowF32 row = shard_row(P, b);
+            const float *q = (col == 0 && n < P.gamma) ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
+            double base = pk.base;
+            bool hit;
+            tok = walk_chunk<RowF32>(pk, row, q, pk.chunk * kSub, min(P.V, pk.chunk * kSub + kSub), base, hit, sh);
+            if (tok < 0) fl |= DSSD_RS_FLAG_INVALID;
+            else tok += P.v_begin;
         }
-        C += m;
     }
-    const bool beyond = owner < 0;  // rounding left no shard above t: the last shard with mass, its last positive entry
-    if (beyond) owner = last_mass;
-    if (owner != P.g) {
-        if (tid == 0) {
-            *token_out = -1;
-            if (flags_out) *flags_out = fl;
-        }
-        return;
+    if (threadIdx.x == 0) {
+        P.token[b] = tok;
+        if (P.flags) P.flags[b] = fl;
     }
-    // this shard holds the target: the chunk first, then the walk inside it
-    const double target = t - before;
-    const double *cs = P.chunk_sum + (size_t)b * P.n_sub * 2 + col;
-    if (tid == 0) {
-        s_i[0] = 0x7fffffff;
-        s_i[1] = -1;
-    }
-    __syncthreads();
-    double carry = 0.0, my_base_first = 0.0, my_base_last = 0.0;
-    int my_first = 0x7fffffff, my_last = -1;
-    for (int base = 0; base < P.n_sub; base += kThreads) {
-        const int c = base + tid;
-        const double m = c < P.n_sub ? cs[2 * c] : 0.0;
-        double tot;
-        const double incl = carry + block_scan(m, s_scan, tot);
-        if (!beyond && c < P.n_sub && incl > target && my_first == 0x7fffffff) {
-            my_first = c;
-            my_base_first = incl - m;
-        }
-        if (c < P.n_sub && m > 0.0) {
-            my_last = c;
-            my_base_last = incl - m;
-        }
-        carry += tot;
-        __syncthreads();
-    }
-    if (my_first != 0x7fffffff) atomicMin(&s_i[0], my_first);
-    if (my_last >= 0) atomicMax(&s_i[1], my_last);
-    __syncthreads();
-    const int first = s_i[0], last = s_i[1];
-    if (first == 0x7fffffff && last < 0) {  // cannot happen while this shard's mass is positive
-        if (tid == 0) {
-            *token_out = -1;
-            if (flags_out) *flags_out = fl | DSSD_RS_FLAG_INVALID;
-        }
-        return;
-    }
-    if (first != 0x7fffffff ? (my_first == first) : (my_last == last)) {
-        Pick pk;
-        pk.ok = 1;
-        pk.beyond = first == 0x7fffffff;
-        pk.chunk = pk.beyond ? last : first;
-        pk.base = pk.beyond ? my_base_last : my_base_first;
-        pk.target = target;
-        s_pick = pk;
-    }
-    __syncthreads();
-    const Pick pk = s_pick;
-    const RowF32 row = shard_row(P, b);
-    const float *q = (col == 0 && n < P.gamma) ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
-    walk_chunk<RowF32>(pk, P.V, row, q, fl, P.v_begin, token_out, flags_out, s_scan, s_i);
 }
-
 
 }  // namespace
 
 size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base)
 {
-    // the kernel sets all of it to 0xFF before use: counters then read "logical 0" (raw + 1) and
-    // the chunk sums read "not yet"
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        size_t o = off;
-        off += (bytes + 255) & ~(size_t)255;
-        return o;
-    };
-    const size_t o_ticket = take(256);  // the two ticket counters, on separate 128-byte lines
-    const int n_sub = (V + kResampleSub - 1) / kResampleSub;
-    const size_t o_sum = take((size_t)B * (size_t)n_sub * sizeof(double));
+    // one sum per chunk; batches whose sums would take more than the built-in scratch of
+    // dssd_device_resample_static keep one per tile, whose chunks the draw then looks at in turn
+    const size_t chunks = ((size_t)V + kSub - 1) / kSub, tiles = ((size_t)V + kTile - 1) / kTile;
+    const bool fine = (size_t)B * chunks * sizeof(double) <= (size_t)DSSD_STATIC_SCRATCH_BYTES;
+    const size_t n_sub = fine ? chunks : tiles;
     if (P) {
-        P->ticket = reinterpret_cast<unsigned long long *>(base + o_ticket);
-        P->draw_ticket = reinterpret_cast<unsigned long long *>(base + o_ticket + 128);
-        P->chunk_sum = reinterpret_cast<double *>(base + o_sum);
-        P->fill_bytes = off;
-        if (P->subs != 1) P->subs = 2;
-        P->n_chunks = (n_sub + P->subs - 1) / P->subs;
-        P->n_sub = n_sub;
-        P->total_tickets = (unsigned long long)B * (unsigned long long)P->n_chunks;
+        P->chunk_sum = reinterpret_cast<double *>(base);
+        P->n_sub = (int)n_sub;
+        P->rows_per_sum = fine ? 1 : kRows;
     }
-    return off;
+    return ((size_t)B * n_sub * sizeof(double) + 255) & ~(size_t)255;
 }
 
-// resident CTAs per device, looked up on the first launch made with that device current (the
-// occupancy depends on the compiled kernels only); 0: not looked up yet
-static std::atomic<int> g_resample_resident[64];  // published last (release), read first (acquire)
-static std::atomic<int> g_resample_sms[64];
+namespace {
+
+template <typename RV>
+cudaError_t launch_resample(const ResampleParams &P, unsigned grid, cudaStream_t stream)
+{
+    const cudaError_t e = launch_pdl(resample_mass_kernel<RV>, grid, kThreads, stream, P);
+    return e != cudaSuccess ? e : launch_pdl(resample_draw_kernel<RV>, (unsigned)P.B, kDrawThreads, stream, P);
+}
+
+}  // namespace
 
 cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t stream)
 {
-    cudaError_t err;
-    int dev = 0, sms = 0, occ = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    occ = g_resample_resident[dev].load(std::memory_order_acquire);
-    if (occ == 0) {
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
-        int o[4] = {0, 0, 0, 0};
-        if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[0], resample_kernel<RowF32>, kThreads, 0)) != cudaSuccess) return err;
-        if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[1], resample_kernel<RowF16>, kThreads, 0)) != cudaSuccess) return err;
-        if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[2], resample_kernel<RowLogits<DSSD_F32>>, kThreads, 0)) != cudaSuccess) return err;
-        if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[3], resample_kernel<RowLogits<DSSD_BF16>>, kThreads, 0)) != cudaSuccess) return err;
-        occ = o[0];
-        for (int i = 1; i < 4; ++i) occ = o[i] < occ ? o[i] : occ;
-        if (occ < 1) occ = 1;
-        g_resample_sms[dev].store(sms, std::memory_order_relaxed);
-        g_resample_resident[dev].store(occ, std::memory_order_release);  // a concurrent first call finds either 0 or the final pair
-    }
-    sms = g_resample_sms[dev].load(std::memory_order_relaxed);
-    // two chunk sums per ticket halve the barriers; one per ticket evens out the CTAs' shares when
-    // there are only a few tickets for each
-    {
-        const unsigned long long pairs = (unsigned long long)P.B * (unsigned long long)(((P.V + kResampleSub - 1) / kResampleSub + 1) / 2);
-        P.subs = pairs < 4ull * (unsigned long long)sms * (unsigned long long)occ ? 1 : 2;
-    }
     resample_workspace_layout(P.B, P.V, &P, static_cast<char *>(workspace));
-    P.spin_limit = 1u << 20;
-    const unsigned long long resident = (unsigned long long)sms * (unsigned long long)occ;
-    const unsigned grid = (unsigned)(P.total_tickets < resident ? P.total_tickets : resident);
-    // a cooperative launch: all CTAs are resident at once (grid <= resident), which the kernel's
-    // grid-wide barrier after the clearing of the scratch relies on
-    const void *fn;
+    const unsigned long long n_tiles = ((unsigned long long)P.V + kTile - 1) / kTile;
+    const unsigned long long total = (unsigned long long)P.B * n_tiles;
+    P.tiles = total < kTwoTiles ? 1 : total < kFourTiles ? 2 : kResampleMaxTiles;
+    P.n_ctas = (int)((n_tiles + P.tiles - 1) / P.tiles);
+    const unsigned long long grid = (unsigned long long)P.B * (unsigned long long)P.n_ctas;
+    if (grid > 0x7fffffffull) return cudaErrorInvalidConfiguration;
     if (P.logits) {
-        fn = P.logits_dtype == DSSD_BF16 ? reinterpret_cast<const void *>(resample_kernel<RowLogits<DSSD_BF16>>)
-                                         : reinterpret_cast<const void *>(resample_kernel<RowLogits<DSSD_F32>>);
-    } else if (P.p_half) {
-        fn = reinterpret_cast<const void *>(resample_kernel<RowF16>);
-    } else {
-        fn = reinterpret_cast<const void *>(resample_kernel<RowF32>);
+        return P.logits_dtype == DSSD_BF16 ? launch_resample<RowLogits<DSSD_BF16>>(P, (unsigned)grid, stream)
+                                           : launch_resample<RowLogits<DSSD_F32>>(P, (unsigned)grid, stream);
     }
-    void *args[] = {&P};
-    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kThreads), args, 0, stream);
+    return P.p_half ? launch_resample<RowF16>(P, (unsigned)grid, stream) : launch_resample<RowF32>(P, (unsigned)grid, stream);
 }
 
 size_t shard_resample_workspace_bytes(int B, int V)
 {
-    const size_t n_sub = (size_t)((V + kResampleSub - 1) / kResampleSub);
+    const size_t n_sub = ((size_t)V + kSub - 1) / kSub;
     return (((size_t)B * n_sub * 2 * sizeof(double)) + 255) & ~(size_t)255;
 }
 
 cudaError_t shard_mass_launch(ShardResampleParams &P, void *workspace, cudaStream_t stream)
 {
-    cudaError_t err;
-    int dev = 0, sms = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
-    P.n_sub = (P.V + kResampleSub - 1) / kResampleSub;
+    P.n_sub = (int)(((size_t)P.V + kSub - 1) / kSub);
     P.chunk_sum = static_cast<double *>(workspace);
-    const long long total = (long long)P.B * P.n_sub;
-    const long long resident = (long long)(sms < 1 ? 1 : sms) * kResampleCtas;
-    shard_mass_kernel<<<(unsigned)(total < resident ? total : resident), kThreads, 0, stream>>>(P);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    shard_total_kernel<<<(unsigned)((P.B + kWarps - 1) / kWarps), kThreads, 0, stream>>>(P);
-    return cudaGetLastError();
+    const unsigned long long grid = (unsigned long long)P.B * (((unsigned long long)P.V + kTile - 1) / kTile);
+    if (grid > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+    const cudaError_t e = launch_pdl(shard_mass_kernel, (unsigned)grid, kThreads, stream, P);
+    return e != cudaSuccess ? e : launch_pdl(shard_total_kernel, (unsigned)((P.B + kWarps - 1) / kWarps), kThreads, stream, P);
 }
 
 cudaError_t shard_draw_launch(ShardResampleParams &P, const void *workspace, cudaStream_t stream)
 {
-    P.n_sub = (P.V + kResampleSub - 1) / kResampleSub;
+    P.n_sub = (int)(((size_t)P.V + kSub - 1) / kSub);
     P.chunk_sum = const_cast<double *>(static_cast<const double *>(workspace));
-    shard_draw_kernel<<<(unsigned)P.B, kThreads, 0, stream>>>(P);
-    return cudaGetLastError();
+    return launch_pdl(shard_draw_kernel, (unsigned)P.B, kDrawThreads, stream, P);
 }
 
 }  // namespace dssd
@@ -1084,8 +855,8 @@ extern "C" dssd_status dssd_device_resample_static(const float *p_row, const flo
     P.V = V;
     P.token = token;
     P.flags = flags;
-    // resample_launch refills the part of the scratch it uses (counters and validity patterns),
-    // so what the previous call left behind does not matter
+    // every sum that the draw reads has been written by the same call, so what the previous call left
+    // behind does not matter
     e = dssd::resample_launch(P, scratch, static_cast<cudaStream_t>(cuda_stream));
     if (e != cudaSuccess) {
         dssd::set_last_cuda_error((int)e);

@@ -7,7 +7,8 @@
 
 namespace dssd {
 
-constexpr int kResampleSub = 4096;  // vocabulary entries per chunk sum; a ticket covers one or two of them
+constexpr int kResampleSub = 1024;    // vocabulary entries per chunk sum
+constexpr int kResampleMaxTiles = 4;  // most tiles (of four chunks) per CTA of the mass kernel
 
 struct ResampleParams {
     const void *p_row;   // float32 entries, or IEEE binary16 bit patterns when p_half is set
@@ -29,23 +30,16 @@ struct ResampleParams {
     int select;
     int32_t *token;
     uint32_t *flags;
-    int subs;       // chunk sums per ticket: 2, or 1 when there are few tickets per resident CTA
-    int n_chunks;   // tickets per sequence (subs * kResampleSub entries each)
-    int n_sub;      // chunk sums per sequence
-    unsigned long long total_tickets;
-    // scratch
-    unsigned long long *ticket;       // next chunk ticket
-    unsigned long long *draw_ticket;  // next sequence to draw
-    double *chunk_sum;   // [B, n_sub]
-    size_t fill_bytes;
-    unsigned spin_limit;
-    // test hook (0: off): the chunk sums of sequence test_drop_seq_plus1 - 1 are never stored, and its
-    // draw polls at most test_poll_limit times for a chunk sum
+    int tiles;         // tiles per CTA of the mass kernel
+    int n_ctas;        // such CTAs per sequence
+    int rows_per_sum;  // chunks per stored sum: 1, or 4 (a whole tile) in the largest batches
+    int n_sub;         // stored sums per sequence
+    double *chunk_sum;   // scratch [B, n_sub]
+    // test hook (0: off): the chunk sums of sequence test_drop_seq_plus1 - 1 are formed but never stored
     int test_drop_seq_plus1;
-    unsigned test_poll_limit;
 };
 
-// Carves the scratch (its size does not depend on P->subs, which the caller sets before: 1 or 2).
+// Carves the scratch; returns the bytes needed.  With P == nullptr only computes the size.
 size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base);
 
 cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t stream);

@@ -25,6 +25,14 @@ __device__ __forceinline__ uint4 ld_stream16(const void *p)
     return v;
 }
 
+// the same, 8 bytes
+__device__ __forceinline__ uint2 ld_stream8(const void *p)
+{
+    uint2 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+
 // two floats rounded to IEEE binary16 (nearest even), low half = first
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
 {
@@ -78,6 +86,33 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
 __device__ __forceinline__ void st_release(unsigned *p, unsigned v)
 {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// ---- programmatic dependent launch (see launch.h) -----------------------------------------------
+
+// everything the kernels before this one wrote is visible after it
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// the next kernel's CTAs may be scheduled once every CTA of this one has said so (or has ended)
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Scalar loads that stay behind pdl_wait() (a plain __ldg may be moved across it), served by L2.
+__device__ __forceinline__ uint32_t ld_after_u32(const void *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ld_after(const int32_t *p) { return (int)ld_after_u32(p); }
+__device__ __forceinline__ float ld_after(const float *p) { return __uint_as_float(ld_after_u32(p)); }
+__device__ __forceinline__ unsigned long long ld_after(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_after(const double *p)
+{
+    return __longlong_as_double((long long)ld_after(reinterpret_cast<const unsigned long long *>(p)));
 }
 
 // ---- shared-memory barriers and bulk asynchronous copies (TMA, untiled form) ------------------
@@ -240,7 +275,9 @@ struct Elem<DSSD_F32> {
     static constexpr int kVec = 4;   // elements per 16-byte vector
     __device__ static __forceinline__ float load(const void *row, int64_t i)
     {
-        return __ldg(reinterpret_cast<const float *>(row) + i);
+        float f;
+        asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(f) : "l"(reinterpret_cast<const float *>(row) + i));
+        return f;
     }
     __device__ static __forceinline__ void unpack(const uint4 &v, float *f)
     {
@@ -256,8 +293,9 @@ struct Elem<DSSD_BF16> {
     static constexpr int kVec = 8;
     __device__ static __forceinline__ float load(const void *row, int64_t i)
     {
-        uint32_t h = __ldg(reinterpret_cast<const unsigned short *>(row) + i);
-        return __uint_as_float(h << 16);
+        unsigned short h;
+        asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(h) : "l"(reinterpret_cast<const unsigned short *>(row) + i));
+        return __uint_as_float((uint32_t)h << 16);
     }
     __device__ static __forceinline__ void unpack(const uint4 &v, float *f)
     {

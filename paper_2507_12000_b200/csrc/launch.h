@@ -1,0 +1,30 @@
+// Launches with programmatic dependent launch (internal to the library).
+//
+// Every call of the library is a short chain of kernels on the caller's stream.  Each is launched
+// with the programmatic-stream-serialization attribute: its CTAs may be scheduled while the kernel
+// before it drains, and they wait (griddepcontrol.wait) before they read or write any global memory.
+// The order stays transitive because every kernel launched this way waits before it lets the next
+// one in (griddepcontrol.launch_dependents) and before it ends: a kernel has completed only after
+// the one before it has.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace dssd {
+
+template <class Params>
+cudaError_t launch_pdl(void (*kernel)(Params), unsigned grid, unsigned block, cudaStream_t stream, const Params &params)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, params);
+}
+
+}  // namespace dssd

@@ -1,0 +1,51 @@
+"""The dense draw where its geometry can go wrong: vocabularies at the edges of a chunk (1024 entries) and of
+a tile (4096), batches at the thresholds of tiles per CTA, more chunks than a warp's lanes keep in
+registers, one sum per tile instead of per chunk, aligned and unaligned rows, both payloads; uniforms at
+both ends of their range and rows whose mass sits in single entries."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_12000_b200 import binding
+
+    return binding
+
+
+@pytest.mark.parametrize("Bn,gamma,V,half", [
+    (5, 2, 1, False), (5, 2, 1023, False), (5, 2, 1024, True), (5, 1, 1025, False), (5, 3, 4095, True),
+    (5, 2, 4096, False), (5, 2, 4097, False), (7, 1, 4100, True), (3, 1, 8192, False), (3, 1, 12289, False),
+    (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
+    (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True),
+])
+def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
+    gen = torch.Generator(device="cuda").manual_seed(Bn + V)
+    p = torch.softmax(2.0 * torch.randn(Bn, V, generator=gen, device="cuda"), dim=-1)
+    q = torch.softmax(2.0 * torch.randn(Bn, gamma, V, generator=gen, device="cuda"), dim=-1)
+    if V > 1:
+        p[0] = 0.0
+        p[0, V - 1] = 1.0          # all mass in the last entry
+        p[1] = 0.0
+        p[1, V // 2] = 0.5         # two entries, the draw falls on the second with u = 1/2
+        p[1, V - 1] = 0.5
+    n = (torch.arange(Bn, device="cuda") % (gamma + 1)).to(torch.int32)
+    n[1] = gamma                   # bonus draws, where r = p
+    u = torch.randint(0, 1 << 24, (Bn,), generator=gen, device="cuda").to(torch.float32) * 2.0 ** -24
+    u[1] = 0.5
+    u[2 % Bn] = 0.0
+    u[-1] = 1.0 - 2.0 ** -24
+    if half:
+        p = p.to(torch.float16)
+    out = B.dssd_device_resample(p, q, n, u, gamma)
+    torch.cuda.synchronize()
+    ref = oracle_mod.device_resample(p.float().cpu().numpy(), q.cpu().numpy(), n.cpu().numpy(), u.cpu().numpy(), gamma,
+                                     threads=8)
+    tok = out["token"].cpu().numpy()
+    # both sides add V float64 terms, in different orders: V * 2^-53 relative each
+    bad = (tok != ref["token"]) & ~(ref["margin_cdf"] < V * 2.0 ** -52)
+    assert not bad.any(), (np.nonzero(bad)[0][:8], tok[bad][:8], ref["token"][bad][:8])
+    assert (out["flags"].cpu().numpy().astype(np.uint32) == ref["flags"]).all()
