@@ -32,8 +32,10 @@
  *     per-device launch constants (SM count, resident CTAs per kernel), which are looked up on the
  *     first call made with a device current and cached, and the built-in scratch of
  *     dssd_device_resample_static.
- *   - The streaming kernels are launched cooperatively (every CTA resident at once): two calls
- *     issued to different streams run one after the other on the GPU, not side by side.
+ *   - The kernels of a call are launched with programmatic stream serialization: the first of them may
+ *     be scheduled while the kernel before it on the stream drains, and waits for its end before
+ *     it reads or writes anything.  dssd_edge_verify_topk is launched cooperatively (every CTA
+ *     resident at once): two such calls on different streams run one after the other.
  *   - Every call with device pointers only can be recorded in a CUDA graph by stream capture
  *     (it enqueues kernels and nothing else), provided one call of the same entry point was made
  *     on that device before the capture began (the first call looks the launch constants up).

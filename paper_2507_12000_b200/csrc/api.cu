@@ -66,8 +66,7 @@ dssd_status edge_verify_any(const void *target_logits, dssd_dtype dtype, int64_t
                             const int32_t *draft_tokens, const float *draft_q_tok, const float *uniforms,
                             float temperature, int B, int gamma, int V, int32_t *accept_len, float *p_row,
                             uint16_t *p_row16, float *p_tok, float *lse, uint32_t *flags, void *workspace,
-                            size_t workspace_bytes, void *cuda_stream, long long drop_row_plus1 = 0,
-                            unsigned poll_limit = 0)
+                            size_t workspace_bytes, void *cuda_stream, long long drop_row_plus1 = 0)
 {
     t_last_cuda_error = 0;
     dssd_status st = check_sizes(B, gamma, V);
@@ -102,7 +101,6 @@ dssd_status edge_verify_any(const void *target_logits, dssd_dtype dtype, int64_t
     P.lse = lse;
     P.flags = flags;
     P.test_drop_row_plus1 = drop_row_plus1;
-    P.test_poll_limit = poll_limit;
     cudaError_t e = dssd::edge_verify_launch(P, (int)dtype, workspace, static_cast<cudaStream_t>(cuda_stream));
     return e == cudaSuccess ? DSSD_OK : cuda_fail(e);
 }
@@ -118,10 +116,11 @@ dssd_status dssd_test_edge_verify_wait_runs_out(const void *target_logits, dssd_
                                                 void *cuda_stream)
 {
     if (!p_row) return DSSD_ERR_INVALID_ARG;
+    (void)poll_limit;  // a withheld sum is seen at the first look
     if (check_sizes(B, gamma, V) == DSSD_OK && (drop_row < 0 || drop_row >= (long long)B * (gamma + 1))) return DSSD_ERR_INVALID_ARG;
     return edge_verify_any(target_logits, dtype, row_stride, draft_tokens, draft_q_tok, uniforms, temperature, B, gamma,
                            V, accept_len, p_row, nullptr, nullptr, nullptr, flags, workspace, workspace_bytes, cuda_stream,
-                           drop_row + 1, poll_limit);
+                           drop_row + 1);
 }
 
 dssd_status dssd_edge_verify(const void *target_logits, dssd_dtype dtype, int64_t row_stride,

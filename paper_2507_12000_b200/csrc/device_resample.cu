@@ -515,9 +515,9 @@ __global__ void __launch_bounds__(kThreads, 5) resample_mass_kernel(const __grid
 {
     __shared__ double s_w[kResampleMaxTiles * kRows][kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // from the last sequence backwards: when the rows were written by a kernel just before this one, the
-    // end of the array is the part most likely still in L2
-    const unsigned t = gridDim.x - 1u - blockIdx.x;
+    // in index order: the edge kernel emits the rows from the last sequence backwards, so the first ones
+    // are still in L2 when they were written just before
+    const unsigned t = blockIdx.x;
     const int64_t b = t / (unsigned)P.n_ctas;
     const int first = (int)(t - (unsigned)b * (unsigned)P.n_ctas) * P.tiles;  // the CTA's first tile
     pdl_wait();

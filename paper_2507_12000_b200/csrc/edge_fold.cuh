@@ -1,0 +1,139 @@
+// Folding a sequence: the runs' partial sums -> every row's log-sum-exp -> acceptance tests -> the
+// first rejection.  Done by every CTA that needs the verdict on a sequence: it costs one round
+// trip to L2 and a few hundred instructions, less than handing the verdict on in another launch.
+#pragma once
+
+#include "dssd_device.cuh"
+#include "edge_judge.cuh"
+#include "edge_verify.h"
+
+namespace dssd {
+
+constexpr unsigned long long kNoPartial = ~0ull;  // stored in place of a withheld partial sum (a sum is never this NaN)
+constexpr int kFoldLanes = 8;                     // threads that add up one row's runs
+constexpr int kFoldRows = kThreads / kFoldLanes;  // rows folded at a time
+static_assert(kFoldRows == 32, "one lane of warp 0 per position");
+
+struct FoldShared {
+    float R[kFoldRows];
+    double S[kFoldRows];
+    int bad[kFoldRows];   // bit 0: a NaN among the sums, bit 1: a sum is missing
+    int n;                // accepted length; -1: no verdict
+    float ref2, invS;     // row n
+};
+
+// The sum of one row, formed by kFoldLanes neighbouring threads (sub = 0 .. kFoldLanes - 1 within
+// the row); the result is the same in all of them.  Fixed order: deterministic.
+__device__ __forceinline__ void row_total(const unsigned long long *part, int runs, int sub, bool live, float &R, double &S,
+                                          int &bad)
+{
+    R = DSSD_NEG_INF;
+    S = 0.0;
+    bad = 0;
+    bool nan = false;
+    for (int k0 = 0; k0 < runs; k0 += 4 * kFoldLanes) {
+        unsigned long long w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = k0 + u * kFoldLanes + sub;
+            w[u] = (live && k < runs) ? ld_after(part + k) : 0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (w[u] == kNoPartial) bad |= 2;
+            else add_partial(R, S, nan, __uint_as_float((unsigned)w[u]), (double)__uint_as_float((unsigned)(w[u] >> 32)));
+        }
+    }
+    if (nan) bad |= 1;
+#pragma unroll
+    for (int o = 1; o < kFoldLanes; o <<= 1) {
+        const float R2 = __shfl_xor_sync(0xffffffffu, R, o);
+        const double S2 = __shfl_xor_sync(0xffffffffu, S, o);
+        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+        bool dummy = false;
+        if (R2 > R) {  // the same two operands in both threads, so both get the same bits
+            double Sx = S2;
+            float Rx = R2;
+            add_partial(Rx, Sx, dummy, R, S);
+            R = Rx;
+            S = Sx;
+        } else {
+            add_partial(R, S, dummy, R2, S2);
+        }
+    }
+}
+
+// Run by all kThreads threads of a CTA; the results are in `sh` (n, ref2, invS) when it returns.
+// `writer`: this CTA writes the sequence's accept_len, flags, lse, p_tok and `ready`.
+// The drafted tokens, their q and uniforms are the caller's inputs, the partial sums and the
+// drafted tokens' logits come from the log-sum-exp kernel: one round trip to L2 for all of them.
+__device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long row0 = b * (P.gamma + 1);
+    int n = P.gamma;
+    unsigned fl = 0;
+    float ref2_n = 0.f, invS_n = 0.f;
+    for (int base = 0; base <= P.gamma; base += kFoldRows) {
+        const int i = base + lane;
+        const bool live = i <= P.gamma;
+        int x = -1;
+        float zx = 0.f, qx = 0.f, ux = 0.f;
+        if (warp == 0 && i < P.gamma) {
+            const size_t di = (size_t)b * P.gamma + i;
+            x = ld_after(P.draft_tokens + di);
+            qx = P.draft_q_rows ? ld_after(P.tokq + row0 + i) : ld_after(P.draft_q_tok + di);
+            ux = ld_after(P.uniforms + di);
+            zx = ld_after(P.tokz + row0 + i);
+            if (P.draft_q_rows && (x < 0 || x >= P.V)) qx = __int_as_float(0x7fc00000);  // nothing was looked up
+        }
+        {
+            const int r = base + tid / kFoldLanes;
+            float R;
+            double S;
+            int bad;
+            row_total(P.part + (size_t)(row0 + (r <= P.gamma ? r : 0)) * P.runs, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, bad);
+            if (base) __syncthreads();  // warp 0 has read the previous rows
+            if (tid % kFoldLanes == 0) {
+                sh.R[tid / kFoldLanes] = R;
+                sh.S[tid / kFoldLanes] = S;
+                sh.bad[tid / kFoldLanes] = bad;
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const int bad = sh.bad[lane];
+            float Rs, invS;
+            const unsigned bits = judge_position(P, b, i, live, writer, sh.R[lane], sh.S[lane], (bad & 1) != 0, live && (bad & 2),
+                                                 x, zx, qx, ux, Rs, invS);
+            const unsigned rej = __ballot_sync(0xffffffffu, live && i < P.gamma && !(bits & kBitAccept));
+            if (rej && n == P.gamma) n = base + __ffs(rej) - 1;
+            fl |= (__ballot_sync(0xffffffffu, bits & kBitBadToken) ? DSSD_EDGE_FLAG_BAD_TOKEN : 0u) |
+                  (__ballot_sync(0xffffffffu, bits & kBitNonFinite) ? DSSD_EDGE_FLAG_NONFINITE : 0u) |
+                  (__ballot_sync(0xffffffffu, bits & kBitTimeout) ? DSSD_EDGE_FLAG_TIMEOUT : 0u);
+            if (n >= base && n < base + 32) {
+                ref2_n = __shfl_sync(0xffffffffu, Rs, n - base);
+                invS_n = __shfl_sync(0xffffffffu, invS, n - base);
+            }
+        }
+    }
+    if (tid == 0) {
+        if (fl & DSSD_EDGE_FLAG_TIMEOUT) n = -1;
+        sh.n = n;
+        sh.ref2 = ref2_n;
+        sh.invS = invS_n;
+        if (writer) {
+            P.accept_len[b] = n;
+            if (P.flags) P.flags[b] = fl;
+            ReadySlot s;
+            s.b = (int)b;
+            s.n = n;
+            s.ref2 = ref2_n;
+            s.invS = invS_n;
+            P.ready[b] = s;
+        }
+    }
+    __syncthreads();
+}
+
+}  // namespace dssd

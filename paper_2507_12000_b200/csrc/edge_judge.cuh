@@ -42,16 +42,17 @@ __device__ __forceinline__ double exp2_small(double x)
 // One position i of sequence b, given its row's sum_v 2^(l_v * c1) = S * 2^Rr (float64 S, integer
 // Rr): writes lse and p_i(x_i), evaluates the acceptance test and returns the position's bits;
 // Rs, invS are what the emission of this row would need.  A lane that is not live returns "accepted".
+// `writer`: of the CTAs that judge the same position, the one that writes lse and p_tok.
 template <class Params>
-__device__ __forceinline__ unsigned judge_position(const Params &P, long long b, int i, bool live, float Rr, double S,
-                                                   bool bad, bool timeout, int x, float zx, float qx, float ux,
+__device__ __forceinline__ unsigned judge_position(const Params &P, long long b, int i, bool live, bool writer, float Rr,
+                                                   double S, bool bad, bool timeout, int x, float zx, float qx, float ux,
                                                    float &Rs, float &invS)
 {
     const double c1 = (double)P.c1;
     // the sum has a finite logarithm iff S is positive and finite
     const bool finite = !timeout && !bad && (S > 0.0) && (S < INFINITY) && (Rr != DSSD_NEG_INF);
     unsigned bits = live ? ((finite ? 0u : kBitNonFinite) | (timeout ? kBitTimeout : 0u)) : kBitAccept;
-    if (live && P.lse)
+    if (live && writer && P.lse)
         P.lse[b * (P.gamma + 1) + i] = finite ? (Rr + __log2f((float)S)) * 0.6931471805599453f : __int_as_float(0x7fc00000);
     // 1 / S in float64: the float32 reciprocal refined by one Newton step
     double invS_d = NAN;
@@ -73,7 +74,7 @@ __device__ __forceinline__ unsigned judge_position(const Params &P, long long b,
             else if (q <= 0.0) accept = (p > 0.0) && (u < 1.0);
             else accept = (u < 1.0) && (u * q < p);
         }
-        if (P.p_tok) P.p_tok[(size_t)b * P.gamma + i] = (float)p;
+        if (writer && P.p_tok) P.p_tok[(size_t)b * P.gamma + i] = (float)p;
         bits |= accept ? kBitAccept : 0u;
     }
     invS = finite ? (float)invS_d : __int_as_float(0x7fc00000);

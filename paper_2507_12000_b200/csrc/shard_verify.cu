@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kThreads) shard_combine_kernel(const __grid_co
                 add_partial(Rr, S, bad, __ldg(P.part_ref + (size_t)g * rows + row), __ldg(P.part_sum + (size_t)g * rows + row));
         }
         float Rs, invS;
-        const unsigned bits = judge_position(P, b, i, live, Rr, S, bad, false, x, zx, qx, ux, Rs, invS);
+        const unsigned bits = judge_position(P, b, i, live, true, Rr, S, bad, false, x, zx, qx, ux, Rs, invS);
         const unsigned rej = __ballot_sync(kFull, live && i < P.gamma && !(bits & kBitAccept));
         if (rej && n == P.gamma) n = base + __ffs(rej) - 1;
         fl |= (__ballot_sync(kFull, bits & kBitBadToken) ? DSSD_EDGE_FLAG_BAD_TOKEN : 0u) |

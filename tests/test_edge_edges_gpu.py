@@ -1,0 +1,29 @@
+"""The edge half where its geometry can go wrong: vocabularies at the edges of a tile of the log-sum-exp
+kernel (4096 float32 or 8192 bf16 logits) and of the emission (8192 entries), launches at the thresholds of
+one / two / four tiles per CTA and of folding inside the emission, 32 positions and more per sequence."""
+import pytest
+
+import dssd_inputs as di
+from gpu_util import compare_round
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_12000_b200 import binding
+
+    return binding
+
+
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [
+    ("f32", 2, 2, 1), ("bf16", 2, 2, 7), ("f32", 3, 1, 4095), ("f32", 3, 1, 4096), ("f32", 3, 1, 4099),
+    ("bf16", 3, 2, 8191), ("bf16", 3, 2, 8192), ("bf16", 3, 2, 8193), ("f32", 2, 1, 8200), ("bf16", 2, 0, 16385),
+    ("f32", 4, 31, 3000), ("bf16", 4, 32, 3001), ("f32", 2, 64, 1500),
+    ("bf16", 592, 1, 600), ("bf16", 593, 1, 600), ("f32", 74, 1, 65536), ("f32", 75, 1, 65536),
+    ("f32", 587, 1, 16384), ("f32", 588, 1, 16384), ("f32", 791, 2, 32768), ("f32", 792, 2, 32768),
+    ("bf16", 1600, 2, 36001),
+])
+def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, zipf=V > 8, seed=V + Bn)
+    compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
