@@ -1,0 +1,40 @@
+"""The marshalling module's own checks: what it refuses before the library is called (no GPU needed)."""
+import pytest
+import torch
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_12000_b200 import build
+
+    build.build()
+    from paper_2507_12000_b200 import binding
+
+    return binding
+
+
+def _out(n=1):
+    return {"accept_len": torch.zeros(n, dtype=torch.int32), "p_row": torch.zeros(n, 8), "token": torch.zeros(n, dtype=torch.int32)}
+
+
+def test_refusals(B):
+    tl, ws = torch.zeros(1, 2, 8), torch.zeros(256, dtype=torch.uint8)
+    with pytest.raises(AssertionError):  # not a CUDA tensor
+        B.dssd_edge_verify(tl, None, None, None, 1.0, out=_out(), workspace=ws)
+    with pytest.raises(TypeError):       # not a tensor
+        B.dssd_edge_verify([1.0], None, None, None, 1.0, out=_out(), workspace=ws)
+    with pytest.raises(AssertionError):
+        B.dssd_device_resample(torch.zeros(1, 8), None, torch.zeros(1, dtype=torch.int32), torch.zeros(1), 0, out=_out(), workspace=ws)
+    with pytest.raises(TypeError):       # wrong number of arguments
+        B._marshal.edge_verify(tl)
+    with pytest.raises(KeyError):        # a required output is missing
+        B.dssd_round_host({"target_logits": tl, "uniforms_rs": torch.zeros(1)}, 1.0, ws, out={}, stream=0)
+    with pytest.raises(TypeError):       # half precision logits are no payload of this library
+        B.dssd_round_host({"target_logits": tl.half(), "uniforms_rs": torch.zeros(1)}, 1.0, ws, out=_out(), stream=0)
+
+
+def test_statuses_come_through(B):
+    host = {"target_logits": torch.zeros(1, 1, 8), "uniforms_rs": torch.zeros(1)}
+    with pytest.raises(B.DssdError) as e:  # temperature 0 is refused by the library itself
+        B.dssd_round_host(host, 0.0, torch.zeros(256, dtype=torch.uint8), out=_out(), stream=0)
+    assert e.value.status == B.DSSD_ERR_INVALID_ARG
