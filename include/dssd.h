@@ -29,16 +29,14 @@
  *   - Every pointer is a DEVICE pointer unless its comment says "host".
  *   - The caller owns every buffer.  The library allocates no memory, enqueues its work on the
  *     given CUDA stream and returns without synchronising.  It keeps no state between calls except
- *     per-device launch constants (SM count, resident CTAs per kernel), which are looked up on the
- *     first call made with a device current and cached, and the built-in scratch of
- *     dssd_device_resample_static.
+ *     the built-in scratch of dssd_device_resample_static, whose address is looked up once per device,
+ *     and the emission kernel's resident CTAs in dssd_edge_emit_shard, likewise.
  *   - The kernels of a call are launched with programmatic stream serialization: the first of them may
  *     be scheduled while the kernel before it on the stream drains, and waits for its end before
- *     it reads or writes anything.  dssd_edge_verify_topk is launched cooperatively (every CTA
- *     resident at once): two such calls on different streams run one after the other.
+ *     it reads or writes anything.
  *   - Every call with device pointers only can be recorded in a CUDA graph by stream capture
- *     (it enqueues kernels and nothing else), provided one call of the same entry point was made
- *     on that device before the capture began (the first call looks the launch constants up).
+ *     (it enqueues kernels and nothing else); dssd_device_resample_static provided one call of it was
+ *     made on that device before the capture began.
  *     dssd_round_host synchronises the stream in the middle and cannot be captured.
  *   - Buffers need only their natural alignment; 16-byte aligned rows take the fast path.
  *   - A status other than DSSD_OK means nothing was enqueued (except DSSD_ERR_CUDA, after

@@ -367,7 +367,7 @@ size_t dssd_edge_verify_topk_workspace_bytes(int B, int gamma, int V, int k)
 {
     if (check_sizes(B, gamma, V) != DSSD_OK) return 0;
     if (k < 1 || k > V || k > DSSD_TOPK_MAX) return 0;
-    return dssd::topk_workspace_layout(B, gamma, k, nullptr, nullptr);
+    return dssd::topk_workspace_bytes(B, gamma, V, k);
 }
 
 dssd_status dssd_edge_verify_topk(const void *target_logits, dssd_dtype dtype, int64_t row_stride,

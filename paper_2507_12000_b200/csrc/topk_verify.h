@@ -7,10 +7,6 @@
 
 namespace dssd {
 
-constexpr int kTopkBlock = 2048;     // vocabulary entries per scheduling block
-constexpr int kTopkMergeKeys = 128;  // most keys that one row's pieces hold together
-constexpr int kTopkMaxPieces = 16;   // most CTAs that share one row
-
 struct TopkParams {
     // caller's arrays
     const void *logits;
@@ -25,29 +21,16 @@ struct TopkParams {
     float *p_val;
     float *p_tok;
     uint32_t *flags;
-    // geometry: rows are cut into blocks of kTopkBlock entries, the blocks of all rows are numbered
-    // row by row, and CTA c owns blocks [c * total_blocks / grid, (c + 1) * total_blocks / grid)
-    int nb;                           // blocks per row
-    int max_pieces;                   // list slots per row (a row is shared by at most this many CTAs)
-    unsigned long long total_blocks;  // rows * nb
-    int grid;
-    // workspace
-    unsigned *error;                  // nonzero once a bounded wait has run out (zeroed by the kernel before use)
-    unsigned *seq_done;               // [B] rows of the sequence that have been judged (zeroed by the kernel before use)
-    unsigned *row_done;               // [rows] pieces of the row whose lists have been published (zeroed likewise)
-    unsigned *verdict;                // [rows] accepted / rejected and the row's flag bits, written when the row is judged
-    unsigned long long *lists;        // [rows, max_pieces, k] candidate keys of each piece of a row; once the row has
-                                      // been judged its first slot holds the row's k (index, probability) pairs
-    size_t zero_bytes;
+    // geometry
+    int runs;                         // runs per row (one CTA of the selection kernel each)
+    int run_vecs;                     // 16-byte vectors per run
+    // workspace (no initial contents needed: every word that is read has been written by the call)
+    unsigned long long *lists;        // [rows, runs, k] the run's k best keys, best first, 0 where it has fewer
 };
 
-// slots per row for a given k (depends on k only)
-int topk_max_pieces(int k);
+size_t topk_workspace_bytes(int B, int gamma, int V, int k);
 
-// Carves the workspace; returns the bytes needed.  With P == nullptr only computes the size.
-size_t topk_workspace_layout(int B, int gamma, int k, TopkParams *P, char *base);
-
-// Fills the geometry, clears the counters and launches the kernel on `stream`.
+// Fills the geometry and launches the kernels on `stream`.
 cudaError_t topk_verify_launch(TopkParams &P, int dtype, void *workspace, cudaStream_t stream);
 
 struct TopkResampleParams {

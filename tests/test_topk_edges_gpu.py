@@ -1,0 +1,48 @@
+"""The truncated-support round where its geometry can go wrong: vocabularies at the edges of a tile of the
+selection kernel (4096 float32 or 8192 bf16 logits), launches at the thresholds of one / two / four tiles per
+CTA, the smallest and the largest k, rows whose runs hold fewer than k entries, rows that are masked (mostly
+-inf), and runs whose candidates overflow the buffer."""
+import numpy as np
+import pytest
+
+import dssd_inputs as di
+from test_parity_topk_gpu import compare_topk
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_12000_b200 import binding
+
+    return binding
+
+
+@pytest.mark.parametrize("dtype,Bn,gamma,V,k", [
+    ("f32", 3, 1, 4095, 32), ("f32", 3, 1, 4096, 1), ("f32", 3, 1, 4099, 10), ("bf16", 3, 2, 8191, 32), ("bf16", 3, 2, 8192, 10),
+    ("bf16", 3, 2, 8200, 32), ("bf16", 2, 1, 16400, 32), ("f32", 4, 15, 9000, 10), ("f32", 4, 16, 9001, 10),
+    ("f32", 587, 1, 16384, 10), ("f32", 588, 1, 16384, 10), ("f32", 791, 2, 32768, 4), ("f32", 792, 2, 32768, 32),
+    ("f32", 2, 1, 600001, 32),
+])
+def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V, k):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, seed=V + Bn)
+    compare_topk(B, oracle_mod, di.generate_topk(w, k, threads=16), w.temperature, k)
+
+
+@pytest.mark.parametrize("k", [1, 10, 32])
+def test_masked_and_overflowing_rows(B, oracle_mod, k):
+    """Rows that keep a few entries above -inf (fewer and more than k), runs that repeat one value, and a first
+    tile of equal logits followed by larger ones."""
+    Bn, gamma, V = 5, 2, 30000
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype="f32", temperature=0.9, sigma_d=0.5, seed=k)
+    d = di.generate_topk(w, k, threads=4)
+    tl = d["target_logits"]
+    rng = np.random.default_rng(k)
+    for b, keep in ((0, 5), (1, 40)):
+        mask = np.ones(V, bool)
+        mask[rng.choice(V, keep, replace=False)] = False
+        tl[b][:, mask] = -np.inf
+    tl[2] = np.repeat(np.arange(V // 100, dtype=np.float32), 100)[None]
+    tl[3][:, :4096] = 0.0
+    tl[3][:, 4096:] = np.linspace(0.0, 1.0, V - 4096, dtype=np.float32)[None]
+    compare_topk(B, oracle_mod, d, w.temperature, k)
