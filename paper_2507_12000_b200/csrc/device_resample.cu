@@ -20,15 +20,16 @@
 
 #include "dssd_device.cuh"
 #include "launch.h"
+#include "quads.cuh"
 
 namespace dssd {
 
 namespace {
 
 constexpr int kSub = kResampleSub;      // entries per chunk sum
-constexpr int kRows = 4;                 // chunks per tile: quad number u * kThreads + t of a tile is thread t's u-th
+constexpr int kRows = 4;                 // chunks per tile
 constexpr int kTile = kRows * kSub;      // entries that a CTA streams at a time
-static_assert(kSub == 4 * kThreads, "a chunk is one quad per thread of the mass kernel");
+static_assert(2 * kRows == kWarps && kSub == 2 * 512, "a warp of the mass kernel streams half a chunk, 512 entries");
 // Tiles per CTA of the mass kernel.  Few tiles: one each, so that all SMs share them.  More than about
 // one and a half waves of 740 resident CTAs: two, more than six waves: four, which pays for a CTA's
 // start and its reduction less often.  Measured (us, mass kernel with the draw behind it; 1 / 2 / 4 tiles):
@@ -52,74 +53,36 @@ __device__ __forceinline__ float4 as_f4(const uint4 &v)
 // together with the row's reference exponent and 1 / sum, from which p_v = 2^(l_v c1 - ref2) / S is
 // formed on the fly exactly as the edge kernel forms it when it emits a row.  The kernel is
 // written once over these views.  A "quad" is four consecutive entries.
-__device__ __forceinline__ float half_bits_to_float(unsigned short h) { return __half2float(__ushort_as_half(h)); }
 __device__ __forceinline__ float4 half_quad(uint2 v)
 {
     const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
     const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
     return make_float4(a.x, a.y, b.x, b.y);
 }
-// Loads of a row that an earlier kernel of the chain may have written: they stay behind pdl_wait()
-// and do not go through the read-only path.  Vectors are read once and not kept in L1.
-__device__ __forceinline__ uint4 ld_row16(const void *p)
-{
-    uint4 v;
-    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint2 ld_row8(const void *p)
-{
-    uint2 v;
-    asm volatile("ld.global.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ float ld_row(const float *p)
-{
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ unsigned short ld_row(const uint16_t *p)
-{
-    unsigned short v;
-    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
-    return v;
-}
-
 struct RowF32 {  // p_row as float32
-    typedef uint4 Raw;
-    const float *p;
+    typedef Quads32 Q;
+    static constexpr uint32_t kFill = 0u;
+    const char *row;
     __device__ static __forceinline__ RowF32 make(const ResampleParams &P, int64_t b, int)
     {
         RowF32 r;
-        r.p = reinterpret_cast<const float *>(P.p_row) + (size_t)b * P.V;
+        r.row = static_cast<const char *>(P.p_row) + (size_t)b * P.V * 4;
         return r;
     }
-    __device__ __forceinline__ bool aligned(int e) const { return (reinterpret_cast<uintptr_t>(p + e) & 15u) == 0; }
-    __device__ __forceinline__ float ld(int64_t e) const { return ld_row(p + e); }
-    __device__ __forceinline__ Raw ld_quad_stream(int e0, int64_t quad) const
-    {
-        return ld_row16(p + e0 + 4 * quad);
-    }
-    __device__ __forceinline__ float4 quad(const Raw &v) const { return as_f4(v); }
+    __device__ __forceinline__ float4 quad(const Q::Raw &v) const { return as_f4(v); }
 };
 
 struct RowF16 {  // p_row as binary16 bit patterns
-    typedef uint2 Raw;
-    const uint16_t *p;
+    typedef Quads16 Q;
+    static constexpr uint32_t kFill = 0u;
+    const char *row;
     __device__ static __forceinline__ RowF16 make(const ResampleParams &P, int64_t b, int)
     {
         RowF16 r;
-        r.p = reinterpret_cast<const uint16_t *>(P.p_row) + (size_t)b * P.V;
+        r.row = static_cast<const char *>(P.p_row) + (size_t)b * P.V * 2;
         return r;
     }
-    __device__ __forceinline__ bool aligned(int e) const { return (reinterpret_cast<uintptr_t>(p + e) & 7u) == 0; }
-    __device__ __forceinline__ float ld(int64_t e) const { return half_bits_to_float(ld_row(p + e)); }
-    __device__ __forceinline__ Raw ld_quad_stream(int e0, int64_t quad) const
-    {
-        return ld_row8(p + e0 + 4 * quad);
-    }
-    __device__ __forceinline__ float4 quad(const Raw &v) const { return half_quad(v); }
+    __device__ __forceinline__ float4 quad(const Q::Raw &v) const { return half_quad(v); }
 };
 
 // four consecutive logits: how they are loaded and widened
@@ -127,15 +90,15 @@ template <int DT>
 struct LogitQuad;
 template <>
 struct LogitQuad<DSSD_F32> {
-    typedef uint4 Raw;
-    __device__ static __forceinline__ Raw ld_stream(const void *p) { return ld_stream16(p); }
-    __device__ static __forceinline__ float4 widen(const Raw &v) { return as_f4(v); }
+    typedef Quads32 Q;
+    static constexpr uint32_t kNegInf = 0xff800000u;
+    __device__ static __forceinline__ float4 widen(const uint4 &v) { return as_f4(v); }
 };
 template <>
 struct LogitQuad<DSSD_BF16> {
-    typedef uint2 Raw;
-    __device__ static __forceinline__ Raw ld_stream(const void *p) { return ld_stream8(p); }
-    __device__ static __forceinline__ float4 widen(const Raw &v)
+    typedef Quads16 Q;
+    static constexpr uint32_t kNegInf = 0xff80u;
+    __device__ static __forceinline__ float4 widen(const uint2 &v)
     {
         return make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
     }
@@ -143,7 +106,8 @@ struct LogitQuad<DSSD_BF16> {
 
 template <int DT>
 struct RowLogits {  // row n of the target logits, turned into probabilities on the fly
-    typedef typename LogitQuad<DT>::Raw Raw;
+    typedef typename LogitQuad<DT>::Q Q;
+    static constexpr uint32_t kFill = LogitQuad<DT>::kNegInf;
     const char *row;
     float c1, nref, invS;
     __device__ static __forceinline__ RowLogits make(const ResampleParams &P, int64_t b, int n)
@@ -158,131 +122,59 @@ struct RowLogits {  // row n of the target logits, turned into probabilities on 
         return r;
     }
     __device__ __forceinline__ float prob(float l) const { return ex2(fmaf(l, c1, nref)) * invS; }
-    __device__ __forceinline__ bool aligned(int e) const
-    {
-        return (reinterpret_cast<uintptr_t>(row + (size_t)e * Elem<DT>::kBytes) & (4u * Elem<DT>::kBytes - 1u)) == 0;
-    }
-    __device__ __forceinline__ float ld(int64_t e) const { return prob(Elem<DT>::load(row, e)); }
-    __device__ __forceinline__ Raw ld_quad_stream(int e0, int64_t quad) const
-    {
-        return LogitQuad<DT>::ld_stream(row + ((size_t)e0 + 4 * (size_t)quad) * Elem<DT>::kBytes);
-    }
-    __device__ __forceinline__ float4 quad(const Raw &v) const
+    __device__ __forceinline__ float4 quad(const typename Q::Raw &v) const
     {
         const float4 l = LogitQuad<DT>::widen(v);
         return make_float4(prob(l.x), prob(l.y), prob(l.z), prob(l.w));
     }
 };
 
-// This thread's part of the four chunk sums of the tile that starts at entry e0 (entries up to e1 only).
-// All loads are requested before the first is used.  Where the rows are not aligned, or the tile is
-// not a full one, entries are loaded one by one, neighbouring threads on neighbouring entries of the
-// same chunk.  q is not read without kHasQ (then r = p); with kPlain the sums of p go to `plain`.
-template <bool kHasQ, bool kPlain, typename RV>
-__device__ __forceinline__ void tile_mass(const RV &row, const float *q, int e0, int e1, double (&acc)[kRows], double *plain = nullptr)
+// This thread's part of a chunk sum: the four quads of its warp's half of a chunk, entries base + 128 u +
+// 4 lane .. + 3.  All loads are requested before the first is used.  q is not read without kHasQ (then
+// r = p); with kPlain the sum of p goes to `plain`.
+template <bool kHasQ, bool kPlain, bool kShift, typename RV>
+__device__ __forceinline__ double share_mass(const RV &row, const float *q, int V, long long base, double &plain)
 {
-    const int tid = threadIdx.x;
-    if (e1 - e0 == kTile && row.aligned(e0) && (!kHasQ || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0)) {
-        typename RV::Raw a[kRows];
-        uint4 b[kRows];
+    WarpQuads<typename RV::Q, 4, kShift> a;
+    WarpQuads<Quads32, 4, kShift> b;
+    a.load(row.row, V, base, RV::kFill);
+    if (kHasQ) b.load(reinterpret_cast<const char *>(q), V, base, 0u);
+    double acc = 0.0;
+    plain = 0.0;
 #pragma unroll
-        for (int u = 0; u < kRows; ++u) a[u] = row.ld_quad_stream(e0, tid + u * kThreads);
+    for (int u = 0; u < 4; ++u) {
+        const float4 x = row.quad(a.at(u));
         if (kHasQ) {
-            const float *qp = q + e0 + 4 * tid;
-#pragma unroll
-            for (int u = 0; u < kRows; ++u) b[u] = ld_row16(qp + u * kSub);
+            const float4 y = as_f4(b.at(u));
+            acc += (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
         }
-#pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            const float4 x = row.quad(a[u]);
-            if (kHasQ) {
-                const float4 y = as_f4(b[u]);
-                acc[u] = (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
-            }
-            if (!kHasQ || kPlain) {
-                const double s = ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-                if (kPlain) plain[u] = s;
-                if (!kHasQ) acc[u] = s;
-            }
-        }
-    } else {
-        const int first = e0 + tid, left = e1 - first;
-        float x[4 * kRows], y[4 * kRows];
-#pragma unroll
-        for (int j = 0; j < 4 * kRows; ++j) {
-            x[j] = y[j] = 0.f;
-            if (j * kThreads < left) x[j] = row.ld((int64_t)first + j * kThreads);
-        }
-        if (kHasQ) {
-            const float *qp = q + first;
-#pragma unroll
-            for (int j = 0; j < 4 * kRows; ++j)
-                if (j * kThreads < left) y[j] = ld_row(qp + j * kThreads);
-        }
-#pragma unroll
-        for (int u = 0; u < kRows; ++u) {
-            double r[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                r[j] = (4 * u + j) * kThreads < left ? (kHasQ ? res(x[4 * u + j], y[4 * u + j]) : (double)x[4 * u + j]) : 0.0;
-            acc[u] = (r[0] + r[1]) + (r[2] + r[3]);
-            if (kPlain)
-                plain[u] = ((double)x[4 * u] + (double)x[4 * u + 1]) + ((double)x[4 * u + 2] + (double)x[4 * u + 3]);
+        if (!kHasQ || kPlain) {
+            const double s = ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
+            if (kPlain) plain += s;
+            if (!kHasQ) acc += s;
         }
     }
+    return acc;
 }
 
-// Four sums over the warp at the price of six shuffled doubles: the lane ends up with sum number
-// (bit 4 of the lane) * 2 + (bit 3 of the lane).
-__device__ __forceinline__ double warp_sum4(const double (&x)[4])
+// r for thread t's run of the chunk that starts at entry e0: entries e0 + kRun * t + j in r[j]; 0 beyond the
+// row's end.  All loads are requested before the first is used.
+template <bool kHasQ, bool kShift, typename RV>
+__device__ __forceinline__ void load_run(const RV &row, const float *q, int V, int e0, double (&r)[kRun])
 {
-    const bool hi = threadIdx.x & 16, lo = threadIdx.x & 8;
-    double a = hi ? x[2] : x[0], b = hi ? x[3] : x[1];
-    a += __shfl_xor_sync(0xffffffffu, hi ? x[0] : x[2], 16);
-    b += __shfl_xor_sync(0xffffffffu, hi ? x[1] : x[3], 16);
-    double c = lo ? b : a;
-    c += __shfl_xor_sync(0xffffffffu, lo ? a : b, 8);
+    const long long first = (long long)e0 + kRun * (int)threadIdx.x;
+    ThreadQuads<typename RV::Q, kRun / 4, kShift> a;
+    ThreadQuads<Quads32, kRun / 4, kShift> b;
+    a.load(row.row, V, first, RV::kFill);
+    if (kHasQ) b.load(reinterpret_cast<const char *>(q), V, first, 0u);
 #pragma unroll
-    for (int o = 4; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    return c;
-}
-
-// r for thread t's run of the chunk [e0, e0 + kSub), entries e0 + kRun * t + j in r[j]; 0 from entry e1
-// on.  All loads are requested before the first is used.
-template <bool kHasQ, typename RV>
-__device__ __forceinline__ void load_run(const RV &row, const float *q, int e0, int e1, double (&r)[kRun])
-{
-    const int first = e0 + kRun * (int)threadIdx.x, left = e1 - first;
-    float y[kRun];
-    if (e1 - e0 == kSub && row.aligned(e0) && (!kHasQ || (reinterpret_cast<uintptr_t>(q + e0) & 15u) == 0)) {
-        typename RV::Raw a[kRun / 4];
-#pragma unroll
-        for (int u = 0; u < kRun / 4; ++u) a[u] = row.ld_quad_stream(first, u);
-        if (kHasQ) {
-#pragma unroll
-            for (int u = 0; u < kRun / 4; ++u) {
-                const float4 v = as_f4(ld_row16(q + first + 4 * u));
-                y[4 * u] = v.x, y[4 * u + 1] = v.y, y[4 * u + 2] = v.z, y[4 * u + 3] = v.w;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kRun / 4; ++u) {
-            const float4 x = row.quad(a[u]);
-            r[4 * u] = kHasQ ? res(x.x, y[4 * u]) : (double)x.x;
-            r[4 * u + 1] = kHasQ ? res(x.y, y[4 * u + 1]) : (double)x.y;
-            r[4 * u + 2] = kHasQ ? res(x.z, y[4 * u + 2]) : (double)x.z;
-            r[4 * u + 3] = kHasQ ? res(x.w, y[4 * u + 3]) : (double)x.w;
-        }
-    } else {
-        float x[kRun];
-#pragma unroll
-        for (int j = 0; j < kRun; ++j) {
-            x[j] = y[j] = 0.f;
-            if (j < left) x[j] = row.ld((int64_t)first + j);
-            if (kHasQ && j < left) y[j] = ld_row(q + first + j);
-        }
-#pragma unroll
-        for (int j = 0; j < kRun; ++j) r[j] = j < left ? (kHasQ ? res(x[j], y[j]) : (double)x[j]) : 0.0;
+    for (int u = 0; u < kRun / 4; ++u) {
+        const float4 x = row.quad(a.at(u));
+        const float4 y = kHasQ ? as_f4(b.at(u)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        r[4 * u] = kHasQ ? res(x.x, y.x) : (double)x.x;
+        r[4 * u + 1] = kHasQ ? res(x.y, y.y) : (double)x.y;
+        r[4 * u + 2] = kHasQ ? res(x.z, y.z) : (double)x.z;
+        r[4 * u + 3] = kHasQ ? res(x.w, y.w) : (double)x.w;
     }
 }
 
@@ -401,7 +293,7 @@ __device__ __forceinline__ Pick pick_chunk(const LaneSums &L, Sum sum, bool beyo
     return pk;
 }
 
-// The draw inside the picked chunk, entries [e0, e1), by the whole CTA: the token is the first entry whose
+// The draw inside the picked chunk, which starts at entry e0, by the whole CTA: the token is the first entry whose
 // running mass exceeds the target, else (rounding, or pk.beyond) the last one with mass; -1 when
 // the chunk has none.  `base` moves on by the chunk's mass; `hit`: the target was exceeded.  The result is
 // the same in all threads.  q == nullptr means r = p.
@@ -409,14 +301,14 @@ struct WalkShared {
     double sum[kDrawWarps];
     int tok[kDrawWarps];   // the warp's token; hit in bit 30
 };
-template <typename RV>
-__device__ __forceinline__ int walk_chunk(const Pick &pk, const RV &row, const float *q, int e0, int e1, double &base, bool &hit,
+template <bool kShift, typename RV>
+__device__ __forceinline__ int walk_chunk(const Pick &pk, const RV &row, const float *q, int V, int e0, double &base, bool &hit,
                                           WalkShared &sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double r[kRun], pre[kRun];
-    if (q) load_run<true>(row, q, e0, e1, r);
-    else load_run<false>(row, q, e0, e1, r);
+    if (q) load_run<true, kShift>(row, q, V, e0, r);
+    else load_run<false, kShift>(row, q, V, e0, r);
     unsigned positive = 0;
     double mine = 0.0;
 #pragma unroll
@@ -462,7 +354,7 @@ __device__ __forceinline__ int walk_chunk(const Pick &pk, const RV &row, const f
 }
 
 // The draw for sequence b by one CTA; q == nullptr means r = p.
-template <typename RV>
+template <bool kShift, typename RV>
 __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const float *q, unsigned fl, float u, LaneSums &L,
                      WalkShared &sh)
 {
@@ -479,9 +371,8 @@ __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const fl
         fl |= DSSD_RS_FLAG_FALLBACK;
         __syncthreads();  // every warp has read the sums that are replaced now
         for (int c = tid >> 5; c < P.n_sub; c += kDrawWarps) {
-            double tot = 0.0;
-            const int end = (int)min((long long)P.V, (long long)(c + 1) * width);
-            for (int e = c * width + lane; e < end; e += 32) tot += (double)row.ld(e);
+            double tot = 0.0, none;
+            for (int e = 0; e < width; e += 512) tot += share_mass<false, false, kShift>(row, q, P.V, (long long)c * width + e, none);
             tot = warp_sum(tot);
             if (lane == 0) cs[c] = tot;
         }
@@ -496,7 +387,7 @@ __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const fl
         for (int k = 0; k < P.rows_per_sum && !hit; ++k) {
             const long long e0 = (long long)pk.chunk * width + k * kSub;
             if (e0 >= P.V) break;
-            const int t = walk_chunk<RV>(pk, row, q, (int)e0, (int)min((long long)P.V, e0 + kSub), base, hit, sh);
+            const int t = walk_chunk<kShift>(pk, row, q, P.V, (int)e0, base, hit, sh);
             if (t >= 0) tok = t;
         }
     }
@@ -510,10 +401,10 @@ __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const fl
 // persistent kernel it replaces, with tickets, a cleared scratch and the draws at its end, took 41 us
 // with them; B = 1 V = 50272: 6.5 us for both kernels against 8.9.  48 registers, so five CTAs share an SM
 // and one CTA's reduction lies under the others' loads (four: 36.1 us).
-template <typename RV>
-__global__ void __launch_bounds__(kThreads, 5) resample_mass_kernel(const __grid_constant__ ResampleParams P)
+template <bool kShift, typename RV>
+__global__ void __launch_bounds__(kThreads, kShift ? 4 : 5) resample_mass_kernel(const __grid_constant__ ResampleParams P)
 {
-    __shared__ double s_w[kResampleMaxTiles * kRows][kWarps];
+    __shared__ double s_w[kResampleMaxTiles * kRows][2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // in index order: the edge kernel emits the rows from the last sequence backwards, so the first ones
     // are still in L2 when they were written just before
@@ -528,24 +419,19 @@ __global__ void __launch_bounds__(kThreads, 5) resample_mass_kernel(const __grid
     const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
     const int tiles = min(P.tiles, (P.V + kTile - 1) / kTile - first);
     for (int k = 0; k < tiles; ++k) {
-        const int e0 = (first + k) * kTile, e1 = min(P.V, e0 + kTile);
-        double acc[kRows];
-        if (q) tile_mass<true, false>(row, q, e0, e1, acc);
-        else tile_mass<false, false>(row, q, e0, e1, acc);
-        const double x = warp_sum4(acc);
-        if ((lane & 7) == 0) s_w[k * kRows + (lane >> 3)][warp] = x;
+        const long long base = (long long)(first + k) * kTile + warp * 512;
+        double acc, none;
+        if (q) acc = share_mass<true, false, kShift>(row, q, P.V, base, none);
+        else acc = share_mass<false, false, kShift>(row, q, P.V, base, none);
+        acc = warp_sum(acc);
+        if (lane == 0) s_w[k * kRows + (warp >> 1)][warp & 1] = acc;
     }
     __syncthreads();
     const int sums = tiles * kRows / P.rows_per_sum;
     if (tid < sums) {
         const int c = first * kRows / P.rows_per_sum + tid;
         double tot = 0.0;
-        for (int k = 0; k < P.rows_per_sum; ++k) {
-            double x = 0.0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) x += s_w[tid * P.rows_per_sum + k][w];
-            tot += x;
-        }
+        for (int k = 0; k < P.rows_per_sum; ++k) tot += s_w[tid * P.rows_per_sum + k][0] + s_w[tid * P.rows_per_sum + k][1];
         if (b + 1 == (int64_t)P.test_drop_seq_plus1) tot = __longlong_as_double((long long)kNoSum);
         if (c < P.n_sub) P.chunk_sum[(size_t)b * P.n_sub + c] = tot;
     }
@@ -554,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, 5) resample_mass_kernel(const __grid
 // One CTA per sequence.  Bound by latency: one round trip for the sums, one for the chunk, and the float64
 // additions that depend on one another (4 us at B = 256; a chunk of 4096 entries instead of 1024 took 5.9,
 // one warp per sequence with 32 entries per lane 6.0).
-template <typename RV>
+template <bool kShift, typename RV>
 __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __grid_constant__ ResampleParams P)
 {
     __shared__ WalkShared sh;
@@ -580,7 +466,7 @@ __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __gri
     } else {
         const RV row = RV::make(P, b, n);
         const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
-        draw<RV>(P, b, row, q, q ? 0u : DSSD_RS_FLAG_BONUS, u, L, sh);
+        draw<kShift>(P, b, row, q, q ? 0u : DSSD_RS_FLAG_BONUS, u, L, sh);
     }
 }
 
@@ -599,13 +485,14 @@ __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __gri
 __device__ __forceinline__ RowF32 shard_row(const ShardResampleParams &P, int64_t b)
 {
     RowF32 r;
-    r.p = P.p_row + (size_t)b * (size_t)P.p_stride;
+    r.row = reinterpret_cast<const char *>(P.p_row + (size_t)b * (size_t)P.p_stride);
     return r;
 }
 
+template <bool kShift>
 __global__ void __launch_bounds__(kThreads, 4) shard_mass_kernel(const __grid_constant__ ShardResampleParams P)
 {
-    __shared__ double s_w[2 * kRows][kWarps];
+    __shared__ double s_w[kWarps][2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned n_tiles = (unsigned)((P.V + kTile - 1) / kTile);
     const int64_t b = blockIdx.x / n_tiles;
@@ -614,25 +501,24 @@ __global__ void __launch_bounds__(kThreads, 4) shard_mass_kernel(const __grid_co
     pdl_trigger();
     const int n = ld_after(P.accept_len + b);
     const bool valid = n >= 0 && n <= P.gamma;
-    double acc_r[kRows] = {}, acc_p[kRows] = {};
+    double r = 0.0, p = 0.0;
     if (valid) {
         const RowF32 row = shard_row(P, b);
         const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
-        const int e0 = tile * kTile, e1 = min(P.V, e0 + kTile);
-        if (q) tile_mass<true, true>(row, q, e0, e1, acc_r, acc_p);
-        else tile_mass<false, true>(row, q, e0, e1, acc_r, acc_p);
+        const long long base = (long long)tile * kTile + warp * 512;
+        if (q) r = share_mass<true, true, kShift>(row, q, P.V, base, p);
+        else r = share_mass<false, true, kShift>(row, q, P.V, base, p);
     }
-    const double r = warp_sum4(acc_r), p = warp_sum4(acc_p);
-    if ((lane & 7) == 0) {
-        s_w[2 * (lane >> 3)][warp] = r;
-        s_w[2 * (lane >> 3) + 1][warp] = p;
+    r = warp_sum(r);
+    p = warp_sum(p);
+    if (lane == 0) {
+        s_w[warp][0] = r;
+        s_w[warp][1] = p;
     }
     __syncthreads();
     if (tid < 2 * kRows) {
-        const int c = tile * kRows + tid / 2;
-        double tot = 0.0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) tot += s_w[tid][w];
+        const int k = tid >> 1, c = tile * kRows + k;
+        double tot = s_w[2 * k][tid & 1] + s_w[2 * k + 1][tid & 1];
         if (!valid) tot = __longlong_as_double(0x7ff8000000000000ll);
         if (c < P.n_sub) P.chunk_sum[((size_t)b * P.n_sub + c) * 2 + (tid & 1)] = tot;
     }
@@ -661,6 +547,7 @@ __global__ void __launch_bounds__(kThreads) shard_total_kernel(const __grid_cons
 }
 
 // one CTA per sequence
+template <bool kShift>
 __global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_constant__ ShardResampleParams P)
 {
     __shared__ WalkShared sh;
@@ -715,7 +602,7 @@ __global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_c
             const float *q = (col == 0 && n < P.gamma) ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
             double base = pk.base;
             bool hit;
-            tok = walk_chunk<RowF32>(pk, row, q, pk.chunk * kSub, min(P.V, pk.chunk * kSub + kSub), base, hit, sh);
+            tok = walk_chunk<kShift>(pk, row, q, P.V, pk.chunk * kSub, base, hit, sh);
             if (tok < 0) fl |= DSSD_RS_FLAG_INVALID;
             else tok += P.v_begin;
         }
@@ -745,11 +632,24 @@ size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base)
 
 namespace {
 
+// do the rows of an array start on boundaries of four entries?
+bool quads_aligned(const void *base, int64_t stride, int esz)
+{
+    return reinterpret_cast<uintptr_t>(base) % (4 * esz) == 0 && stride % 4 == 0;
+}
+
+template <typename RV, bool kShift>
+cudaError_t launch_resample_as(const ResampleParams &P, unsigned grid, cudaStream_t stream)
+{
+    const cudaError_t e = launch_pdl(resample_mass_kernel<kShift, RV>, grid, kThreads, stream, P);
+    return e != cudaSuccess ? e : launch_pdl(resample_draw_kernel<kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P);
+}
 template <typename RV>
 cudaError_t launch_resample(const ResampleParams &P, unsigned grid, cudaStream_t stream)
 {
-    const cudaError_t e = launch_pdl(resample_mass_kernel<RV>, grid, kThreads, stream, P);
-    return e != cudaSuccess ? e : launch_pdl(resample_draw_kernel<RV>, (unsigned)P.B, kDrawThreads, stream, P);
+    const bool aligned = (P.logits ? quads_aligned(P.logits, P.row_stride, RV::Q::kBytes) : quads_aligned(P.p_row, P.V, RV::Q::kBytes)) &&
+                         (!P.draft_q || quads_aligned(P.draft_q, P.V, 4));
+    return aligned ? launch_resample_as<RV, false>(P, grid, stream) : launch_resample_as<RV, true>(P, grid, stream);
 }
 
 }  // namespace
@@ -776,13 +676,19 @@ size_t shard_resample_workspace_bytes(int B, int V)
     return (((size_t)B * n_sub * 2 * sizeof(double)) + 255) & ~(size_t)255;
 }
 
+static bool shard_aligned(const ShardResampleParams &P)
+{
+    return quads_aligned(P.p_row, P.p_stride, 4) && (!P.draft_q || quads_aligned(P.draft_q, P.q_stride, 4));
+}
+
 cudaError_t shard_mass_launch(ShardResampleParams &P, void *workspace, cudaStream_t stream)
 {
     P.n_sub = (int)(((size_t)P.V + kSub - 1) / kSub);
     P.chunk_sum = static_cast<double *>(workspace);
     const unsigned long long grid = (unsigned long long)P.B * (((unsigned long long)P.V + kTile - 1) / kTile);
     if (grid > 0x7fffffffull) return cudaErrorInvalidConfiguration;
-    const cudaError_t e = launch_pdl(shard_mass_kernel, (unsigned)grid, kThreads, stream, P);
+    const cudaError_t e = shard_aligned(P) ? launch_pdl(shard_mass_kernel<false>, (unsigned)grid, kThreads, stream, P)
+                                           : launch_pdl(shard_mass_kernel<true>, (unsigned)grid, kThreads, stream, P);
     return e != cudaSuccess ? e : launch_pdl(shard_total_kernel, (unsigned)((P.B + kWarps - 1) / kWarps), kThreads, stream, P);
 }
 
@@ -790,7 +696,8 @@ cudaError_t shard_draw_launch(ShardResampleParams &P, const void *workspace, cud
 {
     P.n_sub = (int)(((size_t)P.V + kSub - 1) / kSub);
     P.chunk_sum = const_cast<double *>(static_cast<const double *>(workspace));
-    return launch_pdl(shard_draw_kernel, (unsigned)P.B, kDrawThreads, stream, P);
+    return shard_aligned(P) ? launch_pdl(shard_draw_kernel<false>, (unsigned)P.B, kDrawThreads, stream, P)
+                            : launch_pdl(shard_draw_kernel<true>, (unsigned)P.B, kDrawThreads, stream, P);
 }
 
 }  // namespace dssd

@@ -20,6 +20,7 @@
 #include "dssd_device.cuh"
 #include "edge_fold.cuh"
 #include "launch.h"
+#include "quads.cuh"
 
 namespace dssd {
 
@@ -251,54 +252,38 @@ __device__ __forceinline__ void emit_raw(OUT *out, const uint4 &w, f32x2 cc, f32
 }
 
 template <int DT>
-struct QuadRaw;
-template <>
-struct QuadRaw<DSSD_F32> {
-    typedef uint4 T;
-    __device__ static __forceinline__ uint4 load(const void *p) { return ld_stream16(p); }
+struct LogitQuads {
+    typedef Quads32 Q;
 };
 template <>
-struct QuadRaw<DSSD_BF16> {
-    typedef uint2 T;
-    __device__ static __forceinline__ uint2 load(const void *p) { return ld_stream8(p); }
+struct LogitQuads<DSSD_BF16> {
+    typedef Quads16 Q;
 };
 
-// OUT[e] for the entries [e0, e1) of a row, e1 - e0 <= kEmitTile.  Both arrays aligned for whole
-// quads of four entries: 8- or 16-byte loads, 16- or 8-byte stores, all of a thread's loads
-// requested before the first is used.  Otherwise entry by entry, neighbouring threads on
-// neighbouring entries, with as many loads in flight.
-template <int DT, class OUT>
-__device__ __forceinline__ void emit_range(const char *rowp, OUT *outp, int e0, int e1, float c1, float ref2, float invS)
+// OUT[e] for the entries [e0, e0 + kEmitTile) of a row that lie in [0, V), where e0 makes the output's quads
+// aligned (it may be negative).  The logits' quads may lie on any element boundary (quads.cuh); all of a
+// thread's loads are requested before the first is used.
+template <int DT, bool kShift, class OUT>
+__device__ __forceinline__ void emit_tile(const char *rowp, OUT *outp, int V, long long e0, float c1, float ref2, float invS)
 {
-    using E = Elem<DT>;
-    const int tid = threadIdx.x;
+    using Q = typename LogitQuads<DT>::Q;
+    constexpr int kN = kEmitTile / 4 / kThreads;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long base = e0 + warp * (128 * kN);
     const float nref = -ref2;
-    int done = e0;
-    if (((reinterpret_cast<uintptr_t>(rowp + (size_t)e0 * E::kBytes) & (4 * E::kBytes - 1)) |
-         (reinterpret_cast<uintptr_t>(outp + e0) & (4 * sizeof(OUT) - 1))) == 0) {
-        const f32x2 cc = pack2(c1, c1), nn = pack2(nref, nref), ss = pack2(invS, invS);
-        const int nq = (e1 - e0) >> 2;
-        constexpr int kQ = kEmitTile / 4 / kThreads;
-        const char *src = rowp + (size_t)e0 * E::kBytes + (size_t)tid * (4 * E::kBytes);
-        OUT *dst = outp + e0 + 4 * tid;
-        typename QuadRaw<DT>::T w[kQ];
+    const f32x2 cc = pack2(c1, c1), nn = pack2(nref, nref), ss = pack2(invS, invS);
+    WarpQuads<Q, kN, kShift> w;
+    w.load(rowp, V, base, 0u);
 #pragma unroll
-        for (int u = 0; u < kQ; ++u)
-            if (tid + u * kThreads < nq) w[u] = QuadRaw<DT>::load(src + u * (kThreads * 4 * E::kBytes));
-#pragma unroll
-        for (int u = 0; u < kQ; ++u)
-            if (tid + u * kThreads < nq) emit_raw(dst + u * (kThreads * 4), w[u], cc, nn, ss);
-        done = e0 + 4 * nq;
-    }
-    constexpr int kU = 8;
-    for (int e = done + tid; e < e1; e += kU * kThreads) {
-        float z[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-            if (e + u * kThreads < e1) z[u] = E::load(rowp, e + u * kThreads);
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-            if (e + u * kThreads < e1) store_one(outp + e + u * kThreads, ex2(fmaf(z[u], c1, nref)) * invS);
+    for (int u = 0; u < kN; ++u) {
+        const typename Q::Raw v = w.at(u);
+        const long long e = base + 128 * u + 4 * lane;
+        if (e >= 0 && e + 4 <= V) {
+            emit_raw(outp + e, v, cc, nn, ss);
+        } else if (e + 4 > 0 && e < V) {  // a quad that crosses an end of the row
+            for (int j = 0; j < 4; ++j)
+                if (e + j >= 0 && e + j < V) store_one(outp + e + j, ex2(fmaf(Elem<DT>::load(rowp, e + j), c1, nref)) * invS);
+        }
     }
 }
 
@@ -313,7 +298,7 @@ __global__ void __launch_bounds__(kThreads) edge_fold_kernel(const __grid_consta
 // Bound by HBM: reads and writes mixed, 234 MB at B = 256 V = 151936 in 36.5 us.
 // One CTA per (sequence, tile of row n), after a fold of its own or (kFold = false) the fold kernel's.
 // The sequences run backwards: the rows that the log-sum-exp kernel read last are the ones still in L2.
-template <int DT, bool kFold>
+template <int DT, bool kFold, bool kShift>
 __global__ void __launch_bounds__(kThreads, 4) edge_emit_kernel(const __grid_constant__ EdgeParams P)
 {
     const unsigned rb = blockIdx.x / (unsigned)P.emit_tiles;
@@ -337,9 +322,16 @@ __global__ void __launch_bounds__(kThreads, 4) edge_emit_kernel(const __grid_con
     }
     if (n < 0 || (P.skip_bonus_row && n == P.gamma)) return;
     const char *rowp = row_ptr<DT>(P, b * (P.gamma + 1) + n);
-    const int e0 = tile * kEmitTile, e1 = min((long long)P.V, (long long)e0 + kEmitTile);
-    if (P.p_row16) emit_range<DT>(rowp, P.p_row16 + (size_t)b * P.V, e0, e1, P.c1, ref2, invS);
-    else emit_range<DT>(rowp, P.p_row + (size_t)b * P.V, e0, e1, P.c1, ref2, invS);
+    // tiles start where the output is aligned
+    if (P.p_row16) {
+        uint16_t *out = P.p_row16 + (size_t)b * P.V;
+        const int off = kShift ? quad_offset<Quads16>(reinterpret_cast<const char *>(out), 0) : 0;
+        emit_tile<DT, kShift>(rowp, out, P.V, (long long)tile * kEmitTile - off, P.c1, ref2, invS);
+    } else {
+        float *out = P.p_row + (size_t)b * P.V;
+        const int off = kShift ? quad_offset<Quads32>(reinterpret_cast<const char *>(out), 0) : 0;
+        emit_tile<DT, kShift>(rowp, out, P.V, (long long)tile * kEmitTile - off, P.c1, ref2, invS);
+    }
 }
 
 // One shard of the vocabulary: the rows' sums and the drafted tokens' logits go out as they are.
@@ -402,19 +394,35 @@ size_t edge_workspace_layout(int B, int gamma, int runs_per_row, EdgeParams *P, 
 
 namespace {
 
+template <int DT, bool kShift>
+cudaError_t launch_emit(const EdgeParams &P, unsigned ctas, bool fold, cudaStream_t stream)
+{
+    return fold ? launch_pdl(edge_emit_kernel<DT, true, kShift>, ctas, kThreads, stream, P)
+                : launch_pdl(edge_emit_kernel<DT, false, kShift>, ctas, kThreads, stream, P);
+}
+
 template <int DT>
-cudaError_t launch_edge(const EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
+cudaError_t launch_edge(EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
 {
     cudaError_t e = launch_pdl(edge_lse_kernel<DT>, lse_ctas, kLseThreads, stream, P);
     if (e != cudaSuccess) return e;
     const unsigned long long rows = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1);
     if (P.shard_sum) return launch_pdl(edge_partial_kernel, (unsigned)((rows + kFoldRows - 1) / kFoldRows), kThreads, stream, P);
     const bool emit = P.p_row || P.p_row16;
+    // rows whose logits and output all start on boundaries of four entries need no shifting
+    const int osz = P.p_row16 ? 2 : 4;
+    const uintptr_t out = P.p_row16 ? reinterpret_cast<uintptr_t>(P.p_row16) : reinterpret_cast<uintptr_t>(P.p_row);
+    const bool aligned = P.V % 4 == 0 && out % (4 * osz) == 0 && P.row_stride % 4 == 0 &&
+                         reinterpret_cast<uintptr_t>(P.logits) % (4 * Elem<DT>::kBytes) == 0;
+    P.emit_tiles = (int)(((long long)P.V + (aligned ? 0 : 3) + kEmitTile - 1) / kEmitTile);
     const unsigned long long ctas = (unsigned long long)P.B * (unsigned long long)P.emit_tiles;
-    if (emit && ctas <= kEmitFoldCtas) return launch_pdl(edge_emit_kernel<DT, true>, (unsigned)ctas, kThreads, stream, P);
-    e = launch_pdl(edge_fold_kernel, (unsigned)P.B, kThreads, stream, P);
-    if (e != cudaSuccess || !emit) return e;
-    return launch_pdl(edge_emit_kernel<DT, false>, (unsigned)ctas, kThreads, stream, P);
+    if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+    const bool fold = emit && ctas <= kEmitFoldCtas;
+    if (!fold) {
+        e = launch_pdl(edge_fold_kernel, (unsigned)P.B, kThreads, stream, P);
+        if (e != cudaSuccess || !emit) return e;
+    }
+    return aligned ? launch_emit<DT, false>(P, (unsigned)ctas, fold, stream) : launch_emit<DT, true>(P, (unsigned)ctas, fold, stream);
 }
 
 }  // namespace
@@ -431,10 +439,7 @@ cudaError_t edge_verify_launch(EdgeParams &P, int dtype, void *workspace, cudaSt
     if (runs < 1) runs = 1;
     P.run_vecs = (int)(per * kLseTile);
     P.runs = (int)runs;
-    P.emit_tiles = (int)(((long long)P.V + kEmitTile - 1) / kEmitTile);
-    if (rows * (unsigned long long)runs > 0x7fffffffull ||
-        (unsigned long long)P.B * (unsigned long long)P.emit_tiles > 0x7fffffffull)
-        return cudaErrorInvalidConfiguration;
+    if (rows * (unsigned long long)runs > 0x7fffffffull) return cudaErrorInvalidConfiguration;
     edge_workspace_layout(P.B, P.gamma, P.runs, &P, static_cast<char *>(workspace));
     const unsigned lse_ctas = (unsigned)(rows * (unsigned long long)runs);
     return dtype == DSSD_BF16 ? launch_edge<DSSD_BF16>(P, lse_ctas, stream) : launch_edge<DSSD_F32>(P, lse_ctas, stream);

@@ -22,7 +22,7 @@ def B():
     ("f32", 4, 31, 3000), ("bf16", 4, 32, 3001), ("f32", 2, 64, 1500),
     ("bf16", 592, 1, 600), ("bf16", 593, 1, 600), ("f32", 74, 1, 65536), ("f32", 75, 1, 65536),
     ("f32", 587, 1, 16384), ("f32", 588, 1, 16384), ("f32", 791, 2, 32768), ("f32", 792, 2, 32768),
-    ("bf16", 1600, 2, 36001),
+    ("bf16", 1600, 2, 36001), ("bf16", 5, 1, 8189), ("bf16", 5, 1, 8190), ("f32", 5, 1, 8191), ("f32", 5, 2, 16385),
 ])
 def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, zipf=V > 8, seed=V + Bn)

@@ -20,7 +20,7 @@ def B():
     (5, 2, 1, False), (5, 2, 1023, False), (5, 2, 1024, True), (5, 1, 1025, False), (5, 3, 4095, True),
     (5, 2, 4096, False), (5, 2, 4097, False), (7, 1, 4100, True), (3, 1, 8192, False), (3, 1, 12289, False),
     (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
-    (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True),
+    (6, 2, 9001, False), (6, 3, 9002, True), (7, 2, 9003, True), (6, 2, 9003, False), (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True),
 ])
 def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
     gen = torch.Generator(device="cuda").manual_seed(Bn + V)
