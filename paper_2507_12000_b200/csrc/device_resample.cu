@@ -36,6 +36,14 @@ static_assert(2 * kRows == kWarps && kSub == 2 * 512, "a warp of the mass kernel
 // B = 256 V = 151936 (9728 tiles) 45.7 / 45.0 / 41.7, B = 64 V = 128256 (2048) 21.4 / 21.4 / 32.1,
 // B = 8 V = 32000 (64) 7.9 / 8.7 / 10.2.
 constexpr unsigned long long kTwoTiles = 1200, kFourTiles = 4800;
+constexpr int kClusterThreads = 512;     // most threads per CTA of the cluster kernel
+constexpr int kClusterMax = 8;           // most CTAs per sequence (the portable cluster size)
+// Most CTAs of a launch of the cluster kernel, about one wave (two CTAs of 256 threads fit an SM).  Measured (us a round, cluster
+// kernel / two kernels): B = 8 V = 32000 (64 CTAs) 10.7 / 12.1, B = 32 (256) 15.6 / 15.5, B = 64 (512) 21.3 / 20.5,
+// B = 100 V = 3001 (100) 12.4 / 15.1. CTAs of 512 threads, for vocabularies beyond 32768, pay off in smaller
+// batches only: B = 1 V = 50272 (8) 10.5 / 11.4, B = 16 V = 50257 (128) 17.7 / 16.2.
+constexpr int kClusterWave = 200;
+constexpr int kClusterSums = kClusterMax * kClusterThreads / 32;
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
 constexpr int kDrawWarps = kDrawThreads / 32;
 constexpr int kRun = kSub / kDrawThreads;  // entries of a chunk per thread
@@ -62,6 +70,7 @@ __device__ __forceinline__ float4 half_quad(uint2 v)
 struct RowF32 {  // p_row as float32
     typedef Quads32 Q;
     static constexpr uint32_t kFill = 0u;
+    static constexpr bool kFixed = true;  // the row does not depend on the accepted length
     const char *row;
     __device__ static __forceinline__ RowF32 make(const ResampleParams &P, int64_t b, int)
     {
@@ -75,6 +84,7 @@ struct RowF32 {  // p_row as float32
 struct RowF16 {  // p_row as binary16 bit patterns
     typedef Quads16 Q;
     static constexpr uint32_t kFill = 0u;
+    static constexpr bool kFixed = true;  // the row does not depend on the accepted length
     const char *row;
     __device__ static __forceinline__ RowF16 make(const ResampleParams &P, int64_t b, int)
     {
@@ -108,6 +118,7 @@ template <int DT>
 struct RowLogits {  // row n of the target logits, turned into probabilities on the fly
     typedef typename LogitQuad<DT>::Q Q;
     static constexpr uint32_t kFill = LogitQuad<DT>::kNegInf;
+    static constexpr bool kFixed = false;
     const char *row;
     float c1, nref, invS;
     __device__ static __forceinline__ RowLogits make(const ResampleParams &P, int64_t b, int n)
@@ -470,6 +481,121 @@ __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __gri
     }
 }
 
+// Small launches: one cluster of 1, 2, 4 or 8 CTAs per sequence does the whole draw and reads every entry
+// once.  Warp g of the cluster holds entries 512 g .. of the row in registers (the layout of share_mass), its
+// sum goes to every CTA's shared memory, and after one cluster barrier every warp picks the 512 entries that
+// hold the target; the warp that holds them finds the token.
+template <bool kShift, typename RV>
+__global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const __grid_constant__ ResampleParams P)
+{
+    __shared__ double s_sum[2][kClusterSums];
+    __shared__ Pick s_pick;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const unsigned csize = (unsigned)P.n_ctas, rank = csize > 1 ? cluster_rank() : 0u;
+    const int64_t b = blockIdx.x / csize;
+    const int g = (int)rank * warps + warp, n_sums = (int)csize * warps;
+    if (csize > 1) cluster_arrive();  // a CTA's shared memory may be written once it is known to run
+    pdl_wait();
+    pdl_trigger();
+    const int n = ld_after(P.accept_len + b);
+    const float u = ld_after(P.uniforms + b);
+    const long long base = 512ll * g;
+    WarpQuads<typename RV::Q, 4, kShift> a;
+    if (RV::kFixed) a.load(RV::make(P, b, 0).row, P.V, base, RV::kFill);  // (on its way before n is back)
+    const bool draws = n >= 0 && n <= P.gamma && selected(P, n);
+    double r[16];
+    const float *q = draws && n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
+    unsigned fl = q ? 0u : DSSD_RS_FLAG_BONUS;
+    const RV row = RV::make(P, b, draws ? n : 0);
+    Pick pk;
+    pk.ok = false;
+    for (int attempt = 0; draws && attempt < 2; ++attempt) {
+        if (!RV::kFixed) a.load(row.row, P.V, base, RV::kFill);
+        double t = 0.0;
+        if (q) {
+            WarpQuads<Quads32, 4, kShift> d;
+            d.load(reinterpret_cast<const char *>(q), P.V, base, 0u);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float4 x = row.quad(a.at(k)), y = as_f4(d.at(k));
+                r[4 * k] = res(x.x, y.x), r[4 * k + 1] = res(x.y, y.y), r[4 * k + 2] = res(x.z, y.z), r[4 * k + 3] = res(x.w, y.w);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float4 x = row.quad(a.at(k));
+                r[4 * k] = x.x, r[4 * k + 1] = x.y, r[4 * k + 2] = x.z, r[4 * k + 3] = x.w;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t += (r[4 * k] + r[4 * k + 1]) + (r[4 * k + 2] + r[4 * k + 3]);
+        t = warp_sum(t);
+        if (csize > 1) {
+            if (attempt == 0) cluster_wait();
+            if (lane < (int)csize) cluster_store(&s_sum[attempt][g], (unsigned)lane, t);
+            cluster_arrive();
+            cluster_wait();
+        } else {
+            if (lane == 0) s_sum[attempt][g] = t;
+            __syncthreads();
+        }
+        // one warp per CTA: its float64 operations would hold up the others' if every warp did them
+        if (warp == 0) {
+            LaneSums L;
+            auto sum = [&](int c) { return s_sum[attempt][c]; };
+            load_sums(L, n_sums, sum);
+            const Pick mine = pick_chunk(L, sum, false, [&](double Z) { return (double)u * Z; });
+            if (lane == 0) s_pick = mine;
+        }
+        __syncthreads();
+        pk = s_pick;
+        if (pk.ok || !q) break;
+        q = nullptr;  // residual has no mass (p == q): draw from p instead
+        fl |= DSSD_RS_FLAG_FALLBACK;
+        __syncthreads();  // the pick has been read
+    }
+    if (!draws && csize > 1) cluster_wait();
+    if (!pk.ok) {
+        if (rank == 0 && threadIdx.x == 0) {
+            const bool invalid = n < 0 || n > P.gamma;
+            if (draws || invalid || P.select == 1) {  // (the bonus token drawn at the edge: the others get their token later)
+                P.token[b] = -1;
+                if (P.flags) P.flags[b] = invalid ? DSSD_RS_FLAG_INVALID : draws ? fl | DSSD_RS_FLAG_INVALID : 0u;
+            }
+        }
+        return;
+    }
+    if (g != pk.chunk) return;
+    // this warp's 512 entries in the order 128 u + 4 lane + j: the first whose running mass exceeds the target,
+    // else (rounding, or pk.beyond) the last with mass
+    double in[4], C = pk.base;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) in[k] = warp_scan((r[4 * k] + r[4 * k + 1]) + (r[4 * k + 2] + r[4 * k + 3]));
+    int tok = -1;
+    bool hit = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double up = __shfl_up_sync(0xffffffffu, in[k], 1);
+        const double c0 = C + (lane ? up : 0.0), c1 = c0 + r[4 * k], c2 = c1 + r[4 * k + 1], c3 = c2 + r[4 * k + 2], c4 = c3 + r[4 * k + 3];
+        const unsigned pos = (r[4 * k] > 0.0 ? 1u : 0u) | (r[4 * k + 1] > 0.0 ? 2u : 0u) | (r[4 * k + 2] > 0.0 ? 4u : 0u) |
+                             (r[4 * k + 3] > 0.0 ? 8u : 0u);
+        const unsigned over = pk.beyond ? 0u : pos & ((c1 > pk.target ? 1u : 0u) | (c2 > pk.target ? 2u : 0u) |
+                                                      (c3 > pk.target ? 4u : 0u) | (c4 > pk.target ? 8u : 0u));
+        const unsigned cross = __ballot_sync(0xffffffffu, over != 0), mass = __ballot_sync(0xffffffffu, pos != 0);
+        const int at = cross ? __ffs(cross) - 1 : mass ? 31 - __clz(mass) : 0;
+        const int j = __shfl_sync(0xffffffffu, over ? __ffs(over) - 1 : 31 - __clz(pos | 1u), at);
+        if (!hit && mass) {
+            tok = 512 * g + 128 * k + 4 * at + j;
+            hit = cross != 0;
+        }
+        C += shfl_f64(in[k], 31);
+    }
+    if (lane == 0) {
+        P.token[b] = tok;
+        if (P.flags) P.flags[b] = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u);
+    }
+}
+
 // ---- one shard of the vocabulary ---------------------------------------------------------------
 //
 // The draw over a row that is spread over G shards takes two steps with one small exchange
@@ -641,6 +767,9 @@ bool quads_aligned(const void *base, int64_t stride, int esz)
 template <typename RV, bool kShift>
 cudaError_t launch_resample_as(const ResampleParams &P, unsigned grid, cudaStream_t stream)
 {
+    if (P.cluster_threads)
+        return launch_pdl(resample_cluster_kernel<kShift, RV>, (unsigned)(P.B * P.n_ctas), (unsigned)P.cluster_threads, stream, P,
+                          0, (unsigned)P.n_ctas);
     const cudaError_t e = launch_pdl(resample_mass_kernel<kShift, RV>, grid, kThreads, stream, P);
     return e != cudaSuccess ? e : launch_pdl(resample_draw_kernel<kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P);
 }
@@ -663,6 +792,16 @@ cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t str
     P.n_ctas = (int)((n_tiles + P.tiles - 1) / P.tiles);
     const unsigned long long grid = (unsigned long long)P.B * (unsigned long long)P.n_ctas;
     if (grid > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+    // small launches: a cluster of CTAs per sequence, while one wave of them holds the batch
+    const long long warps = ((long long)P.V + 511) / 512;  // 512 entries each
+    const int per_cta = warps <= 8 * kClusterMax ? 8 : 16;
+    long long ctas = 1;
+    while (ctas * per_cta < warps) ctas *= 2;
+    P.cluster_threads = 0;
+    if (ctas <= kClusterMax && P.B * ctas <= (per_cta == 8 ? kClusterWave : kClusterWave / 4) && !P.test_drop_seq_plus1) {
+        P.n_ctas = (int)ctas;
+        P.cluster_threads = 32 * (int)(warps < per_cta ? warps : per_cta);
+    }
     if (P.logits) {
         return P.logits_dtype == DSSD_BF16 ? launch_resample<RowLogits<DSSD_BF16>>(P, (unsigned)grid, stream)
                                            : launch_resample<RowLogits<DSSD_F32>>(P, (unsigned)grid, stream);

@@ -17,50 +17,51 @@ static_assert(kFoldRows == 32, "one lane of warp 0 per position");
 struct FoldShared {
     float R[kFoldRows];
     double S[kFoldRows];
-    int bad[kFoldRows];   // bit 0: a NaN among the sums, bit 1: a sum is missing
+    int missing[kFoldRows];
     int n;                // accepted length; -1: no verdict
     float ref2, invS;     // row n
 };
 
-// The sum of one row, formed by kFoldLanes neighbouring threads (sub = 0 .. kFoldLanes - 1 within
-// the row); the result is the same in all of them.  Fixed order: deterministic.
+// The sum of one row, formed by kFoldLanes neighbouring threads (sub = 0 .. kFoldLanes - 1 within the row):
+// the largest reference first, then float64 terms s * 2^(ref - R) by exponent arithmetic, added in a fixed
+// order.  The result, sum_v 2^(l_v c1) = S * 2^R, is the same in all threads of the row; a NaN or an
+// infinite sum stays one, a row without mass gives S = 0.  Short, because every emission CTA of a small
+// launch runs it.
 __device__ __forceinline__ void row_total(const unsigned long long *part, int runs, int sub, bool live, float &R, double &S,
-                                          int &bad)
+                                          bool &missing)
 {
-    R = DSSD_NEG_INF;
-    S = 0.0;
-    bad = 0;
-    bool nan = false;
-    for (int k0 = 0; k0 < runs; k0 += 4 * kFoldLanes) {
-        unsigned long long w[4];
+    constexpr int kHeld = 2;  // words in registers: rows of up to 16 runs need no second look
+    unsigned long long w[kHeld];
+    float top = DSSD_NEG_INF;
+    missing = false;
+    auto word = [&](int k) { return live && k < runs ? ld_after(part + k) : 0ull; };
+    auto look = [&](unsigned long long x) {
+        missing |= x == kNoPartial;
+        if (__uint_as_float((unsigned)(x >> 32)) > 0.f) top = fmaxf(top, __uint_as_float((unsigned)x));
+    };
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int k = k0 + u * kFoldLanes + sub;
-            w[u] = (live && k < runs) ? ld_after(part + k) : 0ull;
-        }
+    for (int u = 0; u < kHeld; ++u) w[u] = word(u * kFoldLanes + sub);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (w[u] == kNoPartial) bad |= 2;
-            else add_partial(R, S, nan, __uint_as_float((unsigned)w[u]), (double)__uint_as_float((unsigned)(w[u] >> 32)));
-        }
-    }
-    if (nan) bad |= 1;
+    for (int u = 0; u < kHeld; ++u) look(w[u]);
+    for (int k = kHeld * kFoldLanes + sub; k < runs; k += kFoldLanes) look(word(k));
+#pragma unroll
+    for (int o = 1; o < kFoldLanes; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    double s = 0.0;
+    auto add = [&](unsigned long long x) {
+        const float v = __uint_as_float((unsigned)(x >> 32));
+        if (v > 0.f && v < INFINITY) s += scale_pow2((double)v, __uint_as_float((unsigned)x) - top);
+        else if (v != 0.f) s += (double)v;
+    };
+#pragma unroll
+    for (int u = 0; u < kHeld; ++u) add(w[u]);
+    for (int k = kHeld * kFoldLanes + sub; k < runs; k += kFoldLanes) add(word(k));
 #pragma unroll
     for (int o = 1; o < kFoldLanes; o <<= 1) {
-        const float R2 = __shfl_xor_sync(0xffffffffu, R, o);
-        const double S2 = __shfl_xor_sync(0xffffffffu, S, o);
-        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-        bool dummy = false;
-        if (R2 > R) {  // the same two operands in both threads, so both get the same bits
-            double Sx = S2;
-            float Rx = R2;
-            add_partial(Rx, Sx, dummy, R, S);
-            R = Rx;
-            S = Sx;
-        } else {
-            add_partial(R, S, dummy, R2, S2);
-        }
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        missing |= __shfl_xor_sync(0xffffffffu, (int)missing, o) != 0;
     }
+    R = top;
+    S = s;
 }
 
 // Run by all kThreads threads of a CTA; the results are in `sh` (n, ref2, invS) when it returns.
@@ -91,20 +92,19 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
             const int r = base + tid / kFoldLanes;
             float R;
             double S;
-            int bad;
-            row_total(P.part + (size_t)(row0 + (r <= P.gamma ? r : 0)) * P.runs, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, bad);
+            bool missing;
+            row_total(P.part + (size_t)(row0 + (r <= P.gamma ? r : 0)) * P.runs, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, missing);
             if (base) __syncthreads();  // warp 0 has read the previous rows
             if (tid % kFoldLanes == 0) {
                 sh.R[tid / kFoldLanes] = R;
                 sh.S[tid / kFoldLanes] = S;
-                sh.bad[tid / kFoldLanes] = bad;
+                sh.missing[tid / kFoldLanes] = missing;
             }
         }
         __syncthreads();
         if (warp == 0) {
-            const int bad = sh.bad[lane];
             float Rs, invS;
-            const unsigned bits = judge_position(P, b, i, live, writer, sh.R[lane], sh.S[lane], (bad & 1) != 0, live && (bad & 2),
+            const unsigned bits = judge_position(P, b, i, live, writer, sh.R[lane], sh.S[lane], false, live && sh.missing[lane],
                                                  x, zx, qx, ux, Rs, invS);
             const unsigned rej = __ballot_sync(0xffffffffu, live && i < P.gamma && !(bits & kBitAccept));
             if (rej && n == P.gamma) n = base + __ffs(rej) - 1;

@@ -353,11 +353,11 @@ __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_con
     }
     float R;
     double S;
-    int bad;
-    row_total(P.part + (size_t)(live ? row : 0) * P.runs, P.runs, sub, live, R, S, bad);
+    bool missing;
+    row_total(P.part + (size_t)(live ? row : 0) * P.runs, P.runs, sub, live, R, S, missing);
     if (live && sub == 0) {
         P.shard_ref[row] = R == DSSD_NEG_INF ? 0.f : R;
-        P.shard_sum[row] = bad ? (double)__int_as_float(0x7fc00000) : S;
+        P.shard_sum[row] = missing || S != S ? (double)__int_as_float(0x7fc00000) : S;
         if (i < P.gamma) P.shard_tok_logit[(size_t)b * P.gamma + i] = (x >= 0 && x < (long long)P.V) ? zx : __int_as_float(0x7fc00000);
     }
 }

@@ -19,7 +19,8 @@ def B():
 @pytest.mark.parametrize("Bn,gamma,V,half", [
     (5, 2, 1, False), (5, 2, 1023, False), (5, 2, 1024, True), (5, 1, 1025, False), (5, 3, 4095, True),
     (5, 2, 4096, False), (5, 2, 4097, False), (7, 1, 4100, True), (3, 1, 8192, False), (3, 1, 12289, False),
-    (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
+    (9, 2, 511, False), (9, 2, 513, True), (25, 1, 32768, False), (26, 1, 32768, False), (3, 2, 32769, False), (6, 1, 65536, True),
+    (7, 1, 65536, False), (4, 2, 65537, False), (200, 1, 900, False), (201, 1, 900, True), (5, 1, 50257, True), (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
     (6, 2, 9001, False), (6, 3, 9002, True), (7, 2, 9003, True), (6, 2, 9003, False), (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True),
 ])
 def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
@@ -48,4 +49,24 @@ def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
     # both sides add V float64 terms, in different orders: V * 2^-53 relative each
     bad = (tok != ref["token"]) & ~(ref["margin_cdf"] < V * 2.0 ** -52)
     assert not bad.any(), (np.nonzero(bad)[0][:8], tok[bad][:8], ref["token"][bad][:8])
+    assert (out["flags"].cpu().numpy().astype(np.uint32) == ref["flags"]).all()
+
+
+@pytest.mark.parametrize("Bn,V", [(5, 3000), (3, 20011), (40, 70001)])
+def test_fallback_and_invalid_lengths(B, oracle_mod, Bn, V):
+    """No residual mass (p == q): drawn from p; lengths outside [0, gamma] and rows without mass: token -1; one
+    cluster per sequence and the two-kernel path."""
+    gamma = 2
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    p = torch.softmax(2.0 * torch.randn(Bn, V, generator=gen, device="cuda"), dim=-1)
+    q = p.view(Bn, 1, V).repeat(1, gamma, 1).contiguous()
+    n = (torch.arange(Bn, device="cuda") % (gamma + 1)).to(torch.int32)
+    n[0], n[1] = -1, gamma + 1
+    p[2] = 0.0
+    u = torch.rand(Bn, generator=gen, device="cuda").clamp_(max=1.0 - 2.0 ** -24)
+    out = B.dssd_device_resample(p, q, n, u, gamma)
+    torch.cuda.synchronize()
+    ref = oracle_mod.device_resample(p.cpu().numpy(), q.cpu().numpy(), n.cpu().numpy(), u.cpu().numpy(), gamma)
+    near = ref["margin_cdf"] < V * 2.0 ** -52  # V float64 additions in another order
+    assert ((out["token"].cpu().numpy() == ref["token"]) | near).all()
     assert (out["flags"].cpu().numpy().astype(np.uint32) == ref["flags"]).all()
