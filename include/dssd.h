@@ -37,7 +37,7 @@
  *   - Every call with device pointers only can be recorded in a CUDA graph by stream capture
  *     (it enqueues kernels and nothing else); dssd_device_resample_static provided one call of it was
  *     made on that device before the capture began.
- *     dssd_round_host synchronises the stream in the middle and cannot be captured.
+ *     dssd_round_host waits for the accepted lengths and cannot be captured.
  *   - Buffers need only their natural alignment; 16-byte aligned rows take the fast path.
  *   - A status other than DSSD_OK means nothing was enqueued (except DSSD_ERR_CUDA, after
  *     which the outputs are undefined).  Data-dependent anomalies never fault or trap: they
@@ -213,11 +213,12 @@ size_t dssd_round_host_arena_bytes(int B, int gamma, int V, dssd_dtype dtype);
  * `cuda_stream`.  The host buffers must stay valid until the stream has finished; use pinned
  * memory for the copies to be asynchronous.
  *
- * Of the draft distributions only the rows the device half reads cross the bus: the call waits
- * on the host for the accepted lengths (one cudaStreamSynchronize in the middle; accept_len is
- * final when the call returns) and then uploads row Q_n of every sequence with a rejection,
- * B * V * 4 bytes at most instead of B * gamma * V * 4.  Because of that wait the call cannot be
- * made while the stream is being captured (DSSD_ERR_CUDA then).
+ * Of the draft distributions only the rows the device half reads cross the bus, B * V * 4 bytes at
+ * most instead of B * gamma * V * 4: row Q_n of every sequence with a rejection.  Pinned host
+ * buffers are mapped, and the kernels read those rows (and the short arrays) and write the results
+ * over the bus themselves; pageable ones are copied.  The call waits on the host for the accepted
+ * lengths (accept_len is final when the call returns) and therefore cannot be made while the stream
+ * is being captured (DSSD_ERR_CUDA then).
  *
  * host inputs:  target_logits [B, gamma+1, V] contiguous, draft_tokens, draft_q_tok, uniforms
  *               [B, gamma], draft_q [B, gamma, V], uniforms_rs [B]

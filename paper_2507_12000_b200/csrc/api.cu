@@ -4,8 +4,10 @@
 
 #include "device_resample.h"
 #include "dssd.h"
+#include "dssd_device.cuh"
 #include "dssd_test_hooks.h"
 #include "edge_verify.h"
+#include "launch.h"
 #include "shard_verify.h"
 #include "topk_verify.h"
 
@@ -66,7 +68,8 @@ dssd_status edge_verify_any(const void *target_logits, dssd_dtype dtype, int64_t
                             const int32_t *draft_tokens, const float *draft_q_tok, const float *uniforms,
                             float temperature, int B, int gamma, int V, int32_t *accept_len, float *p_row,
                             uint16_t *p_row16, float *p_tok, float *lse, uint32_t *flags, void *workspace,
-                            size_t workspace_bytes, void *cuda_stream, long long drop_row_plus1 = 0)
+                            size_t workspace_bytes, void *cuda_stream, long long drop_row_plus1 = 0,
+                            int32_t *accept_copy = nullptr)
 {
     t_last_cuda_error = 0;
     dssd_status st = check_sizes(B, gamma, V);
@@ -95,6 +98,7 @@ dssd_status edge_verify_any(const void *target_logits, dssd_dtype dtype, int64_t
     P.gamma = gamma;
     P.V = V;
     P.accept_len = accept_len;
+    P.accept_copy = accept_copy;
     P.p_row = p_row;
     P.p_row16 = p_row16;
     P.p_tok = p_tok;
@@ -636,6 +640,107 @@ dssd_status dssd_resample_shard_draw(const double *masses, int G, int g, int v_b
     return e == cudaSuccess ? DSSD_OK : cuda_fail(e);
 }
 
+}  // extern "C"
+
+namespace {
+
+// A host array as the GPU reaches it: pinned memory is mapped, so kernels read the rows they need over the
+// bus, and write their results there, without copies of their own.  nullptr for pageable memory.
+template <class T>
+T *mapped(T *host, size_t count)
+{
+    if (!host || count == 0) return nullptr;
+    const char *first = reinterpret_cast<const char *>(host), *last = first + count * sizeof(T) - 1;
+    cudaPointerAttributes a, z;
+    if (cudaPointerGetAttributes(&a, first) != cudaSuccess || cudaPointerGetAttributes(&z, last) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
+    if (static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) != last - first) return nullptr;
+    return static_cast<T *>(a.devicePointer);
+}
+
+// The short input arrays of a round on host buffers, brought to the GPU by one kernel that reads the mapped
+// arrays over the bus (a copy each costs the host 3 us and the stream 2 to 4; a read by the kernels that use
+// them waits for the bus, about 5 us, once in each of them).  Pageable and long arrays are copied.
+struct StageParams {
+    const uint32_t *src[4];
+    uint32_t *dst[4];
+    unsigned end[4];  // words up to and including array i
+};
+constexpr unsigned kStageWords = 16384;  // of one array; beyond, a copy is as quick
+__global__ void __launch_bounds__(256) stage_kernel(const __grid_constant__ StageParams P)
+{
+    dssd::pdl_wait();
+    dssd::pdl_trigger();
+    const unsigned w = blockIdx.x * 256 + threadIdx.x;
+    unsigned begin = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (w >= begin && w < P.end[i]) P.dst[i][w - begin] = dssd::ld_after_u32(P.src[i] + (w - begin));
+        begin = P.end[i];
+    }
+}
+
+class Stage {
+public:
+    explicit Stage(cudaStream_t stream) : s(stream) {}
+    // `count` words of `host` to `device`; call run() before they are used
+    template <class T>
+    cudaError_t add(const T *host, size_t count, T *device)
+    {
+        static_assert(sizeof(T) == 4, "words");
+        const T *m = count <= kStageWords ? mapped(host, count) : nullptr;
+        if (!m) return count ? cudaMemcpyAsync(device, host, count * sizeof(T), cudaMemcpyHostToDevice, s) : cudaSuccess;
+        P.src[n] = reinterpret_cast<const uint32_t *>(m);
+        P.dst[n] = reinterpret_cast<uint32_t *>(device);
+        total += (unsigned)count;
+        P.end[n++] = total;
+        return cudaSuccess;
+    }
+    cudaError_t run()
+    {
+        if (!total) return cudaSuccess;
+        for (int i = n; i < 4; ++i) P.end[i] = total;
+        return dssd::launch_pdl(stage_kernel, (total + 255) / 256, 256u, s, P);
+    }
+
+private:
+    cudaStream_t s;
+    StageParams P{};
+    unsigned total = 0;
+    int n = 0;
+};
+
+// An output array on the GPU: the mapped host array itself, else `device`, which `fetch` copies back.
+template <class T>
+struct Result {
+    T *host, *device, *on_gpu;
+    size_t count;
+    Result(T *h, T *d, size_t n) : host(h), device(d), on_gpu(d), count(n)
+    {
+        if (T *m = mapped(h, n)) on_gpu = m;
+    }
+    cudaError_t fetch(cudaStream_t s) const
+    {
+        if (!host || on_gpu != device) return cudaSuccess;
+        return cudaMemcpyAsync(host, device, count * sizeof(T), cudaMemcpyDeviceToHost, s);
+    }
+};
+
+struct Event {
+    cudaEvent_t e = nullptr;
+    ~Event()
+    {
+        if (e) cudaEventDestroy(e);
+    }
+};
+
+}  // namespace
+
+extern "C" {
+
 size_t dssd_round_host_arena_bytes(int B, int gamma, int V, dssd_dtype dtype)
 {
     if (check_sizes(B, gamma, V) != DSSD_OK) return 0;
@@ -702,33 +807,43 @@ dssd_status dssd_round_host(const void *target_logits, dssd_dtype dtype,
 #define DSSD_TRY(call) \
     if ((e = (call)) != cudaSuccess) return cuda_fail(e)
     DSSD_TRY(cudaMemcpyAsync(d_logits, target_logits, Bz * (g + 1) * Vz * esz, cudaMemcpyHostToDevice, s));
-    if (gamma > 0) {
-        DSSD_TRY(cudaMemcpyAsync(d_tok_in, draft_tokens, Bz * g * 4, cudaMemcpyHostToDevice, s));
-        DSSD_TRY(cudaMemcpyAsync(d_qtok, draft_q_tok, Bz * g * 4, cudaMemcpyHostToDevice, s));
-        DSSD_TRY(cudaMemcpyAsync(d_u, uniforms, Bz * g * 4, cudaMemcpyHostToDevice, s));
-    }
-    DSSD_TRY(cudaMemcpyAsync(d_urs, uniforms_rs, Bz * 4, cudaMemcpyHostToDevice, s));
-    st = dssd_edge_verify(d_logits, dtype, (int64_t)V, gamma ? d_tok_in : nullptr, gamma ? d_qtok : nullptr,
-                          gamma ? d_u : nullptr, temperature, B, gamma, V, d_n, d_prow, nullptr, nullptr,
-                          d_ef, d_ws_e, ws_e, cuda_stream);
+    Stage stage(s);
+    DSSD_TRY(stage.add(draft_tokens, Bz * g, d_tok_in));
+    DSSD_TRY(stage.add(draft_q_tok, Bz * g, d_qtok));
+    DSSD_TRY(stage.add(uniforms, Bz * g, d_u));
+    DSSD_TRY(stage.add(uniforms_rs, Bz, d_urs));
+    DSSD_TRY(stage.run());
+    const Result<uint32_t> r_ef(edge_flags, d_ef, Bz), r_rf(rs_flags, d_rf, Bz);
+    const Result<int32_t> r_token(token, d_token, Bz);
+    int32_t *n_copy = mapped(accept_len, Bz);
+    st = edge_verify_any(d_logits, dtype, (int64_t)V, gamma ? d_tok_in : nullptr, gamma ? d_qtok : nullptr, gamma ? d_u : nullptr, temperature, B, gamma, V, d_n, d_prow, nullptr, nullptr,
+                         nullptr, r_ef.on_gpu, d_ws_e, ws_e, cuda_stream, 0, n_copy);
     if (st != DSSD_OK) return st;
-    // The device half reads row Q_n only: wait for the accepted lengths, then upload those rows
-    // (each to its place in the [B, gamma, V] array, the rest of which is never read).
-    DSSD_TRY(cudaMemcpyAsync(accept_len, d_n, Bz * 4, cudaMemcpyDeviceToHost, s));
-    DSSD_TRY(cudaStreamSynchronize(s));
-    for (size_t b = 0; b < Bz; ++b) {
-        const int n = accept_len[b];
-        if (n < 0 || n >= gamma) continue;  // bonus draw (no Q row), or no draw at all
-        const size_t off = (b * g + (size_t)n) * Vz;
-        DSSD_TRY(cudaMemcpyAsync(d_q + off, draft_q + off, Vz * 4, cudaMemcpyHostToDevice, s));
+    if (!n_copy) DSSD_TRY(cudaMemcpyAsync(accept_len, d_n, Bz * 4, cudaMemcpyDeviceToHost, s));
+    Event edge_done;
+    DSSD_TRY(cudaEventCreateWithFlags(&edge_done.e, cudaEventDisableTiming));
+    DSSD_TRY(cudaEventRecord(edge_done.e, s));
+    // The device half reads row Q_n only.  Mapped rows it reads over the bus itself; of pageable ones the host
+    // uploads those rows once the accepted lengths are back (each to its place in the [B, gamma, V]
+    // array, the rest of which is never read).
+    const float *q = gamma ? mapped(draft_q, Bz * g * Vz) : nullptr;
+    if (gamma && !q) {
+        q = d_q;
+        DSSD_TRY(cudaEventSynchronize(edge_done.e));
+        for (size_t b = 0; b < Bz; ++b) {
+            const int n = accept_len[b];
+            if (n < 0 || n >= gamma) continue;  // bonus draw (no Q row), or no draw at all
+            const size_t off = (b * g + (size_t)n) * Vz;
+            DSSD_TRY(cudaMemcpyAsync(d_q + off, draft_q + off, Vz * 4, cudaMemcpyHostToDevice, s));
+        }
     }
-    st = dssd_device_resample(d_prow, gamma ? d_q : nullptr, d_n, d_urs, B, gamma, V, d_token, d_rf, d_ws_r,
-                              ws_r, cuda_stream);
+    st = dssd_device_resample(d_prow, q, d_n, d_urs, B, gamma, V, r_token.on_gpu, r_rf.on_gpu, d_ws_r, ws_r, cuda_stream);
     if (st != DSSD_OK) return st;
-    DSSD_TRY(cudaMemcpyAsync(token, d_token, Bz * 4, cudaMemcpyDeviceToHost, s));
-    if (edge_flags) DSSD_TRY(cudaMemcpyAsync(edge_flags, d_ef, Bz * 4, cudaMemcpyDeviceToHost, s));
-    if (rs_flags) DSSD_TRY(cudaMemcpyAsync(rs_flags, d_rf, Bz * 4, cudaMemcpyDeviceToHost, s));
+    DSSD_TRY(r_token.fetch(s));
+    DSSD_TRY(r_ef.fetch(s));
+    DSSD_TRY(r_rf.fetch(s));
     if (p_row) DSSD_TRY(cudaMemcpyAsync(p_row, d_prow, Bz * Vz * 4, cudaMemcpyDeviceToHost, s));
+    DSSD_TRY(cudaEventSynchronize(edge_done.e));  // accept_len is final when the call returns
 #undef DSSD_TRY
     return DSSD_OK;
 }
@@ -801,25 +916,34 @@ dssd_status dssd_round_host_topk(const void *target_logits, dssd_dtype dtype,
 #define DSSD_TRY(call) \
     if ((e = (call)) != cudaSuccess) return cuda_fail(e)
     DSSD_TRY(cudaMemcpyAsync(d_logits, target_logits, Bz * (g + 1) * Vz * esz, cudaMemcpyHostToDevice, s));
-    if (gamma > 0) {
-        DSSD_TRY(cudaMemcpyAsync(d_tok_in, draft_tokens, Bz * g * 4, cudaMemcpyHostToDevice, s));
-        DSSD_TRY(cudaMemcpyAsync(d_qtok, draft_q_tok, Bz * g * 4, cudaMemcpyHostToDevice, s));
-        DSSD_TRY(cudaMemcpyAsync(d_u, uniforms, Bz * g * 4, cudaMemcpyHostToDevice, s));
+    Stage stage(s);
+    DSSD_TRY(stage.add(draft_tokens, Bz * g, d_tok_in));
+    DSSD_TRY(stage.add(draft_q_tok, Bz * g, d_qtok));
+    DSSD_TRY(stage.add(uniforms, Bz * g, d_u));
+    DSSD_TRY(stage.add(uniforms_rs, Bz, d_urs));
+    DSSD_TRY(stage.run());
+    const int32_t *qi = nullptr;
+    const float *qv = nullptr;
+    // (of these lists one per sequence is read, once)
+    if (gamma > 0 && !(qi = mapped(q_idx, Bz * g * kz))) {
         DSSD_TRY(cudaMemcpyAsync(d_qidx, q_idx, Bz * g * kz * 4, cudaMemcpyHostToDevice, s));
-        DSSD_TRY(cudaMemcpyAsync(d_qval, q_val, Bz * g * kz * 4, cudaMemcpyHostToDevice, s));
+        qi = d_qidx;
     }
-    DSSD_TRY(cudaMemcpyAsync(d_urs, uniforms_rs, Bz * 4, cudaMemcpyHostToDevice, s));
-    st = dssd_edge_verify_topk(d_logits, dtype, (int64_t)V, gamma ? d_tok_in : nullptr, gamma ? d_qtok : nullptr,
-                               gamma ? d_u : nullptr, temperature, B, gamma, V, k, d_n, d_pidx, d_pval, nullptr,
-                               d_ef, d_ws, ws, cuda_stream);
+    if (gamma > 0 && !(qv = mapped(q_val, Bz * g * kz))) {
+        DSSD_TRY(cudaMemcpyAsync(d_qval, q_val, Bz * g * kz * 4, cudaMemcpyHostToDevice, s));
+        qv = d_qval;
+    }
+    const Result<uint32_t> r_ef(edge_flags, d_ef, Bz), r_rf(rs_flags, d_rf, Bz);
+    const Result<int32_t> r_token(token, d_token, Bz);
+    st = dssd_edge_verify_topk(d_logits, dtype, (int64_t)V, gamma ? d_tok_in : nullptr, gamma ? d_qtok : nullptr, gamma ? d_u : nullptr, temperature, B, gamma, V, k, d_n, d_pidx, d_pval,
+                               nullptr, r_ef.on_gpu, d_ws, ws, cuda_stream);
     if (st != DSSD_OK) return st;
-    st = dssd_device_resample_topk(d_pidx, d_pval, gamma ? d_qidx : nullptr, gamma ? d_qval : nullptr, d_n, d_urs, B,
-                                   gamma, k, d_token, d_rf, cuda_stream);
+    st = dssd_device_resample_topk(d_pidx, d_pval, qi, qv, d_n, d_urs, B, gamma, k, r_token.on_gpu, r_rf.on_gpu, cuda_stream);
     if (st != DSSD_OK) return st;
     DSSD_TRY(cudaMemcpyAsync(accept_len, d_n, Bz * 4, cudaMemcpyDeviceToHost, s));
-    DSSD_TRY(cudaMemcpyAsync(token, d_token, Bz * 4, cudaMemcpyDeviceToHost, s));
-    if (edge_flags) DSSD_TRY(cudaMemcpyAsync(edge_flags, d_ef, Bz * 4, cudaMemcpyDeviceToHost, s));
-    if (rs_flags) DSSD_TRY(cudaMemcpyAsync(rs_flags, d_rf, Bz * 4, cudaMemcpyDeviceToHost, s));
+    DSSD_TRY(r_token.fetch(s));
+    DSSD_TRY(r_ef.fetch(s));
+    DSSD_TRY(r_rf.fetch(s));
     if (p_idx) DSSD_TRY(cudaMemcpyAsync(p_idx, d_pidx, Bz * kz * 4, cudaMemcpyDeviceToHost, s));
     if (p_val) DSSD_TRY(cudaMemcpyAsync(p_val, d_pval, Bz * kz * 4, cudaMemcpyDeviceToHost, s));
 #undef DSSD_TRY

@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const
     pdl_wait();
     pdl_trigger();
     const int n = ld_after(P.accept_len + b);
-    const float u = ld_after(P.uniforms + b);
+    const float u = warp == 0 ? ld_after(P.uniforms + b) : 0.f;
     const long long base = 512ll * g;
     WarpQuads<typename RV::Q, 4, kShift> a;
     if (RV::kFixed) a.load(RV::make(P, b, 0).row, P.V, base, RV::kFill);  // (on its way before n is back)

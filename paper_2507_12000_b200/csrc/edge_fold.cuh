@@ -124,6 +124,7 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
         sh.invS = invS_n;
         if (writer) {
             P.accept_len[b] = n;
+            if (P.accept_copy) P.accept_copy[b] = n;
             if (P.flags) P.flags[b] = fl;
             ReadySlot s;
             s.b = (int)b;

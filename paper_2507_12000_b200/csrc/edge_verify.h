@@ -42,6 +42,7 @@ struct EdgeParams {
     float c1;  // log2(e) / T, rounded to float32; the kernels' temperature scaling throughout
     int B, gamma, V;
     int32_t *accept_len;
+    int32_t *accept_copy;  // optional second copy of accept_len (in host memory that the GPU reaches)
     float *p_row;          // float32 payload, or
     uint16_t *p_row16;     // IEEE binary16 payload (at most one of the two is set)
     float *p_tok;

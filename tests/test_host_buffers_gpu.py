@@ -1,0 +1,61 @@
+"""The rounds on host buffers, pinned (read and written over the bus by the kernels), pageable (copied) and
+mixed, short arrays and arrays beyond what the staging kernel takes: the same results as the device calls."""
+import pytest
+import torch
+
+import dssd_inputs as di
+from gpu_util import to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2507_12000_b200 import binding
+
+    return binding
+
+
+def _host(g, pin):
+    out = {}
+    for i, (k, v) in enumerate(g.items()):
+        t = v.cpu()
+        out[k] = t.pin_memory() if pin == "all" or (pin == "some" and i % 2) else t
+    return out
+
+
+@pytest.mark.parametrize("pin", ["all", "none", "some"])
+@pytest.mark.parametrize("Bn,gamma,V,dtype", [(3, 2, 4001, "bf16"), (40, 3, 9000, "f32"), (9, 0, 3000, "f32"), (6000, 3, 64, "bf16")])
+def test_dense_round(B, pin, Bn, gamma, V, dtype):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, seed=Bn + V)
+    g = to_device(di.generate(w, threads=8))
+    ev = B.dssd_edge_verify(g["target_logits"], g["draft_tokens"], g["draft_q_tok"], g["uniforms"], w.temperature)
+    rs = B.dssd_device_resample(ev["p_row"], g["draft_q"], ev["accept_len"], g["uniforms_rs"], gamma)
+    arena = torch.full((B.dssd_round_host_arena_bytes(Bn, gamma, V, B.DSSD_BF16 if dtype == "bf16" else B.DSSD_F32),), 0x5A,
+                       dtype=torch.uint8, device="cuda")
+    out = {k: torch.zeros(Bn, dtype=torch.int32) for k in ("accept_len", "token", "edge_flags", "rs_flags")}
+    out["p_row"] = torch.zeros(Bn, V)
+    out = _host(out, pin)
+    got = B.dssd_round_host(_host(g, pin), w.temperature, arena, out=out)
+    n_at_return = got["accept_len"].clone()
+    torch.cuda.synchronize()
+    assert torch.equal(n_at_return, ev["accept_len"].cpu())  # final when the call returns
+    assert torch.equal(got["token"], rs["token"].cpu()) and torch.equal(got["p_row"], ev["p_row"].cpu())
+    assert torch.equal(got["edge_flags"], ev["flags"].cpu()) and torch.equal(got["rs_flags"], rs["flags"].cpu())
+
+
+@pytest.mark.parametrize("pin", ["all", "none", "some"])
+def test_topk_round(B, pin):
+    k = 10
+    w = di.custom(B=20, gamma=3, V=9001, dtype="bf16", temperature=0.9, sigma_d=0.5, seed=3)
+    g = to_device(di.generate_topk(w, k, threads=8))
+    ev = B.dssd_edge_verify_topk(g["target_logits"], g["draft_tokens"], g["draft_q_tok"], g["uniforms"], w.temperature, k)
+    rs = B.dssd_device_resample_topk(ev["p_idx"], ev["p_val"], g["q_idx"], g["q_val"], ev["accept_len"], g["uniforms_rs"], w.gamma)
+    arena = torch.full((B.dssd_round_host_topk_arena_bytes(w.B, w.gamma, w.V, k, B.DSSD_BF16),), 0x5A, dtype=torch.uint8, device="cuda")
+    out = {n: torch.zeros(w.B, dtype=torch.int32) for n in ("accept_len", "token", "edge_flags", "rs_flags")}
+    out["p_idx"], out["p_val"] = torch.zeros(w.B, k, dtype=torch.int32), torch.zeros(w.B, k)
+    got = B.dssd_round_host_topk(_host(g, pin), w.temperature, k, arena, out=_host(out, pin))
+    torch.cuda.synchronize()
+    for name, want in (("accept_len", ev["accept_len"]), ("token", rs["token"]), ("edge_flags", ev["flags"]), ("rs_flags", rs["flags"]),
+                       ("p_idx", ev["p_idx"]), ("p_val", ev["p_val"])):
+        assert torch.equal(got[name], want.cpu()), name
