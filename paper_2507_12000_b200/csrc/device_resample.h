@@ -54,6 +54,7 @@ struct ShardResampleParams {
     const int32_t *accept_len;
     int B, gamma, V;
     int n_sub;              // chunk sums per sequence
+    int cluster;            // CTAs per sequence of the cluster kernel
     double *chunk_sum;      // scratch [B, n_sub, 2]: residual mass and plain mass of every chunk
     // mass
     double *mass;           // [B, 2] out: the slice's residual mass and plain mass

@@ -19,8 +19,8 @@
 
 #include "dssd_device.cuh"
 #include "edge_fold.cuh"
+#include "emit.cuh"
 #include "launch.h"
-#include "quads.cuh"
 
 namespace dssd {
 
@@ -211,81 +211,7 @@ __global__ void __launch_bounds__(kLseThreads, 8) edge_lse_kernel(const __grid_c
     }
 }
 
-// ---- emission --------------------------------------------------------------------------------
-
-// default stores: the rows written last are still in L2 when the draw reads them
-__device__ __forceinline__ void store_quad(float *o, float a, float b, float c, float d)
-{
-    *reinterpret_cast<float4 *>(o) = make_float4(a, b, c, d);
-}
-__device__ __forceinline__ void store_quad(uint16_t *o, float a, float b, float c, float d)
-{
-    *reinterpret_cast<uint2 *>(o) = make_uint2(pack_half2(a, b), pack_half2(c, d));
-}
-__device__ __forceinline__ void store_one(float *o, float a) { *o = a; }
-__device__ __forceinline__ void store_one(uint16_t *o, float a) { *o = to_half_bits(a); }
-
-// out[0..3] = 2^(z * c1 - ref2) * invS for four logits, as two packed pairs
-template <class OUT>
-__device__ __forceinline__ void emit_quad(OUT *out, float z0, float z1, float z2, float z3, f32x2 cc, f32x2 nn, f32x2 ss)
-{
-    float a, b, c, d;
-    unpack2(fma2(pack2(z0, z1), cc, nn), a, b);
-    unpack2(fma2(pack2(z2, z3), cc, nn), c, d);
-    unpack2(mul2(pack2(ex2(a), ex2(b)), ss), a, b);
-    unpack2(mul2(pack2(ex2(c), ex2(d)), ss), c, d);
-    store_quad(out, a, b, c, d);
-}
-
-__device__ __forceinline__ void emit_raw(float *out, const uint2 &w, f32x2 cc, f32x2 nn, f32x2 ss)
-{
-    emit_quad(out, bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y), cc, nn, ss);
-}
-__device__ __forceinline__ void emit_raw(uint16_t *out, const uint2 &w, f32x2 cc, f32x2 nn, f32x2 ss)
-{
-    emit_quad(out, bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y), cc, nn, ss);
-}
-template <class OUT>
-__device__ __forceinline__ void emit_raw(OUT *out, const uint4 &w, f32x2 cc, f32x2 nn, f32x2 ss)
-{
-    emit_quad(out, __uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w), cc, nn, ss);
-}
-
-template <int DT>
-struct LogitQuads {
-    typedef Quads32 Q;
-};
-template <>
-struct LogitQuads<DSSD_BF16> {
-    typedef Quads16 Q;
-};
-
-// OUT[e] for the entries [e0, e0 + kEmitTile) of a row that lie in [0, V), where e0 makes the output's quads
-// aligned (it may be negative).  The logits' quads may lie on any element boundary (quads.cuh); all of a
-// thread's loads are requested before the first is used.
-template <int DT, bool kShift, class OUT>
-__device__ __forceinline__ void emit_tile(const char *rowp, OUT *outp, int V, long long e0, float c1, float ref2, float invS)
-{
-    using Q = typename LogitQuads<DT>::Q;
-    constexpr int kN = kEmitTile / 4 / kThreads;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long base = e0 + warp * (128 * kN);
-    const float nref = -ref2;
-    const f32x2 cc = pack2(c1, c1), nn = pack2(nref, nref), ss = pack2(invS, invS);
-    WarpQuads<Q, kN, kShift> w;
-    w.load(rowp, V, base, 0u);
-#pragma unroll
-    for (int u = 0; u < kN; ++u) {
-        const typename Q::Raw v = w.at(u);
-        const long long e = base + 128 * u + 4 * lane;
-        if (e >= 0 && e + 4 <= V) {
-            emit_raw(outp + e, v, cc, nn, ss);
-        } else if (e + 4 > 0 && e < V) {  // a quad that crosses an end of the row
-            for (int j = 0; j < 4; ++j)
-                if (e + j >= 0 && e + j < V) store_one(outp + e + j, ex2(fmaf(Elem<DT>::load(rowp, e + j), c1, nref)) * invS);
-        }
-    }
-}
+// ---- emission (emit.cuh) ----------------------------------------------------------------------
 
 __global__ void __launch_bounds__(kThreads) edge_fold_kernel(const __grid_constant__ EdgeParams P)
 {
@@ -322,16 +248,8 @@ __global__ void __launch_bounds__(kThreads, 4) edge_emit_kernel(const __grid_con
     }
     if (n < 0 || (P.skip_bonus_row && n == P.gamma)) return;
     const char *rowp = row_ptr<DT>(P, b * (P.gamma + 1) + n);
-    // tiles start where the output is aligned
-    if (P.p_row16) {
-        uint16_t *out = P.p_row16 + (size_t)b * P.V;
-        const int off = kShift ? quad_offset<Quads16>(reinterpret_cast<const char *>(out), 0) : 0;
-        emit_tile<DT, kShift>(rowp, out, P.V, (long long)tile * kEmitTile - off, P.c1, ref2, invS);
-    } else {
-        float *out = P.p_row + (size_t)b * P.V;
-        const int off = kShift ? quad_offset<Quads32>(reinterpret_cast<const char *>(out), 0) : 0;
-        emit_tile<DT, kShift>(rowp, out, P.V, (long long)tile * kEmitTile - off, P.c1, ref2, invS);
-    }
+    if (P.p_row16) emit_tile<DT, kShift>(rowp, P.p_row16 + (size_t)b * P.V, P.V, tile, P.c1, ref2, invS);
+    else emit_tile<DT, kShift>(rowp, P.p_row + (size_t)b * P.V, P.V, tile, P.c1, ref2, invS);
 }
 
 // One shard of the vocabulary: the rows' sums and the drafted tokens' logits go out as they are.
@@ -409,12 +327,9 @@ cudaError_t launch_edge(EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
     const unsigned long long rows = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1);
     if (P.shard_sum) return launch_pdl(edge_partial_kernel, (unsigned)((rows + kFoldRows - 1) / kFoldRows), kThreads, stream, P);
     const bool emit = P.p_row || P.p_row16;
-    // rows whose logits and output all start on boundaries of four entries need no shifting
-    const int osz = P.p_row16 ? 2 : 4;
-    const uintptr_t out = P.p_row16 ? reinterpret_cast<uintptr_t>(P.p_row16) : reinterpret_cast<uintptr_t>(P.p_row);
-    const bool aligned = P.V % 4 == 0 && out % (4 * osz) == 0 && P.row_stride % 4 == 0 &&
-                         reinterpret_cast<uintptr_t>(P.logits) % (4 * Elem<DT>::kBytes) == 0;
-    P.emit_tiles = (int)(((long long)P.V + (aligned ? 0 : 3) + kEmitTile - 1) / kEmitTile);
+    const bool aligned = emit_aligned(P.logits, P.row_stride, Elem<DT>::kBytes, P.p_row16 ? (const void *)P.p_row16 : P.p_row, P.V,
+                                      P.p_row16 ? 2 : 4);
+    P.emit_tiles = emit_tiles(P.V, aligned);
     const unsigned long long ctas = (unsigned long long)P.B * (unsigned long long)P.emit_tiles;
     if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
     const bool fold = emit && ctas <= kEmitFoldCtas;

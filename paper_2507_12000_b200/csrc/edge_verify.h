@@ -10,13 +10,14 @@ namespace dssd {
 constexpr int kLseThreads = 128;                     // threads per CTA of the log-sum-exp kernel
 constexpr int kLseLoads = 8;                         // 16-byte loads a thread has in flight
 constexpr int kLseTile = kLseThreads * kLseLoads;    // 16-byte vectors of one pass over the CTA (16 KB)
-// Tiles per CTA of the log-sum-exp kernel: one in small launches, so that all SMs share the work; from four
-// waves of 1184 resident CTAs on two, from sixteen on four, so that a CTA's start and reduction are paid
-// for less often.  Measured (us, 1 / 2 / 4 / 8 tiles): B = 256 gamma = 4 V = 151936 bf16 (24 320 tiles)
-// 72.0 / 66.8 / 64.5 / 67.5, B = 64 gamma = 8 V = 128256 bf16 (9216) 30.6 / 28.7 / 28.5 / 28.8, B = 300
-// gamma = 4 V = 30011 bf16 (6000) 22.5 / 21.8 / 23.3, B = 8 gamma = 4 V = 32000 bf16 (160) 3.2 / 4.0 / 5.9.
-constexpr unsigned long long kLseTwoTiles = 4700, kLseFourTiles = 19000;
-constexpr int kEmitTile = 8192;                      // entries of row n that one CTA emits
+// Tiles per CTA of the log-sum-exp kernel: one in small launches, so that all SMs share the work; from about
+// three waves of 1184 resident CTAs on two, from sixteen on four, so that a CTA's start and reduction are
+// paid for less often.  Measured (us, partial sums of a shard, 1 / 2 / 4 tiles): 256 x 5 rows of 151936 bf16
+// (24 320 tiles) 74.1 / 66.2 / 62.3, 64 x 9 of 128256 bf16 (9216) 31.3 / 29.2 / 28.7, 300 x 5 of 30011 bf16 (6000)
+// 22.5 / 21.4 / 21.9, 256 x 5 of 18992 bf16 (3840) 16.0 / 15.4 / 15.9, 64 x 5 of 50256 float32 (4160) 14.0 / 14.0 /
+// 14.6, 30 x 5 of 128256 bf16 (2400) 11.8 / 11.7 / 12.2.  Runs of equal length instead of full tiles and a rest
+// are slower (24 320 tiles: 66.0 with four).
+constexpr unsigned long long kLseTwoTiles = 3000, kLseFourTiles = 19000;
 // Up to one wave of emission CTAs (four per SM) each folds its sequence itself, which saves a launch (B = 8
 // V = 32000: 12.1 us a round against 13.3); beyond that a fold per wave costs more than a kernel that
 // folds every sequence once (B = 256 V = 151936: emission 49.9 us against 3.1 + 36.5).

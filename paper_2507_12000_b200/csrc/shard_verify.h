@@ -40,8 +40,9 @@ struct EmitShardParams {
     int B, gamma, V;  // V: entries of the slice
     float *p_row;     // [B, V] with p_stride elements between rows
     int64_t p_stride;
+    int tiles;  // emission CTAs per sequence (filled by the launch)
 };
 
-cudaError_t shard_emit_launch(const EmitShardParams &P, int dtype, cudaStream_t stream);
+cudaError_t shard_emit_launch(EmitShardParams &P, int dtype, cudaStream_t stream);
 
 }  // namespace dssd
