@@ -119,6 +119,11 @@ __device__ __forceinline__ void cluster_store(double *p, unsigned rank, double v
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "d"(v) : "memory");
 }
 
+__device__ __forceinline__ void cluster_store(unsigned long long *p, unsigned rank, unsigned long long v)
+{
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "l"(v) : "memory");
+}
+
 // Scalar loads that stay behind pdl_wait() (a plain __ldg may be moved across it), served by L2.
 __device__ __forceinline__ uint32_t ld_after_u32(const void *p)
 {

@@ -26,15 +26,15 @@ struct FoldShared {
 // the largest reference first, then float64 terms s * 2^(ref - R) by exponent arithmetic, added in a fixed
 // order.  The result, sum_v 2^(l_v c1) = S * 2^R, is the same in all threads of the row; a NaN or an
 // infinite sum stays one, a row without mass gives S = 0.  Short, because every emission CTA of a small
-// launch runs it.
-__device__ __forceinline__ void row_total(const unsigned long long *part, int runs, int sub, bool live, float &R, double &S,
-                                          bool &missing)
+// launch runs it.  part(k) loads run k's word.
+template <class Part>
+__device__ __forceinline__ void row_total(Part part, int runs, int sub, bool live, float &R, double &S, bool &missing)
 {
     constexpr int kHeld = 2;  // words in registers: rows of up to 16 runs need no second look
     unsigned long long w[kHeld];
     float top = DSSD_NEG_INF;
     missing = false;
-    auto word = [&](int k) { return live && k < runs ? ld_after(part + k) : 0ull; };
+    auto word = [&](int k) { return live && k < runs ? part(k) : 0ull; };
     auto look = [&](unsigned long long x) {
         missing |= x == kNoPartial;
         if (__uint_as_float((unsigned)(x >> 32)) > 0.f) top = fmaxf(top, __uint_as_float((unsigned)x));
@@ -64,37 +64,34 @@ __device__ __forceinline__ void row_total(const unsigned long long *part, int ru
     S = s;
 }
 
+// What the acceptance test of a position takes besides its row's sum.
+struct Drafted {
+    int x;          // the drafted token
+    float z, q, u;  // its logit in the row, its draft probability, the position's uniform
+};
+
 // Run by all kThreads threads of a CTA; the results are in `sh` (n, ref2, invS) when it returns.
 // `writer`: this CTA writes the sequence's accept_len, flags, lse, p_tok and `ready`.
-// The drafted tokens, their q and uniforms are the caller's inputs, the partial sums and the
-// drafted tokens' logits come from the log-sum-exp kernel: one round trip to L2 for all of them.
-__device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh)
+// part(i, k) gives the partial sum of run k of row i of the sequence, drafted(i) what belongs to position i.
+template <class Part, class Draft>
+__device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh, Part part, Draft drafted)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long row0 = b * (P.gamma + 1);
     int n = P.gamma;
     unsigned fl = 0;
     float ref2_n = 0.f, invS_n = 0.f;
     for (int base = 0; base <= P.gamma; base += kFoldRows) {
+        if (base) __syncthreads();  // warp 0 has read the previous rows
         const int i = base + lane;
         const bool live = i <= P.gamma;
-        int x = -1;
-        float zx = 0.f, qx = 0.f, ux = 0.f;
-        if (warp == 0 && i < P.gamma) {
-            const size_t di = (size_t)b * P.gamma + i;
-            x = ld_after(P.draft_tokens + di);
-            qx = P.draft_q_rows ? ld_after(P.tokq + row0 + i) : ld_after(P.draft_q_tok + di);
-            ux = ld_after(P.uniforms + di);
-            zx = ld_after(P.tokz + row0 + i);
-            if (P.draft_q_rows && (x < 0 || x >= P.V)) qx = __int_as_float(0x7fc00000);  // nothing was looked up
-        }
+        Drafted d = {-1, 0.f, 0.f, 0.f};
+        if (warp == 0 && i < P.gamma) d = drafted(i);
         {
             const int r = base + tid / kFoldLanes;
             float R;
             double S;
             bool missing;
-            row_total(P.part + (size_t)(row0 + (r <= P.gamma ? r : 0)) * P.runs, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, missing);
-            if (base) __syncthreads();  // warp 0 has read the previous rows
+            row_total([&](int k) { return part(r, k); }, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, missing);
             if (tid % kFoldLanes == 0) {
                 sh.R[tid / kFoldLanes] = R;
                 sh.S[tid / kFoldLanes] = S;
@@ -103,9 +100,10 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
         }
         __syncthreads();
         if (warp == 0) {
+            if (P.draft_q_rows && (d.x < 0 || d.x >= P.V)) d.q = __int_as_float(0x7fc00000);  // nothing was looked up
             float Rs, invS;
             const unsigned bits = judge_position(P, b, i, live, writer, sh.R[lane], sh.S[lane], false, live && sh.missing[lane],
-                                                 x, zx, qx, ux, Rs, invS);
+                                                 d.x, d.z, d.q, d.u, Rs, invS);
             const unsigned rej = __ballot_sync(0xffffffffu, live && i < P.gamma && !(bits & kBitAccept));
             if (rej && n == P.gamma) n = base + __ffs(rej) - 1;
             fl |= (__ballot_sync(0xffffffffu, bits & kBitBadToken) ? DSSD_EDGE_FLAG_BAD_TOKEN : 0u) |
@@ -135,6 +133,23 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
         }
     }
     __syncthreads();
+}
+
+// The same with what the log-sum-exp kernel left in the workspace: one round trip to L2 for the partial sums,
+// the drafted tokens' logits and the caller's arrays.
+__device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh)
+{
+    const long long row0 = b * (P.gamma + 1);
+    fold_sequence(P, b, writer, sh, [&](int i, int k) { return ld_after(P.part + (size_t)(row0 + i) * P.runs + k); },
+                  [&](int i) {
+                      const size_t di = (size_t)b * P.gamma + i;
+                      Drafted d;
+                      d.x = ld_after(P.draft_tokens + di);
+                      d.q = P.draft_q_rows ? ld_after(P.tokq + row0 + i) : ld_after(P.draft_q_tok + di);
+                      d.u = ld_after(P.uniforms + di);
+                      d.z = ld_after(P.tokz + row0 + i);
+                      return d;
+                  });
 }
 
 }  // namespace dssd

@@ -1,4 +1,4 @@
-// Edge half of the verification round: two kernels whose CTAs the hardware schedules.
+// Edge half of the verification round, as two or three kernels whose CTAs the hardware schedules.
 //
 //   edge_lse_kernel   one CTA per run of one target row (16 to 64 KB of logits): an online maximum and
 //                     sum of 2^(l * c1 - ref) per thread in float32, reduced to the run's (ref, sum)
@@ -10,10 +10,17 @@
 //   edge_emit_kernel  one CTA per tile of row n of a sequence: reads its tile of row n again and writes
 //                     p_row = 2^(l * c1 - ref) / S.
 //
-// The end of a kernel is the only synchronisation: no counter, no flag, no wait on another CTA,
+//
+// Where a sequence's rows are few or short for the number of sequences, one kernel does it all instead:
+//
+//   edge_cluster_kernel  a CTA or a cluster of CTAs per sequence; the partial sums go through shared memory.
+//
+// The end of a kernel (and the cluster's barrier) is the only synchronisation: no counter, no flag, no wait on another CTA,
 // nothing in the workspace that has to be cleared.  A kernel's CTAs are scheduled while the one
 // before it drains (launch.h).
 #include "edge_verify.h"
+
+#include <atomic>
 
 #include <math.h>
 
@@ -25,6 +32,9 @@
 namespace dssd {
 
 namespace {
+
+constexpr int kSegVecs = 32 * kLseLoads;  // 16-byte vectors of a warp's segment of a row in the cluster kernel (4 KB)
+constexpr int kPieceQuads = 4;            // quads per lane that a warp emits at a time there (eight: 0.4 us slower at B = 8 V = 32000)
 
 template <int DT>
 __device__ __forceinline__ const char *row_ptr(const EdgeParams &P, long long row)
@@ -106,6 +116,32 @@ __device__ __forceinline__ void add_tile(Online &o, const uint4 (&v)[kLseLoads],
     for (int u = 0; u < kLseLoads; ++u) add_vec<DT>(o, v[u], cc, nn);
 }
 
+// one entry more
+__device__ __forceinline__ void add_extra(Online &o, float extra, float c1)
+{
+    if (extra > DSSD_NEG_INF || extra != extra) {
+        online_raise(o, extra, c1);
+        o.s0 = add2(o.s0, pack2(ex2(fmaf(extra, c1, -o.ref)), 0.f));
+    }
+}
+
+// the warp's (ref, sum): exact power-of-two scaling; a NaN sum stays one
+__device__ __forceinline__ void online_total(const Online &o, float &R, float &s)
+{
+    float a, b;
+    unpack2(add2(add2(o.s0, o.s1), add2(o.s2, o.s3)), a, b);
+    s = a + b;
+    const float r = o.m == DSSD_NEG_INF ? DSSD_NEG_INF : o.ref;
+    R = warp_max(r);
+    s = warp_sum(r == DSSD_NEG_INF ? (s != s ? s : 0.f) : s * ex2(r - R));
+}
+
+__device__ __forceinline__ unsigned long long partial_word(float R, float s)
+{
+    if (s != s) s = __int_as_float(0x7fc00000);
+    return (unsigned long long)__float_as_uint(R == DSSD_NEG_INF ? 0.f : R) | ((unsigned long long)__float_as_uint(s) << 32);
+}
+
 // Bound by HBM: 128 threads with eight 16-byte loads in flight each, eight CTAs per SM (64 registers) read
 // B = 256 gamma = 4 V = 151936 bf16 (389 MB) in 63 us and B = 1024 gamma = 16 V = 50272 float32 (3.5 GB) in
 // 500 us, 7.0 TB/s; a pure read of the same shape takes 60 and 497 us, so the exponentials are nearly
@@ -177,17 +213,9 @@ __global__ void __launch_bounds__(kLseThreads, 8) edge_lse_kernel(const __grid_c
             if (P.draft_q_rows) qx = ld_after(P.draft_q_rows + ((size_t)seq * P.gamma + pos) * (size_t)P.V + (size_t)x);
         }
     }
-    if (extra > DSSD_NEG_INF || extra != extra) {
-        online_raise(o, extra, c1);
-        o.s0 = add2(o.s0, pack2(ex2(fmaf(extra, c1, -o.ref)), 0.f));
-    }
-    float a, b;
-    unpack2(add2(add2(o.s0, o.s1), add2(o.s2, o.s3)), a, b);
-    float s = a + b;
-    const float r = o.m == DSSD_NEG_INF ? DSSD_NEG_INF : o.ref;
-    // the warp's, then the CTA's (ref, sum): exact power-of-two scaling; a NaN sum stays one
-    const float R = warp_max(r);
-    s = warp_sum(r == DSSD_NEG_INF ? (s != s ? s : 0.f) : s * ex2(r - R));
+    add_extra(o, extra, c1);
+    float R, s;  // the warp's, then the CTA's
+    online_total(o, R, s);
     if ((tid & 31) == 0) s_warp[tid >> 5] = make_float2(R, s);
     __syncthreads();
     if (tid == 0) {
@@ -200,10 +228,7 @@ __global__ void __launch_bounds__(kLseThreads, 8) edge_lse_kernel(const __grid_c
             const float2 c = s_warp[w];
             t += c.x == DSSD_NEG_INF ? (c.y != c.y ? c.y : 0.f) : c.y * ex2(c.x - Rt);
         }
-        if (t != t) t = __int_as_float(0x7fc00000);
-        const unsigned long long word = (unsigned long long)__float_as_uint(Rt == DSSD_NEG_INF ? 0.f : Rt) |
-                                        ((unsigned long long)__float_as_uint(t) << 32);
-        P.part[blockIdx.x] = (long long)row + 1 == P.test_drop_row_plus1 ? kNoPartial : word;
+        P.part[blockIdx.x] = (long long)row + 1 == P.test_drop_row_plus1 ? kNoPartial : partial_word(Rt, t);
         if (owned) {
             P.tokz[row] = zx;
             if (P.draft_q_rows) P.tokq[row] = qx;
@@ -252,6 +277,106 @@ __global__ void __launch_bounds__(kThreads, 4) edge_emit_kernel(const __grid_con
     else emit_tile<DT, kShift>(rowp, P.p_row + (size_t)b * P.V, P.V, tile, P.c1, ref2, invS);
 }
 
+// ---- small launches: one cluster of CTAs per sequence ---------------------------------------------
+
+// One warp's part of a row: the kLseLoads * 32 vectors from v0 on, and the entries outside the vectors that
+// belong to them.  The result is the warp's (ref, sum), the same in all lanes.
+template <int DT>
+__device__ __forceinline__ void warp_lse(const char *rowp, int V, int seg, int segs, float c1, float &R, float &s)
+{
+    using E = Elem<DT>;
+    const int lane = threadIdx.x & 31;
+    const long long rowbytes = (long long)V * E::kBytes;
+    int head = (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(rowp) & 15u)) & 15u);
+    if (head > rowbytes) head = (int)rowbytes;
+    const int nvec = (int)((rowbytes - head) >> 4);
+    const uint4 *src = reinterpret_cast<const uint4 *>(rowp + head);
+    const int i = seg * kSegVecs + lane;
+    uint4 v[kLseLoads];
+    if (seg * kSegVecs + kSegVecs <= nvec) {
+#pragma unroll
+        for (int u = 0; u < kLseLoads; ++u) v[u] = ld_stream16(src + i + 32 * u);
+    } else {
+#pragma unroll
+        for (int u = 0; u < kLseLoads; ++u) {
+            v[u] = neg_inf_vec<DT>();
+            if (i + 32 * u < nvec) v[u] = ld_stream16(src + i + 32 * u);
+        }
+    }
+    float extra = DSSD_NEG_INF;  // the up to seven entries before the vectors: lanes 0 .. 6; those after them: lanes 16 .. 22
+    if (seg == 0 && lane < head / E::kBytes) extra = E::load(rowp, lane);
+    if (seg + 1 == segs && lane >= 16) {
+        const int e = (int)((head + ((long long)nvec << 4)) / E::kBytes) + lane - 16;
+        if (e < V) extra = E::load(rowp, e);
+    }
+    Online o;
+    o.m = DSSD_NEG_INF;
+    o.ref = 0.f;
+    o.s0 = o.s1 = o.s2 = o.s3 = 0ull;
+    add_tile<DT>(o, v, c1);
+    add_extra(o, extra, c1);
+    online_total(o, R, s);
+}
+
+template <int DT, bool kShift, class OUT>
+__device__ __forceinline__ void emit_pieces(const char *rowp, OUT *outp, int V, int g, int n_warps, float c1, float ref2, float invS)
+{
+    const long long lead = kShift ? emit_lead(outp) : 0;
+    for (long long e = 128ll * kPieceQuads * g - lead; e < V; e += 128ll * kPieceQuads * n_warps)
+        emit_piece<DT, kShift, kPieceQuads>(rowp, outp, V, e, c1, ref2, invS);
+}
+
+// One cluster of up to kEdgeClusterMax CTAs per sequence does the whole of it.  Warp g of the cluster's takes the segments
+// g, g + warps, .. of the sequence's rows; every segment's (ref, sum) goes to every CTA's shared memory, and after
+// one cluster barrier every CTA folds the sequence for itself and emits its part of row n.
+template <int DT, bool kShift>
+__global__ void __launch_bounds__(kThreads, 4) edge_cluster_kernel(const __grid_constant__ EdgeParams P)
+{
+    __shared__ unsigned long long s_part[kEdgeClusterParts];
+    __shared__ Drafted s_draft[kFoldRows];
+    __shared__ FoldShared sh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned csize = (unsigned)P.cluster, rank = csize > 1 ? cluster_rank() : 0u;
+    const long long b = blockIdx.x / csize, row0 = b * (P.gamma + 1);
+    const int g = warp * (int)csize + (int)rank, n_warps = (int)csize * kWarps;
+    if (csize > 1) {  // a CTA's shared memory may be written once it is known to run
+        cluster_arrive();
+        cluster_wait();
+    }
+    pdl_wait();
+    pdl_trigger();
+    // the last warp has the fewest segments: it looks the drafted tokens up
+    if (warp == kWarps - 1 && lane < P.gamma) {
+        const size_t di = (size_t)b * P.gamma + lane;
+        Drafted d;
+        d.x = ld_after(P.draft_tokens + di);
+        d.q = ld_after(P.draft_q_tok + di);
+        d.u = ld_after(P.uniforms + di);
+        d.z = d.x >= 0 && d.x < P.V ? Elem<DT>::load(row_ptr<DT>(P, row0 + lane), d.x) : 0.f;
+        s_draft[lane] = d;
+    }
+    for (int t = g; t < P.runs * (P.gamma + 1); t += n_warps) {
+        const int i = t / P.runs;
+        float R, s;
+        warp_lse<DT>(row_ptr<DT>(P, row0 + i), P.V, t - i * P.runs, P.runs, P.c1, R, s);
+        const unsigned long long word = row0 + i + 1 == P.test_drop_row_plus1 ? kNoPartial : partial_word(R, s);
+        if (csize == 1) s_part[t] = word;
+        else if (lane < (int)csize) cluster_store(&s_part[t], (unsigned)lane, word);
+    }
+    if (csize > 1) {
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    fold_sequence(P, b, rank == 0, sh, [&](int i, int k) { return s_part[i * P.runs + k]; }, [&](int i) { return s_draft[i]; });
+    const int n = sh.n;
+    if (n < 0 || (P.skip_bonus_row && n == P.gamma)) return;
+    const char *rowp = row_ptr<DT>(P, row0 + n);
+    if (P.p_row16) emit_pieces<DT, kShift>(rowp, P.p_row16 + (size_t)b * P.V, P.V, g, n_warps, P.c1, sh.ref2, sh.invS);
+    else if (P.p_row) emit_pieces<DT, kShift>(rowp, P.p_row + (size_t)b * P.V, P.V, g, n_warps, P.c1, sh.ref2, sh.invS);
+}
+
 // One shard of the vocabulary: the rows' sums and the drafted tokens' logits go out as they are.
 __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_constant__ EdgeParams P)
 {
@@ -272,7 +397,7 @@ __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_con
     float R;
     double S;
     bool missing;
-    row_total(P.part + (size_t)(live ? row : 0) * P.runs, P.runs, sub, live, R, S, missing);
+    row_total([&](int k) { return ld_after(P.part + (size_t)row * P.runs + k); }, P.runs, sub, live, R, S, missing);
     if (live && sub == 0) {
         P.shard_ref[row] = R == DSSD_NEG_INF ? 0.f : R;
         P.shard_sum[row] = missing || S != S ? (double)__int_as_float(0x7fc00000) : S;
@@ -320,6 +445,84 @@ cudaError_t launch_emit(const EdgeParams &P, unsigned ctas, bool fold, cudaStrea
 }
 
 template <int DT>
+bool outputs_aligned(const EdgeParams &P)
+{
+    return emit_aligned(P.logits, P.row_stride, Elem<DT>::kBytes, P.p_row16 ? (const void *)P.p_row16 : P.p_row, P.V, P.p_row16 ? 2 : 4);
+}
+
+template <int DT>
+cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
+{
+    const unsigned grid = (unsigned)P.B * (unsigned)P.cluster;
+    return outputs_aligned<DT>(P) ? launch_pdl(edge_cluster_kernel<DT, false>, grid, kThreads, stream, P, 0, (unsigned)P.cluster)
+                                  : launch_pdl(edge_cluster_kernel<DT, true>, grid, kThreads, stream, P, 0, (unsigned)P.cluster);
+}
+
+// Clusters beyond the portable size have to be allowed for each kernel, and a device (or the part of one that the
+// process was given) may not have a processing cluster of that many SMs: asked once per device.
+template <int DT, bool kShift>
+bool wide_clusters()
+{
+    void (*kernel)(EdgeParams) = edge_cluster_kernel<DT, kShift>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kEdgeClusterWide;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kEdgeClusterWide);
+    cfg.blockDim = dim3(kThreads);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
+}
+int most_cluster_ctas()
+{
+    static std::atomic<int> known[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return kEdgeCluster;
+    int most = known[dev].load(std::memory_order_relaxed);
+    if (!most) {
+        const bool wide = wide_clusters<DSSD_F32, false>() && wide_clusters<DSSD_F32, true>() && wide_clusters<DSSD_BF16, false>() &&
+                          wide_clusters<DSSD_BF16, true>();
+        if (!wide) cudaGetLastError();
+        most = wide ? kEdgeClusterWide : kEdgeCluster;
+        known[dev].store(most, std::memory_order_relaxed);
+    }
+    return most;
+}
+
+// at most c CTAs per sequence, no more than `wave` in all, at least one
+long long fit(long long c, long long wave, int B)
+{
+    const long long most = wave / B;
+    return c < most ? c : most > 1 ? most : 1;
+}
+
+// CTAs per sequence of the cluster kernel, or 0 where the separate kernels are the better ones (edge_verify.h).
+int cluster_ctas(const EdgeParams &P, int esz, long long segs)
+{
+    const long long parts = segs * (P.gamma + 1);
+    if (P.shard_sum || P.draft_q_rows || P.gamma >= kFoldRows || parts > kEdgeClusterParts) return 0;
+    long long c = (parts + kWarps - 1) / kWarps;
+    c = fit(c, kEdgeWave, P.B);
+    if (c > 2) c = fit(c, kEdgeClusterWave, P.B);
+    if (c > kEdgeCluster) {
+        const long long wide = fit(c, kEdgeWideWave, P.B);
+        c = wide > kEdgeCluster ? wide : kEdgeCluster;
+        if (c > kEdgeCluster && c > most_cluster_ctas()) c = most_cluster_ctas();
+    }
+    const double work = (double)(parts * (esz == 2 ? 2 : 1)) + (P.p_row || P.p_row16 ? (double)P.V / (128 * kPieceQuads) : 0.0);
+    if (c > kEdgeCluster && work > kEdgeWideRounds * (double)(kWarps * c)) c = kEdgeCluster;
+    if (c > kEdgeCluster) return (int)c;
+    const long long ctas = P.B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
+    const double fill = (double)ctas / (double)(waves * kEdgeWave);
+    const double limit = fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0;
+    return work <= limit * (double)(kWarps * c) ? (int)c : 0;
+}
+
+template <int DT>
 cudaError_t launch_edge(EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
 {
     cudaError_t e = launch_pdl(edge_lse_kernel<DT>, lse_ctas, kLseThreads, stream, P);
@@ -327,8 +530,7 @@ cudaError_t launch_edge(EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
     const unsigned long long rows = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1);
     if (P.shard_sum) return launch_pdl(edge_partial_kernel, (unsigned)((rows + kFoldRows - 1) / kFoldRows), kThreads, stream, P);
     const bool emit = P.p_row || P.p_row16;
-    const bool aligned = emit_aligned(P.logits, P.row_stride, Elem<DT>::kBytes, P.p_row16 ? (const void *)P.p_row16 : P.p_row, P.V,
-                                      P.p_row16 ? 2 : 4);
+    const bool aligned = outputs_aligned<DT>(P);
     P.emit_tiles = emit_tiles(P.V, aligned);
     const unsigned long long ctas = (unsigned long long)P.B * (unsigned long long)P.emit_tiles;
     if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
@@ -348,6 +550,13 @@ cudaError_t edge_verify_launch(EdgeParams &P, int dtype, void *workspace, cudaSt
     const unsigned long long rows = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1);
     P.c1 = (float)(1.4426950408889634 / (double)P.temperature);
     const long long nvec = (long long)P.V * esz / 16;
+    const long long segs = nvec > kSegVecs ? (nvec + kSegVecs - 1) / kSegVecs : 1;
+    P.cluster = cluster_ctas(P, esz, segs);
+    if (P.cluster) {
+        edge_workspace_layout(P.B, P.gamma, 1, &P, static_cast<char *>(workspace));  // (the partial sums stay on the chip)
+        P.runs = (int)segs;
+        return dtype == DSSD_BF16 ? launch_cluster<DSSD_BF16>(P, stream) : launch_cluster<DSSD_F32>(P, stream);
+    }
     const unsigned long long tiles = rows * (unsigned long long)((nvec + kLseTile - 1) / kLseTile);
     const long long per = tiles < kLseTwoTiles ? 1 : tiles < kLseFourTiles ? 2 : 4;
     long long runs = (nvec + per * kLseTile - 1) / (per * kLseTile);

@@ -18,10 +18,29 @@ constexpr int kLseTile = kLseThreads * kLseLoads;    // 16-byte vectors of one p
 // 14.6, 30 x 5 of 128256 bf16 (2400) 11.8 / 11.7 / 12.2.  Runs of equal length instead of full tiles and a rest
 // are slower (24 320 tiles: 66.0 with four).
 constexpr unsigned long long kLseTwoTiles = 3000, kLseFourTiles = 19000;
-// Up to one wave of emission CTAs (four per SM) each folds its sequence itself, which saves a launch (B = 8
-// V = 32000: 12.1 us a round against 13.3); beyond that a fold per wave costs more than a kernel that
-// folds every sequence once (B = 256 V = 151936: emission 49.9 us against 3.1 + 36.5).
+// Where the separate kernels run, up to one wave of emission CTAs (four per SM) each fold their sequence themselves, which
+// saves a launch (B = 1 V = 50272: 0.5 to 1 us on the GPU and 3 us of host time); beyond that a fold per wave costs
+// more than a kernel that folds every sequence once (B = 256 V = 151936: emission 49.9 us against 3.1 + 36.5).
 constexpr unsigned long long kEmitFoldCtas = 592;
+
+// The cluster kernel does the log-sum-exps, the fold and the emission in one launch.  It takes as many CTAs per sequence as
+// have a segment (4 KB of logits) for each of their warps, as a cluster can have - eight, or sixteen while a warp's work
+// stays below kEdgeWideRounds - and as fit a wave: four CTAs per SM, somewhat less for clusters of three and more, which
+// do not pack the GPU's processing clusters completely (B = 113 V = 51071 float32, five each, 565 CTAs: 40.1 against 31.3
+// in separate kernels; B = 31 V = 33584, sixteen each, 496 CTAs: 11.1 against 9.3).  The unit of work is 1024 entries
+// summed or 512 emitted by a warp; how much of it per warp still pays depends on how full the wave is, since a
+// warp's loads wait for one another from segment to segment and only other CTAs on the SM fill the gaps.  Measured (us per
+// call, cluster kernel / separate kernels):
+//   few CTAs:  B = 1 gamma = 8 V = 2176 bf16 4.2 / 6.1, B = 8 gamma = 4 V = 32000 bf16 4.8 / 6.5, B = 16 5.4 / 7.0;
+//              beyond the limits B = 1 gamma = 8 V = 50272 float32 7.9 / 5.7, B = 2 gamma = 9 V = 36496 float32 6.9 / 6.3
+//   one CTA per sequence:  B = 520 gamma = 1 V = 1172 bf16 5.0 / 11.6, B = 979 gamma = 1 V = 4880 bf16 11.8 / 17.5,
+//              B = 318 gamma = 4 V = 9792 bf16 16.3 / 20.2; beyond B = 661 gamma = 1 V = 72431 bf16 110 / 86
+//   full wave:  B = 89 gamma = 4 V = 18896 float32 9.6 / 13.0, B = 64 gamma = 4 V = 128256 bf16 26.5 / 29.7,
+//              B = 128 gamma = 4 V = 50272 float32 30.7 / 32.3; beyond B = 166 gamma = 11 V = 53648 bf16 52.8 / 48.8.
+constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
+constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, more
+constexpr double kEdgeWideRounds = 2.8;
+constexpr int kEdgeClusterParts = 3072;                  // segments of a sequence (24 KB of shared memory)
 
 // What the draw needs to know about a folded sequence when no row is written.
 struct ReadySlot {
@@ -58,8 +77,9 @@ struct EdgeParams {
     float *shard_tok_logit;   // [B, gamma]; NaN where the token lies outside the shard
     int v_begin;
     // geometry
-    int runs;                 // runs per row (one CTA of the log-sum-exp kernel each)
+    int runs;                 // runs per row (one CTA of the log-sum-exp kernel each), segments in the cluster kernel
     int run_vecs;             // 16-byte vectors per run
+    int cluster;              // CTAs per sequence of the cluster kernel (0: separate kernels)
     int emit_tiles;           // tiles (emission CTAs) per sequence
     // test hook (0: off): the partial sums of row test_drop_row_plus1 - 1 are formed but never stored
     long long test_drop_row_plus1;

@@ -72,18 +72,21 @@ struct LogitQuads<DSSD_BF16> {
     typedef Quads16 Q;
 };
 
-// outp[e] = 2^(l_e * c1 - ref2) * invS for the entries e of one tile of a row of V entries, by a CTA of kThreads
-// threads.  Tiles start where the output's quads are aligned; the logits' quads may lie on any element
-// boundary (quads.cuh).  All of a thread's loads are requested before the first is used.
-template <int DT, bool kShift, class OUT>
-__device__ __forceinline__ void emit_tile(const char *rowp, OUT *outp, int V, int tile, float c1, float ref2, float invS)
+// entries of the quad that crosses the start of an unaligned output row and lie before it
+template <class OUT>
+__device__ __forceinline__ int emit_lead(const OUT *outp)
 {
-    using OQ = typename OutQuads<OUT>::Q;
-    const long long e0 = (long long)tile * kEmitTile - (kShift ? quad_offset<OQ>(reinterpret_cast<const char *>(outp), 0) : 0);
+    return quad_offset<typename OutQuads<OUT>::Q>(reinterpret_cast<const char *>(outp), 0);
+}
+
+// outp[e] = 2^(l_e * c1 - ref2) * invS for the 128 kN entries from `base` on that lie in a row of V entries, by a warp.
+// `base` is where the output's quads are aligned; the logits' quads may lie on any element
+// boundary (quads.cuh).  All of a thread's loads are requested before the first is used.
+template <int DT, bool kShift, int kN, class OUT>
+__device__ __forceinline__ void emit_piece(const char *rowp, OUT *outp, int V, long long base, float c1, float ref2, float invS)
+{
     using Q = typename LogitQuads<DT>::Q;
-    constexpr int kN = kEmitTile / 4 / kThreads;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long base = e0 + warp * (128 * kN);
+    const int lane = threadIdx.x & 31;
     const float nref = -ref2;
     const f32x2 cc = pack2(c1, c1), nn = pack2(nref, nref), ss = pack2(invS, invS);
     WarpQuads<Q, kN, kShift> w;
@@ -99,6 +102,15 @@ __device__ __forceinline__ void emit_tile(const char *rowp, OUT *outp, int V, in
                 if (e + j >= 0 && e + j < V) store_one(outp + e + j, ex2(fmaf(Elem<DT>::load(rowp, e + j), c1, nref)) * invS);
         }
     }
+}
+
+// One tile of a row by a CTA of kThreads threads.
+template <int DT, bool kShift, class OUT>
+__device__ __forceinline__ void emit_tile(const char *rowp, OUT *outp, int V, int tile, float c1, float ref2, float invS)
+{
+    constexpr int kN = kEmitTile / 4 / kThreads;
+    const long long e0 = (long long)tile * kEmitTile - (kShift ? emit_lead(outp) : 0);
+    emit_piece<DT, kShift, kN>(rowp, outp, V, e0 + (int)(threadIdx.x >> 5) * (128 * kN), c1, ref2, invS);
 }
 
 }  // namespace dssd

@@ -27,3 +27,17 @@ def B():
 def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, zipf=V > 8, seed=V + Bn)
     compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
+
+
+# One launch for small sequences: vocabularies at the edges of a warp's segment (1024 float32 or 2048 bf16 logits) and
+# of what it emits (512 entries), one CTA per sequence, clusters of two, eight, nine and sixteen, the last
+# batch of a wave, the most positions, and the sizes next to the limits where the separate kernels take over.
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [
+    ("f32", 1, 1, 1023), ("f32", 1, 3, 1024), ("f32", 3, 3, 1025), ("f32", 3, 15, 1027), ("bf16", 2, 3, 2047), ("bf16", 2, 3, 2048),
+    ("bf16", 2, 7, 2049), ("bf16", 3, 3, 2055), ("bf16", 1, 7, 16384), ("bf16", 1, 8, 16384), ("f32", 36, 15, 8192), ("f32", 37, 15, 8195),
+    ("f32", 38, 15, 8192), ("f32", 73, 7, 8192), ("bf16", 74, 7, 16389), ("bf16", 296, 5, 5000), ("bf16", 297, 5, 5000), ("f32", 593, 3, 2500),
+    ("f32", 30, 30, 2000), ("f32", 3, 31, 2100), ("bf16", 3, 32, 2100), ("f32", 185, 31, 12289), ("bf16", 8, 5, 81776), ("bf16", 4, 2, 58880),
+])
+def test_one_launch_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, zipf=True, seed=V + Bn)
+    compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
