@@ -43,6 +43,10 @@ constexpr int kClusterMax = 8;           // most CTAs per sequence (the portable
 // B = 100 V = 3001 (100) 12.4 / 15.1. CTAs of 512 threads, for vocabularies beyond 32768, pay off in smaller
 // batches only: B = 1 V = 50272 (8) 10.5 / 11.4, B = 16 V = 50257 (128) 17.7 / 16.2.
 constexpr int kClusterWave = 200;
+// One CTA per sequence, vocabularies up to 4096, has no cluster to wait for and pays off up to about two waves of (at 128
+// registers) 512 threads per SM: B = 1000 V = 1024 4.7 / 12.4, B = 1000 V = 2000 7.9 / 12.6, B = 600 V = 4001 10.7 / 11.9; beyond,
+// B = 1000 V = 4001 16.1 / 15.1 (the draw alone).
+constexpr long long kSingleThreads = 153600;
 constexpr int kClusterSums = kClusterMax * kClusterThreads / 32;
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
 constexpr int kDrawWarps = kDrawThreads / 32;
@@ -872,9 +876,12 @@ cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t str
     const int per_cta = warps <= 8 * kClusterMax ? 8 : 16;
     const long long ctas = (warps + per_cta - 1) / per_cta;
     P.cluster_threads = 0;
-    if (ctas <= kClusterMax && P.B * ctas <= (per_cta == 8 ? kClusterWave : kClusterWave / 4) && !P.test_drop_seq_plus1) {
+    const int threads = 32 * (int)(warps < per_cta ? warps : per_cta);
+    const bool small = ctas == 1 ? (long long)P.B * threads <= kSingleThreads
+                                 : ctas <= kClusterMax && P.B * ctas <= (per_cta == 8 ? kClusterWave : kClusterWave / 4);
+    if (small && !P.test_drop_seq_plus1) {
         P.n_ctas = (int)ctas;
-        P.cluster_threads = 32 * (int)(warps < per_cta ? warps : per_cta);
+        P.cluster_threads = threads;
     }
     if (P.logits) {
         return P.logits_dtype == DSSD_BF16 ? launch_resample<RowLogits<DSSD_BF16>>(P, (unsigned)grid, stream)
