@@ -267,8 +267,13 @@ dssd_status dssd_dsd_verify(const void *target_logits, dssd_dtype dtype, int64_t
     E.V = V;
     E.accept_len = accept_len;
     E.flags = edge_flags;  // no row: nothing is emitted
+    E.draw_token = token;
+    E.draw_flags = rs_flags;
+    E.draw_uniforms = uniforms_rs;
+    E.draw_rejected = 1;
     cudaError_t e = dssd::edge_verify_launch(E, (int)dtype, ws_edge, s);
     if (e != cudaSuccess) return cuda_fail(e);
+    if (E.cluster) return DSSD_OK;  // drawn in the same launch
 
     dssd::ResampleParams R{};
     R.logits = target_logits;
@@ -335,8 +340,12 @@ dssd_status dssd_edge_verify_bonus(const void *target_logits, dssd_dtype dtype, 
     E.lse = lse;
     E.flags = flags;
     E.skip_bonus_row = 1;  // rows of fully accepted sequences are not emitted
+    E.draw_token = token;
+    E.draw_flags = token_flags;
+    E.draw_uniforms = uniforms_bonus;
     cudaError_t e = dssd::edge_verify_launch(E, (int)dtype, ws_edge, s);
     if (e != cudaSuccess) return cuda_fail(e);
+    if (E.cluster) return DSSD_OK;  // drawn in the same launch
 
     // the bonus draws, from row gamma's logits and what the edge kernel left about that row
     dssd::ResampleParams R{};

@@ -12,15 +12,14 @@
 // All sums are float64, so the token differs from an index-order float64 scan only when u' * Z
 // lies within rounding (about 1e-13 relative) of a CDF step.
 #include "device_resample.h"
-#include "edge_verify.h"
 
 #include <mutex>
 
 #include <math.h>
 
+#include "draw.cuh"
 #include "dssd_device.cuh"
 #include "launch.h"
-#include "quads.cuh"
 
 namespace dssd {
 
@@ -51,126 +50,6 @@ constexpr int kClusterSums = kClusterMax * kClusterThreads / 32;
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
 constexpr int kDrawWarps = kDrawThreads / 32;
 constexpr int kRun = kSub / kDrawThreads;  // entries of a chunk per thread
-constexpr int kKeep = 8;                 // chunk sums that a lane keeps: enough for 256 chunks without a second look
-
-__device__ __forceinline__ double res(float p, float q) { return fmax(0.0, (double)p - (double)q); }
-
-__device__ __forceinline__ float4 as_f4(const uint4 &v)
-{
-    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
-}
-
-// The row p comes as float32, as IEEE binary16 bit patterns (the 16-bit payload), or - for the
-// fused verification of Algorithm 1, where no row is ever written - as the target logits of row n
-// together with the row's reference exponent and 1 / sum, from which p_v = 2^(l_v c1 - ref2) / S is
-// formed on the fly exactly as the edge kernel forms it when it emits a row.  The kernel is
-// written once over these views.  A "quad" is four consecutive entries.
-__device__ __forceinline__ float4 half_quad(uint2 v)
-{
-    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-struct RowF32 {  // p_row as float32
-    typedef Quads32 Q;
-    static constexpr uint32_t kFill = 0u;
-    static constexpr bool kFixed = true;  // the row does not depend on the accepted length
-    const char *row;
-    __device__ static __forceinline__ RowF32 make(const ResampleParams &P, int64_t b, int)
-    {
-        RowF32 r;
-        r.row = static_cast<const char *>(P.p_row) + (size_t)b * P.V * 4;
-        return r;
-    }
-    __device__ __forceinline__ float4 quad(const Q::Raw &v) const { return as_f4(v); }
-};
-
-struct RowF16 {  // p_row as binary16 bit patterns
-    typedef Quads16 Q;
-    static constexpr uint32_t kFill = 0u;
-    static constexpr bool kFixed = true;  // the row does not depend on the accepted length
-    const char *row;
-    __device__ static __forceinline__ RowF16 make(const ResampleParams &P, int64_t b, int)
-    {
-        RowF16 r;
-        r.row = static_cast<const char *>(P.p_row) + (size_t)b * P.V * 2;
-        return r;
-    }
-    __device__ __forceinline__ float4 quad(const Q::Raw &v) const { return half_quad(v); }
-};
-
-// four consecutive logits: how they are loaded and widened
-template <int DT>
-struct LogitQuad;
-template <>
-struct LogitQuad<DSSD_F32> {
-    typedef Quads32 Q;
-    static constexpr uint32_t kNegInf = 0xff800000u;
-    __device__ static __forceinline__ float4 widen(const uint4 &v) { return as_f4(v); }
-};
-template <>
-struct LogitQuad<DSSD_BF16> {
-    typedef Quads16 Q;
-    static constexpr uint32_t kNegInf = 0xff80u;
-    __device__ static __forceinline__ float4 widen(const uint2 &v)
-    {
-        return make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
-    }
-};
-
-template <int DT>
-struct RowLogits {  // row n of the target logits, turned into probabilities on the fly
-    typedef typename LogitQuad<DT>::Q Q;
-    static constexpr uint32_t kFill = LogitQuad<DT>::kNegInf;
-    static constexpr bool kFixed = false;
-    const char *row;
-    float c1, nref, invS;
-    __device__ static __forceinline__ RowLogits make(const ResampleParams &P, int64_t b, int n)
-    {
-        RowLogits r;
-        r.row = reinterpret_cast<const char *>(P.logits) +
-                ((size_t)b * (size_t)(P.gamma + 1) + (size_t)n) * (size_t)P.row_stride * Elem<DT>::kBytes;
-        const ReadySlot *s = reinterpret_cast<const ReadySlot *>(P.ready) + b;
-        r.c1 = P.c1;
-        r.nref = -ld_after(&s->ref2);
-        r.invS = ld_after(&s->invS);
-        return r;
-    }
-    __device__ __forceinline__ float prob(float l) const { return ex2(fmaf(l, c1, nref)) * invS; }
-    __device__ __forceinline__ float4 quad(const typename Q::Raw &v) const
-    {
-        const float4 l = LogitQuad<DT>::widen(v);
-        return make_float4(prob(l.x), prob(l.y), prob(l.z), prob(l.w));
-    }
-};
-
-// This thread's part of a chunk sum: the four quads of its warp's half of a chunk, entries base + 128 u +
-// 4 lane .. + 3.  All loads are requested before the first is used.  q is not read without kHasQ (then
-// r = p); with kPlain the sum of p goes to `plain`.
-template <bool kHasQ, bool kPlain, bool kShift, typename RV>
-__device__ __forceinline__ double share_mass(const RV &row, const float *q, int V, long long base, double &plain)
-{
-    WarpQuads<typename RV::Q, 4, kShift> a;
-    WarpQuads<Quads32, 4, kShift> b;
-    a.load(row.row, V, base, RV::kFill);
-    if (kHasQ) b.load(reinterpret_cast<const char *>(q), V, base, 0u);
-    double acc = 0.0;
-    plain = 0.0;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const float4 x = row.quad(a.at(u));
-        if (kHasQ) {
-            const float4 y = as_f4(b.at(u));
-            acc += (res(x.x, y.x) + res(x.y, y.y)) + (res(x.z, y.z) + res(x.w, y.w));
-        }
-        if (!kHasQ || kPlain) {
-            const double s = ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-            if (kPlain) plain += s;
-            if (!kHasQ) acc += s;
-        }
-    }
-    return acc;
-}
 
 // r for thread t's run of the chunk that starts at entry e0: entries e0 + kRun * t + j in r[j]; 0 beyond the
 // row's end.  All loads are requested before the first is used.
@@ -193,119 +72,10 @@ __device__ __forceinline__ void load_run(const RV &row, const float *q, int V, i
     }
 }
 
-constexpr unsigned long long kNoSum = ~0ull;  // stored in place of a withheld chunk sum (a sum is never this NaN)
-
 // is a sequence with accepted length n (0 <= n <= gamma) one this launch draws for?
 __device__ __forceinline__ bool selected(const ResampleParams &P, int n)
 {
     return P.select == 0 || (P.select == 1 ? n == P.gamma : n < P.gamma);
-}
-
-__device__ __forceinline__ bool missing(double m) { return (unsigned long long)__double_as_longlong(m) == kNoSum; }
-
-// Where in a row the draw falls.
-struct Pick {
-    bool ok;        // the row's mass Z is positive and finite
-    bool late;      // a chunk sum is missing
-    bool beyond;    // no chunk prefix exceeds the target: take the last positive entry
-    int chunk;
-    double base;    // mass before that chunk
-    double target;  // the running mass that the token's must exceed
-};
-
-__device__ __forceinline__ double warp_scan(double x)  // inclusive, in lane order
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double up = __shfl_up_sync(0xffffffffu, x, o);
-        if ((int)(threadIdx.x & 31) >= o) x += up;
-    }
-    return x;
-}
-
-__device__ __forceinline__ double shfl_f64(double x, int src) { return __shfl_sync(0xffffffffu, x, src); }
-
-// The chunk sums that lane l of a warp looks at: a contiguous share of the n_sub, the first kKeep of
-// them in registers.  sum(c) loads chunk sum c.
-struct LaneSums {
-    int c0, c1;
-    double m[kKeep];
-};
-template <class Sum>
-__device__ __forceinline__ void load_sums(LaneSums &L, int n_sub, Sum sum)
-{
-    const int per = (n_sub + 31) / 32;
-    L.c0 = min(n_sub, (int)(threadIdx.x & 31) * per);
-    L.c1 = min(n_sub, L.c0 + per);
-#pragma unroll
-    for (int k = 0; k < kKeep; ++k) L.m[k] = L.c0 + k < L.c1 ? sum(L.c0 + k) : 0.0;
-}
-
-// Every warp does the same, so nothing is exchanged: a prefix over the lanes' shares gives Z, and the
-// first chunk whose inclusive prefix exceeds target(Z) - the last one with mass when there is none - is
-// the pick.  `beyond` set by the caller means that no prefix is known to exceed the target.  The
-// float64 additions that depend on one another are what this costs: the prefix within a lane's share is
-// formed once and compared in parallel.
-template <class Sum, class Target>
-__device__ __forceinline__ Pick pick_chunk(const LaneSums &L, Sum sum, bool beyond, Target target)
-{
-    const int lane = threadIdx.x & 31;
-    double pre[kKeep];
-    double s = 0.0;
-    bool late = false;
-    unsigned positive = 0;
-#pragma unroll
-    for (int k = 0; k < kKeep; ++k) {
-        s += L.m[k];
-        pre[k] = s;
-        late |= missing(L.m[k]);
-        positive |= L.m[k] > 0.0 ? 1u << k : 0u;
-    }
-    for (int c = L.c0 + kKeep; c < L.c1; ++c) {
-        const double x = sum(c);
-        s += x;
-        late |= missing(x);
-    }
-    const double incl = warp_scan(s);
-    const double up = __shfl_up_sync(0xffffffffu, incl, 1);
-    const double excl = lane ? up : 0.0;
-    Pick pk;
-    const double Z = shfl_f64(incl, 31);
-    pk.late = __any_sync(0xffffffffu, late);
-    pk.ok = (Z > 0.0) && (Z < INFINITY);
-    pk.target = target(Z);
-    const unsigned cross = beyond ? 0u : __ballot_sync(0xffffffffu, s > 0.0 && incl > pk.target);
-    const unsigned mass = __ballot_sync(0xffffffffu, s > 0.0);
-    pk.beyond = cross == 0;
-    const int owner = cross ? __ffs(cross) - 1 : mass ? 31 - __clz(mass) : 0;
-    // the lane's own chunks: the first that crosses, else the last with mass
-    int k = 0;
-    unsigned over = 0;
-#pragma unroll
-    for (int j = 0; j < kKeep; ++j) over |= cross && excl + pre[j] > pk.target ? 1u << j : 0u;
-    over &= positive;
-    bool hit = over != 0;
-    if (hit) k = __ffs(over) - 1;
-    else if (positive) k = 31 - __clz(positive);
-    double base = excl;
-#pragma unroll
-    for (int j = 1; j < kKeep; ++j)
-        if (j == k) base = excl + pre[j - 1];
-    if (lane == owner && !hit) {  // (beyond kKeep chunks per lane only)
-        double C = excl + pre[kKeep - 1];
-        for (int c = L.c0 + kKeep; c < L.c1 && !hit; ++c) {
-            const double x = sum(c);
-            if (x > 0.0) {
-                k = c - L.c0;
-                base = C;
-                hit = cross != 0 && C + x > pk.target;
-            }
-            C += x;
-        }
-    }
-    pk.chunk = __shfl_sync(0xffffffffu, L.c0 + k, owner);
-    pk.base = shfl_f64(base, owner);
-    return pk;
 }
 
 // The draw inside the picked chunk, which starts at entry e0, by the whole CTA: the token is the first entry whose
@@ -486,118 +256,38 @@ __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __gri
 }
 
 // Small launches: one cluster of up to eight CTAs per sequence does the whole draw and reads every entry
-// once.  Warp g of the cluster holds entries 512 g .. of the row in registers (the layout of share_mass), its
-// sum goes to every CTA's shared memory, and after one cluster barrier every warp picks the 512 entries that
-// hold the target; the warp that holds them finds the token.
+// once (draw_held).
 template <bool kShift, typename RV>
 __global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const __grid_constant__ ResampleParams P)
 {
-    __shared__ double s_sum[2][kClusterSums];
+    __shared__ double s_sum[2 * kClusterSums];
     __shared__ Pick s_pick;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const unsigned csize = (unsigned)P.n_ctas, rank = csize > 1 ? cluster_rank() : 0u;
     const int64_t b = blockIdx.x / csize;
-    const int g = (int)rank * warps + warp, n_sums = (int)csize * warps;
-    if (csize > 1) cluster_arrive();  // a CTA's shared memory may be written once it is known to run
+    const int g = (int)rank * warps + warp;
+    if (csize > 1) {  // a CTA's shared memory may be written once it is known to run
+        cluster_arrive();
+        cluster_wait();
+    }
     pdl_wait();
     pdl_trigger();
     const int n = ld_after(P.accept_len + b);
     const float u = warp == 0 ? ld_after(P.uniforms + b) : 0.f;
-    const long long base = 512ll * g;
     WarpQuads<typename RV::Q, 4, kShift> a;
-    if (RV::kFixed) a.load(RV::make(P, b, 0).row, P.V, base, RV::kFill);  // (on its way before n is back)
-    const bool draws = n >= 0 && n <= P.gamma && selected(P, n);
-    double r[16];
-    const float *q = draws && n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
-    unsigned fl = q ? 0u : DSSD_RS_FLAG_BONUS;
-    const RV row = RV::make(P, b, draws ? n : 0);
-    Pick pk;
-    pk.ok = false;
-    for (int attempt = 0; draws && attempt < 2; ++attempt) {
-        if (!RV::kFixed) a.load(row.row, P.V, base, RV::kFill);
-        double t = 0.0;
-        if (q) {
-            WarpQuads<Quads32, 4, kShift> d;
-            d.load(reinterpret_cast<const char *>(q), P.V, base, 0u);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float4 x = row.quad(a.at(k)), y = as_f4(d.at(k));
-                r[4 * k] = res(x.x, y.x), r[4 * k + 1] = res(x.y, y.y), r[4 * k + 2] = res(x.z, y.z), r[4 * k + 3] = res(x.w, y.w);
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float4 x = row.quad(a.at(k));
-                r[4 * k] = x.x, r[4 * k + 1] = x.y, r[4 * k + 2] = x.z, r[4 * k + 3] = x.w;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) t += (r[4 * k] + r[4 * k + 1]) + (r[4 * k + 2] + r[4 * k + 3]);
-        t = warp_sum(t);
-        if (csize > 1) {
-            if (attempt == 0) cluster_wait();
-            if (lane < (int)csize) cluster_store(&s_sum[attempt][g], (unsigned)lane, t);
-            cluster_arrive();
-            cluster_wait();
-        } else {
-            if (lane == 0) s_sum[attempt][g] = t;
-            __syncthreads();
-        }
-        // one warp per CTA: its float64 operations would hold up the others' if every warp did them
-        if (warp == 0) {
-            LaneSums L;
-            auto sum = [&](int c) { return s_sum[attempt][c]; };
-            load_sums(L, n_sums, sum);
-            const Pick mine = pick_chunk(L, sum, false, [&](double Z) { return (double)u * Z; });
-            if (lane == 0) s_pick = mine;
-        }
-        __syncthreads();
-        pk = s_pick;
-        if (pk.ok || !q) break;
-        q = nullptr;  // residual has no mass (p == q): draw from p instead
-        fl |= DSSD_RS_FLAG_FALLBACK;
-        __syncthreads();  // the pick has been read
-    }
-    if (!draws && csize > 1) cluster_wait();
-    if (!pk.ok) {
-        if (rank == 0 && threadIdx.x == 0) {
-            const bool invalid = n < 0 || n > P.gamma;
-            if (draws || invalid || P.select == 1) {  // (the bonus token drawn at the edge: the others get their token later)
-                P.token[b] = -1;
-                if (P.flags) P.flags[b] = invalid ? DSSD_RS_FLAG_INVALID : draws ? fl | DSSD_RS_FLAG_INVALID : 0u;
-            }
+    if (RV::kFixed) a.load(RV::make(P, b, 0).row, P.V, 512ll * g, RV::kFill);  // (on its way before n is back)
+    const bool invalid = n < 0 || n > P.gamma;
+    if (invalid || !selected(P, n)) {
+        if (rank == 0 && threadIdx.x == 0 && (invalid || P.select == 1)) {  // (the bonus token drawn at the edge: the others get their token later)
+            P.token[b] = -1;
+            if (P.flags) P.flags[b] = invalid ? DSSD_RS_FLAG_INVALID : 0u;
         }
         return;
     }
-    if (g != pk.chunk) return;
-    // this warp's 512 entries in the order 128 u + 4 lane + j: the first whose running mass exceeds the target,
-    // else (rounding, or pk.beyond) the last with mass
-    double in[4], C = pk.base;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) in[k] = warp_scan((r[4 * k] + r[4 * k + 1]) + (r[4 * k + 2] + r[4 * k + 3]));
-    int tok = -1;
-    bool hit = false;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double up = __shfl_up_sync(0xffffffffu, in[k], 1);
-        const double c0 = C + (lane ? up : 0.0), c1 = c0 + r[4 * k], c2 = c1 + r[4 * k + 1], c3 = c2 + r[4 * k + 2], c4 = c3 + r[4 * k + 3];
-        const unsigned pos = (r[4 * k] > 0.0 ? 1u : 0u) | (r[4 * k + 1] > 0.0 ? 2u : 0u) | (r[4 * k + 2] > 0.0 ? 4u : 0u) |
-                             (r[4 * k + 3] > 0.0 ? 8u : 0u);
-        const unsigned over = pk.beyond ? 0u : pos & ((c1 > pk.target ? 1u : 0u) | (c2 > pk.target ? 2u : 0u) |
-                                                      (c3 > pk.target ? 4u : 0u) | (c4 > pk.target ? 8u : 0u));
-        const unsigned cross = __ballot_sync(0xffffffffu, over != 0), mass = __ballot_sync(0xffffffffu, pos != 0);
-        const int at = cross ? __ffs(cross) - 1 : mass ? 31 - __clz(mass) : 0;
-        const int j = __shfl_sync(0xffffffffu, over ? __ffs(over) - 1 : 31 - __clz(pos | 1u), at);
-        if (!hit && mass) {
-            tok = 512 * g + 128 * k + 4 * at + j;
-            hit = cross != 0;
-        }
-        C += shfl_f64(in[k], 31);
-    }
-    if (lane == 0) {
-        P.token[b] = tok;
-        if (P.flags) P.flags[b] = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u);
-    }
+    const RV row = RV::make(P, b, n);
+    if (!RV::kFixed) a.load(row.row, P.V, 512ll * g, RV::kFill);
+    const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
+    draw_held<kShift>(row, a, q, P.V, g, (int)csize * warps, csize, rank, u, s_sum, s_pick, P.token + b, P.flags ? P.flags + b : nullptr);
 }
 
 // ---- one shard of the vocabulary ---------------------------------------------------------------

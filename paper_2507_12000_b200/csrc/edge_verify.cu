@@ -24,6 +24,7 @@
 
 #include <math.h>
 
+#include "draw.cuh"
 #include "dssd_device.cuh"
 #include "edge_fold.cuh"
 #include "emit.cuh"
@@ -326,11 +327,97 @@ __device__ __forceinline__ void emit_pieces(const char *rowp, OUT *outp, int V, 
         emit_piece<DT, kShift, kPieceQuads>(rowp, outp, V, e, c1, ref2, invS);
 }
 
-// One cluster of up to kEdgeClusterMax CTAs per sequence does the whole of it.  Warp g of the cluster's takes the segments
+// The draw from row n of sequence b, by the cluster that has folded it: where its warps can hold the row (draw_held) as
+// the kernel of small draws does it; else the sums of segments of 512 entries go to the first CTA's shared memory,
+// and after a cluster barrier its first warp picks the segment, fetches it again and walks it.
+struct DrawShared {
+    double sum[kEdgeDrawSegs];
+    Pick pick;
+    int again;
+};
+static_assert(kEdgeDrawSegs >= 2 * kEdgeClusterWide * kWarps, "draw_held keeps two sets of sums");
+template <int DT, bool kShift, bool kHeld>
+__device__ __forceinline__ void draw_here(const EdgeParams &P, long long b, const char *rowp, int n, float ref2, float invS, unsigned csize,
+                                          unsigned rank, DrawShared &sh)
+{
+    [[maybe_unused]] const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, segs = (P.V + 511) / 512;
+    const float *q = n < P.gamma ? P.draft_q_rows + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
+    [[maybe_unused]] unsigned fl = q ? 0u : DSSD_RS_FLAG_BONUS;
+    RowLogits<DT> row;
+    row.row = rowp;
+    row.c1 = P.c1;
+    row.nref = -ref2;
+    row.invS = invS;
+    const float u = warp == 0 ? ld_after(P.draw_uniforms + b) : 0.f;
+    WarpQuads<typename RowLogits<DT>::Q, 4, kShift> a;
+    if constexpr (kHeld) {
+        const int g = warp * (int)csize + (int)rank;
+        a.load(rowp, P.V, 512ll * g, RowLogits<DT>::kFill);
+        draw_held<kShift>(row, a, q, P.V, g, kWarps * (int)csize, csize, rank, u, sh.sum, sh.pick, P.draw_token + b,
+                          P.draw_flags ? P.draw_flags + b : nullptr);
+    } else {
+        for (int g = warp * (int)csize + (int)rank; g < segs; g += kWarps * (int)csize) {
+            double none, t;
+            if (q) t = share_mass<true, false, kShift>(row, q, P.V, 512ll * g, none);
+            else t = share_mass<false, false, kShift>(row, q, P.V, 512ll * g, none);
+            t = warp_sum(t);
+            if (lane == 0) {
+                if (csize > 1) cluster_store(&sh.sum[g], 0u, t);
+                else sh.sum[g] = t;
+            }
+        }
+        if (csize > 1) {
+            cluster_arrive();
+            cluster_wait();
+        } else {
+            __syncthreads();
+        }
+        if (rank) return;
+        Pick pk;
+        auto pick = [&]() {
+            LaneSums L;
+            auto sum = [&](int c) { return sh.sum[c]; };
+            load_sums(L, segs, sum);
+            pk = pick_chunk(L, sum, false, [&](double Z) { return (double)u * Z; });
+        };
+        if (warp == 0) {
+            pick();
+            if (lane == 0) sh.again = !pk.ok && q;
+        }
+        __syncthreads();
+        if (sh.again) {  // the residual has no mass (p == q): draw from p instead; rare, so by this CTA alone
+            q = nullptr;
+            fl |= DSSD_RS_FLAG_FALLBACK;
+            for (int g = warp; g < segs; g += kWarps) {
+                double none;
+                const double t = warp_sum(share_mass<false, false, kShift>(row, q, P.V, 512ll * g, none));
+                if (lane == 0) sh.sum[g] = t;
+            }
+            __syncthreads();
+            if (warp == 0) pick();
+        }
+        if (warp) return;
+        int tok = -1;
+        if (pk.ok) {
+            double r[16];
+            a.load(rowp, P.V, 512ll * pk.chunk, RowLogits<DT>::kFill);
+            segment_residuals<kShift>(row, a, q, P.V, 512ll * pk.chunk, r);
+            tok = walk_segment(pk, r, pk.chunk);
+        }
+        if (lane == 0) {
+            P.draw_token[b] = tok;
+            if (P.draw_flags) P.draw_flags[b] = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u);
+        }
+    }
+}
+
+// One cluster of up to sixteen CTAs per sequence does the whole of it.  Warp g of the cluster's takes the segments
 // g, g + warps, .. of the sequence's rows; every segment's (ref, sum) goes to every CTA's shared memory, and after
-// one cluster barrier every CTA folds the sequence for itself and emits its part of row n.
-template <int DT, bool kShift>
-__global__ void __launch_bounds__(kThreads, 4) edge_cluster_kernel(const __grid_constant__ EdgeParams P)
+// one cluster barrier every CTA folds the sequence for itself and emits its part of row n.  kDraw = 1, 2: the call wants
+// tokens too (of every sequence, or of the fully accepted ones); 2 holds the row in registers meanwhile, which
+// saves fetching a segment again (B = 8 V = 32000 fused 7.9 us against 8.6) but costs half of the CTAs per SM.
+template <int DT, bool kShift, int kDraw>
+__global__ void __launch_bounds__(kThreads, kDraw == 2 ? 2 : 4) edge_cluster_kernel(const __grid_constant__ EdgeParams P)
 {
     __shared__ unsigned long long s_part[kEdgeClusterParts];
     __shared__ Drafted s_draft[kFoldRows];
@@ -350,9 +437,13 @@ __global__ void __launch_bounds__(kThreads, 4) edge_cluster_kernel(const __grid_
         const size_t di = (size_t)b * P.gamma + lane;
         Drafted d;
         d.x = ld_after(P.draft_tokens + di);
-        d.q = ld_after(P.draft_q_tok + di);
         d.u = ld_after(P.uniforms + di);
-        d.z = d.x >= 0 && d.x < P.V ? Elem<DT>::load(row_ptr<DT>(P, row0 + lane), d.x) : 0.f;
+        d.q = d.z = 0.f;
+        if (!P.draft_q_rows) d.q = ld_after(P.draft_q_tok + di);
+        if (d.x >= 0 && d.x < P.V) {
+            d.z = Elem<DT>::load(row_ptr<DT>(P, row0 + lane), d.x);
+            if (P.draft_q_rows) d.q = ld_after(P.draft_q_rows + di * (size_t)P.V + d.x);
+        }
         s_draft[lane] = d;
     }
     for (int t = g; t < P.runs * (P.gamma + 1); t += n_warps) {
@@ -371,7 +462,18 @@ __global__ void __launch_bounds__(kThreads, 4) edge_cluster_kernel(const __grid_
     }
     fold_sequence(P, b, rank == 0, sh, [&](int i, int k) { return s_part[i * P.runs + k]; }, [&](int i) { return s_draft[i]; });
     const int n = sh.n;
-    if (n < 0 || (P.skip_bonus_row && n == P.gamma)) return;
+    if (kDraw) {
+        __shared__ DrawShared sd;
+        if (n == P.gamma || (n >= 0 && P.draw_rejected)) {
+            draw_here<DT, kShift, kDraw == 2>(P, b, row_ptr<DT>(P, row0 + n), n, sh.ref2, sh.invS, csize, rank, sd);
+            return;
+        }
+        if (rank == 0 && threadIdx.x == 0) {  // no verdict, or a token that the device half draws
+            P.draw_token[b] = -1;
+            if (P.draw_flags) P.draw_flags[b] = n < 0 ? DSSD_RS_FLAG_INVALID : 0u;
+        }
+    }
+    if (n < 0) return;
     const char *rowp = row_ptr<DT>(P, row0 + n);
     if (P.p_row16) emit_pieces<DT, kShift>(rowp, P.p_row16 + (size_t)b * P.V, P.V, g, n_warps, P.c1, sh.ref2, sh.invS);
     else if (P.p_row) emit_pieces<DT, kShift>(rowp, P.p_row + (size_t)b * P.V, P.V, g, n_warps, P.c1, sh.ref2, sh.invS);
@@ -450,20 +552,29 @@ bool outputs_aligned(const EdgeParams &P)
     return emit_aligned(P.logits, P.row_stride, Elem<DT>::kBytes, P.p_row16 ? (const void *)P.p_row16 : P.p_row, P.V, P.p_row16 ? 2 : 4);
 }
 
-template <int DT>
+template <int DT, int kDraw>
 cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 {
     const unsigned grid = (unsigned)P.B * (unsigned)P.cluster;
-    return outputs_aligned<DT>(P) ? launch_pdl(edge_cluster_kernel<DT, false>, grid, kThreads, stream, P, 0, (unsigned)P.cluster)
-                                  : launch_pdl(edge_cluster_kernel<DT, true>, grid, kThreads, stream, P, 0, (unsigned)P.cluster);
+    const bool aligned = outputs_aligned<DT>(P) && (!P.draw_rejected || reinterpret_cast<uintptr_t>(P.draft_q_rows) % 16 == 0);
+    return aligned ? launch_pdl(edge_cluster_kernel<DT, false, kDraw>, grid, kThreads, stream, P, 0, (unsigned)P.cluster)
+                   : launch_pdl(edge_cluster_kernel<DT, true, kDraw>, grid, kThreads, stream, P, 0, (unsigned)P.cluster);
+}
+
+template <int DT>
+cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
+{
+    if (!P.draw_token) return launch_cluster<DT, 0>(P, stream);
+    const bool held = P.B * P.cluster <= kEdgeHeldWave && P.V <= 512 * kWarps * P.cluster;
+    return held ? launch_cluster<DT, 2>(P, stream) : launch_cluster<DT, 1>(P, stream);
 }
 
 // Clusters beyond the portable size have to be allowed for each kernel, and a device (or the part of one that the
 // process was given) may not have a processing cluster of that many SMs: asked once per device.
-template <int DT, bool kShift>
+template <int DT, bool kShift, int kDraw>
 bool wide_clusters()
 {
-    void (*kernel)(EdgeParams) = edge_cluster_kernel<DT, kShift>;
+    void (*kernel)(EdgeParams) = edge_cluster_kernel<DT, kShift, kDraw>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -477,6 +588,12 @@ bool wide_clusters()
     int n = 0;
     return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
 }
+template <int kDraw>
+bool wide_clusters()
+{
+    return wide_clusters<DSSD_F32, false, kDraw>() && wide_clusters<DSSD_F32, true, kDraw>() && wide_clusters<DSSD_BF16, false, kDraw>() &&
+           wide_clusters<DSSD_BF16, true, kDraw>();
+}
 int most_cluster_ctas()
 {
     static std::atomic<int> known[64];
@@ -484,8 +601,7 @@ int most_cluster_ctas()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return kEdgeCluster;
     int most = known[dev].load(std::memory_order_relaxed);
     if (!most) {
-        const bool wide = wide_clusters<DSSD_F32, false>() && wide_clusters<DSSD_F32, true>() && wide_clusters<DSSD_BF16, false>() &&
-                          wide_clusters<DSSD_BF16, true>();
+        const bool wide = wide_clusters<0>() && wide_clusters<1>() && wide_clusters<2>();
         if (!wide) cudaGetLastError();
         most = wide ? kEdgeClusterWide : kEdgeCluster;
         known[dev].store(most, std::memory_order_relaxed);
@@ -504,7 +620,7 @@ long long fit(long long c, long long wave, int B)
 int cluster_ctas(const EdgeParams &P, int esz, long long segs)
 {
     const long long parts = segs * (P.gamma + 1);
-    if (P.shard_sum || P.draft_q_rows || P.gamma >= kFoldRows || parts > kEdgeClusterParts) return 0;
+    if (P.shard_sum || P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kEdgeDrawSegs)) return 0;
     long long c = (parts + kWarps - 1) / kWarps;
     c = fit(c, kEdgeWave, P.B);
     if (c > 2) c = fit(c, kEdgeClusterWave, P.B);
@@ -513,7 +629,7 @@ int cluster_ctas(const EdgeParams &P, int esz, long long segs)
         c = wide > kEdgeCluster ? wide : kEdgeCluster;
         if (c > kEdgeCluster && c > most_cluster_ctas()) c = most_cluster_ctas();
     }
-    const double work = (double)(parts * (esz == 2 ? 2 : 1)) + (P.p_row || P.p_row16 ? (double)P.V / (128 * kPieceQuads) : 0.0);
+    const double work = (double)(parts * (esz == 2 ? 2 : 1)) + (P.p_row || P.p_row16 || P.draw_token ? (double)P.V / (128 * kPieceQuads) : 0.0);
     if (c > kEdgeCluster && work > kEdgeWideRounds * (double)(kWarps * c)) c = kEdgeCluster;
     if (c > kEdgeCluster) return (int)c;
     const long long ctas = P.B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;

@@ -40,7 +40,9 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
 constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, more
 constexpr double kEdgeWideRounds = 2.8;
-constexpr int kEdgeClusterParts = 3072;                  // segments of a sequence (24 KB of shared memory)
+constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
+constexpr int kEdgeDrawSegs = 1024;                      // segments of 512 entries of a row that the cluster kernel draws from (8 KB)
+constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory; the limits on the work allow 900)
 
 // What the draw needs to know about a folded sequence when no row is written.
 struct ReadySlot {
@@ -69,6 +71,13 @@ struct EdgeParams {
     float *lse;
     uint32_t *flags;
     int skip_bonus_row;    // 1: no row is emitted for fully accepted sequences (n == gamma)
+    // a token per sequence as well, if the cluster kernel runs (P.cluster != 0 after the launch; otherwise the caller draws):
+    // from row gamma for fully accepted sequences and, with draw_rejected, from max(0, p - q) of row n for the others,
+    // which get token -1 and flags 0 without it.  draw_rejected needs draft_q_rows.
+    int32_t *draw_token;
+    uint32_t *draw_flags;
+    const float *draw_uniforms;  // [B]
+    int draw_rejected;
     // one shard of the vocabulary (entries v_begin .. v_begin + V - 1 of every row): when shard_sum is
     // set only each row's partial sum is formed, sum_v 2^(l_v c1) = shard_sum * 2^shard_ref, and the
     // logits of the drafted tokens the shard holds are looked up; nothing is tested or emitted

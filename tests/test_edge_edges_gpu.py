@@ -5,6 +5,8 @@ import pytest
 
 import dssd_inputs as di
 from gpu_util import compare_round
+from test_parity_bonus_gpu import compare_bonus
+from test_parity_dsd_gpu import compare_dsd
 
 pytestmark = pytest.mark.gpu
 
@@ -41,3 +43,20 @@ def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
 def test_one_launch_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, zipf=True, seed=V + Bn)
     compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
+
+
+# The same launch with the draw in it (bonus at the edge; fused verification): rows held by the cluster's warps, with 16
+# CTAs and with one, and streamed, at the batch where the one ends and the other begins; segments of 512 entries at their
+# edges; residuals without mass, which fall back to the row itself.
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [
+    ("f32", 1, 2, 511), ("f32", 2, 2, 512), ("bf16", 3, 3, 513), ("bf16", 2, 1, 4096), ("bf16", 2, 1, 4097), ("f32", 3, 5, 16383),
+    ("bf16", 8, 4, 32000), ("f32", 4, 7, 20006), ("f32", 100, 3, 2048), ("f32", 101, 3, 2048), ("bf16", 200, 2, 1500), ("bf16", 201, 2, 1501),
+    ("f32", 64, 4, 9001), ("bf16", 592, 3, 3001), ("bf16", 600, 3, 6000), ("f32", 66, 15, 6240), ("f32", 130, 3, 33000),
+])
+def test_draws_in_the_same_launch(B, oracle_mod, dtype, Bn, gamma, V):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.4, zipf=True, seed=V + Bn)
+    d = di.generate(w, threads=16)
+    compare_bonus(B, oracle_mod, d, w.temperature, threads=16)
+    d["draft_q"][: (Bn + 1) // 2] = 1.0  # rejected nearly always, and max(0, p - q) is 0 everywhere
+    d["draft_q_tok"][: (Bn + 1) // 2] = 1.0
+    compare_dsd(B, oracle_mod, d, w.temperature, threads=16)
