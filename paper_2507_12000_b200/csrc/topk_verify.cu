@@ -39,6 +39,12 @@ constexpr int kSelThreads = 128;
 constexpr int kSelLoads = 8;                         // 16-byte loads a thread has in flight
 constexpr int kSelTile = kSelThreads * kSelLoads;    // 16-byte vectors of one pass over the CTA (16 KB)
 constexpr int kCand = 1024;                          // candidates that a CTA can hold
+// The first threshold: the k-th of 32 groups' maxima is tight and cheap for small k (k = 10: about 12 candidates per tile)
+// but near its smallest group for large ones (k = 32: 110 candidates, and ranking m of them costs m * m), where a bound
+// from all threads' maxima leaves 50.  More than kRefine candidates are cut back once more by the maxima over the whole
+// run.  B = 256 gamma = 4 V = 151936 bf16 k = 32: 85 us against 553 without both.
+constexpr int kGroupsUpTo = 12;
+constexpr int kRefine = 96;
 constexpr int kFoldWarps = 16;                       // most warps (rows at a time) of the fold kernel
 constexpr int kMergeCap = 256;                       // keys that a warp ranks when it merges a row's runs
 constexpr unsigned long long kBadList = ~0ull;       // first key of a run that held a NaN or +inf
@@ -122,7 +128,8 @@ struct Vec<DSSD_BF16> {
 struct SelectShared {
     unsigned long long key[kCand];
     unsigned long long top[32];
-    float grp[32];
+    uint4 grp[kSelThreads / 4];  // thresholds are taken from these maxima: of 32 groups, or of the threads
+    uint32_t tau[kSelThreads / 32];
     unsigned count;  // candidates found (more than kCand: some were dropped)
     int bad;         // the run holds a NaN or +inf
 };
@@ -131,6 +138,29 @@ __device__ __forceinline__ void push(SelectShared &sh, unsigned long long key)
 {
     const unsigned at = atomicAdd(&sh.count, 1u);
     if (at < (unsigned)kCand) sh.key[at] = key;
+}
+
+// A lower bound on the k-th largest of the threads' values x, each of which is an entry of its own: the smallest over
+// the warps of the ceil(k / 4)-th largest in the warp (k <= 32).  Cheaper than the k-th largest itself: the values
+// are compared within a warp only, as integers that carry the lane in their last bits.
+__device__ __forceinline__ float bound_of_threads(SelectShared &sh, float x, int k)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t mine = (ord(x) & ~31u) | (uint32_t)lane;
+    reinterpret_cast<uint32_t *>(sh.grp)[tid] = mine;
+    __syncwarp();
+    int rank = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const uint4 o = sh.grp[warp * 8 + j];
+        rank += (o.x > mine) + (o.y > mine) + (o.z > mine) + (o.w > mine);
+    }
+    if (rank == (k - 1) / 4) sh.tau[warp] = mine & ~31u;
+    __syncthreads();
+    uint32_t t = sh.tau[0];
+#pragma unroll
+    for (int w = 1; w < kSelThreads / 32; ++w) t = min(t, sh.tau[w]);
+    return t <= ord(DSSD_NEG_INF) ? DSSD_NEG_INF : unord(t);  // (below -inf there are NaNs)
 }
 
 // The k largest of the m keys in sh.key, best first, to sh.top (0 where there are fewer); by the whole CTA.
@@ -146,6 +176,28 @@ __device__ __forceinline__ void rank_keys(SelectShared &sh, int m, int k)
         if (rank < k) sh.top[rank] = x;
     }
     __syncthreads();
+}
+
+// Drops candidates that cannot be among the k best: the k-th largest of the threads' maxima over the whole run bounds
+// the k-th logit much more tightly than the first tile's did, and ranking costs the square of what is left.
+__device__ __noinline__ int refine(SelectShared &sh, int m, float top, int k)
+{
+    const int tid = threadIdx.x;
+    const float tau = bound_of_threads(sh, top == top ? top : DSSD_NEG_INF, k);
+    unsigned long long held[kCand / kSelThreads];
+#pragma unroll
+    for (int i = 0; i < kCand / kSelThreads; ++i) {
+        held[i] = 0ull;
+        if (i * kSelThreads + tid < m) held[i] = sh.key[i * kSelThreads + tid];
+    }
+    if (tid == 0) sh.count = 0;
+    __syncthreads();
+    const unsigned long long floor = (unsigned long long)ord(tau) << 32;
+#pragma unroll
+    for (int i = 0; i < kCand / kSelThreads; ++i)
+        if (held[i] != 0ull && held[i] >= floor) sh.key[atomicAdd(&sh.count, 1u)] = held[i];
+    __syncthreads();
+    return (int)sh.count;
 }
 
 // The run again, where the candidates did not fit: entry by entry, at most one per thread and step.
@@ -235,21 +287,26 @@ __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __gr
         top = max_nan(top, tm);
         unsigned hot = 0;
         if (first) {
-            // 32 groups of four threads: each group's maximum is one distinct entry
-            float g = tm == tm ? tm : DSSD_NEG_INF;
-            g = fmaxf(g, __shfl_xor_sync(kFullMask, g, 1));
-            g = fmaxf(g, __shfl_xor_sync(kFullMask, g, 2));
-            if ((tid & 3) == 0) sh.grp[tid >> 2] = g;
-            __syncthreads();
-            const float mine = sh.grp[lane];
-            int rank = 0;
+            const float x = tm == tm ? tm : DSSD_NEG_INF;
+            if (k > kGroupsUpTo) {
+                tau = bound_of_threads(sh, x, k);
+            } else {
+                // 32 groups of four threads: each group's maximum is one distinct entry
+                float g = fmaxf(x, __shfl_xor_sync(kFullMask, x, 1));
+                g = fmaxf(g, __shfl_xor_sync(kFullMask, g, 2));
+                float *grp = reinterpret_cast<float *>(sh.grp);
+                if ((tid & 3) == 0) grp[tid >> 2] = g;
+                __syncthreads();
+                const float mine = grp[lane];
+                int rank = 0;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float o = sh.grp[j];
-                rank += (o > mine) || (o == mine && j < lane);
+                for (int j = 0; j < 32; ++j) {
+                    const float o = grp[j];
+                    rank += (o > mine) || (o == mine && j < lane);
+                }
+                const unsigned hit = __ballot_sync(kFullMask, rank == k - 1);
+                tau = __shfl_sync(kFullMask, mine, __ffs(hit) - 1);
             }
-            const unsigned hit = __ballot_sync(kFullMask, rank == k - 1);
-            tau = __shfl_sync(kFullMask, mine, __ffs(hit) - 1);
             if (extra_at >= 0 && extra >= tau) push(sh, make_key(extra, extra_at));
 #pragma unroll
             for (int u = 0; u < kSelLoads; ++u) hot |= vm[u] >= tau && base + tid + u * kSelThreads < v1 ? 1u << u : 0u;
@@ -262,10 +319,18 @@ __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __gr
             const int at = base + tid + (__ffs(hot) - 1) * kSelThreads;
             hot &= hot - 1u;
             const uint4 v = ld_stream16(src + at);  // from L2: the registers have moved on
+            unsigned mask = 0;
 #pragma unroll
             for (int j = 0; j < E; ++j) {
                 const float f = Vec<DT>::elem(v, j);
-                if (first ? f >= tau : f > tau) push(sh, make_key(f, idx0 + at * E + j));
+                mask |= (first ? f >= tau : f > tau) ? 1u << j : 0u;
+            }
+            unsigned to = atomicAdd(&sh.count, (unsigned)__popc(mask));
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                if (!(mask >> j & 1u)) continue;
+                if (to < (unsigned)kCand) sh.key[to] = make_key(Vec<DT>::elem(v, j), idx0 + at * E + j);
+                ++to;
             }
         }
         first = false;
@@ -278,6 +343,7 @@ __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __gr
         select_slowly<DT>(sh, rowp, e0, e1, k);
         m = (int)sh.count;
     }
+    if (m > kRefine) m = refine(sh, m, top, k);
     rank_keys(sh, m, k);
     if (tid < k) {
         unsigned long long key = sh.top[tid];
@@ -308,8 +374,11 @@ __device__ __forceinline__ RowDist dist_from_keys(const TopkParams &P, unsigned 
     const double z = (double)val / T;
     const double mx = __shfl_sync(kFullMask, z, 0);
     const double e = lane < k ? exp(z - mx) : 0.0;
-    double S = 0.0;
-    for (int r = 0; r < k; ++r) S += __shfl_sync(kFullMask, e, r);
+    double S = 0.0;  // in rank order; the lanes beyond k add 0
+    for (int r = 0; r < k; r += 4) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) S += __shfl_sync(kFullMask, e, r + j);
+    }
     d.idx = lane < k ? key_index(key) : -1;
     d.prob = e / S;
     return d;
@@ -326,7 +395,7 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x)
 }
 
 struct MergeShared {
-    unsigned long long key[kMergeCap];
+    unsigned long long key[kMergeCap + 8];
     unsigned long long top[32];
 };
 
@@ -338,10 +407,10 @@ __device__ __forceinline__ unsigned long long merged_keys(const unsigned long lo
     const int lane = threadIdx.x & 31;
     if (runs == 1) return lane < k ? ld_after(src + lane) : 0ull;
     const int m = runs * k;
-    // one round trip for the lists' ends and (up to 128 of them) their keys
-    unsigned long long x[4];
+    // one round trip for the lists' ends and (up to 256 of them) their keys
+    unsigned long long x[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) x[u] = 32 * u + lane < m ? ld_after(src + 32 * u + lane) : 0ull;
+    for (int u = 0; u < 8; ++u) x[u] = 32 * u + lane < m ? ld_after(src + 32 * u + lane) : 0ull;
     unsigned long long bound = 0ull;
     bool bad = false;
     for (int r = lane; r < runs; r += 32) {
@@ -355,16 +424,16 @@ __device__ __forceinline__ unsigned long long merged_keys(const unsigned long lo
     int c = 0;
     for (int i0 = 0;;) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
             const unsigned keep = __ballot_sync(kFullMask, x[u] >= bound);
             const int at = c + __popc(keep & ((1u << lane) - 1u));
             if (x[u] >= bound && at < kMergeCap) sh.key[at] = x[u];
             c += __popc(keep);
         }
-        i0 += 128;
+        i0 += 256;
         if (i0 >= m) break;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = i0 + 32 * u + lane < m ? ld_after(src + i0 + 32 * u + lane) : 0ull;
+        for (int u = 0; u < 8; ++u) x[u] = i0 + 32 * u + lane < m ? ld_after(src + i0 + 32 * u + lane) : 0ull;
     }
     __syncwarp();
     if (c > kMergeCap) {  // lists that interleave evenly: one best key after the other
@@ -380,10 +449,15 @@ __device__ __forceinline__ unsigned long long merged_keys(const unsigned long lo
         }
         return mine;
     }
+    if (lane < 8) sh.key[c + lane] = 0ull;  // the ranking goes in steps of eight
+    __syncwarp();
     for (int i = lane; i < c; i += 32) {
         const unsigned long long y = sh.key[i];
         int rank = 0;
-        for (int j = 0; j < c; ++j) rank += sh.key[j] > y;
+        for (int j0 = 0; j0 < c; j0 += 8) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) rank += sh.key[j0 + j] > y;
+        }
         if (rank < k) sh.top[rank] = y;
     }
     __syncwarp();
@@ -480,19 +554,19 @@ __device__ __forceinline__ double shfl_f64(double v, int src) { return __shfl_sy
 // returns the position, or -1 when the mass is not positive and finite
 __device__ __forceinline__ int warp_inverse_cdf(double r, int k, double u)
 {
-    double Z = 0.0;
-    for (int e = 0; e < k; ++e) Z += shfl_f64(r, e);
-    if (!(Z > 0.0) || !(Z < INFINITY)) return -1;
-    const double t = u * Z;
-    double C = 0.0;
-    int last_pos = -1, hit = -1;
-    for (int e = 0; e < k; ++e) {
-        const double re = shfl_f64(r, e);
-        C += re;
-        if (re > 0.0) last_pos = e;
-        if (hit < 0 && C > t) hit = e;
+    const int lane = threadIdx.x & 31;
+    double C = 0.0, mine = 0.0;  // the running mass in index order (lanes beyond k hold 0); this lane's
+    for (int e0 = 0; e0 < k; e0 += 4) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            C += shfl_f64(r, e0 + j);
+            if (lane == e0 + j) mine = C;
+        }
     }
-    return hit >= 0 ? hit : last_pos;
+    if (!(C > 0.0) || !(C < INFINITY)) return -1;
+    const unsigned hit = __ballot_sync(kFullMask, lane < k && mine > u * C);
+    const unsigned positive = __ballot_sync(kFullMask, r > 0.0);
+    return hit ? __ffs(hit) - 1 : 31 - __clz(positive);
 }
 
 __global__ void __launch_bounds__(kThreads) topk_resample_kernel(const __grid_constant__ TopkResampleParams P)
@@ -506,7 +580,7 @@ __global__ void __launch_bounds__(kThreads) topk_resample_kernel(const __grid_co
     if (b >= P.B) return;
     const int n = ld_after(P.accept_len + b);
     const double u = (double)ld_after(P.uniforms + b);
-    const int pi = lane < k ? ld_after(P.p_idx + (size_t)b * k + lane) : 0;
+    const int pi = lane < k ? ld_after(P.p_idx + (size_t)b * k + lane) : 0x7fffffff;
     const float pv = lane < k ? ld_after(P.p_val + (size_t)b * k + lane) : 0.f;
     const bool has_row = !__any_sync(kFullMask, lane < k && pi < 0);
     unsigned fl = 0u;
@@ -516,7 +590,10 @@ __global__ void __launch_bounds__(kThreads) topk_resample_kernel(const __grid_co
     } else {
         // P's entries in increasing vocabulary index (indices are distinct)
         int rank = 0;
-        for (int e = 0; e < k; ++e) rank += __shfl_sync(kFullMask, pi, e) < pi;
+        for (int e0 = 0; e0 < k; e0 += 4) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) rank += __shfl_sync(kFullMask, pi, e0 + j) < pi;
+        }
         if (lane < k) {
             s_idx[warp][rank] = pi;
             s_val[warp][rank] = pv;
@@ -533,10 +610,13 @@ __global__ void __launch_bounds__(kThreads) topk_resample_kernel(const __grid_co
             const int qi = lane < k ? ld_after(P.q_idx + qo + lane) : -1;
             const float qv = lane < k ? ld_after(P.q_val + qo + lane) : 0.f;
             float sq = 0.f;
-            for (int f = k - 1; f >= 0; --f) {  // the first listed match wins
-                const int fi = __shfl_sync(kFullMask, qi, f);
-                const float fv = __shfl_sync(kFullMask, qv, f);
-                if (fi == sid) sq = fv;
+            for (int f0 = (k - 1) & ~3; f0 >= 0; f0 -= 4) {  // the first listed match wins
+#pragma unroll
+                for (int j = 3; j >= 0; --j) {
+                    const int fi = __shfl_sync(kFullMask, qi, f0 + j);
+                    const float fv = __shfl_sync(kFullMask, qv, f0 + j);
+                    if (fi == sid) sq = fv;
+                }
             }
             const double r = lane < k ? fmax(0.0, sp - (double)sq) : 0.0;
             pos = warp_inverse_cdf(r, k, u);

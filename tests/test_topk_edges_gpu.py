@@ -22,7 +22,7 @@ def B():
     ("f32", 3, 1, 4095, 32), ("f32", 3, 1, 4096, 1), ("f32", 3, 1, 4099, 10), ("bf16", 3, 2, 8191, 32), ("bf16", 3, 2, 8192, 10),
     ("bf16", 3, 2, 8200, 32), ("bf16", 2, 1, 16400, 32), ("f32", 4, 15, 9000, 10), ("f32", 4, 16, 9001, 10),
     ("f32", 587, 1, 16384, 10), ("f32", 588, 1, 16384, 10), ("f32", 791, 2, 32768, 4), ("f32", 792, 2, 32768, 32),
-    ("f32", 2, 1, 600001, 32),
+    ("f32", 2, 1, 600001, 32), ("bf16", 3, 2, 8200, 12), ("bf16", 3, 2, 8200, 13), ("f32", 3, 2, 200, 20), ("bf16", 800, 2, 65536, 32),
 ])
 def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V, k):
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, seed=V + Bn)
