@@ -513,14 +513,15 @@ __global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_c
 size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base)
 {
     // one sum per chunk; batches whose sums would take more than the built-in scratch of
-    // dssd_device_resample_static keep one per tile, whose chunks the draw then looks at in turn
-    const size_t chunks = ((size_t)V + kSub - 1) / kSub, tiles = ((size_t)V + kTile - 1) / kTile;
-    const bool fine = (size_t)B * chunks * sizeof(double) <= (size_t)DSSD_STATIC_SCRATCH_BYTES;
-    const size_t n_sub = fine ? chunks : tiles;
+    // dssd_device_resample_static keep one per two chunks or per tile, which the draw then looks at in turn
+    int rows = 1;
+    auto sums = [&]() { return ((size_t)V + (size_t)(rows * kSub) - 1) / (size_t)(rows * kSub); };
+    while (rows < kRows && (size_t)B * sums() * sizeof(double) > (size_t)DSSD_STATIC_SCRATCH_BYTES) rows *= 2;
+    const size_t n_sub = sums();
     if (P) {
         P->chunk_sum = reinterpret_cast<double *>(base);
         P->n_sub = (int)n_sub;
-        P->rows_per_sum = fine ? 1 : kRows;
+        P->rows_per_sum = rows;
     }
     return ((size_t)B * n_sub * sizeof(double) + 255) & ~(size_t)255;
 }

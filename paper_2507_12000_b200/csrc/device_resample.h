@@ -33,7 +33,7 @@ struct ResampleParams {
     int tiles;         // tiles per CTA of the mass kernel
     int n_ctas;        // such CTAs per sequence
     int cluster_threads;  // threads per CTA of the cluster kernel (n_ctas per sequence), 0: mass kernel and draw kernel
-    int rows_per_sum;  // chunks per stored sum: 1, or 4 (a whole tile) in the largest batches
+    int rows_per_sum;  // chunks per stored sum: 1, or 2 or 4 (a whole tile) in the largest batches
     int n_sub;         // stored sums per sequence
     double *chunk_sum;   // scratch [B, n_sub]
     // test hook (0: off): the chunk sums of sequence test_drop_seq_plus1 - 1 are formed but never stored

@@ -22,7 +22,7 @@ def B():
     (9, 2, 511, False), (9, 2, 513, True), (25, 1, 32768, False), (26, 1, 32768, False), (3, 2, 32769, False), (6, 1, 65536, True),
     (7, 1, 65536, False), (4, 2, 65537, False), (200, 1, 900, False), (201, 1, 900, True), (5, 1, 50257, True), (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
     (600, 1, 4096, False), (601, 1, 4096, True), (1200, 1, 2047, True), (1201, 1, 2047, False), (2400, 1, 1024, False), (2401, 1, 1024, False),
-    (6, 2, 9001, False), (6, 3, 9002, True), (7, 2, 9003, True), (6, 2, 9003, False), (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True),
+    (6, 2, 9001, False), (6, 3, 9002, True), (7, 2, 9003, True), (6, 2, 9003, False), (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True), (32768, 1, 4097, False), (32769, 1, 8193, True),
 ])
 def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
     gen = torch.Generator(device="cuda").manual_seed(Bn + V)
