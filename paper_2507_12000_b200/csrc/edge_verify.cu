@@ -74,6 +74,37 @@ __device__ __forceinline__ void add_pair(f32x2 &acc, float a, float b, f32x2 cc,
     acc = add2(acc, pack2(ex2(x), ex2(y)));
 }
 
+// x within [-127, 128]; a NaN stays one
+__device__ __forceinline__ float clamp_nan(float x)
+{
+    float r;
+    asm("{\n\t.reg .f32 t;\n\tmax.NaN.f32 t, %1, 0fC2FE0000;\n\tmin.NaN.f32 %0, t, 0f43000000;\n\t}" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The same without the special-function unit, which bf16 rows keep four fifths busy: 2^x = 2^n 2^f with n = rint(x)
+// and a polynomial for 2^f, |f| <= 1/2, of degree 6, fitted for the least relative error by Remez exchange (1.9e-9; 8e-8 with float32
+// roundings, the unit's own error is 2^-22).  Adding kRound leaves n + 127 in the last bits, which shifted up are the
+// float 2^n: 0 for n = -127 and infinity for n = 128, where the unit's results end too.  A NaN stays one.
+__device__ __forceinline__ void add_pair_by_fma(f32x2 &acc, float a, float b, f32x2 cc, f32x2 nn)
+{
+    constexpr float kRound = 12582912.f + 127.f;
+    float x, y, tx, ty;
+    unpack2(fma2(pack2(a, b), cc, nn), x, y);
+    const f32x2 z = pack2(clamp_nan(x), clamp_nan(y));
+    const f32x2 t = add2(z, pack2(kRound, kRound));
+    const f32x2 f = fma2(add2(t, pack2(-kRound, -kRound)), pack2(-1.f, -1.f), z);
+    unpack2(t, tx, ty);
+    f32x2 p = pack2(1.534581242594868e-4f, 1.534581242594868e-4f);
+    p = fma2(p, f, pack2(1.3399930903688073e-3f, 1.3399930903688073e-3f));
+    p = fma2(p, f, pack2(9.618489071726799e-3f, 9.618489071726799e-3f));
+    p = fma2(p, f, pack2(5.550328642129898e-2f, 5.550328642129898e-2f));
+    p = fma2(p, f, pack2(2.4022646248340607e-1f, 2.4022646248340607e-1f));
+    p = fma2(p, f, pack2(6.931471824645996e-1f, 6.931471824645996e-1f));
+    p = fma2(p, f, pack2(1.f, 1.f));
+    acc = fma2(p, pack2(__uint_as_float(__float_as_uint(tx) << 23), __uint_as_float(__float_as_uint(ty) << 23)), acc);
+}
+
 template <int DT>
 __device__ __forceinline__ float vec_max(const uint4 &v)
 {
@@ -84,14 +115,16 @@ __device__ __forceinline__ float vec_max(const uint4 &v)
     return fmaxf(fmaxf(__uint_as_float(v.x), __uint_as_float(v.y)), fmaxf(__uint_as_float(v.z), __uint_as_float(v.w)));
 }
 
-template <int DT>
+// kFma: a quarter of a bf16 vector's terms on the FMA pipe
+template <int DT, bool kFma>
 __device__ __forceinline__ void add_vec(Online &o, const uint4 &v, f32x2 cc, f32x2 nn)
 {
     if (DT == DSSD_BF16) {
         add_pair(o.s0, bf16_lo(v.x), bf16_hi(v.x), cc, nn);
         add_pair(o.s1, bf16_lo(v.y), bf16_hi(v.y), cc, nn);
         add_pair(o.s2, bf16_lo(v.z), bf16_hi(v.z), cc, nn);
-        add_pair(o.s3, bf16_lo(v.w), bf16_hi(v.w), cc, nn);
+        if (kFma) add_pair_by_fma(o.s3, bf16_lo(v.w), bf16_hi(v.w), cc, nn);
+        else add_pair(o.s3, bf16_lo(v.w), bf16_hi(v.w), cc, nn);
     } else {
         add_pair(o.s0, __uint_as_float(v.x), __uint_as_float(v.y), cc, nn);
         add_pair(o.s1, __uint_as_float(v.z), __uint_as_float(v.w), cc, nn);
@@ -113,8 +146,12 @@ __device__ __forceinline__ void add_tile(Online &o, const uint4 (&v)[kLseLoads],
     for (int u = 1; u < kLseLoads; ++u) bm = fmaxf(bm, vec_max<DT>(v[u]));
     online_raise(o, bm, c1);
     const f32x2 cc = pack2(c1, c1), nn = pack2(-o.ref, -o.ref);
+    // every second vector: B = 256 gamma = 4 V = 151936 63.3 us against 64.5 without and 63.9 with every vector
 #pragma unroll
-    for (int u = 0; u < kLseLoads; ++u) add_vec<DT>(o, v[u], cc, nn);
+    for (int u = 0; u < kLseLoads; u += 2) {
+        add_vec<DT, true>(o, v[u], cc, nn);
+        add_vec<DT, false>(o, v[u + 1], cc, nn);
+    }
 }
 
 // one entry more

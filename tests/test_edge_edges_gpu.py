@@ -60,3 +60,27 @@ def test_draws_in_the_same_launch(B, oracle_mod, dtype, Bn, gamma, V):
     d["draft_q"][: (Bn + 1) // 2] = 1.0  # rejected nearly always, and max(0, p - q) is 0 everywhere
     d["draft_q_tok"][: (Bn + 1) // 2] = 1.0
     compare_dsd(B, oracle_mod, d, w.temperature, threads=16)
+
+
+@pytest.mark.parametrize("dtype,V,stride", [("bf16", 4096, 1), ("bf16", 40000, 97), ("f32", 4096, 1)])
+def test_every_entry_of_a_vector_counts(B, dtype, V, stride):
+    """Some terms of a row's sum are formed by a polynomial, the others by the special-function unit: a NaN is seen in
+    every position, -inf and terms far below the largest weigh nothing, and a row of one entry above -inf is 1 there."""
+    import torch
+
+    Bn, dt = 40, torch.bfloat16 if dtype == "bf16" else torch.float32
+    at = torch.arange(Bn, device="cuda") * stride
+    rows = torch.arange(Bn, device="cuda")
+    none = torch.empty(Bn, 0, device="cuda")
+    run = lambda z: B.dssd_edge_verify(z.view(Bn, 1, V), none.int(), none, none, 1.0)
+    z = torch.zeros(Bn, V, dtype=dt, device="cuda")
+    z[rows, at] = float("nan")
+    assert (run(z)["flags"] == B.EDGE_FLAG_NONFINITE).all()
+    for low in (float("-inf"), -1.0e4, -200.0, -90.0):
+        z = torch.full((Bn, V), low, dtype=dt, device="cuda")
+        z[rows, at] = 1.5
+        ev = run(z)
+        assert (ev["flags"] == 0).all()
+        assert ((ev["p_row"][rows, at] - 1.0).abs() <= 3e-7).all() and ((ev["lse"][:, 0] - 1.5).abs() <= 1e-6).all()
+    z = torch.zeros(Bn, V, dtype=dt, device="cuda")  # equal entries: n in all positions
+    assert ((run(z)["p_row"] * V - 1.0).abs() <= 2e-6).all()
