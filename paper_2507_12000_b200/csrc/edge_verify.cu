@@ -544,6 +544,53 @@ __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_con
     }
 }
 
+// The same in one launch, chosen as the cluster kernel is: the partial sums go to the first CTA's shared memory.
+template <int DT>
+__global__ void __launch_bounds__(kThreads, 4) edge_partial_cluster_kernel(const __grid_constant__ EdgeParams P)
+{
+    __shared__ unsigned long long s_part[kEdgeClusterParts];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned csize = (unsigned)P.cluster, rank = csize > 1 ? cluster_rank() : 0u;
+    const long long b = blockIdx.x / csize, row0 = b * (P.gamma + 1);
+    if (csize > 1) {  // the first CTA's shared memory may be written once it is known to run
+        cluster_arrive();
+        cluster_wait();
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (rank == 0 && warp == kWarps - 1 && lane < P.gamma) {
+        const size_t di = (size_t)b * P.gamma + lane;
+        const long long x = (long long)ld_after(P.draft_tokens + di) - (long long)P.v_begin;
+        P.shard_tok_logit[di] = x >= 0 && x < (long long)P.V ? Elem<DT>::load(row_ptr<DT>(P, row0 + lane), x) : __int_as_float(0x7fc00000);
+    }
+    for (int t = warp * (int)csize + (int)rank; t < P.runs * (P.gamma + 1); t += kWarps * (int)csize) {
+        const int i = t / P.runs;
+        float R, s;
+        warp_lse<DT>(row_ptr<DT>(P, row0 + i), P.V, t - i * P.runs, P.runs, P.c1, R, s);
+        const unsigned long long word = row0 + i + 1 == P.test_drop_row_plus1 ? kNoPartial : partial_word(R, s);
+        if (lane == 0) {
+            if (csize > 1) cluster_store(&s_part[t], 0u, word);
+            else s_part[t] = word;
+        }
+    }
+    if (csize > 1) {
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    if (rank) return;
+    const int i = tid / kFoldLanes, sub = tid % kFoldLanes;
+    float R;
+    double S;
+    bool missing;
+    row_total([&](int k) { return s_part[i * P.runs + k]; }, P.runs, sub, i <= P.gamma, R, S, missing);
+    if (i <= P.gamma && sub == 0) {
+        P.shard_ref[row0 + i] = R == DSSD_NEG_INF ? 0.f : R;
+        P.shard_sum[row0 + i] = missing || S != S ? (double)__int_as_float(0x7fc00000) : S;
+    }
+}
+
 }  // namespace
 
 int edge_max_runs_per_row(int V)
@@ -601,6 +648,8 @@ cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 template <int DT>
 cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 {
+    if (P.shard_sum)
+        return launch_pdl(edge_partial_cluster_kernel<DT>, (unsigned)P.B * (unsigned)P.cluster, kThreads, stream, P, 0, (unsigned)P.cluster);
     if (!P.draw_token) return launch_cluster<DT, 0>(P, stream);
     const bool held = P.B * P.cluster <= kEdgeHeldWave && P.V <= 512 * kWarps * P.cluster;
     return held ? launch_cluster<DT, 2>(P, stream) : launch_cluster<DT, 1>(P, stream);
@@ -608,10 +657,8 @@ cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 
 // Clusters beyond the portable size have to be allowed for each kernel, and a device (or the part of one that the
 // process was given) may not have a processing cluster of that many SMs: asked once per device.
-template <int DT, bool kShift, int kDraw>
-bool wide_clusters()
+bool wide_clusters(void (*kernel)(EdgeParams))
 {
-    void (*kernel)(EdgeParams) = edge_cluster_kernel<DT, kShift, kDraw>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -625,11 +672,15 @@ bool wide_clusters()
     int n = 0;
     return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
 }
-template <int kDraw>
+template <int DT, int kDraw>
 bool wide_clusters()
 {
-    return wide_clusters<DSSD_F32, false, kDraw>() && wide_clusters<DSSD_F32, true, kDraw>() && wide_clusters<DSSD_BF16, false, kDraw>() &&
-           wide_clusters<DSSD_BF16, true, kDraw>();
+    return wide_clusters(edge_cluster_kernel<DT, false, kDraw>) && wide_clusters(edge_cluster_kernel<DT, true, kDraw>);
+}
+template <int DT>
+bool wide_clusters()
+{
+    return wide_clusters<DT, 0>() && wide_clusters<DT, 1>() && wide_clusters<DT, 2>() && wide_clusters(edge_partial_cluster_kernel<DT>);
 }
 int most_cluster_ctas()
 {
@@ -638,7 +689,7 @@ int most_cluster_ctas()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return kEdgeCluster;
     int most = known[dev].load(std::memory_order_relaxed);
     if (!most) {
-        const bool wide = wide_clusters<0>() && wide_clusters<1>() && wide_clusters<2>();
+        const bool wide = wide_clusters<DSSD_F32>() && wide_clusters<DSSD_BF16>();
         if (!wide) cudaGetLastError();
         most = wide ? kEdgeClusterWide : kEdgeCluster;
         known[dev].store(most, std::memory_order_relaxed);
@@ -657,7 +708,7 @@ long long fit(long long c, long long wave, int B)
 int cluster_ctas(const EdgeParams &P, int esz, long long segs)
 {
     const long long parts = segs * (P.gamma + 1);
-    if (P.shard_sum || P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kEdgeDrawSegs)) return 0;
+    if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kEdgeDrawSegs)) return 0;
     long long c = (parts + kWarps - 1) / kWarps;
     c = fit(c, kEdgeWave, P.B);
     if (c > 2) c = fit(c, kEdgeClusterWave, P.B);
@@ -667,10 +718,11 @@ int cluster_ctas(const EdgeParams &P, int esz, long long segs)
         if (c > kEdgeCluster && c > most_cluster_ctas()) c = most_cluster_ctas();
     }
     const double work = (double)(parts * (esz == 2 ? 2 : 1)) + (P.p_row || P.p_row16 || P.draw_token ? (double)P.V / (128 * kPieceQuads) : 0.0);
-    if (c > kEdgeCluster && work > kEdgeWideRounds * (double)(kWarps * c)) c = kEdgeCluster;
+    if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
     if (c > kEdgeCluster) return (int)c;
     const long long ctas = P.B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
     const double fill = (double)ctas / (double)(waves * kEdgeWave);
+    if (P.shard_sum) return work <= (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0) * (double)(kWarps * c) ? (int)c : 0;
     const double limit = fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0;
     return work <= limit * (double)(kWarps * c) ? (int)c : 0;
 }

@@ -37,9 +37,12 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //              B = 318 gamma = 4 V = 9792 bf16 16.3 / 20.2; beyond B = 661 gamma = 1 V = 72431 bf16 110 / 86
 //   full wave:  B = 89 gamma = 4 V = 18896 float32 9.6 / 13.0, B = 64 gamma = 4 V = 128256 bf16 26.5 / 29.7,
 //              B = 128 gamma = 4 V = 50272 float32 30.7 / 32.3; beyond B = 166 gamma = 11 V = 53648 bf16 52.8 / 48.8.
+// A shard's partial sums have no emission to share a launch with and pay off up to less work per warp: B = 256 gamma = 4 V = 18992
+// bf16 13.5 / 14.2, B = 503 gamma = 3 V = 5936 float32 8.5 / 11.1, B = 620 gamma = 15 V = 792 bf16 9.7 / 28.4; beyond B = 173 gamma = 3
+// V = 67023 float32 40.5 / 30.5, B = 2 gamma = 2 V = 79648 float32 5.4 / 4.6.
 constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
 constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, more
-constexpr double kEdgeWideRounds = 2.8;
+constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
 constexpr int kEdgeDrawSegs = 1024;                      // segments of 512 entries of a row that the cluster kernel draws from (8 KB)
 constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory; the limits on the work allow 900)
