@@ -38,24 +38,20 @@ UNIT = "rows/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 
-# DRAM traffic of the dominant kernel from ncu (dram__bytes_read.sum + dram__bytes_write.sum,
-# bytes per launch), valid only for the kernel source whose hash is recorded with it.
+# DRAM traffic of the edge call from ncu (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the kernel
+# sources whose hash is recorded with it.
 NCU_TRAFFIC = {
-    # profiles/edge_verify_kernel_c4.md: 428.4 MB read (389.0 MB of logits + 51 % of the second read of row n)
-    # and 96.6 MB written inside the kernel; the other 59.0 MB of p_row were still in L2 when the kernel ended
-    # and reach DRAM after it.  "bytes" counts all of p_row.
-    "c4": {"bytes": 428413440 + 155582464, "kernel_hash": "174f9e8708fc9d97",
-           "note": "dram__bytes_read.sum 428.4 MB + all 155.6 MB of p_row (96.6 MB of it written inside the "
-                   "kernel, the rest still in L2 at its end); reads are 1.10x the logits: the second read of "
-                   "row n misses L2 for 51 % of its bytes",
-           "counted_inside_kernel": 428413440 + 96619264},
+    # profiles/edge_call_c4.md: log-sum-exp kernel 389.0 MB read, fold 0.03, emission 71.0 MB read and 141.0 MB written
+    # inside it; the other 14.6 MB of p_row were still in L2 when it ended.  "bytes" counts all of p_row.
+    "c4": {"bytes": 389025280 + 31744 + 71031552 + 155582464, "kernel_hash": "94b44e9f62f356a1",
+           "note": "dram__bytes_read.sum 460.1 MB + all 155.6 MB of p_row; reads are 1.18x the logits: the second read of "
+                   "row n misses L2 for 91 % of its bytes",
+           "counted_inside_kernel": 389025280 + 31744 + 71031552 + 6894848 + 141007360},
 }
 
 
-# the same for topk_verify_kernel (k = 10)
+# the same for the two kernels of the top-k edge call (k = 10)
 NCU_TRAFFIC_TOPK = {
-    # profiles/topk_verify_kernel_c4.md: 389.1 MB read + 3.4 MB written
-    "c4": {"bytes": 389107968 + 3403264, "kernel_hash": "191879487eaaf336"},
 }
 
 
@@ -69,10 +65,23 @@ def _kernel_hash_topk() -> str:
 
 def _kernel_hash() -> str:
     h = hashlib.sha256()
-    for f in ("edge_verify.cu", "edge_verify.h", "edge_judge.cuh", "dssd_device.cuh"):
+    for f in ("edge_verify.cu", "edge_verify.h", "edge_fold.cuh", "emit.cuh", "edge_judge.cuh", "dssd_device.cuh"):
         with open(os.path.join(ROOT, "paper_2507_12000_b200", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
+
+
+def _launches_per_step(step) -> int:
+    """The library's kernels in one step, counted by the profiler after the timed region."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    step()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        step()
+        torch.cuda.synchronize()
+    return sum(1 for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA and "dssd::" in e.name)
 
 
 def _peaks():
@@ -346,6 +355,7 @@ def run_ours(args, w: di.Workload, light: bool = False):
     sampler.stop_flag = True
     sampler.join(timeout=1.0)
     clocks = sampler.summary(t_host0, t_host1)
+    launches = _launches_per_step(lambda: step(0))
     n_gpu = ev_out["accept_len"].cpu().numpy()
     n_bonus = int((n_gpu == gamma).sum())
 
@@ -492,7 +502,7 @@ def run_ours(args, w: di.Workload, light: bool = False):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": max(args.warmup, 3),
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "f32", "data": "synthetic", "config": _config(w, args),
-        "roofline": {"bound": "hbm", "kernel": "edge_verify_kernel", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "edge call (edge_lse_kernel, edge_fold_kernel, edge_emit_kernel; small launches edge_cluster_kernel)", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
                      "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS,
                      "algorithmic_bytes_per_launch": edge_bytes, "avg_launch_ms": edge_avg_ms,
@@ -513,14 +523,14 @@ def run_ours(args, w: di.Workload, light: bool = False):
         "cpu_baseline": cpu,
         "parity": parity,
         "e2e": e2e,
-        "gpu_launches": (3 if bonus_edge else 2) * K * len(loops),
+        "gpu_launches": launches * K * len(loops),
         "clocks": clocks,
     }
     if bonus_edge:
         line["config"]["workload"] = line["config"]["workload"].replace(
             f"{w.name}:", f"{w.name}, bonus token drawn at the edge (Algorithm 2 as printed):")
         line["config"]["fully_accepted_sequences"] = n_bonus
-        line["roofline"]["kernel"] = "edge_verify_kernel + resample_kernel<RowLogits> (dssd_edge_verify_bonus)"
+        line["roofline"]["kernel"] = "edge call and bonus draw (dssd_edge_verify_bonus)"
     if world > 1:
         dist.destroy_process_group()
     return line
@@ -639,6 +649,7 @@ def run_ours_topk(args, w: di.Workload):
     sampler.stop_flag = True
     sampler.join(timeout=1.0)
     clocks = sampler.summary(t_host0, t_host1)
+    launches = _launches_per_step(lambda: step(sets[0]))
     n_gpu = ev_out["accept_len"].cpu().numpy()
     tok_gpu = rs_out["token"].cpu().numpy()
 
@@ -708,7 +719,7 @@ def run_ours_topk(args, w: di.Workload):
         "metric": METRIC, "value": world * rows / (ms_per_step * 1e-3), "unit": UNIT, "n_gpus": world, "steps": K,
         "warmup": max(args.warmup, 3), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f64", "data": "synthetic", "config": _config_topk(w, args),
-        "roofline": {"bound": "hbm", "kernel": "topk_verify_kernel", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "topk_select_kernel + topk_fold_kernel", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
                      "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS,
                      "algorithmic_bytes_per_launch": edge_bytes, "avg_launch_ms": edge_avg_ms,
@@ -721,7 +732,7 @@ def run_ours_topk(args, w: di.Workload):
         "e2e": {"value": world * rows / (e2e_ms / e2e_steps * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "steps": e2e_steps, "ms_per_step": e2e_ms / e2e_steps},
         "timed": {"loops": len(loops), "device_ms": sum(lp["total_ms"] for lp in loops), "reported": "median loop"},
-        "gpu_launches": 2 * K * len(loops),
+        "gpu_launches": launches * K * len(loops),
         "clocks": clocks,
     }
     print(json.dumps(line))
@@ -793,6 +804,7 @@ def run_ours_fused(args, w: di.Workload):
     sampler.stop_flag = True
     sampler.join(timeout=1.0)
     clocks = sampler.summary(t_host0, t_host1)
+    launches = _launches_per_step(lambda: step(sets[0]))
     n_gpu = out["accept_len"].cpu().numpy()
     tok_gpu = out["token"].cpu().numpy()
     n_bonus = int((n_gpu == gamma).sum())
@@ -870,7 +882,7 @@ def run_ours_fused(args, w: di.Workload):
         "metric": METRIC, "value": world * rows / (ms_per_step * 1e-3), "unit": UNIT, "n_gpus": world, "steps": K,
         "warmup": max(args.warmup, 3), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic", "config": cfg,
-        "roofline": {"bound": "hbm", "kernel": "edge_verify_kernel + resample_kernel (one call)", "achieved": achieved,
+        "roofline": {"bound": "hbm", "kernel": "edge kernels and draw (one call)", "achieved": achieved,
                      "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
                      "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS, "algorithmic_bytes_per_launch": call_bytes,
                      "avg_launch_ms": avg_ms, "min_launch_ms": min(call_ms), "traffic": None},
@@ -878,7 +890,7 @@ def run_ours_fused(args, w: di.Workload):
         "e2e": {"value": world * rows / (e2e_ms / e2e_steps * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": 2 * Bn * 4, "steps": e2e_steps, "ms_per_step": e2e_ms / e2e_steps},
         "timed": {"loops": len(loops), "device_ms": sum(lp["total_ms"] for lp in loops), "reported": "median loop"},
-        "gpu_launches": 2 * K * len(loops), "clocks": clocks,
+        "gpu_launches": launches * K * len(loops), "clocks": clocks,
     }))
     if world > 1:
         dist.destroy_process_group()
@@ -986,6 +998,7 @@ def run_ours_sharded(args, w: di.Workload):
     sampler.stop_flag = True
     sampler.join(timeout=1.0)
     clocks = sampler.summary(t_host0, t_host1)
+    launches = _launches_per_step(lambda: list(calls()))
     ms_per_step = loop["total_ms"] / K
     per_call = dict(zip(names, loop["per_call_ms"]))
     # the same steps (flush included) replayed from a CUDA graph: the four small calls are launch- and
@@ -1052,7 +1065,7 @@ def run_ours_sharded(args, w: di.Workload):
         "metric": METRIC, "value": w.rows / (ms_per_step * 1e-3), "unit": UNIT, "n_gpus": 1, "steps": K,
         "warmup": max(args.warmup, 3), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "strong",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic", "config": cfg,
-        "roofline": {"bound": "hbm", "kernel": "edge_verify_kernel (partial sums of one shard)", "achieved": achieved,
+        "roofline": {"bound": "hbm", "kernel": "partial sums of one shard", "achieved": achieved,
                      "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
                      "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS, "algorithmic_bytes_per_launch": part_bytes,
                      "avg_launch_ms": per_call["partial"], "traffic": None},
@@ -1060,7 +1073,7 @@ def run_ours_sharded(args, w: di.Workload):
         "step_gbs": step_bytes / (ms_per_step * 1e-3) / 1e9,
         "timed": {"loops": len(loops), "device_ms": sum(lp["total_ms"] for lp in loops), "reported": "median loop"},
         "graph": graph_rec,
-        "cpu_baseline": cpu, "parity": parity, "e2e": None, "gpu_launches": 7 * K * len(loops), "clocks": clocks,
+        "cpu_baseline": cpu, "parity": parity, "e2e": None, "gpu_launches": launches * K * len(loops), "clocks": clocks,
     }))
 
 

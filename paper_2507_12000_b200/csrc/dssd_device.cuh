@@ -25,14 +25,6 @@ __device__ __forceinline__ uint4 ld_stream16(const void *p)
     return v;
 }
 
-// the same, 8 bytes
-__device__ __forceinline__ uint2 ld_stream8(const void *p)
-{
-    uint2 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-    return v;
-}
-
 // two floats rounded to IEEE binary16 (nearest even), low half = first
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
 {
@@ -41,52 +33,6 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
 }
 
 __device__ __forceinline__ unsigned short to_half_bits(float x) { return __half_as_ushort(__float2half_rn(x)); }
-
-// 8-byte streaming store (evict-first)
-__device__ __forceinline__ void st_stream8(void *p, uint32_t a, uint32_t b)
-{
-    asm volatile("st.global.cs.v2.b32 [%0], {%1,%2};" ::"l"(p), "r"(a), "r"(b) : "memory");
-}
-
-// 16-byte streaming store (evict-first): output that this kernel never reads back.
-__device__ __forceinline__ void st_stream16(void *p, float a, float b, float c, float d)
-{
-    asm volatile("st.global.cs.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
-                 : "memory");
-}
-
-// 8-byte relaxed, GPU-scope accesses: single-copy atomic, always served by L2.  Used for slots
-// that carry their own validity (a pre-filled pattern), so no fence is needed around them.
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_relaxed_u64(void *p, unsigned long long v)
-{
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_release(unsigned *p, unsigned v)
-{
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 
 // ---- programmatic dependent launch (see launch.h) -----------------------------------------------
 
@@ -142,100 +88,6 @@ __device__ __forceinline__ unsigned long long ld_after(const unsigned long long 
 __device__ __forceinline__ double ld_after(const double *p)
 {
     return __longlong_as_double((long long)ld_after(reinterpret_cast<const unsigned long long *>(p)));
-}
-
-// ---- shared-memory barriers and bulk asynchronous copies (TMA, untiled form) ------------------
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-// makes freshly initialised barriers visible to the asynchronous copy engine
-__device__ __forceinline__ void mbar_init_fence()
-{
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-// Bounded wait for the phase with the given parity; false when the limit ran out.  Each try
-// suspends the thread until the phase completes or about `kMbarSuspendNs` have passed, so a
-// waiting warp takes almost no issue slots from the working ones.
-constexpr unsigned kMbarSuspendNs = 4000;
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned limit)
-{
-    for (unsigned it = 0; it < limit; ++it) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity), "r"(kMbarSuspendNs)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-// Orders this thread's earlier generic-proxy accesses to shared memory before later accesses
-// of the asynchronous proxy (a bulk copy that overwrites a buffer the warp has just read).
-__device__ __forceinline__ void fence_proxy_async()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ uint64_t l2_policy_evict_first()
-{
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-// global -> shared bulk copy; src, dst 16-byte aligned, bytes a multiple of 16; completion is
-// signalled on the barrier as `bytes` transaction bytes
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar,
-                                              uint64_t policy)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-        ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy)
-        : "memory");
-}
-
-__device__ __forceinline__ uint4 lds16(uint32_t addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
-
-__device__ __forceinline__ uint2 lds8(uint32_t addr)
-{
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-    return v;
 }
 
 // ---- arithmetic --------------------------------------------------------------------------
@@ -301,41 +153,21 @@ struct Elem;
 template <>
 struct Elem<DSSD_F32> {
     static constexpr int kBytes = 4;
-    static constexpr int kVec = 4;   // elements per 16-byte vector
     __device__ static __forceinline__ float load(const void *row, int64_t i)
     {
         float f;
         asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(f) : "l"(reinterpret_cast<const float *>(row) + i));
         return f;
     }
-    __device__ static __forceinline__ void unpack(const uint4 &v, float *f)
-    {
-        f[0] = __uint_as_float(v.x);
-        f[1] = __uint_as_float(v.y);
-        f[2] = __uint_as_float(v.z);
-        f[3] = __uint_as_float(v.w);
-    }
 };
 template <>
 struct Elem<DSSD_BF16> {
     static constexpr int kBytes = 2;
-    static constexpr int kVec = 8;
     __device__ static __forceinline__ float load(const void *row, int64_t i)
     {
         unsigned short h;
         asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(h) : "l"(reinterpret_cast<const unsigned short *>(row) + i));
         return __uint_as_float((uint32_t)h << 16);
-    }
-    __device__ static __forceinline__ void unpack(const uint4 &v, float *f)
-    {
-        f[0] = bf16_lo(v.x);
-        f[1] = bf16_hi(v.x);
-        f[2] = bf16_lo(v.y);
-        f[3] = bf16_hi(v.y);
-        f[4] = bf16_lo(v.z);
-        f[5] = bf16_hi(v.z);
-        f[6] = bf16_lo(v.w);
-        f[7] = bf16_hi(v.w);
     }
 };
 
