@@ -1,4 +1,5 @@
-// Device half of the verification round: residual (or bonus) inverse-CDF draw, as two kernels.
+// Device half of the verification round: residual (or bonus) inverse-CDF draw, as two kernels, or as one where
+// the batch is small (resample_cluster_kernel: a cluster of CTAs per sequence holds the row in registers).
 //
 //   resample_mass_kernel  one CTA per (sequence, one to four tiles of kTile entries): streams its part of
 //                         p_row[b] and of Q_n[b], forms r = max(0, p - q) (or r = p for the bonus draw)
@@ -7,8 +8,8 @@
 //                         and the chunk that holds u' * Z; every thread fetches its run of that chunk, a
 //                         second prefix finds the thread and its run gives the token.
 //
-// Plain stores and the order of the two launches (launch.h) connect them: no ticket, no wait, nothing
-// in the scratch that has to be cleared.
+// Plain stores and the order of the launches (launch.h) connect them; nothing in the scratch has to be
+// cleared.
 // All sums are float64, so the token differs from an index-order float64 scan only when u' * Z
 // lies within rounding (about 1e-13 relative) of a CDF step.
 #include "device_resample.h"
