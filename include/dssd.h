@@ -38,6 +38,8 @@
  *     (it enqueues kernels and nothing else); dssd_device_resample_static provided one call of it was
  *     made on that device before the capture began.
  *     dssd_round_host waits for the accepted lengths and cannot be captured.
+ *   - The *_bytes functions never decrease when a size grows: a workspace or an arena made for the largest sizes
+ *     of a program serves all smaller ones.
  *   - Buffers need only their natural alignment; 16-byte aligned rows take the fast path.
  *   - A status other than DSSD_OK means nothing was enqueued (except DSSD_ERR_CUDA, after
  *     which the outputs are undefined).  Data-dependent anomalies never fault or trap: they

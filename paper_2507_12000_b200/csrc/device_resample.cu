@@ -524,7 +524,11 @@ size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base)
         P->n_sub = (int)n_sub;
         P->rows_per_sum = rows;
     }
-    return ((size_t)B * n_sub * sizeof(double) + 255) & ~(size_t)255;
+    // The size is enough for every smaller batch and vocabulary too, also where those keep more sums per row: they do
+    // so up to that scratch's size only.
+    const size_t need = (size_t)B * n_sub * sizeof(double), finest = (size_t)B * (((size_t)V + kSub - 1) / kSub) * sizeof(double);
+    const size_t smaller = finest < (size_t)DSSD_STATIC_SCRATCH_BYTES ? finest : (size_t)DSSD_STATIC_SCRATCH_BYTES;
+    return ((need > smaller ? need : smaller) + 255) & ~(size_t)255;
 }
 
 namespace {

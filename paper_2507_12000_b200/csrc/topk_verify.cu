@@ -648,13 +648,20 @@ static void topk_geometry(int B, int gamma, int V, int esz, int &runs, int &run_
     run_vecs = (int)(per * kSelTile);
 }
 
+// Enough for every launch of no more sequences, positions, vocabulary entries and k than these, of either type: a
+// workspace made for the largest batch serves the smaller ones.  A launch of t tiles keeps t lists below kSelTwoTiles,
+// rows * ceil(n / 2) <= t of them below kSelFourTiles (n tiles per row) and rows * ceil(n / 4) beyond; each bound grows with
+// rows and n, and so does the largest of the three.
 size_t topk_workspace_bytes(int B, int gamma, int V, int k)
 {
-    int r2, r4, vecs;
-    topk_geometry(B, gamma, V, 2, r2, vecs);
-    topk_geometry(B, gamma, V, 4, r4, vecs);
-    const size_t runs = (size_t)(r2 > r4 ? r2 : r4);
-    return ((size_t)B * (size_t)(gamma + 1) * runs * (size_t)k * 8 + 255) & ~(size_t)255;
+    const unsigned long long rows = (unsigned long long)B * (unsigned long long)(gamma + 1);
+    unsigned long long n = ((unsigned long long)V * 4 / 16 + kSelTile - 1) / kSelTile;
+    if (n < 1) n = 1;
+    auto least = [](unsigned long long a, unsigned long long b) { return a < b ? a : b; };
+    unsigned long long lists = least(rows * n, kSelTwoTiles), two = least(rows * ((n + 1) / 2), kSelFourTiles);
+    if (two > lists) lists = two;
+    if (rows * n >= kSelFourTiles && rows * ((n + 3) / 4) > lists) lists = rows * ((n + 3) / 4);
+    return ((size_t)lists * (size_t)k * 8 + 255) & ~(size_t)255;
 }
 
 cudaError_t topk_verify_launch(TopkParams &P, int dtype, void *workspace, cudaStream_t stream)

@@ -67,6 +67,33 @@ def test_workspace_sizes(B):
     assert B.dssd_round_host_arena_bytes(8, 4, 32000, 7) == 0
 
 
+def test_sizes_never_decrease(B):
+    """A workspace made for a program's largest sizes serves its smaller ones: no size function decreases when a
+    size grows, in particular where a launch starts to keep fewer sums or lists per row."""
+    L = B.lib
+    ints = ctypes.c_int
+    L.dssd_edge_partial_workspace_bytes.restype = ctypes.c_size_t
+    L.dssd_edge_partial_workspace_bytes.argtypes = [ints, ints, ints]
+    plain = [L.dssd_edge_verify_workspace_bytes, L.dssd_device_resample_workspace_bytes, L.dssd_dsd_verify_workspace_bytes,
+             L.dssd_edge_verify_bonus_workspace_bytes, L.dssd_edge_partial_workspace_bytes,
+             L.dssd_resample_shard_workspace_bytes]
+    sizes = [(lambda b, g, v, k, f=f: f(b, g, v)) for f in plain]
+    sizes += [lambda b, g, v, k, t=t: L.dssd_round_host_arena_bytes(b, g, v, t) for t in (B.DSSD_F32, B.DSSD_BF16)]
+    sizes += [lambda b, g, v, k: L.dssd_edge_verify_topk_workspace_bytes(b, g, v, k)]
+    sizes += [lambda b, g, v, k, t=t: L.dssd_round_host_topk_arena_bytes(b, g, v, k, t) for t in (B.DSSD_F32, B.DSSD_BF16)]
+    walks = [[(b, 4, v, 10) for b in range(1, 1300)] for v in (32000, 128256, 151936)]
+    walks += [[(b, g, v, 10) for g in range(0, 70)] for b, v in ((64, 50272), (17, 151936), (300, 30011))]
+    walks += [[(b, 4, v, 10) for v in range(32, 400000, 511)] for b in (1, 30, 300, 1000)]
+    walks += [[(1, 2, 1 << e, 10) for e in range(5, 31)]]
+    walks += [[(64, 4, 50272, k) for k in range(1, 33)]]
+    for size in sizes:
+        for walk in walks:
+            got = [size(*c) for c in walk]
+            assert all(x > 0 for x in got)
+            down = [(walk[i], got[i], walk[i + 1], got[i + 1]) for i in range(len(got) - 1) if got[i + 1] < got[i]]
+            assert not down, down[:3]
+
+
 def test_bad_arguments_are_rejected_before_any_launch(B):
     L = B.lib
     buf = (ctypes.c_char * 4096)()
