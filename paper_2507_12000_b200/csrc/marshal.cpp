@@ -189,6 +189,18 @@ QShard q_shard(PyObject *o, int64_t B, int64_t gamma, int64_t Vs)
     return {q.numel() ? static_cast<const float *>(q.data_ptr()) : nullptr, row_stride(q, "rows of draft_q_shard must be equally spaced")};
 }
 
+// The library's call without the interpreter lock, once every argument has been read: a round on host buffers waits for
+// the GPU and copies from pageable memory, and any launch waits while the stream's queue is full.  Other threads run
+// meanwhile, a host callback on the stream among them.
+template <class... P, class... A>
+dssd_status call(dssd_status (*fn)(P...), A... args)
+{
+    PyThreadState *const state = PyEval_SaveThread();
+    const dssd_status st = fn(args...);
+    PyEval_RestoreThread(state);
+    return st;
+}
+
 // ---- one function per entry point: (arguments ...) -> status -----------------------------------
 
 // target_logits, draft_tokens, draft_q_tok, uniforms, temperature, out, workspace, stream, half
@@ -207,9 +219,9 @@ dssd_status edge_verify(PyObject *const *a)
     uint32_t *fl = maybe<uint32_t>(a[5], "flags");
     void *s = stream(a[7]);
     if (half)
-        return lib.dssd_edge_verify_p16(r.data, r.dtype, r.stride, tok, q, u, T, r.B, r.gamma, r.V, n,
+        return call(lib.dssd_edge_verify_p16, r.data, r.dtype, r.stride, tok, q, u, T, r.B, r.gamma, r.V, n,
                                         static_cast<uint16_t *>(p.data_ptr()), pt, lse, fl, ws.data, ws.bytes, s);
-    return lib.dssd_edge_verify(r.data, r.dtype, r.stride, tok, q, u, T, r.B, r.gamma, r.V, n,
+    return call(lib.dssd_edge_verify, r.data, r.dtype, r.stride, tok, q, u, T, r.B, r.gamma, r.V, n,
                                 static_cast<float *>(p.data_ptr()), pt, lse, fl, ws.data, ws.bytes, s);
 }
 
@@ -235,9 +247,9 @@ dssd_status device_resample(PyObject *const *a)
     uint32_t *fl = maybe<uint32_t>(a[5], "flags");
     void *s = stream(a[7]);
     if (p.scalar_type() == at::kHalf)
-        return lib.dssd_device_resample_p16(static_cast<const uint16_t *>(p.data_ptr()), q, n, u, B, gamma, V, tok, fl, ws.data,
+        return call(lib.dssd_device_resample_p16, static_cast<const uint16_t *>(p.data_ptr()), q, n, u, B, gamma, V, tok, fl, ws.data,
                                             ws.bytes, s);
-    return lib.dssd_device_resample(static_cast<const float *>(p.data_ptr()), q, n, u, B, gamma, V, tok, fl, ws.data, ws.bytes, s);
+    return call(lib.dssd_device_resample, static_cast<const float *>(p.data_ptr()), q, n, u, B, gamma, V, tok, fl, ws.data, ws.bytes, s);
 }
 
 // the same for the rejected sequences only
@@ -247,7 +259,7 @@ dssd_status device_resample_rejected(PyObject *const *a)
     const int B = (int)p.size(0), V = (int)p.size(1), gamma = size_arg(a[4]);
     const float *q = draft_rows(a[1], B, gamma, V);
     const Space ws = space(a[6]);
-    return lib.dssd_device_resample_rejected(static_cast<const float *>(p.data_ptr()), q,
+    return call(lib.dssd_device_resample_rejected, static_cast<const float *>(p.data_ptr()), q,
                                              static_cast<const int32_t *>(tensor(a[2]).data_ptr()),
                                              static_cast<const float *>(tensor(a[3]).data_ptr()), B, gamma, V,
                                              need<int32_t>(a[5], "token"), maybe<uint32_t>(a[5], "flags"), ws.data, ws.bytes,
@@ -259,7 +271,7 @@ dssd_status device_resample_static(PyObject *const *a)
 {
     const at::Tensor &p = payload(a[0], false);
     const int B = (int)p.size(0), V = (int)p.size(1), gamma = size_arg(a[4]);
-    return lib.dssd_device_resample_static(static_cast<const float *>(p.data_ptr()), gamma > 0 ? ptr_as<const float>(a[1]) : nullptr,
+    return call(lib.dssd_device_resample_static, static_cast<const float *>(p.data_ptr()), gamma > 0 ? ptr_as<const float>(a[1]) : nullptr,
                                            static_cast<const int32_t *>(tensor(a[2]).data_ptr()),
                                            static_cast<const float *>(tensor(a[3]).data_ptr()), B, gamma, V,
                                            need<int32_t>(a[5], "token"), maybe<uint32_t>(a[5], "flags"), stream(a[6]));
@@ -270,7 +282,7 @@ dssd_status edge_verify_topk(PyObject *const *a)
 {
     const Rows r = rows(a[0]);
     const Space ws = space(a[7]);
-    return lib.dssd_edge_verify_topk(r.data, r.dtype, r.stride, ptr_as<const int32_t>(a[1]), ptr_as<const float>(a[2]),
+    return call(lib.dssd_edge_verify_topk, r.data, r.dtype, r.stride, ptr_as<const int32_t>(a[1]), ptr_as<const float>(a[2]),
                                      ptr_as<const float>(a[3]), (float)number(a[4]), r.B, r.gamma, r.V, size_arg(a[5]),
                                      need<int32_t>(a[6], "accept_len"), need<int32_t>(a[6], "p_idx"), need<float>(a[6], "p_val"),
                                      maybe<float>(a[6], "p_tok"), maybe<uint32_t>(a[6], "flags"), ws.data, ws.bytes, stream(a[8]));
@@ -295,7 +307,7 @@ dssd_status device_resample_topk(PyObject *const *a)
         qi = ptr_as<const int32_t>(a[2]);
         qv = ptr_as<const float>(a[3]);
     }
-    return lib.dssd_device_resample_topk(static_cast<const int32_t *>(pi.data_ptr()), static_cast<const float *>(pv.data_ptr()), qi, qv,
+    return call(lib.dssd_device_resample_topk, static_cast<const int32_t *>(pi.data_ptr()), static_cast<const float *>(pv.data_ptr()), qi, qv,
                                          static_cast<const int32_t *>(tensor(a[4]).data_ptr()),
                                          static_cast<const float *>(tensor(a[5]).data_ptr()), B, gamma, k,
                                          need<int32_t>(a[7], "token"), maybe<uint32_t>(a[7], "flags"), stream(a[8]));
@@ -307,7 +319,7 @@ dssd_status dsd_verify(PyObject *const *a)
     const Rows r = rows(a[0]);
     const float *q = draft_rows(a[1], r.B, r.gamma, r.V);
     const Space ws = space(a[7]);
-    return lib.dssd_dsd_verify(r.data, r.dtype, r.stride, q, ptr_as<const int32_t>(a[2]), ptr_as<const float>(a[3]),
+    return call(lib.dssd_dsd_verify, r.data, r.dtype, r.stride, q, ptr_as<const int32_t>(a[2]), ptr_as<const float>(a[3]),
                                static_cast<const float *>(tensor(a[4]).data_ptr()), (float)number(a[5]), r.B, r.gamma, r.V,
                                need<int32_t>(a[6], "accept_len"), need<int32_t>(a[6], "token"),
                                maybe<uint32_t>(a[6], "edge_flags"), maybe<uint32_t>(a[6], "rs_flags"), ws.data, ws.bytes,
@@ -319,7 +331,7 @@ dssd_status edge_verify_bonus(PyObject *const *a)
 {
     const Rows r = rows(a[0]);
     const Space ws = space(a[7]);
-    return lib.dssd_edge_verify_bonus(r.data, r.dtype, r.stride, ptr_as<const int32_t>(a[1]), ptr_as<const float>(a[2]),
+    return call(lib.dssd_edge_verify_bonus, r.data, r.dtype, r.stride, ptr_as<const int32_t>(a[1]), ptr_as<const float>(a[2]),
                                       ptr_as<const float>(a[3]), static_cast<const float *>(tensor(a[4]).data_ptr()),
                                       (float)number(a[5]), r.B, r.gamma, r.V, need<int32_t>(a[6], "accept_len"),
                                       need<float>(a[6], "p_row"), need<int32_t>(a[6], "token"), maybe<float>(a[6], "p_tok"),
@@ -332,7 +344,7 @@ dssd_status round_host(PyObject *const *a)
 {
     const Rows r = rows(item(a[0], "target_logits"), false);
     const Space ar = space(a[2]);
-    return lib.dssd_round_host(r.data, r.dtype, maybe<const int32_t>(a[0], "draft_tokens"), maybe<const float>(a[0], "draft_q_tok"),
+    return call(lib.dssd_round_host, r.data, r.dtype, maybe<const int32_t>(a[0], "draft_tokens"), maybe<const float>(a[0], "draft_q_tok"),
                                maybe<const float>(a[0], "uniforms"), maybe<const float>(a[0], "draft_q"),
                                need<const float>(a[0], "uniforms_rs"), (float)number(a[1]), r.B, r.gamma, r.V,
                                need<int32_t>(a[3], "accept_len"), need<int32_t>(a[3], "token"),
@@ -345,7 +357,7 @@ dssd_status round_host_topk(PyObject *const *a)
 {
     const Rows r = rows(item(a[0], "target_logits"), false);
     const Space ar = space(a[3]);
-    return lib.dssd_round_host_topk(r.data, r.dtype, maybe<const int32_t>(a[0], "draft_tokens"),
+    return call(lib.dssd_round_host_topk, r.data, r.dtype, maybe<const int32_t>(a[0], "draft_tokens"),
                                     maybe<const float>(a[0], "draft_q_tok"), maybe<const float>(a[0], "uniforms"),
                                     maybe<const int32_t>(a[0], "q_idx"), maybe<const float>(a[0], "q_val"),
                                     need<const float>(a[0], "uniforms_rs"), (float)number(a[1]), r.B, r.gamma, r.V, size_arg(a[2]),
@@ -359,7 +371,7 @@ dssd_status edge_partial(PyObject *const *a)
 {
     const Rows r = rows(a[0]);
     const Space ws = space(a[5]);
-    return lib.dssd_edge_partial(r.data, r.dtype, r.stride, ptr_as<const int32_t>(a[1]), size_arg(a[2]), (float)number(a[3]), r.B,
+    return call(lib.dssd_edge_partial, r.data, r.dtype, r.stride, ptr_as<const int32_t>(a[1]), size_arg(a[2]), (float)number(a[3]), r.B,
                                  r.gamma, r.V, need<float>(a[4], "part_ref"), need<double>(a[4], "part_sum"),
                                  ptr_as<float>(item(a[4], "tok_logit")), ws.data, ws.bytes, stream(a[6]));
 }
@@ -375,7 +387,7 @@ dssd_status edge_combine(PyObject *const *a)
     const int G = (int)pr.size(0), B = (int)pr.size(1), gamma = (int)pr.size(2) - 1;
     require(tl.is_contiguous() && tl.scalar_type() == at::kFloat && tl.numel() == (int64_t)G * B * gamma,
             "tok_logit must be a contiguous float32 [G, B, gamma] tensor");
-    return lib.dssd_edge_combine(static_cast<const float *>(pr.data_ptr()), static_cast<const double *>(ps.data_ptr()),
+    return call(lib.dssd_edge_combine, static_cast<const float *>(pr.data_ptr()), static_cast<const double *>(ps.data_ptr()),
                                  ptr_as<const float>(a[2]), G, ptr_as<const int32_t>(a[3]), ptr_as<const float>(a[4]),
                                  ptr_as<const float>(a[5]), (float)number(a[6]), B, gamma, size_arg(a[7]),
                                  need<int32_t>(a[8], "accept_len"), need<float>(a[8], "row_scale"), maybe<float>(a[8], "p_tok"),
@@ -388,7 +400,7 @@ dssd_status edge_emit_shard(PyObject *const *a)
     const Rows r = rows(a[0]);
     const at::Tensor &o = tensor(a[4]);
     require(o.dim() == 2 && o.size(0) == r.B && o.size(1) == r.V, "out must be a [B, V_shard] tensor");
-    return lib.dssd_edge_emit_shard(r.data, r.dtype, r.stride, static_cast<const int32_t *>(tensor(a[1]).data_ptr()),
+    return call(lib.dssd_edge_emit_shard, r.data, r.dtype, r.stride, static_cast<const int32_t *>(tensor(a[1]).data_ptr()),
                                     static_cast<const float *>(tensor(a[2]).data_ptr()), (float)number(a[3]), r.B, r.gamma, r.V,
                                     static_cast<float *>(o.data_ptr()), rows_2d(o), stream(a[5]));
 }
@@ -401,7 +413,7 @@ dssd_status resample_shard_mass(PyObject *const *a)
     const int B = (int)p.size(0), Vs = (int)p.size(1), gamma = size_arg(a[3]);
     const QShard q = q_shard(a[1], B, gamma, Vs);
     const Space ws = space(a[5]);
-    return lib.dssd_resample_shard_mass(static_cast<const float *>(p.data_ptr()), ps, q.data, q.stride,
+    return call(lib.dssd_resample_shard_mass, static_cast<const float *>(p.data_ptr()), ps, q.data, q.stride,
                                         static_cast<const int32_t *>(tensor(a[2]).data_ptr()), B, gamma, Vs,
                                         static_cast<double *>(tensor(a[4]).data_ptr()), ws.data, ws.bytes, stream(a[6]));
 }
@@ -416,7 +428,7 @@ dssd_status resample_shard_draw(PyObject *const *a)
     const int B = (int)p.size(0), Vs = (int)p.size(1), gamma = size_arg(a[7]);
     const QShard q = q_shard(a[4], B, gamma, Vs);
     const Space ws = space(a[8]);
-    return lib.dssd_resample_shard_draw(static_cast<const double *>(m.data_ptr()), (int)m.size(0), size_arg(a[1]), size_arg(a[2]),
+    return call(lib.dssd_resample_shard_draw, static_cast<const double *>(m.data_ptr()), (int)m.size(0), size_arg(a[1]), size_arg(a[2]),
                                         static_cast<const float *>(p.data_ptr()), ps, q.data, q.stride,
                                         static_cast<const int32_t *>(tensor(a[5]).data_ptr()),
                                         static_cast<const float *>(tensor(a[6]).data_ptr()), B, gamma, Vs,

@@ -1,4 +1,10 @@
-"""The marshalling module's own checks: what it refuses before the library is called (no GPU needed)."""
+"""The marshalling module's own checks: what it refuses before the library is called, and how it calls (no GPU needed)."""
+import ctypes
+import re
+import subprocess
+import threading
+import time
+
 import pytest
 import torch
 
@@ -38,3 +44,45 @@ def test_statuses_come_through(B):
     with pytest.raises(B.DssdError) as e:  # temperature 0 is refused by the library itself
         B.dssd_round_host(host, 0.0, torch.zeros(256, dtype=torch.uint8), out=_out(), stream=0)
     assert e.value.status == B.DSSD_ERR_INVALID_ARG
+
+
+@pytest.fixture()
+def slow_library(B, tmp_path):
+    """In the library's place one whose every entry point takes 0.2 s and succeeds."""
+    calls = re.findall(r"X\((dssd_\w+)\)", open(B._PKG + "/csrc/marshal.cpp").read())
+    src = tmp_path / "slow.c"
+    src.write_text("#include <unistd.h>\n" + "".join(f"int {n}(void) {{ usleep(200000); return 0; }}\n" for n in calls))
+    so = tmp_path / "libslow.so"
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
+    slow = ctypes.CDLL(str(so))
+    B._marshal.bind(slow._handle)
+    yield slow
+    B._marshal.bind(B.lib._handle)
+
+
+@pytest.mark.parametrize("topk", [False, True])
+def test_other_threads_run_during_a_call(B, slow_library, topk):
+    host = {"target_logits": torch.zeros(1, 1, 8), "uniforms_rs": torch.zeros(1)}
+    arena, out = torch.zeros(256, dtype=torch.uint8), _out()
+    started, stop, during = threading.Event(), threading.Event(), []
+
+    def count():
+        started.set()
+        while not stop.is_set():
+            during.append(time.monotonic())
+            time.sleep(0.002)
+
+    t = threading.Thread(target=count)
+    t.start()
+    started.wait()
+    begin = time.monotonic()
+    if topk:
+        B.dssd_round_host_topk(host, 1.0, 4, arena, out=out, stream=0)
+    else:
+        B.dssd_round_host(host, 1.0, arena, out=out, stream=0)
+    end = time.monotonic()
+    stop.set()
+    t.join()
+    # a thread that waits for the lock may run once on either side of the call, and no more
+    assert end - begin > 0.19
+    assert sum(begin + 0.02 < x < end - 0.02 for x in during) > 5
