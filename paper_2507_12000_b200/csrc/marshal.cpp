@@ -9,6 +9,8 @@
 
 #include <dlfcn.h>
 
+#include <vector>
+
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -61,10 +63,19 @@ T *ptr_as(PyObject *o)
     return static_cast<T *>(ptr(o));
 }
 
-// out["name"]; a missing key is an error for a required output and NULL for an optional one
+// References that a mapping other than a dict gave out, kept until the call that asked for them returns.
+thread_local std::vector<PyObject *> kept;
+PyObject *keep(PyObject *v)
+{
+    if (v == nullptr) throw Raised();
+    kept.push_back(v);
+    return v;
+}
+
+// out["name"]; a missing key is an error
 PyObject *item(PyObject *out, const char *name)
 {
-    if (!PyDict_Check(out)) raise(PyExc_TypeError, "out must be a dict");
+    if (!PyDict_CheckExact(out)) return keep(PyMapping_GetItemString(out, name));
     PyObject *v = PyDict_GetItemString(out, name);
     if (v == nullptr) {
         PyErr_SetString(PyExc_KeyError, name);
@@ -77,11 +88,11 @@ T *need(PyObject *out, const char *name)
 {
     return static_cast<T *>(tensor(item(out, name)).data_ptr());
 }
+// out.get("name"): NULL where there is none
 template <class T>
 T *maybe(PyObject *out, const char *name)
 {
-    if (!PyDict_Check(out)) raise(PyExc_TypeError, "out must be a dict");
-    return ptr_as<T>(PyDict_GetItemString(out, name));
+    return ptr_as<T>(PyDict_CheckExact(out) ? PyDict_GetItemString(out, name) : keep(PyObject_CallMethod(out, "get", "s", name)));
 }
 
 double number(PyObject *o)
@@ -98,12 +109,12 @@ long integer(PyObject *o)
 }
 int size_arg(PyObject *o) { return (int)integer(o); }
 
-// None: torch's current stream; else a torch stream or a cudaStream_t as an integer
+// None: torch's current stream; else a torch stream, or a cudaStream_t as an integer or an object that converts to one
 void *stream(PyObject *o)
 {
     if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
     if (PyLong_Check(o)) return PyLong_AsVoidPtr(o);
-    PyObject *h = PyObject_GetAttrString(o, "cuda_stream");
+    PyObject *h = PyObject_HasAttrString(o, "cuda_stream") ? PyObject_GetAttrString(o, "cuda_stream") : PyNumber_Long(o);
     if (h == nullptr) throw Raised();
     void *s = PyLong_AsVoidPtr(h);
     Py_DECREF(h);
@@ -445,14 +456,23 @@ PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n)
         PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", kArgs, n);
         return nullptr;
     }
+    const size_t before = kept.size();
+    PyObject *result = nullptr;
     try {
-        return PyLong_FromLong(fn(args));
+        result = PyLong_FromLong(fn(args));
     } catch (const Raised &) {
-        return nullptr;
     } catch (const std::exception &e) {
         PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
     }
+    while (kept.size() > before) {  // (after an error too: the references' owners may run Python code of their own)
+        PyObject *type, *value, *trace;
+        PyErr_Fetch(&type, &value, &trace);
+        PyObject *v = kept.back();
+        kept.pop_back();
+        Py_DECREF(v);
+        PyErr_Restore(type, value, trace);
+    }
+    return result;
 }
 
 // the handle that dlopen gave for libdssd.so

@@ -1,4 +1,5 @@
 """The marshalling module's own checks: what it refuses before the library is called, and how it calls (no GPU needed)."""
+import collections
 import ctypes
 import re
 import subprocess
@@ -48,10 +49,14 @@ def test_statuses_come_through(B):
 
 @pytest.fixture()
 def slow_library(B, tmp_path):
-    """In the library's place one whose every entry point takes 0.2 s and succeeds."""
+    """In the library's place one whose every entry point takes 0.2 s, notes its last argument and succeeds."""
     calls = re.findall(r"X\((dssd_\w+)\)", open(B._PKG + "/csrc/marshal.cpp").read())
     src = tmp_path / "slow.c"
-    src.write_text("#include <unistd.h>\n" + "".join(f"int {n}(void) {{ usleep(200000); return 0; }}\n" for n in calls))
+    host = ("const void *target_logits, int dtype, const void *a, const void *b, const void *c, const void *d, const void *e, float T, "
+            "int B, int gamma, int V, void *f, void *g, void *h, void *i, void *j, void *arena, unsigned long bytes, void *stream")
+    src.write_text("#include <unistd.h>\nvoid *last_stream;\n" + "".join(
+        f"int {n}({host}) {{ last_stream = stream; usleep(200000); return 0; }}\n" if n == "dssd_round_host" else
+        f"int {n}(void) {{ usleep(200000); return 0; }}\n" for n in calls))
     so = tmp_path / "libslow.so"
     subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
     slow = ctypes.CDLL(str(so))
@@ -86,3 +91,34 @@ def test_other_threads_run_during_a_call(B, slow_library, topk):
     # a thread that waits for the lock may run once on either side of the call, and no more
     assert end - begin > 0.19
     assert sum(begin + 0.02 < x < end - 0.02 for x in during) > 5
+
+
+class _Handle:
+    """A stream as other packages wrap it: converts to the integer."""
+
+    def __int__(self):
+        return 0x1234
+
+
+@pytest.mark.parametrize("stream,value", [(0x1234, 0x1234), (_Handle(), 0x1234), (0, None)])
+def test_streams(B, slow_library, stream, value):
+    host = {"target_logits": torch.zeros(1, 1, 8), "uniforms_rs": torch.zeros(1)}
+    B.dssd_round_host(host, 1.0, torch.zeros(256, dtype=torch.uint8), out=_out(), stream=stream)
+    assert ctypes.c_void_p.in_dll(slow_library, "last_stream").value == value
+    with pytest.raises((TypeError, AttributeError)):
+        B.dssd_round_host(host, 1.0, torch.zeros(256, dtype=torch.uint8), out=_out(), stream=object())
+
+
+def test_mappings_other_than_dict(B, slow_library):
+    """Anything with [] and get: tensors that only the mapping's answer holds live until the call returns."""
+    class Made(collections.UserDict):
+        def __getitem__(self, name):
+            return super().__getitem__(name).clone()
+
+    host = Made(target_logits=torch.zeros(1, 1, 8), uniforms_rs=torch.zeros(1))
+    out = collections.UserDict(_out())
+    assert B.dssd_round_host(host, 1.0, torch.zeros(256, dtype=torch.uint8), out=out, stream=0) is out
+    with pytest.raises(KeyError):
+        B.dssd_round_host(host, 1.0, torch.zeros(256, dtype=torch.uint8), out=collections.UserDict(), stream=0)
+    with pytest.raises((TypeError, AttributeError)):
+        B.dssd_round_host(host, 1.0, torch.zeros(256, dtype=torch.uint8), out=[1], stream=0)
