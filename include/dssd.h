@@ -218,7 +218,7 @@ size_t dssd_round_host_arena_bytes(int B, int gamma, int V, dssd_dtype dtype);
  * Of the draft distributions only the rows the device half reads cross the bus, B * V * 4 bytes at
  * most instead of B * gamma * V * 4: row Q_n of every sequence with a rejection.  Pinned host
  * buffers are mapped, and the kernels read those rows (and the short arrays) and write the results
- * over the bus themselves; pageable ones are copied.  The call waits on the host for the accepted
+ * over the bus themselves; a buffer of which any part is pageable is copied.  The call waits on the host for the accepted
  * lengths (accept_len is final when the call returns) and therefore cannot be made while the stream
  * is being captured (DSSD_ERR_CUDA then).
  *

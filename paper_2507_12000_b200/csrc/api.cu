@@ -1,4 +1,5 @@
 // C ABI of the library: argument checks, workspace carving, launches.  See include/dssd.h.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -653,21 +654,58 @@ dssd_status dssd_resample_shard_draw(const double *masses, int G, int g, int v_b
 
 namespace {
 
+// One pinned range of host memory: where it starts on the host, its length, and `p` as the GPU reaches it; false
+// for an address that lies in none (pageable or managed memory).  The runtime's query of an address does not tell how
+// far the range goes; the driver's does, and it finds nothing at an unregistered address without failing.
+struct Pinned {
+    uintptr_t begin;
+    size_t bytes;
+    char *device;
+};
+bool pinned_range(const char *p, Pinned &r)
+{
+    typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Query query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<Query>(fn) : nullptr;
+    }();
+    if (!query) return false;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr device = 0, begin = 0;
+    size_t bytes = 0;
+    CUpointer_attribute which[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &managed, &device, &begin, &bytes};
+    if (query(5, which, to, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+    if (type != CU_MEMORYTYPE_HOST || managed || !device || begin > reinterpret_cast<uintptr_t>(p)) return false;
+    r.begin = begin;
+    r.bytes = bytes;
+    r.device = reinterpret_cast<char *>(device);
+    return r.begin + r.bytes > reinterpret_cast<uintptr_t>(p);
+}
+
 // A host array as the GPU reaches it: pinned memory is mapped, so kernels read the rows they need over the
-// bus, and write their results there, without copies of their own.  nullptr for pageable memory.
+// bus, and write their results there, without copies of their own.  nullptr where any part of it is pageable: an array
+// may begin and end in registered ranges and have a gap between them, so all its ranges are looked at.
 template <class T>
 T *mapped(T *host, size_t count)
 {
     if (!host || count == 0) return nullptr;
-    const char *first = reinterpret_cast<const char *>(host), *last = first + count * sizeof(T) - 1;
-    cudaPointerAttributes a, z;
-    if (cudaPointerGetAttributes(&a, first) != cudaSuccess || cudaPointerGetAttributes(&z, last) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    constexpr int kMost = 64;  // ranges; an array registered in more pieces is copied
+    const char *const first = reinterpret_cast<const char *>(host), *const end = first + count * sizeof(T);
+    char *device = nullptr;
+    const char *p = first;
+    for (int i = 0; p < end; ++i) {
+        Pinned r;
+        if (i == kMost || !pinned_range(p, r)) return nullptr;
+        if (i == 0) device = r.device;
+        else if (r.device != device + (p - first)) return nullptr;
+        p = reinterpret_cast<const char *>(r.begin + r.bytes);
     }
-    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
-    if (static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) != last - first) return nullptr;
-    return static_cast<T *>(a.devicePointer);
+    return reinterpret_cast<T *>(device);
 }
 
 // The short input arrays of a round on host buffers, brought to the GPU by one kernel that reads the mapped

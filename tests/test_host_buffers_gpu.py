@@ -59,3 +59,35 @@ def test_topk_round(B, pin):
     for name, want in (("accept_len", ev["accept_len"]), ("token", rs["token"]), ("edge_flags", ev["flags"]), ("rs_flags", rs["flags"]),
                        ("p_idx", ev["p_idx"]), ("p_val", ev["p_val"])):
         assert torch.equal(got[name], want.cpu()), name
+
+
+@pytest.mark.parametrize("pages", [[(0, 3), (9, 12)], [(0, 5), (5, 12)], [(0, 12)], [(2, 12)]])
+def test_draft_rows_pinned_in_pieces(B, pages):
+    """draft_q of 12 rows of one page each, of which only some pages are registered: read in place where all are (in one range or in
+    two that follow one another), else copied row by row, also where its first and last bytes are pinned."""
+    Bn, gamma, V = 3, 4, 1024
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype="f32", temperature=0.9, sigma_d=1.0, seed=8)
+    g = to_device(di.generate(w, threads=8))
+    arena = torch.empty(B.dssd_round_host_arena_bytes(Bn, gamma, V, B.DSSD_F32), dtype=torch.uint8, device="cuda")
+    host = _host(g, "all")
+    raw = torch.empty(13 * 4096, dtype=torch.uint8)
+    at = -raw.data_ptr() % 4096
+    host["draft_q"] = raw[at:at + 12 * 4096].view(torch.float32).view(Bn, gamma, V).copy_(host["draft_q"])
+    base, rt = host["draft_q"].data_ptr(), torch.cuda.cudart()
+    for a, b in pages:
+        assert int(rt.cudaHostRegister(base + a * 4096, (b - a) * 4096, 0)) == 0
+    try:
+        for n_at in range(gamma + 1):  # the rejection at every position in turn
+            host["uniforms"].fill_(0.0)
+            host["uniforms"][:, n_at:] = 1.0
+            n = torch.full((Bn,), n_at, dtype=torch.int32, device="cuda")
+            ev = B.dssd_edge_verify(g["target_logits"], g["draft_tokens"], g["draft_q_tok"], host["uniforms"].cuda(), w.temperature)
+            assert torch.equal(ev["accept_len"], n)
+            rs = B.dssd_device_resample(ev["p_row"], g["draft_q"], n, g["uniforms_rs"], gamma)
+            got = B.dssd_round_host(host, w.temperature, arena)
+            torch.cuda.synchronize()
+            assert torch.equal(got["accept_len"], n.cpu()) and torch.equal(got["token"], rs["token"].cpu())
+            assert torch.equal(got["rs_flags"], rs["flags"].cpu())
+    finally:
+        for a, _ in pages:
+            assert int(rt.cudaHostUnregister(base + a * 4096)) == 0
