@@ -30,7 +30,7 @@
  *   - The caller owns every buffer.  The library allocates no memory, enqueues its work on the
  *     given CUDA stream and returns without synchronising.  It keeps no state between calls except
  *     the built-in scratch of dssd_device_resample_static, whose address is looked up once per device,
- *     and the emission kernel's resident CTAs in dssd_edge_emit_shard, likewise.
+ *     and, once per context, whether the device takes clusters of sixteen CTAs.
  *   - The kernels of a call are launched with programmatic stream serialization: the first of them may
  *     be scheduled while the kernel before it on the stream drains, and waits for its end before
  *     it reads or writes anything.

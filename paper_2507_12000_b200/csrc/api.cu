@@ -665,13 +665,7 @@ struct Pinned {
 bool pinned_range(const char *p, Pinned &r)
 {
     typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
-    static const Query query = [] {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult found;
-        const cudaError_t e = cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found);
-        if (e != cudaSuccess) cudaGetLastError();
-        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<Query>(fn) : nullptr;
-    }();
+    static const Query query = dssd::driver_call<Query>("cuPointerGetAttributes");
     if (!query) return false;
     unsigned type = 0, managed = 0;
     CUdeviceptr device = 0, begin = 0;

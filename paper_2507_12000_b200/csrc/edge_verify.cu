@@ -22,6 +22,7 @@
 
 #include <atomic>
 
+#include <cuda.h>
 #include <math.h>
 
 #include "draw.cuh"
@@ -656,7 +657,8 @@ cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 }
 
 // Clusters beyond the portable size have to be allowed for each kernel, and a device (or the part of one that the
-// process was given) may not have a processing cluster of that many SMs: asked once per device.
+// process was given) may not have a processing cluster of that many SMs: asked once per context, which holds the
+// permission.  A device that was reset, or a second context on it, is asked again.
 bool wide_clusters(void (*kernel)(EdgeParams))
 {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
@@ -684,16 +686,21 @@ bool wide_clusters()
 }
 int most_cluster_ctas()
 {
-    static std::atomic<int> known[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return kEdgeCluster;
-    int most = known[dev].load(std::memory_order_relaxed);
-    if (!most) {
-        const bool wide = wide_clusters<DSSD_F32>() && wide_clusters<DSSD_BF16>();
-        if (!wide) cudaGetLastError();
-        most = wide ? kEdgeClusterWide : kEdgeCluster;
-        known[dev].store(most, std::memory_order_relaxed);
-    }
+    typedef CUresult (*ContextId)(CUcontext, unsigned long long *);
+    static const ContextId context_id = driver_call<ContextId>("cuCtxGetId");
+    static std::atomic<unsigned long long> known[16];  // (id + 1) * 32 + the answer; 0: empty
+    static std::atomic<unsigned> turn;
+    unsigned long long id = 0;  // (an id is never given twice)
+    const bool has_id = context_id && context_id(nullptr, &id) == CUDA_SUCCESS;
+    if (has_id)
+        for (const auto &k : known) {
+            const unsigned long long w = k.load(std::memory_order_acquire);
+            if (w / 32 == id + 1) return (int)(w % 32);
+        }
+    const bool wide = wide_clusters<DSSD_F32>() && wide_clusters<DSSD_BF16>();
+    if (!wide) cudaGetLastError();
+    const int most = wide ? kEdgeClusterWide : kEdgeCluster;
+    if (has_id) known[turn.fetch_add(1, std::memory_order_relaxed) % 16].store((id + 1) * 32 + (unsigned long long)most, std::memory_order_release);
     return most;
 }
 

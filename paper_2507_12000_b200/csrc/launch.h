@@ -32,4 +32,15 @@ cudaError_t launch_pdl(void (*kernel)(Params), unsigned grid, unsigned block, cu
     return cudaLaunchKernelEx(&cfg, kernel, params);
 }
 
+// An entry point of the driver, which the library is not linked against; nullptr if there is none of that name.
+template <class Fn>
+Fn driver_call(const char *name)
+{
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const cudaError_t e = cudaGetDriverEntryPoint(name, &fn, cudaEnableDefault, &found);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(fn) : nullptr;
+}
+
 }  // namespace dssd
