@@ -121,8 +121,9 @@ size_t dssd_edge_verify_workspace_bytes(int B, int gamma, int V);
  * power-of-two scaling.  p_i(x_i) = 2^(l_x * c1 - ref) / S and the test u * q < p are evaluated in
  * float64.  The result is within about 1e-6 relative of the exact softmax as long as
  * |l| * log2(e) / T stays well inside the float32 range (the rounding of c1 alone contributes
- * 6e-8 * |l_v / T - E_p[l / T]| to ln p); rows whose scaled logits overflow float32 are flagged
- * DSSD_EDGE_FLAG_NONFINITE.  u == 1 never accepts; q <= 0 accepts iff p > 0; a NaN q or an
+ * 6e-8 * |l_v / T - E_p[l / T]| to ln p).  A logit whose scaled value lies below float32's range (a mask of the
+ * type's lowest value) weighs nothing, as -inf does; rows with a scaled logit above the range, or with none inside it, are
+ * flagged DSSD_EDGE_FLAG_NONFINITE.  u == 1 never accepts; q <= 0 accepts iff p > 0; a NaN q or an
  * out-of-range token rejects.
  *
  * target_logits  [B, gamma+1, V] of `dtype`, unit stride along V, `row_stride` elements between

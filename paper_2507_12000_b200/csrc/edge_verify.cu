@@ -56,6 +56,7 @@ __device__ __forceinline__ void online_raise(Online &o, float bm, float c1)
 {
     if (bm > o.m) {
         const float nref = rintf(bm * c1);
+        if (nref == DSSD_NEG_INF) return;  // all of them lie below float32's range (a mask of the type's lowest value): like -inf
         const float f = (o.m == DSSD_NEG_INF) ? 0.f : ex2(o.ref - nref);  // an exact power of two
         const f32x2 ff = pack2(f, f);
         o.s0 = mul2(o.s0, ff);

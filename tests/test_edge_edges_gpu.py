@@ -84,3 +84,27 @@ def test_every_entry_of_a_vector_counts(B, dtype, V, stride):
         assert ((ev["p_row"][rows, at] - 1.0).abs() <= 3e-7).all() and ((ev["lse"][:, 0] - 1.5).abs() <= 1e-6).all()
     z = torch.zeros(Bn, V, dtype=dt, device="cuda")  # equal entries: n in all positions
     assert ((run(z)["p_row"] * V - 1.0).abs() <= 2e-6).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("Bn,gamma,V", [(1, 0, 40000), (8, 4, 32000), (300, 4, 30011), (40, 8, 70001), (256, 4, 151936)])
+def test_masks_of_the_lowest_value_weigh_nothing(B, dtype, Bn, gamma, V):
+    """Masks of the type's lowest value, whose scaled logits are below float32's range, give bit for bit what masks of -inf
+    give, wherever they begin and end: whole tiles of a thread, its first ones, all but one entry."""
+    import torch
+
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    z = torch.randn(Bn, gamma + 1, V, device="cuda", generator=torch.Generator("cuda").manual_seed(V)).to(dt)
+    x = torch.zeros(Bn, gamma, dtype=torch.int32, device="cuda")
+    half = torch.full((Bn, gamma), 0.5, device="cuda")
+    for a, b in ((0, V // 2), (0, 24576), (8192, V), (16384, 32768), (V // 3, V), (1, V), (0, V - 1)):
+        got = []
+        for low in (torch.finfo(dt).min, float("-inf")):
+            masked = z.clone()
+            masked[:, :, a:b] = low
+            got.append(B.dssd_edge_verify(masked, x, half, half, 1.0))
+        assert (got[0]["flags"] == 0).all()
+        for k in ("accept_len", "p_row", "lse", "flags", "p_tok"):
+            assert torch.equal(got[0][k], got[1][k]), (k, a, b)
+    rows = torch.full((Bn, gamma + 1, V), torch.finfo(dt).min, dtype=dt, device="cuda")  # nothing inside the range
+    assert (B.dssd_edge_verify(rows, x, half, half, 1.0)["flags"] == B.EDGE_FLAG_NONFINITE).all()
