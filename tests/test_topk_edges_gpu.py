@@ -46,3 +46,27 @@ def test_masked_and_overflowing_rows(B, oracle_mod, k):
     tl[3][:, :4096] = 0.0
     tl[3][:, 4096:] = np.linspace(0.0, 1.0, V - 4096, dtype=np.float32)[None]
     compare_topk(B, oracle_mod, d, w.temperature, k)
+
+
+@pytest.mark.parametrize("k", [1, 9, 10, 32])
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [("f32", 9, 1, 30011), ("bf16", 9, 1, 30011), ("bf16", 520, 2, 32768), ("f32", 520, 4, 33003)])
+def test_ties_and_masks(B, oracle_mod, dtype, Bn, gamma, V, k):
+    """Runs whose candidates overflow: masks of several values (ties at the threshold, of which the lowest indices count) that end
+    anywhere, ascending rows, few distinct values, and rows with more candidates above any bound from the threads'
+    maxima than fit; in rows at every alignment, in runs of one, two and four tiles."""
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype="f32", temperature=0.9, sigma_d=0.5, seed=k)
+    d = di.generate_topk(w, k, threads=16)
+    tl = d["target_logits"]
+    rng = np.random.default_rng(k)
+    at = np.arange(V)
+    for i, low in ((0, -1.0e9), (1, -10000.3), (2, np.finfo(np.float32).min), (3, -np.inf)):
+        tl[i][:, rng.random(V) < 0.9995 if i % 2 else at >= 17] = low
+    tl[4][:] = np.linspace(-1.0, 1.0, V, dtype=np.float32)
+    tl[5][:] = 0.1234567
+    tl[6][:] = rng.integers(0, 3, V)
+    tl[7][:] = np.where(at // 4 % 128 < 32, 0.0, 1.0 + at / V)
+    tl[8][:, : V // 2], tl[8][:, V // 2:] = -0.0, 0.0
+    if dtype == "bf16":
+        with np.errstate(over="ignore"):
+            d["target_logits"] = (np.where(np.abs(tl) == np.finfo(np.float32).max, np.sign(tl) * 3.3e38, tl).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
+    compare_topk(B, oracle_mod, d, w.temperature, k)
