@@ -48,7 +48,8 @@ constexpr int kGroupsUpTo = 12;
 constexpr int kRefine = 96;
 constexpr int kFoldWarps = 16;                       // most warps (rows at a time) of the fold kernel
 constexpr int kMergeCap = 256;                       // keys that a warp ranks when it merges a row's runs
-constexpr unsigned long long kBadList = ~0ull;       // first key of a run that held a NaN or +inf
+constexpr int kMergeLists = 64;                      // lists that it notes before it looks at their keys
+constexpr unsigned long long kBadList = ~0ull;       // every key of a run that held a NaN or +inf
 constexpr unsigned kFullMask = 0xffffffffu;
 
 __device__ __forceinline__ float max_nan(float a, float b)
@@ -124,6 +125,31 @@ struct Vec<DSSD_BF16> {
         const uint32_t w = j < 4 ? (j < 2 ? v.x : v.y) : (j < 6 ? v.z : v.w);
         return (j & 1) ? bf16_hi(w) : bf16_lo(w);
     }
+};
+
+// A CTA's run: the vectors v0 .. v1 - 1 of its row, which start at the row's first 16-byte boundary (entry idx0), and, in the
+// row's first and last run, the entries before and after the vectors; entries e0 .. e1 - 1 in all.
+template <int DT>
+struct Run {
+    const char *rowp;
+    const uint4 *src;
+    int run, idx0, nvec, v0, v1;
+    __device__ __forceinline__ explicit Run(const TopkParams &P)
+    {
+        const unsigned row = blockIdx.x / (unsigned)P.runs;
+        run = (int)(blockIdx.x - row * (unsigned)P.runs);
+        rowp = static_cast<const char *>(P.logits) + (size_t)row * (size_t)P.row_stride * Vec<DT>::kEsz;
+        const long long rowbytes = (long long)P.V * Vec<DT>::kEsz;
+        int head = (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(rowp) & 15u)) & 15u);
+        if (head > rowbytes) head = (int)rowbytes;
+        nvec = (int)((rowbytes - head) >> 4);
+        v0 = min(nvec, run * P.run_vecs);
+        v1 = run + 1 == P.runs ? nvec : min(nvec, v0 + P.run_vecs);
+        src = reinterpret_cast<const uint4 *>(rowp + head);
+        idx0 = head / Vec<DT>::kEsz;
+    }
+    __device__ __forceinline__ int e0() const { return run == 0 ? 0 : idx0 + v0 * Vec<DT>::E; }
+    __device__ __forceinline__ int e1(const TopkParams &P) const { return run + 1 == P.runs ? P.V : idx0 + v1 * Vec<DT>::E; }
 };
 
 struct SelectShared {
@@ -207,11 +233,14 @@ __device__ __noinline__ int refine(SelectShared &sh, int m, float top, int k)
 // vector by vector in index order.  Two passes over the run at most, from L2.  B = 256 gamma = 4 V = 32000 bf16,
 // nine tenths masked, k = 10: 61 us, entry by entry (select_slowly) 791; ascending rows 267 and 6592.  false: more are above t than fit.
 template <int DT>
-__device__ __noinline__ bool select_again(SelectShared &sh, const char *rowp, int idx0, int v0, int v1, int e0, int e1, float top, int k)
+__device__ __noinline__ bool select_again(SelectShared &sh, const TopkParams &P, float top)
 {
     constexpr int E = Vec<DT>::E;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint4 *src = reinterpret_cast<const uint4 *>(rowp + (size_t)idx0 * Vec<DT>::kEsz);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = P.k;
+    const Run<DT> R(P);
+    const char *rowp = R.rowp;
+    const uint4 *src = R.src;
+    const int idx0 = R.idx0, v0 = R.v0, v1 = R.v1, e0 = R.e0(), e1 = R.e1(P);
     const int ev0 = idx0 + v0 * E, ev1 = idx0 + v1 * E;  // the entries in vectors
     const uint32_t mine = ord(top == top ? top : DSSD_NEG_INF);
     int rank = 0;
@@ -280,9 +309,12 @@ __device__ __noinline__ bool select_again(SelectShared &sh, const char *rowp, in
 
 // The run again, where that did not do either: entry by entry, at most one per thread and step.
 template <int DT>
-__device__ __noinline__ void select_slowly(SelectShared &sh, const char *rowp, int e0, int e1, int k)
+__device__ __noinline__ void select_slowly(SelectShared &sh, const TopkParams &P)
 {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, k = P.k;
+    const Run<DT> R(P);
+    const char *rowp = R.rowp;
+    const int e0 = R.e0(), e1 = R.e1(P);
     unsigned long long floor = 0ull;  // keys up to here are not among the k best
     __syncthreads();
     if (tid == 0) sh.count = 0;
@@ -310,25 +342,17 @@ __device__ __noinline__ void select_slowly(SelectShared &sh, const char *rowp, i
 // replaces (a ring per CTA, one selection warp that inserted candidates one by one, rows judged in the
 // same warp) took 79 us for this and the fold together, and 18.8 us at B = 1 gamma = 8 V = 50272 where
 // both kernels now take 7.7.  Ten CTAs per SM (48 registers); eight 61.9, twelve 65 us (spills).
-// One CTA per (row, run).  A row's vectors start at
-// its first 16-byte boundary; the entries before it belong to the first run, those after the last whole
-// vector to the last run.
+// One CTA per (row, run).
 template <int DT>
 __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __grid_constant__ TopkParams P)
 {
-    constexpr int E = Vec<DT>::E, kEsz = Vec<DT>::kEsz;
+    constexpr int E = Vec<DT>::E;
     __shared__ SelectShared sh;
     const int tid = threadIdx.x, lane = tid & 31, k = P.k;
-    const unsigned row = blockIdx.x / (unsigned)P.runs;
-    const int run = (int)(blockIdx.x - row * (unsigned)P.runs);
-    const char *rowp = static_cast<const char *>(P.logits) + (size_t)row * (size_t)P.row_stride * kEsz;
-    const long long rowbytes = (long long)P.V * kEsz;
-    int head = (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(rowp) & 15u)) & 15u);
-    if (head > rowbytes) head = (int)rowbytes;
-    const int nvec = (int)((rowbytes - head) >> 4);
-    const int v0 = min(nvec, run * P.run_vecs), v1 = run + 1 == P.runs ? nvec : min(nvec, v0 + P.run_vecs);
-    const uint4 *src = reinterpret_cast<const uint4 *>(rowp + head);
-    const int idx0 = head / kEsz;  // index of the first vector's first entry
+    const Run<DT> R(P);
+    const char *rowp = R.rowp;
+    const uint4 *src = R.src;
+    const int run = R.run, nvec = R.nvec, v0 = R.v0, v1 = R.v1, idx0 = R.idx0;
     if (tid == 0) {
         sh.count = 0;
         sh.bad = 0;
@@ -417,15 +441,14 @@ __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __gr
     __syncthreads();
     int m = (int)sh.count;
     if (m > kCand) {
-        const int e0 = run == 0 ? 0 : idx0 + v0 * E, e1 = run + 1 == P.runs ? P.V : idx0 + v1 * E;
-        if (!select_again<DT>(sh, rowp, idx0, v0, v1, e0, e1, top, k)) select_slowly<DT>(sh, rowp, e0, e1, k);
+        if (!select_again<DT>(sh, P, top)) select_slowly<DT>(sh, P);
         m = (int)sh.count;
     }
     if (m > kRefine) m = refine(sh, m, top, k);
     rank_keys(sh, m, k);
     if (tid < k) {
         unsigned long long key = sh.top[tid];
-        if (sh.bad) key = tid == 0 ? kBadList : 0ull;
+        if (sh.bad) key = kBadList;
         P.lists[(size_t)blockIdx.x * k + tid] = key;
     }
 }
@@ -475,58 +498,13 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x)
 struct MergeShared {
     unsigned long long key[kMergeCap + 8];
     unsigned long long top[32];
+    int list[kMergeLists];
 };
 
-// One warp: merges the lists of the row's runs; returns key r of the row's support in lane r (kBadList in
-// lane 0 marks a row with a NaN or +inf).  The largest of the lists' last keys bounds the row's k-th key
-// from below; the keys that reach it - few more than k - are ranked by counting.
-__device__ __forceinline__ unsigned long long merged_keys(const unsigned long long *src, int runs, int k, MergeShared &sh)
+// One warp: the k largest of the c <= kMergeCap keys in sh.key (at least k), best first, to sh.top.
+__device__ __forceinline__ void rank_merged(MergeShared &sh, int c, int k)
 {
     const int lane = threadIdx.x & 31;
-    if (runs == 1) return lane < k ? ld_after(src + lane) : 0ull;
-    const int m = runs * k;
-    // one round trip for the lists' ends and (up to 256 of them) their keys
-    unsigned long long x[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = 32 * u + lane < m ? ld_after(src + 32 * u + lane) : 0ull;
-    unsigned long long bound = 0ull;
-    bool bad = false;
-    for (int r = lane; r < runs; r += 32) {
-        const unsigned long long last = ld_after(src + (size_t)r * k + k - 1), best = ld_after(src + (size_t)r * k);
-        bad |= best == kBadList;
-        bound = last > bound ? last : bound;
-    }
-    if (__any_sync(kFullMask, bad)) return lane == 0 ? kBadList : 0ull;
-    bound = warp_max_u64(bound);
-    if (bound == 0ull) bound = 1ull;  // no list is full: every key counts, empty slots do not
-    int c = 0;
-    for (int i0 = 0;;) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const unsigned keep = __ballot_sync(kFullMask, x[u] >= bound);
-            const int at = c + __popc(keep & ((1u << lane) - 1u));
-            if (x[u] >= bound && at < kMergeCap) sh.key[at] = x[u];
-            c += __popc(keep);
-        }
-        i0 += 256;
-        if (i0 >= m) break;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = i0 + 32 * u + lane < m ? ld_after(src + i0 + 32 * u + lane) : 0ull;
-    }
-    __syncwarp();
-    if (c > kMergeCap) {  // lists that interleave evenly: one best key after the other
-        unsigned long long prev = ~0ull, mine = 0ull;
-        for (int r = 0; r < k; ++r) {
-            unsigned long long best = 0ull;
-            for (int i = lane; i < m; i += 32) {
-                const unsigned long long y = ld_after(src + i);
-                if (y < prev && y > best) best = y;
-            }
-            prev = warp_max_u64(best);
-            if (lane == r) mine = prev;
-        }
-        return mine;
-    }
     if (lane < 8) sh.key[c + lane] = 0ull;  // the ranking goes in steps of eight
     __syncwarp();
     for (int i = lane; i < c; i += 32) {
@@ -539,6 +517,146 @@ __device__ __forceinline__ unsigned long long merged_keys(const unsigned long lo
         if (rank < k) sh.top[rank] = y;
     }
     __syncwarp();
+}
+
+// One warp: merges the lists of a row of many runs; returns key r of the row's support in lane r (kBadList in lane 0 marks a
+// row with a NaN or +inf).  Of the lists' j-th keys - one per lane, the largest of the lane's lists - the r-th largest,
+// r * j >= k, bounds the row's k-th key from below: r lists hold j keys each that reach it.  So does the largest of their last
+// keys, the better bound where one run holds most of the row's best (masked and ascending rows).  The keys that
+// reach it are few more than k, ranked by counting; if more come than fit, those that have come are cut back to their k best,
+// the last of which is a better bound.  All keys are looked at where they are few (four round trips), else only the
+// lists whose first key reaches the bound, hardly ever more than k of the hundreds.
+// (With the lists' last keys alone for a bound, far lower where many lists interleave, the edge call took
+// 75 us at k = 32 B = 1 gamma = 4 V = 128256 float32, 32 lists per row, now 12.1; k = 10 B = 1 gamma = 2 V = 4194304 217, now 30.)
+__device__ __forceinline__ unsigned long long merge_many(const unsigned long long *src, int runs, int k, MergeShared &sh)
+{
+    const int lane = threadIdx.x & 31, m = runs * k;
+    const bool all = m <= 1024;
+    // one round trip for the first 256 keys and what the bound is taken from
+    unsigned long long x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = all && 32 * u + lane < m ? ld_after(src + 32 * u + lane) : 0ull;
+    const int half = ((runs < 32 ? runs : 32) + 1) / 2;
+    const int j = (k + half - 1) / half, r = (k + j - 1) / j;
+    unsigned long long best = 0ull, last = 0ull;
+    bool bad = false;
+    for (int q0 = lane; q0 < runs; q0 += 256) {
+        unsigned long long y[8], z[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool there = q0 + 32 * u < runs;
+            y[u] = there ? ld_after(src + (size_t)(q0 + 32 * u) * k + j - 1) : 0ull;
+            z[u] = there ? ld_after(src + (size_t)(q0 + 32 * u) * k + k - 1) : 0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            bad |= y[u] == kBadList;
+            best = y[u] > best ? y[u] : best;
+            last = z[u] > last ? z[u] : last;
+        }
+    }
+    if (__any_sync(kFullMask, bad)) return lane == 0 ? kBadList : 0ull;
+    sh.top[lane] = best;
+    __syncwarp();
+    int place = 0;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const unsigned long long o = sh.top[i];
+        place += o > best || (o == best && i < lane);
+    }
+    unsigned long long bound = __shfl_sync(kFullMask, best, __ffs(__ballot_sync(kFullMask, place == r - 1)) - 1);
+    last = warp_max_u64(last);
+    if (last > bound) bound = last;
+    if (bound == 0ull) bound = 1ull;  // too few lists of j keys: every key counts, empty slots do not
+    int c = 0;
+    auto append = [&](unsigned long long y) {
+        unsigned keep = __ballot_sync(kFullMask, y >= bound);
+        if (!keep) return;
+        if (c + __popc(keep) > kMergeCap) {
+            __syncwarp();
+            rank_merged(sh, c, k);
+            bound = sh.top[k - 1];
+            if (lane < k) sh.key[lane] = sh.top[lane];
+            __syncwarp();
+            c = k;
+            keep = __ballot_sync(kFullMask, y >= bound);
+        }
+        if (y >= bound) sh.key[c + __popc(keep & ((1u << lane) - 1u))] = y;
+        c += __popc(keep);
+    };
+    if (all) {
+        for (int i0 = 0;;) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) append(x[u]);
+            i0 += 256;
+            if (i0 >= m) break;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = i0 + 32 * u + lane < m ? ld_after(src + i0 + 32 * u + lane) : 0ull;
+        }
+    } else {
+        int lists = 0;  // noted in sh.list, their keys not looked at yet
+        auto take = [&]() {
+            __syncwarp();
+            for (int i0 = 0; i0 < lists * k; i0 += 256) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int i = i0 + 32 * u + lane;
+                    x[u] = i < lists * k ? ld_after(src + (size_t)sh.list[i / k] * k + i % k) : 0ull;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) append(x[u]);
+            }
+            lists = 0;
+            __syncwarp();
+        };
+        for (int q0 = 0; q0 < runs; q0 += 256) {
+            unsigned long long y[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) y[u] = q0 + 32 * u + lane < runs ? ld_after(src + (size_t)(q0 + 32 * u + lane) * k) : 0ull;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const unsigned reach = __ballot_sync(kFullMask, y[u] >= bound);
+                if (lists + __popc(reach) > kMergeLists) take();
+                if (reach >> lane & 1u) sh.list[lists + __popc(reach & ((1u << lane) - 1u))] = q0 + 32 * u + lane;
+                lists += __popc(reach);
+            }
+        }
+        take();
+    }
+    __syncwarp();
+    rank_merged(sh, c, k);
+    const unsigned long long key = lane < k ? sh.top[lane] : 0ull;
+    __syncwarp();
+    return key;
+}
+
+// The same where the keys fit a warp's registers and k is small: the largest of the lists' last keys is bound enough (7 runs,
+// k = 5, B = 32 gamma = 4 V = 50257 bf16: the edge call 10.2 us, with merge_many 11.9; k = 32: 19.1 and 14.4).
+constexpr int kMergeFew = 256;
+__device__ __forceinline__ unsigned long long merge_few(const unsigned long long *src, int runs, int k, MergeShared &sh)
+{
+    const int lane = threadIdx.x & 31, m = runs * k;
+    // one round trip for the lists' ends and their keys
+    unsigned long long x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = 32 * u + lane < m ? ld_after(src + 32 * u + lane) : 0ull;
+    unsigned long long bound = 0ull;
+    for (int r = lane; r < runs; r += 32) {
+        const unsigned long long last = ld_after(src + (size_t)r * k + k - 1);
+        bound = last > bound ? last : bound;
+    }
+    bound = warp_max_u64(bound);
+    if (bound == kBadList) return lane == 0 ? kBadList : 0ull;
+    if (bound == 0ull) bound = 1ull;  // no list is full: every key counts, empty slots do not
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const unsigned keep = __ballot_sync(kFullMask, x[u] >= bound);
+        if (x[u] >= bound) sh.key[c + __popc(keep & ((1u << lane) - 1u))] = x[u];
+        c += __popc(keep);
+    }
+    __syncwarp();
+    rank_merged(sh, c, k);
     const unsigned long long key = lane < k ? sh.top[lane] : 0ull;
     __syncwarp();
     return key;
@@ -565,8 +683,11 @@ __device__ __forceinline__ bool judge(const TopkParams &P, const RowDist &d, int
 }
 
 // One CTA per sequence, a warp per row (the rows in turns when there are more than kFoldWarps).  Bound by
-// latency: one round trip for the lists and the float64 operations that depend on one another.
-__global__ void __launch_bounds__(32 * kFoldWarps) topk_fold_kernel(const __grid_constant__ TopkParams P)
+// latency: one round trip for the lists and the float64 operations that depend on one another.  More sequences than are resident
+// at 128 registers run with 64 (kCtas = 2): B = 8192 gamma = 2 V = 4096 k = 4 84 us for the edge call against 93; one wave is
+// quicker with 128: B = 256 gamma = 4 V = 151936 k = 10 67.2 against 67.9.
+template <bool kMany, int kCtas>
+__global__ void __launch_bounds__(32 * kFoldWarps, kCtas) topk_fold_kernel(const __grid_constant__ TopkParams P)
 {
     extern __shared__ unsigned char smem[];
     MergeShared *merge = reinterpret_cast<MergeShared *>(smem);
@@ -592,7 +713,10 @@ __global__ void __launch_bounds__(32 * kFoldWarps) topk_fold_kernel(const __grid
                 u = ld_after(P.uniforms + o);
                 q = ld_after(P.draft_q_tok + o);
             }
-            const unsigned long long key = merged_keys(P.lists + ((size_t)b * rows + j) * P.runs * k, P.runs, k, merge[warp]);
+            const unsigned long long *lists = P.lists + ((size_t)b * rows + j) * P.runs * k;
+            const unsigned long long key = P.runs == 1 ? (lane < k ? ld_after(lists + lane) : 0ull)
+                                           : kMany     ? merge_many(lists, P.runs, k, merge[warp])
+                                                       : merge_few(lists, P.runs, k, merge[warp]);
             d = dist_from_keys(P, key);
             unsigned row_fl = d.bad ? DSSD_EDGE_FLAG_NONFINITE : 0u;
             bool accept = true;
@@ -752,7 +876,10 @@ cudaError_t topk_verify_launch(TopkParams &P, int dtype, void *workspace, cudaSt
                                              : launch_pdl(topk_select_kernel<DSSD_F32>, (unsigned)grid, kSelThreads, stream, P);
     if (e != cudaSuccess) return e;
     const int warps = P.gamma + 1 < kFoldWarps ? P.gamma + 1 : kFoldWarps;
-    return launch_pdl(topk_fold_kernel, (unsigned)P.B, 32u * (unsigned)warps, stream, P, (size_t)warps * sizeof(MergeShared));
+    const bool many = (long long)P.runs * P.k > kMergeFew || P.k > kGroupsUpTo;
+    const bool waves = (long long)P.B * warps > 148 * kFoldWarps;
+    return launch_pdl(many ? topk_fold_kernel<true, 1> : waves ? topk_fold_kernel<false, 2> : topk_fold_kernel<false, 1>, (unsigned)P.B,
+                      32u * (unsigned)warps, stream, P, (size_t)warps * sizeof(MergeShared));
 }
 
 cudaError_t topk_resample_launch(const TopkResampleParams &P, cudaStream_t stream)

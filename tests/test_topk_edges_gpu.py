@@ -70,3 +70,18 @@ def test_ties_and_masks(B, oracle_mod, dtype, Bn, gamma, V, k):
         with np.errstate(over="ignore"):
             d["target_logits"] = (np.where(np.abs(tl) == np.finfo(np.float32).max, np.sign(tl) * 3.3e38, tl).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
     compare_topk(B, oracle_mod, d, w.temperature, k)
+
+
+@pytest.mark.parametrize("V,k", [(9 * 4096, 29), (33 * 4096 + 5, 8), (30 * 4096, 32), (33 * 4096, 32), (300 * 4096 + 1, 1), (300 * 4096, 10),
+                                 (300 * 4096 + 3, 32), (2100 * 4096, 12)])
+def test_rows_of_many_runs(B, oracle_mod, V, k):
+    """Merging the lists of many runs (4096 float32 entries each), all keys and only those of the lists that matter: equal shares, rows
+    whose best entries lie in fewer of the merging lanes than the bound needs (so that hundreds of keys and lists reach it), ascending
+    rows, and rows with fewer than k entries above -inf."""
+    w = di.custom(B=4, gamma=0 if V > 5000000 else 1, V=V, dtype="f32", temperature=0.9, sigma_d=0.5, seed=k)
+    d = di.generate_topk(w, k, threads=16)
+    tl, run = d["target_logits"], np.arange(V) // 4096
+    tl[1] += np.where(run % 32 < 15, 50.0, 0.0).astype(np.float32)
+    tl[2][:] = np.linspace(-3.0, 9.0, V, dtype=np.float32)
+    tl[3][:, np.arange(V) % 9001 != 0] = -np.inf
+    compare_topk(B, oracle_mod, d, w.temperature, k)
