@@ -47,6 +47,7 @@ constexpr int kCand = 1024;                          // candidates that a CTA ca
 constexpr int kGroupsUpTo = 12;
 constexpr int kRefine = 96;
 constexpr int kFoldWarps = 16;                       // most warps (rows at a time) of the fold kernel
+constexpr int kFoldTurns = 2;                        // most turns; beyond, topk_rows_kernel
 constexpr int kMergeCap = 256;                       // keys that a warp ranks when it merges a row's runs
 constexpr int kMergeLists = 64;                      // lists that it notes before it looks at their keys
 constexpr unsigned long long kBadList = ~0ull;       // every key of a run that held a NaN or +inf
@@ -682,6 +683,41 @@ __device__ __forceinline__ bool judge(const TopkParams &P, const RowDist &d, int
     return (ratio == ratio) && (u < (ratio < 1.0 ? ratio : 1.0));
 }
 
+// One row, by a warp: its support's distribution from the lists of its runs (their merged keys in `key`), the acceptance test if
+// a token was drafted for it.  Bit 0 of the result: accepted, flag bits from bit 8 on.
+template <bool kMany>
+__device__ __forceinline__ unsigned fold_row(const TopkParams &P, int b, int j, MergeShared &sh, RowDist &d, unsigned long long &key)
+{
+    const int lane = threadIdx.x & 31, k = P.k;
+    int x = 0;
+    float u = 0.f, q = 0.f;
+    if (j < P.gamma) {
+        const size_t o = (size_t)b * P.gamma + j;
+        x = ld_after(P.draft_tokens + o);
+        u = ld_after(P.uniforms + o);
+        q = ld_after(P.draft_q_tok + o);
+    }
+    const unsigned long long *lists = P.lists + ((size_t)b * (P.gamma + 1) + j) * P.runs * k;
+    key = P.runs == 1 ? (lane < k ? ld_after(lists + lane) : 0ull) : kMany ? merge_many(lists, P.runs, k, sh) : merge_few(lists, P.runs, k, sh);
+    d = dist_from_keys(P, key);
+    unsigned fl = d.bad ? DSSD_EDGE_FLAG_NONFINITE : 0u;
+    bool accept = true;
+    if (j < P.gamma) {
+        double p;
+        accept = judge(P, d, x, (double)u, (double)q, fl, p);
+        if (lane == 0 && P.p_tok) P.p_tok[(size_t)b * P.gamma + j] = (float)p;
+    }
+    return (accept ? 1u : 0u) | (fl << 8);
+}
+
+__device__ __forceinline__ void write_pairs(const TopkParams &P, int b, const RowDist &d)
+{
+    const int lane = threadIdx.x & 31, k = P.k;
+    if (lane >= k) return;
+    P.p_idx[(size_t)b * k + lane] = d.bad ? -1 : d.idx;
+    P.p_val[(size_t)b * k + lane] = d.bad ? NAN : (float)d.prob;
+}
+
 // One CTA per sequence, a warp per row (the rows in turns when there are more than kFoldWarps).  Bound by
 // latency: one round trip for the lists and the float64 operations that depend on one another.  More sequences than are resident
 // at 128 registers run with 64 (kCtas = 2): B = 8192 gamma = 2 V = 4096 k = 4 84 us for the edge call against 93; one wave is
@@ -692,7 +728,7 @@ __global__ void __launch_bounds__(32 * kFoldWarps, kCtas) topk_fold_kernel(const
     extern __shared__ unsigned char smem[];
     MergeShared *merge = reinterpret_cast<MergeShared *>(smem);
     __shared__ unsigned s_verdict[kFoldWarps];  // bit 0: accepted, flag bits from bit 8 on
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5, k = P.k;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int b = blockIdx.x, rows = P.gamma + 1;
     pdl_wait();
     pdl_trigger();
@@ -704,44 +740,67 @@ __global__ void __launch_bounds__(32 * kFoldWarps, kCtas) topk_fold_kernel(const
         d.idx = -1;
         d.prob = NAN;
         d.bad = false;
+        unsigned mine = 1u;
         if (j < rows) {
-            int x = 0;
-            float u = 0.f, q = 0.f;
-            if (j < P.gamma) {
-                const size_t o = (size_t)b * P.gamma + j;
-                x = ld_after(P.draft_tokens + o);
-                u = ld_after(P.uniforms + o);
-                q = ld_after(P.draft_q_tok + o);
-            }
-            const unsigned long long *lists = P.lists + ((size_t)b * rows + j) * P.runs * k;
-            const unsigned long long key = P.runs == 1 ? (lane < k ? ld_after(lists + lane) : 0ull)
-                                           : kMany     ? merge_many(lists, P.runs, k, merge[warp])
-                                                       : merge_few(lists, P.runs, k, merge[warp]);
-            d = dist_from_keys(P, key);
-            unsigned row_fl = d.bad ? DSSD_EDGE_FLAG_NONFINITE : 0u;
-            bool accept = true;
-            if (j < P.gamma) {
-                double p;
-                accept = judge(P, d, x, (double)u, (double)q, row_fl, p);
-                if (lane == 0 && P.p_tok) P.p_tok[(size_t)b * P.gamma + j] = (float)p;
-            }
-            if (lane == 0) s_verdict[warp] = (accept ? 1u : 0u) | (row_fl << 8);
-        } else if (lane == 0) {
-            s_verdict[warp] = 1u;
+            unsigned long long key;
+            mine = fold_row<kMany>(P, b, j, merge[warp], d, key);
         }
+        if (lane == 0) s_verdict[warp] = mine;
         __syncthreads();
         const unsigned v = lane < warps ? s_verdict[lane] : 1u;
         fl |= __reduce_or_sync(kFullMask, v >> 8);
         const unsigned rej = __ballot_sync(kFullMask, !(v & 1u));
         const bool open = n == P.gamma;  // no rejection before this batch
         if (rej && open) n = base + __ffs(rej) - 1;
-        if (open && n == j && lane < k) {  // row n is this warp's
-            P.p_idx[(size_t)b * k + lane] = d.bad ? -1 : d.idx;
-            P.p_val[(size_t)b * k + lane] = d.bad ? NAN : (float)d.prob;
-        }
+        if (open && n == j) write_pairs(P, b, d);  // row n is this warp's
         __syncthreads();
     }
     if (threadIdx.x == 0) {
+        P.accept_len[b] = n;
+        if (P.flags) P.flags[b] = fl;
+    }
+}
+
+// The same in two steps for many positions, which the kernel above takes in turns: a warp per row leaves the row's verdict and, in
+// the place of its first list, its merged keys; a warp per sequence finds row n.  B = 2 gamma = 200 V = 32000 k = 10: the edge call
+// PLACE_E us, in turns 53.6; gamma = 64 PLACE_F and 22.7; gamma = 31 PLACE_G and 12.6.
+template <bool kMany>
+__global__ void __launch_bounds__(32 * kFoldWarps, 1) topk_rows_kernel(const __grid_constant__ TopkParams P)
+{
+    extern __shared__ unsigned char smem[];
+    MergeShared *merge = reinterpret_cast<MergeShared *>(smem);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long row = (long long)blockIdx.x * kFoldWarps + warp;
+    pdl_wait();
+    pdl_trigger();
+    if (row >= (long long)P.B * (P.gamma + 1)) return;
+    const int b = (int)(row / (P.gamma + 1)), j = (int)(row - (long long)b * (P.gamma + 1));
+    RowDist d;
+    unsigned long long key;
+    const unsigned verdict = fold_row<kMany>(P, b, j, merge[warp], d, key);
+    if (lane < P.k) P.lists[(size_t)row * P.runs * P.k + lane] = key;
+    if (lane == 0) P.verdict[row] = verdict;
+}
+
+__global__ void __launch_bounds__(kThreads) topk_first_kernel(const __grid_constant__ TopkParams P)
+{
+    const int lane = threadIdx.x & 31;
+    const long long b = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    pdl_wait();
+    pdl_trigger();
+    if (b >= P.B) return;
+    const size_t row0 = (size_t)b * (P.gamma + 1);
+    int n = P.gamma;
+    unsigned fl = 0;
+    for (int base = 0; base <= P.gamma; base += 32) {
+        const unsigned v = base + lane <= P.gamma ? ld_after_u32(P.verdict + row0 + base + lane) : 1u;
+        fl |= __reduce_or_sync(kFullMask, v >> 8);
+        const unsigned rej = __ballot_sync(kFullMask, !(v & 1u));
+        if (rej && n == P.gamma) n = base + __ffs(rej) - 1;
+    }
+    const RowDist d = dist_from_keys(P, lane < P.k ? ld_after(P.lists + (row0 + n) * P.runs * P.k + lane) : 0ull);
+    write_pairs(P, (int)b, d);
+    if (lane == 0) {
         P.accept_len[b] = n;
         if (P.flags) P.flags[b] = fl;
     }
@@ -854,7 +913,7 @@ static void topk_geometry(int B, int gamma, int V, int esz, int &runs, int &run_
 // workspace made for the largest batch serves the smaller ones.  A launch of t tiles keeps t lists below kSelTwoTiles,
 // rows * ceil(n / 2) <= t of them below kSelFourTiles (n tiles per row) and rows * ceil(n / 4) beyond; each bound grows with
 // rows and n, and so does the largest of the three.
-size_t topk_workspace_bytes(int B, int gamma, int V, int k)
+static size_t list_bytes(int B, int gamma, int V, int k)
 {
     const unsigned long long rows = (unsigned long long)B * (unsigned long long)(gamma + 1);
     unsigned long long n = ((unsigned long long)V * 4 / 16 + kSelTile - 1) / kSelTile;
@@ -866,10 +925,16 @@ size_t topk_workspace_bytes(int B, int gamma, int V, int k)
     return ((size_t)lists * (size_t)k * 8 + 255) & ~(size_t)255;
 }
 
+size_t topk_workspace_bytes(int B, int gamma, int V, int k)
+{
+    return list_bytes(B, gamma, V, k) + (((size_t)B * (size_t)(gamma + 1) * 4 + 255) & ~(size_t)255);
+}
+
 cudaError_t topk_verify_launch(TopkParams &P, int dtype, void *workspace, cudaStream_t stream)
 {
     topk_geometry(P.B, P.gamma, P.V, dtype == DSSD_BF16 ? 2 : 4, P.runs, P.run_vecs);
     P.lists = static_cast<unsigned long long *>(workspace);
+    P.verdict = reinterpret_cast<uint32_t *>(static_cast<char *>(workspace) + list_bytes(P.B, P.gamma, P.V, P.k));
     const unsigned long long grid = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1) * (unsigned long long)P.runs;
     if (grid > 0x7fffffffull) return cudaErrorInvalidConfiguration;
     const cudaError_t e = dtype == DSSD_BF16 ? launch_pdl(topk_select_kernel<DSSD_BF16>, (unsigned)grid, kSelThreads, stream, P)
@@ -877,6 +942,12 @@ cudaError_t topk_verify_launch(TopkParams &P, int dtype, void *workspace, cudaSt
     if (e != cudaSuccess) return e;
     const int warps = P.gamma + 1 < kFoldWarps ? P.gamma + 1 : kFoldWarps;
     const bool many = (long long)P.runs * P.k > kMergeFew || P.k > kGroupsUpTo;
+    if (P.gamma + 1 > kFoldTurns * kFoldWarps) {
+        const unsigned ctas = (unsigned)(((long long)P.B * (P.gamma + 1) + kFoldWarps - 1) / kFoldWarps);
+        const cudaError_t r = launch_pdl(many ? topk_rows_kernel<true> : topk_rows_kernel<false>, ctas, 32u * kFoldWarps, stream, P,
+                                         kFoldWarps * sizeof(MergeShared));
+        return r != cudaSuccess ? r : launch_pdl(topk_first_kernel, ((unsigned)P.B + kWarps - 1) / kWarps, kThreads, stream, P);
+    }
     const bool waves = (long long)P.B * warps > 148 * kFoldWarps;
     return launch_pdl(many ? topk_fold_kernel<true, 1> : waves ? topk_fold_kernel<false, 2> : topk_fold_kernel<false, 1>, (unsigned)P.B,
                       32u * (unsigned)warps, stream, P, (size_t)warps * sizeof(MergeShared));

@@ -26,6 +26,7 @@ struct TopkParams {
     int run_vecs;                     // 16-byte vectors per run
     // workspace (no initial contents needed: every word that is read has been written by the call)
     unsigned long long *lists;        // [rows, runs, k] the run's k best keys, best first, 0 where it has fewer
+    uint32_t *verdict;                // [rows] many positions only: the row's verdict
 };
 
 size_t topk_workspace_bytes(int B, int gamma, int V, int k);

@@ -85,3 +85,19 @@ def test_rows_of_many_runs(B, oracle_mod, V, k):
     tl[2][:] = np.linspace(-3.0, 9.0, V, dtype=np.float32)
     tl[3][:, np.arange(V) % 9001 != 0] = -np.inf
     compare_topk(B, oracle_mod, d, w.temperature, k)
+
+
+@pytest.mark.parametrize("Bn,gamma,V,k", [(3, 31, 9000, 10), (3, 32, 9000, 10), (2, 63, 20000, 32), (9, 64, 300, 5), (2, 200, 70000, 12),
+                                          (1, 1000, 64, 13)])
+def test_many_positions(B, oracle_mod, Bn, gamma, V, k):
+    """Positions in turns and, beyond two turns, judged by a kernel of their own: rejections at any position, rows without a
+    distribution before and after them, draft tokens out of range."""
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype="f32", temperature=0.9, sigma_d=0.2, seed=k)
+    d = di.generate_topk(w, k, threads=16)
+    d["uniforms"][0] = 0.0  # accepted wherever the token is in the support
+    for i in range(1, Bn):
+        d["uniforms"][i, : gamma * i // Bn] = 0.0
+        d["uniforms"][i, gamma * i // Bn] = 1.0
+    d["target_logits"][0, gamma // 2, 7] = np.nan
+    d["draft_tokens"][-1, -1] = V
+    compare_topk(B, oracle_mod, d, w.temperature, k)
