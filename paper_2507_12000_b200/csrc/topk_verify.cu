@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(32 * kFoldWarps, kCtas) topk_fold_kernel(const
 
 // The same in two steps for many positions, which the kernel above takes in turns: a warp per row leaves the row's verdict and, in
 // the place of its first list, its merged keys; a warp per sequence finds row n.  B = 2 gamma = 200 V = 32000 k = 10: the edge call
-// PLACE_E us, in turns 53.6; gamma = 64 PLACE_F and 22.7; gamma = 31 PLACE_G and 12.6.
+// 17.0 us, in turns 54.5; gamma = 64 12.0 and 21.7; gamma = 31, two turns, 11.8.
 template <bool kMany>
 __global__ void __launch_bounds__(32 * kFoldWarps, 1) topk_rows_kernel(const __grid_constant__ TopkParams P)
 {
