@@ -64,6 +64,39 @@ __device__ __forceinline__ void row_total(Part part, int runs, int sub, bool liv
     S = s;
 }
 
+// The same by a whole warp, for rows of hundreds of runs: 256 words on their way at a time.
+constexpr int kFoldWide = 64;  // runs beyond which it is used, by kernels of their own (edge_verify.cu: launch_edge)
+template <class Part>
+__device__ __forceinline__ void row_total_wide(Part part, int runs, float &R, double &S, bool &missing)
+{
+    const int lane = threadIdx.x & 31;
+    float top = DSSD_NEG_INF;
+    double s = 0.0;
+    missing = false;
+    auto all = [&](auto use) {
+        for (int k0 = lane; k0 < runs; k0 += 256) {
+            unsigned long long x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = k0 + 32 * u < runs ? part(k0 + 32 * u) : 0ull;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) use(x[u]);
+        }
+    };
+    all([&](unsigned long long x) {
+        missing |= x == kNoPartial;
+        if (__uint_as_float((unsigned)(x >> 32)) > 0.f) top = fmaxf(top, __uint_as_float((unsigned)x));
+    });
+    top = warp_max(top);
+    all([&](unsigned long long x) {
+        const float v = __uint_as_float((unsigned)(x >> 32));
+        if (v > 0.f && v < INFINITY) s += scale_pow2((double)v, __uint_as_float((unsigned)x) - top);
+        else if (v != 0.f) s += (double)v;
+    });
+    S = warp_sum(s);
+    R = top;
+    missing = __any_sync(0xffffffffu, missing);
+}
+
 // What the acceptance test of a position takes besides its row's sum.
 struct Drafted {
     int x;          // the drafted token
@@ -73,7 +106,7 @@ struct Drafted {
 // Run by all kThreads threads of a CTA; the results are in `sh` (n, ref2, invS) when it returns.
 // `writer`: this CTA writes the sequence's accept_len, flags, lse, p_tok and `ready`.
 // part(i, k) gives the partial sum of run k of row i of the sequence, drafted(i) what belongs to position i.
-template <class Part, class Draft>
+template <bool kWide, class Part, class Draft>
 __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh, Part part, Draft drafted)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -86,7 +119,19 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
         const bool live = i <= P.gamma;
         Drafted d = {-1, 0.f, 0.f, 0.f};
         if (warp == 0 && i < P.gamma) d = drafted(i);
-        {
+        if (kWide) {
+            for (int w = warp; w < kFoldRows && base + w <= P.gamma; w += kWarps) {
+                float R;
+                double S;
+                bool missing;
+                row_total_wide([&](int k) { return part(base + w, k); }, P.runs, R, S, missing);
+                if (lane == 0) {
+                    sh.R[w] = R;
+                    sh.S[w] = S;
+                    sh.missing[w] = missing;
+                }
+            }
+        } else {
             const int r = base + tid / kFoldLanes;
             float R;
             double S;
@@ -137,10 +182,11 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
 
 // The same with what the log-sum-exp kernel left in the workspace: one round trip to L2 for the partial sums,
 // the drafted tokens' logits and the caller's arrays.
+template <bool kWide>
 __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh)
 {
     const long long row0 = b * (P.gamma + 1);
-    fold_sequence(P, b, writer, sh, [&](int i, int k) { return ld_after(P.part + (size_t)(row0 + i) * P.runs + k); },
+    fold_sequence<kWide>(P, b, writer, sh, [&](int i, int k) { return ld_after(P.part + (size_t)(row0 + i) * P.runs + k); },
                   [&](int i) {
                       const size_t di = (size_t)b * P.gamma + i;
                       Drafted d;

@@ -278,12 +278,15 @@ __global__ void __launch_bounds__(kLseThreads, 8) edge_lse_kernel(const __grid_c
 
 // ---- emission (emit.cuh) ----------------------------------------------------------------------
 
+// kWide: more than kFoldWide runs per row (B = 1 gamma = 2 float32, the edge call, eight threads per row / a warp: V = 16777216
+// 189.6 / 67.8 us, V = 67108864 471 / 228, V = 1048576 18.8 / 9.7, V = 300000 11.4 / 8.5)
+template <bool kWide>
 __global__ void __launch_bounds__(kThreads) edge_fold_kernel(const __grid_constant__ EdgeParams P)
 {
     __shared__ FoldShared sh;
     pdl_wait();
     pdl_trigger();
-    fold_sequence(P, blockIdx.x, true, sh);
+    fold_sequence<kWide>(P, blockIdx.x, true, sh);
 }
 
 // Bound by HBM: reads and writes mixed, 234 MB at B = 256 V = 151936 in 36.5 us.
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 4) edge_emit_kernel(const __grid_con
     float ref2, invS;
     if (kFold) {
         __shared__ FoldShared sh;
-        fold_sequence(P, b, tile == 0, sh);
+        fold_sequence<false>(P, b, tile == 0, sh);
         n = sh.n;
         ref2 = sh.ref2;
         invS = sh.invS;
@@ -499,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, kDraw == 2 ? 2 : 4) edge_cluster_ker
     } else {
         __syncthreads();
     }
-    fold_sequence(P, b, rank == 0, sh, [&](int i, int k) { return s_part[i * P.runs + k]; }, [&](int i) { return s_draft[i]; });
+    fold_sequence<false>(P, b, rank == 0, sh, [&](int i, int k) { return s_part[i * P.runs + k]; }, [&](int i) { return s_draft[i]; });
     const int n = sh.n;
     if (kDraw) {
         __shared__ DrawShared sd;
@@ -518,12 +521,14 @@ __global__ void __launch_bounds__(kThreads, kDraw == 2 ? 2 : 4) edge_cluster_ker
     else if (P.p_row) emit_pieces<DT, kShift>(rowp, P.p_row + (size_t)b * P.V, P.V, g, n_warps, P.c1, sh.ref2, sh.invS);
 }
 
-// One shard of the vocabulary: the rows' sums and the drafted tokens' logits go out as they are.
+// One shard of the vocabulary: the rows' sums and the drafted tokens' logits go out as they are.  kWide: a warp per row.
+template <bool kWide>
 __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_constant__ EdgeParams P)
 {
+    constexpr int kLanes = kWide ? 32 : kFoldLanes;
     const long long rows = (long long)P.B * (P.gamma + 1);
-    const long long row = (long long)blockIdx.x * kFoldRows + threadIdx.x / kFoldLanes;
-    const int sub = threadIdx.x % kFoldLanes;
+    const long long row = (long long)blockIdx.x * (kThreads / kLanes) + threadIdx.x / kLanes;
+    const int sub = threadIdx.x % kLanes;
     const bool live = row < rows;
     pdl_wait();
     pdl_trigger();
@@ -538,7 +543,9 @@ __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_con
     float R;
     double S;
     bool missing;
-    row_total([&](int k) { return ld_after(P.part + (size_t)row * P.runs + k); }, P.runs, sub, live, R, S, missing);
+    auto part = [&](int k) { return ld_after(P.part + (size_t)row * P.runs + k); };
+    if (kWide) row_total_wide(part, live ? P.runs : 0, R, S, missing);
+    else row_total(part, P.runs, sub, live, R, S, missing);
     if (live && sub == 0) {
         P.shard_ref[row] = R == DSSD_NEG_INF ? 0.f : R;
         P.shard_sum[row] = missing || S != S ? (double)__int_as_float(0x7fc00000) : S;
@@ -741,15 +748,19 @@ cudaError_t launch_edge(EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
     cudaError_t e = launch_pdl(edge_lse_kernel<DT>, lse_ctas, kLseThreads, stream, P);
     if (e != cudaSuccess) return e;
     const unsigned long long rows = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1);
-    if (P.shard_sum) return launch_pdl(edge_partial_kernel, (unsigned)((rows + kFoldRows - 1) / kFoldRows), kThreads, stream, P);
+    const bool wide = P.runs > kFoldWide;
+    if (P.shard_sum)
+        return wide ? launch_pdl(edge_partial_kernel<true>, (unsigned)((rows + kWarps - 1) / kWarps), kThreads, stream, P)
+                    : launch_pdl(edge_partial_kernel<false>, (unsigned)((rows + kFoldRows - 1) / kFoldRows), kThreads, stream, P);
     const bool emit = P.p_row || P.p_row16;
     const bool aligned = outputs_aligned<DT>(P);
     P.emit_tiles = emit_tiles(P.V, aligned);
     const unsigned long long ctas = (unsigned long long)P.B * (unsigned long long)P.emit_tiles;
     if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
-    const bool fold = emit && ctas <= kEmitFoldCtas;
+    const bool fold = emit && ctas <= kEmitFoldCtas && !wide;
     if (!fold) {
-        e = launch_pdl(edge_fold_kernel, (unsigned)P.B, kThreads, stream, P);
+        e = wide ? launch_pdl(edge_fold_kernel<true>, (unsigned)P.B, kThreads, stream, P)
+                 : launch_pdl(edge_fold_kernel<false>, (unsigned)P.B, kThreads, stream, P);
         if (e != cudaSuccess || !emit) return e;
     }
     return aligned ? launch_emit<DT, false>(P, (unsigned)ctas, fold, stream) : launch_emit<DT, true>(P, (unsigned)ctas, fold, stream);

@@ -34,7 +34,7 @@ def B():
 
 
 @pytest.mark.parametrize("dtype,Bn,gamma,V,drop_row", [("bf16", 200, 3, 9001, 417), ("f32", 40, 8, 70001, 0),
-                                                        ("bf16", 7, 2, 300000, 20)])
+                                                        ("bf16", 7, 2, 300000, 20), ("f32", 3, 2, 400001, 4)])
 def test_a_partial_sum_that_never_arrives(B, dtype, Bn, gamma, V, drop_row):
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.8, seed=V)
     g = to_device(di.generate(w, threads=4))

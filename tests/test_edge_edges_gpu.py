@@ -31,6 +31,16 @@ def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
     compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
 
 
+# Rows of more runs than eight threads add up in two looks (64 of 4096 float32 or 8192 bf16 logits): a warp per row in the fold, more
+# rows than warps, more than 32 positions.
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [
+    ("f32", 1, 2, 262144), ("f32", 1, 2, 262148), ("f32", 2, 40, 300001), ("bf16", 3, 9, 540001), ("f32", 1, 1, 1100003), ("bf16", 1, 1, 5000001),
+])
+def test_rows_of_many_runs(B, oracle_mod, dtype, Bn, gamma, V):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.3, zipf=True, seed=V + Bn)
+    compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
+
+
 # One launch for small sequences: vocabularies at the edges of a warp's segment (1024 float32 or 2048 bf16 logits) and
 # of what it emits (512 entries), one CTA per sequence, clusters of two, eight, nine and sixteen, the last
 # batch of a wave, the most positions, and the sizes next to the limits where the separate kernels take over.
