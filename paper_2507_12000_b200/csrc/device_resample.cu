@@ -139,8 +139,18 @@ __device__ __forceinline__ int walk_chunk(const Pick &pk, const RV &row, const f
     return tok;
 }
 
+// The pick among n_sub chunks; kLong: there are many more than a warp's lanes keep.  (A draw of V = 300000, 293 sums: 7.5 us without,
+// 7.9 with; V = 1048576, 1024 sums: 10.4 and 8.7.)
+constexpr int kLongSums = 512;
+template <bool kLong, class Sum, class Target>
+__device__ __forceinline__ Pick pick_of(const LaneSums &L, Sum sum, bool beyond, Target target)
+{
+    if constexpr (kLong) return pick_long(L, sum, beyond, target);
+    else return pick_chunk(L, sum, beyond, target);
+}
+
 // The draw for sequence b by one CTA; q == nullptr means r = p.
-template <bool kShift, typename RV>
+template <bool kLong, bool kShift, typename RV>
 __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const float *q, unsigned fl, float u, LaneSums &L,
                      WalkShared &sh)
 {
@@ -149,7 +159,7 @@ __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const fl
     double *cs = P.chunk_sum + (size_t)b * P.n_sub;
     auto sum = [&](int c) { return ld_after(cs + c); };
     auto target = [&](double Z) { return (double)u * Z; };
-    Pick pk = pick_chunk(L, sum, false, target);
+    Pick pk = pick_of<kLong>(L, sum, false, target);
     if (!pk.ok && !pk.late && q) {
         // The residual has no mass (p == q): draw from p instead.  Rare, so its sums are formed here, a warp
         // at each, where the others were.
@@ -164,7 +174,7 @@ __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const fl
         }
         __syncthreads();
         load_sums(L, P.n_sub, sum);
-        pk = pick_chunk(L, sum, false, target);
+        pk = pick_of<kLong>(L, sum, false, target);
     }
     int tok = -1;
     if (pk.ok && !pk.late) {
@@ -225,8 +235,9 @@ __global__ void __launch_bounds__(kThreads, kShift ? 4 : 5) resample_mass_kernel
 
 // One CTA per sequence.  Bound by latency: one round trip for the sums, one for the chunk, and the float64
 // additions that depend on one another (4 us at B = 256; a chunk of 4096 entries instead of 1024 took 5.9,
-// one warp per sequence with 32 entries per lane 6.0).
-template <bool kShift, typename RV>
+// one warp per sequence with 32 entries per lane 6.0).  kLong: rows of many sums (the draw of B = 1 float32, V = 16777216
+// 107 to 124 us where every lane added and searched its share one load after the other, now 37 to 39; V = 67108864 298 to 334, now 124).
+template <bool kLong, bool kShift, typename RV>
 __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __grid_constant__ ResampleParams P)
 {
     __shared__ WalkShared sh;
@@ -252,7 +263,7 @@ __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __gri
     } else {
         const RV row = RV::make(P, b, n);
         const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
-        draw<kShift>(P, b, row, q, q ? 0u : DSSD_RS_FLAG_BONUS, u, L, sh);
+        draw<kLong, kShift>(P, b, row, q, q ? 0u : DSSD_RS_FLAG_BONUS, u, L, sh);
     }
 }
 
@@ -427,8 +438,8 @@ __global__ void __launch_bounds__(kThreads) shard_total_kernel(const __grid_cons
     }
 }
 
-// one CTA per sequence
-template <bool kShift>
+// one CTA per sequence; kLong: slices of many chunks
+template <bool kLong, bool kShift>
 __global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_constant__ ShardResampleParams P)
 {
     __shared__ WalkShared sh;
@@ -493,7 +504,7 @@ __global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_c
             // this shard holds the target: the chunk first, then the walk inside it
             auto sum = [&](int c) { return ld_after(cs + 2 * c + col); };
             if (col) load_sums(L, P.n_sub, sum);
-            const Pick pk = pick_chunk(L, sum, beyond, [&](double) { return t - before; });
+            const Pick pk = pick_of<kLong>(L, sum, beyond, [&](double) { return t - before; });
             const RowF32 row = shard_row(P, b);
             const float *q = (col == 0 && n < P.gamma) ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.q_stride : nullptr;
             double base = pk.base;
@@ -513,11 +524,11 @@ __global__ void __launch_bounds__(kDrawThreads) shard_draw_kernel(const __grid_c
 
 size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base)
 {
-    // one sum per chunk; batches whose sums would take more than the built-in scratch of
-    // dssd_device_resample_static keep one per two chunks or per tile, which the draw then looks at in turn
+    // one sum per chunk; rows of more than 1024 chunks, and batches whose sums would take more than the built-in scratch of
+    // dssd_device_resample_static, keep one per two chunks or per tile, which the draw then looks at in turn
     int rows = 1;
     auto sums = [&]() { return ((size_t)V + (size_t)(rows * kSub) - 1) / (size_t)(rows * kSub); };
-    while (rows < kRows && (size_t)B * sums() * sizeof(double) > (size_t)DSSD_STATIC_SCRATCH_BYTES) rows *= 2;
+    while (rows < kRows && (sums() > 1024 || (size_t)B * sums() * sizeof(double) > (size_t)DSSD_STATIC_SCRATCH_BYTES)) rows *= 2;
     const size_t n_sub = sums();
     if (P) {
         P->chunk_sum = reinterpret_cast<double *>(base);
@@ -546,7 +557,9 @@ cudaError_t launch_resample_as(const ResampleParams &P, unsigned grid, cudaStrea
         return launch_pdl(resample_cluster_kernel<kShift, RV>, (unsigned)(P.B * P.n_ctas), (unsigned)P.cluster_threads, stream, P,
                           0, (unsigned)P.n_ctas);
     const cudaError_t e = launch_pdl(resample_mass_kernel<kShift, RV>, grid, kThreads, stream, P);
-    return e != cudaSuccess ? e : launch_pdl(resample_draw_kernel<kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P);
+    if (e != cudaSuccess) return e;
+    return P.n_sub > kLongSums ? launch_pdl(resample_draw_kernel<true, kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P)
+                                : launch_pdl(resample_draw_kernel<false, kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P);
 }
 template <typename RV>
 cudaError_t launch_resample(const ResampleParams &P, unsigned grid, cudaStream_t stream)
@@ -621,8 +634,11 @@ cudaError_t shard_draw_launch(ShardResampleParams &P, const void *workspace, cud
 {
     P.n_sub = (int)(((size_t)P.V + kSub - 1) / kSub);
     P.chunk_sum = const_cast<double *>(static_cast<const double *>(workspace));
-    return shard_aligned(P) ? launch_pdl(shard_draw_kernel<false>, (unsigned)P.B, kDrawThreads, stream, P)
-                            : launch_pdl(shard_draw_kernel<true>, (unsigned)P.B, kDrawThreads, stream, P);
+    if (P.n_sub > kLongSums)
+        return shard_aligned(P) ? launch_pdl(shard_draw_kernel<true, false>, (unsigned)P.B, kDrawThreads, stream, P)
+                                : launch_pdl(shard_draw_kernel<true, true>, (unsigned)P.B, kDrawThreads, stream, P);
+    return shard_aligned(P) ? launch_pdl(shard_draw_kernel<false, false>, (unsigned)P.B, kDrawThreads, stream, P)
+                            : launch_pdl(shard_draw_kernel<false, true>, (unsigned)P.B, kDrawThreads, stream, P);
 }
 
 }  // namespace dssd

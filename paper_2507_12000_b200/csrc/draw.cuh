@@ -265,6 +265,59 @@ __device__ __forceinline__ Pick pick_chunk(const LaneSums &L, Sum sum, bool beyo
     return pk;
 }
 
+// The same for more than 32 kKeep chunks (vocabularies beyond 262144): the lane whose share holds the target is found first, and
+// then its share is what all lanes look at, as often as it takes.  load_sums has loaded the first chunks of every share.
+template <class Sum, class Target>
+__device__ __forceinline__ Pick pick_long(LaneSums L, Sum sum, bool beyond, Target target)
+{
+    const int lane = threadIdx.x & 31;
+    Pick pk;
+    double base = 0.0;  // mass before the chunks that are looked at
+    for (bool first = true;; first = false) {
+        double s = 0.0;
+        bool late = false;
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            s += L.m[k];
+            late |= missing(L.m[k]);
+        }
+        for (int c = L.c0 + kKeep; c < L.c1; c += kKeep) {
+            double x[kKeep];
+#pragma unroll
+            for (int k = 0; k < kKeep; ++k) x[k] = c + k < L.c1 ? sum(c + k) : 0.0;
+#pragma unroll
+            for (int k = 0; k < kKeep; ++k) {
+                s += x[k];
+                late |= missing(x[k]);
+            }
+        }
+        const double incl = warp_scan(s);
+        const double up = __shfl_up_sync(0xffffffffu, incl, 1);
+        const double excl = lane ? base + up : base;
+        if (first) {
+            const double Z = shfl_f64(incl, 31);
+            pk.late = __any_sync(0xffffffffu, late);
+            pk.ok = (Z > 0.0) && (Z < INFINITY);
+            pk.target = target(Z);
+        }
+        const unsigned cross = beyond ? 0u : __ballot_sync(0xffffffffu, s > 0.0 && base + incl > pk.target);
+        const unsigned mass = __ballot_sync(0xffffffffu, s > 0.0);
+        beyond |= cross == 0;  // (in a later look: by rounding; the share's last mass then)
+        if (first) pk.beyond = beyond;
+        const int owner = cross ? __ffs(cross) - 1 : mass ? 31 - __clz(mass) : 0;
+        const int at = __shfl_sync(0xffffffffu, L.c0, owner), n = __shfl_sync(0xffffffffu, L.c1, owner) - at;
+        base = shfl_f64(excl, owner);
+        if (n <= 1) {
+            pk.chunk = at;
+            pk.base = base;
+            return pk;
+        }
+        load_sums(L, n, [&](int c) { return sum(at + c); });
+        L.c0 += at;
+        L.c1 += at;
+    }
+}
+
 // The draw inside a segment of 512 entries, by a warp: of segment g's entries in r (segment_residuals) the first whose
 // running mass exceeds the target, else (rounding, or pk.beyond) the last with mass; -1: none has.
 __device__ __forceinline__ int walk_segment(const Pick &pk, const double (&r)[16], int g)

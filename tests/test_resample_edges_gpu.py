@@ -23,6 +23,7 @@ def B():
     (7, 1, 65536, False), (4, 2, 65537, False), (200, 1, 900, False), (201, 1, 900, True), (5, 1, 50257, True), (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
     (600, 1, 4096, False), (601, 1, 4096, True), (1200, 1, 2047, True), (1201, 1, 2047, False), (2400, 1, 1024, False), (2401, 1, 1024, False),
     (6, 2, 9001, False), (6, 3, 9002, True), (7, 2, 9003, True), (6, 2, 9003, False), (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True), (32768, 1, 4097, False), (32769, 1, 8193, True),
+    (3, 1, 1 << 19, False), (3, 1, (1 << 19) + 1, False), (4, 1, 1 << 20, False), (4, 1, (1 << 20) + 1, True), (3, 1, (1 << 21) + 3, False), (3, 1, 5000001, False),
 ])
 def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
     gen = torch.Generator(device="cuda").manual_seed(Bn + V)
@@ -53,7 +54,7 @@ def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
     assert (out["flags"].cpu().numpy().astype(np.uint32) == ref["flags"]).all()
 
 
-@pytest.mark.parametrize("Bn,V", [(5, 3000), (3, 20011), (40, 70001)])
+@pytest.mark.parametrize("Bn,V", [(5, 3000), (3, 20011), (40, 70001), (4, 300001), (4, 1100001)])
 def test_fallback_and_invalid_lengths(B, oracle_mod, Bn, V):
     """No residual mass (p == q): drawn from p; lengths outside [0, gamma] and rows without mass: token -1; one
     cluster per sequence and the two-kernel path."""
