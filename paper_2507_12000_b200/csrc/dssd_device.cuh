@@ -50,9 +50,18 @@ __device__ __forceinline__ unsigned cluster_rank()
     return r;
 }
 // every thread of every CTA of the cluster arrives once per phase; what was stored before an arrival, in
-// any CTA's shared memory, is visible after the wait
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// any CTA's shared memory, is visible after the wait.  Both want the warp's threads together, which after divergent code is
+// not to be had without saying so.
+__device__ __forceinline__ void cluster_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // stores to the variable at the same place in the shared memory of the cluster's CTA `rank`
 __device__ __forceinline__ uint32_t cluster_addr(const void *p, unsigned rank)
 {
