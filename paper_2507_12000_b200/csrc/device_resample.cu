@@ -149,21 +149,6 @@ __device__ __forceinline__ Pick pick_of(const LaneSums &L, Sum sum, bool beyond,
     else return pick_chunk(L, sum, beyond, target);
 }
 
-// This thread's part of the sum of p over the chunk that starts at entry `base`; all loads are requested before the first is used.
-template <bool kShift, typename RV>
-__device__ __forceinline__ double plain_mass(const RV &row, int V, long long base)
-{
-    WarpQuads<typename RV::Q, kSub / 128, kShift> a;
-    a.load(row.row, V, base, RV::kFill);
-    double acc = 0.0;
-#pragma unroll
-    for (int u = 0; u < kSub / 128; ++u) {
-        const float4 x = row.quad(a.at(u));
-        acc += ((double)x.x + (double)x.y) + ((double)x.z + (double)x.w);
-    }
-    return acc;
-}
-
 // The draw for sequence b by one CTA; q == nullptr means r = p.
 template <bool kLong, bool kShift, typename RV>
 __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const float *q, unsigned fl, float u, LaneSums &L,
@@ -182,8 +167,8 @@ __device__ void draw(const ResampleParams &P, int64_t b, const RV &row, const fl
         fl |= DSSD_RS_FLAG_FALLBACK;
         __syncthreads();  // every warp has read the sums that are replaced now
         for (int c = tid >> 5; c < P.n_sub; c += kDrawWarps) {
-            double tot = 0.0;
-            for (int e = 0; e < width; e += kSub) tot += plain_mass<kShift>(row, P.V, (long long)c * width + e);
+            double tot = 0.0, none;
+            for (int e = 0; e < width; e += 512) tot += share_mass<false, false, kShift>(row, q, P.V, (long long)c * width + e, none);
             tot = warp_sum(tot);
             if (lane == 0) cs[c] = tot;
         }
