@@ -128,31 +128,6 @@ struct Vec<DSSD_BF16> {
     }
 };
 
-// A CTA's run: the vectors v0 .. v1 - 1 of its row, which start at the row's first 16-byte boundary (entry idx0), and, in the
-// row's first and last run, the entries before and after the vectors; entries e0 .. e1 - 1 in all.
-template <int DT>
-struct Run {
-    const char *rowp;
-    const uint4 *src;
-    int run, idx0, nvec, v0, v1;
-    __device__ __forceinline__ explicit Run(const TopkParams &P)
-    {
-        const unsigned row = blockIdx.x / (unsigned)P.runs;
-        run = (int)(blockIdx.x - row * (unsigned)P.runs);
-        rowp = static_cast<const char *>(P.logits) + (size_t)row * (size_t)P.row_stride * Vec<DT>::kEsz;
-        const long long rowbytes = (long long)P.V * Vec<DT>::kEsz;
-        int head = (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(rowp) & 15u)) & 15u);
-        if (head > rowbytes) head = (int)rowbytes;
-        nvec = (int)((rowbytes - head) >> 4);
-        v0 = min(nvec, run * P.run_vecs);
-        v1 = run + 1 == P.runs ? nvec : min(nvec, v0 + P.run_vecs);
-        src = reinterpret_cast<const uint4 *>(rowp + head);
-        idx0 = head / Vec<DT>::kEsz;
-    }
-    __device__ __forceinline__ int e0() const { return run == 0 ? 0 : idx0 + v0 * Vec<DT>::E; }
-    __device__ __forceinline__ int e1(const TopkParams &P) const { return run + 1 == P.runs ? P.V : idx0 + v1 * Vec<DT>::E; }
-};
-
 struct SelectShared {
     unsigned long long key[kCand];
     unsigned long long top[32];
@@ -234,14 +209,11 @@ __device__ __noinline__ int refine(SelectShared &sh, int m, float top, int k)
 // vector by vector in index order.  Two passes over the run at most, from L2.  B = 256 gamma = 4 V = 32000 bf16,
 // nine tenths masked, k = 10: 61 us, entry by entry (select_slowly) 791; ascending rows 267 and 6592.  false: more are above t than fit.
 template <int DT>
-__device__ __noinline__ bool select_again(SelectShared &sh, const TopkParams &P, float top)
+__device__ __noinline__ bool select_again(SelectShared &sh, const char *rowp, int idx0, int v0, int v1, int e0, int e1, float top, int k)
 {
     constexpr int E = Vec<DT>::E;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = P.k;
-    const Run<DT> R(P);
-    const char *rowp = R.rowp;
-    const uint4 *src = R.src;
-    const int idx0 = R.idx0, v0 = R.v0, v1 = R.v1, e0 = R.e0(), e1 = R.e1(P);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint4 *src = reinterpret_cast<const uint4 *>(rowp + (size_t)idx0 * Vec<DT>::kEsz);
     const int ev0 = idx0 + v0 * E, ev1 = idx0 + v1 * E;  // the entries in vectors
     const uint32_t mine = ord(top == top ? top : DSSD_NEG_INF);
     int rank = 0;
@@ -310,12 +282,9 @@ __device__ __noinline__ bool select_again(SelectShared &sh, const TopkParams &P,
 
 // The run again, where that did not do either: entry by entry, at most one per thread and step.
 template <int DT>
-__device__ __noinline__ void select_slowly(SelectShared &sh, const TopkParams &P)
+__device__ __noinline__ void select_slowly(SelectShared &sh, const char *rowp, int e0, int e1, int k)
 {
-    const int tid = threadIdx.x, k = P.k;
-    const Run<DT> R(P);
-    const char *rowp = R.rowp;
-    const int e0 = R.e0(), e1 = R.e1(P);
+    const int tid = threadIdx.x;
     unsigned long long floor = 0ull;  // keys up to here are not among the k best
     __syncthreads();
     if (tid == 0) sh.count = 0;
@@ -343,17 +312,25 @@ __device__ __noinline__ void select_slowly(SelectShared &sh, const TopkParams &P
 // replaces (a ring per CTA, one selection warp that inserted candidates one by one, rows judged in the
 // same warp) took 79 us for this and the fold together, and 18.8 us at B = 1 gamma = 8 V = 50272 where
 // both kernels now take 7.7.  Ten CTAs per SM (48 registers); eight 61.9, twelve 65 us (spills).
-// One CTA per (row, run).
+// One CTA per (row, run).  A row's vectors start at
+// its first 16-byte boundary; the entries before it belong to the first run, those after the last whole
+// vector to the last run.
 template <int DT>
 __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __grid_constant__ TopkParams P)
 {
-    constexpr int E = Vec<DT>::E;
+    constexpr int E = Vec<DT>::E, kEsz = Vec<DT>::kEsz;
     __shared__ SelectShared sh;
     const int tid = threadIdx.x, lane = tid & 31, k = P.k;
-    const Run<DT> R(P);
-    const char *rowp = R.rowp;
-    const uint4 *src = R.src;
-    const int run = R.run, nvec = R.nvec, v0 = R.v0, v1 = R.v1, idx0 = R.idx0;
+    const unsigned row = blockIdx.x / (unsigned)P.runs;
+    const int run = (int)(blockIdx.x - row * (unsigned)P.runs);
+    const char *rowp = static_cast<const char *>(P.logits) + (size_t)row * (size_t)P.row_stride * kEsz;
+    const long long rowbytes = (long long)P.V * kEsz;
+    int head = (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(rowp) & 15u)) & 15u);
+    if (head > rowbytes) head = (int)rowbytes;
+    const int nvec = (int)((rowbytes - head) >> 4);
+    const int v0 = min(nvec, run * P.run_vecs), v1 = run + 1 == P.runs ? nvec : min(nvec, v0 + P.run_vecs);
+    const uint4 *src = reinterpret_cast<const uint4 *>(rowp + head);
+    const int idx0 = head / kEsz;  // index of the first vector's first entry
     if (tid == 0) {
         sh.count = 0;
         sh.bad = 0;
@@ -442,7 +419,8 @@ __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __gr
     __syncthreads();
     int m = (int)sh.count;
     if (m > kCand) {
-        if (!select_again<DT>(sh, P, top)) select_slowly<DT>(sh, P);
+        const int e0 = run == 0 ? 0 : idx0 + v0 * E, e1 = run + 1 == P.runs ? P.V : idx0 + v1 * E;
+        if (!select_again<DT>(sh, rowp, idx0, v0, v1, e0, e1, top, k)) select_slowly<DT>(sh, rowp, e0, e1, k);
         m = (int)sh.count;
     }
     if (m > kRefine) m = refine(sh, m, top, k);
