@@ -65,7 +65,7 @@ def _kernel_hash_topk() -> str:
 
 def _kernel_hash() -> str:
     h = hashlib.sha256()
-    for f in ("edge_verify.cu", "edge_verify.h", "edge_fold.cuh", "emit.cuh", "edge_judge.cuh", "dssd_device.cuh"):
+    for f in ("edge_verify.cu", "edge_verify.h", "edge_fold.cuh", "emit.cuh", "quads.cuh", "draw.cuh", "edge_judge.cuh", "dssd_device.cuh"):
         with open(os.path.join(ROOT, "paper_2507_12000_b200", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -76,13 +76,14 @@ typedef enum {
 #define DSSD_EDGE_FLAG_BAD_TOKEN 1u /* some x_i outside [0, V): that position is rejected        */
 #define DSSD_EDGE_FLAG_NONFINITE 2u /* some row of the sequence has no finite log-sum-exp (NaN,  \
                                        +inf, or all -inf): that position is rejected, its row is NaN */
-#define DSSD_EDGE_FLAG_TIMEOUT 4u   /* internal wait ran out; p_row of this sequence was not written */
+#define DSSD_EDGE_FLAG_TIMEOUT 4u   /* a partial sum is missing; p_row of this sequence was not written.  Nothing in the    \
+                                       present kernels waits for a sum, so only the test hooks bring this about */
 
 /* flags written by dssd_device_resample, one word per sequence */
 #define DSSD_RS_FLAG_BONUS 1u    /* n == gamma: token drawn from P_{gamma+1}                       */
 #define DSSD_RS_FLAG_FALLBACK 2u /* residual mass sum max(0, p - q) <= 0: token drawn from p instead */
 #define DSSD_RS_FLAG_INVALID 4u  /* no positive mass at all, or n outside [0, gamma]: token = -1    */
-#define DSSD_RS_FLAG_TIMEOUT 8u  /* internal wait ran out: token = -1 (set together with INVALID)    */
+#define DSSD_RS_FLAG_TIMEOUT 8u  /* a chunk sum is missing: token = -1 (set together with INVALID); as above, test hooks only */
 
 /* Human-readable name of a status (static storage, never NULL). */
 const char *dssd_status_string(int status);
@@ -115,11 +116,13 @@ size_t dssd_edge_verify_workspace_bytes(int B, int gamma, int V);
  * dssd_device_resample can draw the bonus token; a caller that wants the paper's byte saving
  * simply does not transmit it.
  *
- * Arithmetic: with c1 = float32(log2(e) / T), every term 2^(l_v * c1 - ref) is formed in float32
- * (one fused multiply-add, one ex2 of relative error 2^-22) and added up in float32 per lane, at
- * most a few hundred terms per accumulator; the per-lane sums are combined in float64 by exact
- * power-of-two scaling.  p_i(x_i) = 2^(l_x * c1 - ref) / S and the test u * q < p are evaluated in
- * float64.  The result is within about 1e-6 relative of the exact softmax as long as
+ * Arithmetic: with c1 = float32(log2(e) / T), every term 2^(l_v * c1 - ref) is formed in float32: one fused
+ * multiply-add and one ex2 of relative error 2^-22, or, for an eighth of a bf16 row's terms, a polynomial of relative
+ * error 8e-8.  Terms are added in float32 per thread (at most 32 to an accumulator), then per warp and per CTA, over a
+ * run of at most 64 KB of logits; the runs' sums are combined in float64.  All references are integers, so every
+ * rescaling is exact.  p_i(x_i) = 2^(l_x * c1 - ref) / S and the test u * q < p are evaluated in
+ * float64.  The result is within about 1e-6 relative of the exact softmax (rows of 151936
+ * entries with logits N(0, 1): 6e-7 at most, 1.4e-7 rms) as long as
  * |l| * log2(e) / T stays well inside the float32 range (the rounding of c1 alone contributes
  * 6e-8 * |l_v / T - E_p[l / T]| to ln p).  A logit whose scaled value lies below float32's range (a mask of the
  * type's lowest value) weighs nothing, as -inf does; rows with a scaled logit above the range, or with none inside it, are
@@ -132,7 +135,7 @@ size_t dssd_edge_verify_workspace_bytes(int B, int gamma, int V);
  * draft_q_tok    [B, gamma] float32    q_i(x_i)     (may be NULL iff gamma == 0)
  * uniforms       [B, gamma] float32    u_i in [0,1) (may be NULL iff gamma == 0)
  * temperature    T > 0, finite
- * accept_len     [B] int32     out: n in [0, gamma]; -1 (with DSSD_EDGE_FLAG_TIMEOUT) if an internal wait ran out
+ * accept_len     [B] int32     out: n in [0, gamma]; -1 (with DSSD_EDGE_FLAG_TIMEOUT) if a partial sum is missing
  * p_row          [B, V] float32 out: P_n(.)
  * p_tok          [B, gamma] float32   out, optional (NULL ok): p_i(x_i)
  * lse            [B, gamma+1] float32 out, optional (NULL ok): ln sum_v exp(l_v / T)

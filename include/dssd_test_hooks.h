@@ -36,7 +36,8 @@ dssd_status dssd_test_edge_verify_wait_runs_out(const void *target_logits, dssd_
                                                 void *cuda_stream);
 
 /*
- * dssd_device_resample in which the chunk sums of sequence `drop_seq` (0 <= drop_seq < B) are
+ * dssd_device_resample, always by its mass and its draw kernel (small batches otherwise take one launch, which hands
+ * no sum on through memory), in which the chunk sums of sequence `drop_seq` (0 <= drop_seq < B) are
  * computed but never stored.  (The sums are read after the kernel that forms them has ended, so a
  * missing one is seen at the first look; `poll_limit` is not used.)  That sequence ends with token = -1 and DSSD_RS_FLAG_TIMEOUT | DSSD_RS_FLAG_INVALID; every other
  * sequence is drawn for as usual.  Arguments otherwise as dssd_device_resample.

@@ -1,6 +1,7 @@
 """The edge half where its geometry can go wrong: vocabularies at the edges of a tile of the log-sum-exp
-kernel (4096 float32 or 8192 bf16 logits) and of the emission (8192 entries), launches at the thresholds of
-one / two / four tiles per CTA and of folding inside the emission, 32 positions and more per sequence."""
+kernel (4096 float32 or 8192 bf16 logits), of a segment of the one-launch kernel and of the emission (8192 entries), launches
+at the thresholds of one / two / four tiles per CTA and of folding inside the emission, 32 positions and more per
+sequence.  (Sequences of 33 positions and more always take the separate kernels.)"""
 import pytest
 
 import dssd_inputs as di
@@ -27,7 +28,20 @@ def B():
     ("bf16", 1600, 2, 36001), ("bf16", 5, 1, 8189), ("bf16", 5, 1, 8190), ("f32", 5, 1, 8191), ("f32", 5, 2, 16385),
 ])
 def test_round_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
+    """Whichever kernels the sizes take."""
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, zipf=V > 8, seed=V + Bn)
+    compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
+
+
+# The separate kernels: rows shorter than a vector, a tile and its neighbours, one, two and four tiles per CTA (2970 and 3003, 18975 and
+# 19008 tiles in all), folds in the emission and in a kernel of their own (592 and 593 emission CTAs).
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [
+    ("f32", 2, 32, 1), ("bf16", 2, 32, 7), ("f32", 3, 32, 4095), ("f32", 3, 32, 4096), ("f32", 3, 32, 4099), ("bf16", 3, 33, 8191),
+    ("bf16", 3, 33, 8192), ("bf16", 3, 33, 8193), ("bf16", 2, 32, 8200), ("f32", 2, 40, 16385), ("f32", 90, 32, 4096), ("f32", 91, 32, 4096),
+    ("f32", 575, 32, 4096), ("f32", 576, 32, 4096), ("bf16", 592, 32, 600), ("bf16", 593, 32, 600), ("f32", 40, 8, 70001), ("f32", 300, 4, 16384),
+])
+def test_separate_kernels_at_the_edges(B, oracle_mod, dtype, Bn, gamma, V):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.3, zipf=V > 8, seed=V + Bn)
     compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
 
 

@@ -80,8 +80,8 @@ def test_strided_and_unaligned_rows(B, oracle_mod):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_same_tokens_as_the_split_calls(B, oracle_mod, dtype):
-    """More sequences than SMs, so that the split edge call takes the streaming kernel too: the
-    fused call then forms bit-identical probabilities and must return identical results."""
+    """Sizes at which the split and the fused edge call both take the separate kernels: the fused call
+    then forms bit-identical probabilities and must return identical results."""
     w = di.custom(B=300, gamma=4, V=30011, dtype=dtype, temperature=0.7, sigma_d=0.5, seed=12)
     d = di.generate(w, threads=4)
     n, tok, g, tl = compare_dsd(B, oracle_mod, d, w.temperature)

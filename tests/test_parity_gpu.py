@@ -32,13 +32,13 @@ def test_tiny_grid(B, oracle_mod, dtype):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_tiny_vocabularies_through_the_streaming_kernel(B, oracle_mod, dtype):
-    """More sequences than SMs, so that the persistent streaming kernel (not the one-CTA-per-
-    sequence kernel of small launches) sees vocabularies around vector and stage boundaries."""
+    """More sequences than SMs, in one launch and (34 positions) in the separate kernels that stream long rows: vocabularies around
+    vector and segment boundaries."""
     seed = 900
     for V in (1, 7, 33, 1025, 16389):
-        for gamma in (0, 3):
+        for gamma in (0, 3, 33):
             seed += 1
-            w = di.custom(B=150, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=1.0, zipf=V > 8, seed=seed)
+            w = di.custom(B=150 if gamma < 33 else 20, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=1.0, zipf=V > 8, seed=seed)
             compare_round(B, oracle_mod, di.generate(w, threads=4), w.temperature, threads=4)
 
 
@@ -100,16 +100,16 @@ def test_sweep_points_sampled(B, oracle_mod):
             compare_round(B, oracle_mod, di.generate(w, threads=8), w.temperature)
 
 
-@pytest.mark.parametrize("Bn", [3, 151])  # one CTA per sequence / the streaming kernel
-def test_strided_and_unaligned_rows(B, oracle_mod, Bn):
+@pytest.mark.parametrize("Bn,gamma", [(3, 2), (151, 2), (20, 33)])  # clusters of CTAs, one CTA per sequence / separate kernels
+def test_strided_and_unaligned_rows(B, oracle_mod, Bn, gamma):
     for dtype, V, off in (("f32", 1000, 1), ("bf16", 4097, 3), ("bf16", 20000, 1), ("f32", 9001, 2)):
-        w = di.custom(B=Bn, gamma=2, V=V, dtype=dtype, seed=V)
+        w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, seed=V)
         d = di.generate(w)
         ref = oracle_mod.verify_round(d, w.temperature)
         g = to_device(d)
-        stride = V + 5
-        buf = torch.zeros(Bn * 3 * stride + 16, dtype=g["target_logits"].dtype, device="cuda")
-        view = buf[off:off + Bn * 3 * stride].view(Bn, 3, stride)[:, :, :V]
+        stride, n_rows = V + 5, gamma + 1
+        buf = torch.zeros(Bn * n_rows * stride + 16, dtype=g["target_logits"].dtype, device="cuda")
+        view = buf[off:off + Bn * n_rows * stride].view(Bn, n_rows, stride)[:, :, :V]
         view.copy_(g["target_logits"])
         assert view.data_ptr() % 16 != 0
         ev = B.dssd_edge_verify(view, g["draft_tokens"], g["draft_q_tok"], g["uniforms"], w.temperature)
@@ -176,8 +176,8 @@ def test_anomalies_are_flagged_not_faulted(B, oracle_mod):
 @pytest.mark.parametrize("Bn,V", [(6, 9000), (200, 4500)])
 def test_first_rejection_beyond_32_positions(B, oracle_mod, Bn, V):
     """Long runs of accepted positions: first rejection exactly at 31, 32, 33, at the last position, at 0,
-    and no rejection at all (u = 0 accepts whatever has p > 0; u close to 1 with q = 1 rejects), through
-    the small-launch kernel (few sequences) and the streaming kernel (many)."""
+    and no rejection at all (u = 0 accepts whatever has p > 0; u close to 1 with q = 1 rejects), in
+    the separate kernels (which more than 32 positions take), few sequences and many."""
     gamma = 45
     rejects = [31, 32, 33, 44, None, 0]
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype="bf16", temperature=0.9, sigma_d=0.4, seed=43)

@@ -66,14 +66,13 @@ def compare_p16(B, O, d, T, logits_view=None, threads=4):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_small_vocabularies_both_kernels(B, oracle_mod, dtype):
-    """Bn = 2 goes through the one-cluster-per-sequence kernel, Bn = 150 through the streaming kernel."""
+    """Few and many sequences in one launch, and 34 positions, which take the separate kernels."""
     seed = 500
     for V in (1, 3, 7, 33, 1000, 1025, 16389):
-        for gamma in (0, 3):
-            for Bn in (2, 150):
-                seed += 1
-                w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=1.0, zipf=V > 8, seed=seed)
-                compare_p16(B, oracle_mod, di.generate(w, threads=4), w.temperature)
+        for gamma, Bn in ((0, 2), (0, 150), (3, 2), (3, 150), (33, 6)):
+            seed += 1
+            w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=1.0, zipf=V > 8, seed=seed)
+            compare_p16(B, oracle_mod, di.generate(w, threads=4), w.temperature)
 
 
 @pytest.mark.parametrize("dtype,V,gamma,Bn", [

@@ -207,7 +207,7 @@ def test_one_shard_is_the_dense_round(B):
     rs = B.dssd_device_resample(ev["p_row"], g["draft_q"], ev["accept_len"], g["uniforms_rs"], w.gamma)
     torch.cuda.synchronize()
     assert torch.equal(out["ev"]["accept_len"], ev["accept_len"])
-    assert torch.equal(out["p_row"], ev["p_row"])  # same sums (streaming kernel), same emission arithmetic
+    assert torch.equal(out["p_row"], ev["p_row"])  # same sums, same emission arithmetic
     assert (out["tokens"][0] == rs["token"].cpu().numpy()).all()
     assert (out["flags"][0] == rs["flags"].cpu().numpy().astype(np.uint32)).all()
 

@@ -72,7 +72,8 @@ def _same(a, b):
         assert torch.equal(x, y), k
 
 
-@pytest.mark.parametrize("shape", [(3, 2, 5000), (200, 3, 9001)])  # cluster kernel / streaming kernel
+# the edge in one launch, one and several CTAs per sequence / in separate kernels, which keep their sums in the workspace
+@pytest.mark.parametrize("shape", [(3, 2, 5000), (200, 3, 9001), (20, 33, 9001)])
 def test_garbage_and_stale_workspaces(B, shape):
     Bn, gamma, V = shape
     w = di.custom(B=Bn, gamma=gamma, V=V, dtype="bf16", temperature=0.9, sigma_d=0.6, seed=Bn)
@@ -110,8 +111,9 @@ def test_garbage_and_stale_workspaces(B, shape):
         _same(cur[name], ref[name])
 
 
-def test_replay_from_a_cuda_graph(B):
-    w = di.custom(B=160, gamma=3, V=12000, dtype="bf16", temperature=0.8, sigma_d=0.6, seed=77)
+@pytest.mark.parametrize("shape", [(160, 3, 12000), (20, 33, 9001)])  # one launch / separate kernels
+def test_replay_from_a_cuda_graph(B, shape):
+    w = di.custom(B=shape[0], gamma=shape[1], V=shape[2], dtype="bf16", temperature=0.8, sigma_d=0.6, seed=77)
     g = to_device(di.generate(w, threads=4))
     gk = to_device(di.generate_topk(w, 10, threads=4))
     n = max(B.dssd_dsd_verify_workspace_bytes(w.B, w.gamma, w.V), B.dssd_edge_verify_topk_workspace_bytes(w.B, w.gamma, w.V, 10))
