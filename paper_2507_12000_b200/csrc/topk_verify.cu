@@ -611,7 +611,8 @@ __device__ __forceinline__ unsigned long long merge_many(const unsigned long lon
 
 // The same where the keys fit a warp's registers and k is small: the largest of the lists' last keys is bound enough (7 runs,
 // k = 5, B = 32 gamma = 4 V = 50257 bf16: the edge call 10.2 us, with merge_many 11.9; k = 32: 19.1 and 14.4).
-constexpr int kMergeFew = 256;
+// Up to kMergeSmall keys at any k: 4 runs, k = 20, a round of B = 112 gamma = 7 V = 25792 bf16 23.5 us, with merge_many 25.4.
+constexpr int kMergeFew = 256, kMergeSmall = 96;
 __device__ __forceinline__ unsigned long long merge_few(const unsigned long long *src, int runs, int k, MergeShared &sh)
 {
     const int lane = threadIdx.x & 31, m = runs * k;
@@ -919,7 +920,8 @@ cudaError_t topk_verify_launch(TopkParams &P, int dtype, void *workspace, cudaSt
                                              : launch_pdl(topk_select_kernel<DSSD_F32>, (unsigned)grid, kSelThreads, stream, P);
     if (e != cudaSuccess) return e;
     const int warps = P.gamma + 1 < kFoldWarps ? P.gamma + 1 : kFoldWarps;
-    const bool many = (long long)P.runs * P.k > kMergeFew || P.k > kGroupsUpTo;
+    const long long keys = (long long)P.runs * P.k;
+    const bool many = keys > kMergeFew || (P.k > kGroupsUpTo && keys > kMergeSmall);
     if (P.gamma + 1 > kFoldTurns * kFoldWarps) {
         const unsigned ctas = (unsigned)(((long long)P.B * (P.gamma + 1) + kFoldWarps - 1) / kFoldWarps);
         const cudaError_t r = launch_pdl(many ? topk_rows_kernel<true> : topk_rows_kernel<false>, ctas, 32u * kFoldWarps, stream, P,

@@ -72,7 +72,7 @@ def test_ties_and_masks(B, oracle_mod, dtype, Bn, gamma, V, k):
     compare_topk(B, oracle_mod, d, w.temperature, k)
 
 
-@pytest.mark.parametrize("V,k", [(9 * 4096, 29), (33 * 4096 + 5, 8), (30 * 4096, 32), (33 * 4096, 32), (300 * 4096 + 1, 1), (300 * 4096, 10),
+@pytest.mark.parametrize("V,k", [(4 * 4096, 20), (5 * 4096, 20), (3 * 4096, 32), (9 * 4096, 29), (33 * 4096 + 5, 8), (30 * 4096, 32), (33 * 4096, 32), (300 * 4096 + 1, 1), (300 * 4096, 10),
                                  (300 * 4096 + 3, 32), (2100 * 4096, 12)])
 def test_rows_of_many_runs(B, oracle_mod, V, k):
     """Merging the lists of many runs (4096 float32 entries each), all keys and only those of the lists that matter: equal shares, rows
