@@ -9,6 +9,7 @@
 #include "dssd_test_hooks.h"
 #include "edge_verify.h"
 #include "launch.h"
+#include "quads.cuh"
 #include "shard_verify.h"
 #include "topk_verify.h"
 
@@ -702,20 +703,46 @@ T *mapped(T *host, size_t count)
     return reinterpret_cast<T *>(device);
 }
 
-// The short input arrays of a round on host buffers, brought to the GPU by one kernel that reads the mapped
+// The input arrays of a round on host buffers, brought to the GPU by one kernel that reads the mapped
 // arrays over the bus (a copy each costs the host 3 us and the stream 2 to 4; a read by the kernels that use
 // them waits for the bus, about 5 us, once in each of them).  Pageable and long arrays are copied.
+//
+// Bound by the bus: the logits of B = 8 gamma = 4 V = 32000 bf16 (2.6 MB), four 16-byte loads per thread in flight, where a
+// copy took 64 us and the kernel after it started 7 us later: a round 82.6 us against 92; B = 6 gamma = 3 V = 33498 bf16
+// (1.6 MB) 61.5 and 75, B = 6 gamma = 8 V = 8048 float32 (1.7 MB) 55.7 and 63.2, B = 2 gamma = 2 V = 3000 float32 24.7 and 28.5.  The
+// copy engine moves long arrays faster: B = 16 gamma = 4 V = 50272 float32 (16 MB) 378 against 363.
 struct StageParams {
     const uint32_t *src[4];
     uint32_t *dst[4];
     unsigned end[4];  // words up to and including array i
+    unsigned word_ctas;   // CTAs for them; the others bring
+    const uint4 *rows;    // the logits
+    uint4 *rows_to;
+    unsigned vecs;        // their whole vectors of 16 bytes
+    unsigned rest;        // bytes after these
 };
 constexpr unsigned kStageWords = 16384;  // of one array; beyond, a copy is as quick
-__global__ void __launch_bounds__(256) stage_kernel(const __grid_constant__ StageParams P)
+constexpr size_t kStageRowBytes = 4 << 20;
+constexpr int kStageThreads = 256, kStageLoads = 4;
+__global__ void __launch_bounds__(kStageThreads) stage_kernel(const __grid_constant__ StageParams P)
 {
     dssd::pdl_wait();
     dssd::pdl_trigger();
-    const unsigned w = blockIdx.x * 256 + threadIdx.x;
+    if (blockIdx.x >= P.word_ctas) {
+        const unsigned i = (blockIdx.x - P.word_ctas) * (kStageThreads * kStageLoads) + threadIdx.x;
+        uint4 v[kStageLoads];
+#pragma unroll
+        for (int u = 0; u < kStageLoads; ++u)
+            if (i + u * kStageThreads < P.vecs) v[u] = dssd::ld_row16(P.rows + i + u * kStageThreads);
+#pragma unroll
+        for (int u = 0; u < kStageLoads; ++u)
+            if (i + u * kStageThreads < P.vecs) P.rows_to[i + u * kStageThreads] = v[u];
+        if (blockIdx.x == P.word_ctas && threadIdx.x < P.rest)
+            reinterpret_cast<unsigned char *>(P.rows_to + P.vecs)[threadIdx.x] =
+                dssd::ld_row_u8(reinterpret_cast<const unsigned char *>(P.rows + P.vecs) + threadIdx.x);
+        return;
+    }
+    const unsigned w = blockIdx.x * kStageThreads + threadIdx.x;
     unsigned begin = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -740,11 +767,24 @@ public:
         P.end[n++] = total;
         return cudaSuccess;
     }
+    // the logits: `bytes` of `host` to `device`, which starts on a boundary of 16 bytes
+    cudaError_t add_rows(const void *host, size_t bytes, void *device)
+    {
+        const char *m = bytes <= kStageRowBytes ? mapped(static_cast<const char *>(host), bytes) : nullptr;
+        if (!m || reinterpret_cast<uintptr_t>(m) % 16) return cudaMemcpyAsync(device, host, bytes, cudaMemcpyHostToDevice, s);
+        P.rows = reinterpret_cast<const uint4 *>(m);
+        P.rows_to = static_cast<uint4 *>(device);
+        P.vecs = (unsigned)(bytes / 16);
+        P.rest = (unsigned)(bytes % 16);
+        return cudaSuccess;
+    }
     cudaError_t run()
     {
-        if (!total) return cudaSuccess;
+        if (!total && !P.rows) return cudaSuccess;
         for (int i = n; i < 4; ++i) P.end[i] = total;
-        return dssd::launch_pdl(stage_kernel, (total + 255) / 256, 256u, s, P);
+        P.word_ctas = (total + kStageThreads - 1) / kStageThreads;
+        const unsigned row_ctas = P.rows ? P.vecs / (kStageThreads * kStageLoads) + 1 : 0;
+        return dssd::launch_pdl(stage_kernel, P.word_ctas + row_ctas, (unsigned)kStageThreads, s, P);
     }
 
 private:
@@ -847,8 +887,8 @@ dssd_status dssd_round_host(const void *target_logits, dssd_dtype dtype,
     cudaError_t e;
 #define DSSD_TRY(call) \
     if ((e = (call)) != cudaSuccess) return cuda_fail(e)
-    DSSD_TRY(cudaMemcpyAsync(d_logits, target_logits, Bz * (g + 1) * Vz * esz, cudaMemcpyHostToDevice, s));
     Stage stage(s);
+    DSSD_TRY(stage.add_rows(target_logits, Bz * (g + 1) * Vz * esz, d_logits));
     DSSD_TRY(stage.add(draft_tokens, Bz * g, d_tok_in));
     DSSD_TRY(stage.add(draft_q_tok, Bz * g, d_qtok));
     DSSD_TRY(stage.add(uniforms, Bz * g, d_u));
@@ -956,8 +996,8 @@ dssd_status dssd_round_host_topk(const void *target_logits, dssd_dtype dtype,
     cudaError_t e;
 #define DSSD_TRY(call) \
     if ((e = (call)) != cudaSuccess) return cuda_fail(e)
-    DSSD_TRY(cudaMemcpyAsync(d_logits, target_logits, Bz * (g + 1) * Vz * esz, cudaMemcpyHostToDevice, s));
     Stage stage(s);
+    DSSD_TRY(stage.add_rows(target_logits, Bz * (g + 1) * Vz * esz, d_logits));
     DSSD_TRY(stage.add(draft_tokens, Bz * g, d_tok_in));
     DSSD_TRY(stage.add(draft_q_tok, Bz * g, d_qtok));
     DSSD_TRY(stage.add(uniforms, Bz * g, d_u));

@@ -40,6 +40,13 @@ __device__ __forceinline__ uint32_t ld_row_u16(const void *p)
     return v;
 }
 
+__device__ __forceinline__ unsigned char ld_row_u8(const void *p)
+{
+    unsigned short v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return (unsigned char)v;
+}
+
 struct Quads32 {  // 4-byte entries
     typedef uint4 Raw;
     static constexpr int kBytes = 4;

@@ -91,3 +91,29 @@ def test_draft_rows_pinned_in_pieces(B, pages):
     finally:
         for a, _ in pages:
             assert int(rt.cudaHostUnregister(base + a * 4096)) == 0
+
+
+@pytest.mark.parametrize("Bn,gamma,V,dtype,offset", [
+    (1, 0, 5, "bf16", 0),       # shorter than one vector
+    (5, 1, 4096, "bf16", 0),    # whole CTAs of the kernel that reads them over the bus
+    (3, 1, 8193, "bf16", 0),    # a vector and two bytes more than that
+    (3, 1, 8193, "bf16", 3),    # not on a boundary of 16 bytes: copied
+    (2, 1, 262144, "f32", 0),   # the longest logits that are read over the bus ...
+    (2, 1, 262145, "f32", 0),   # ... and longer ones
+])
+def test_pinned_logits(B, Bn, gamma, V, dtype, offset):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.5, seed=V + offset)
+    g = to_device(di.generate(w, threads=8))
+    ev = B.dssd_edge_verify(g["target_logits"], g["draft_tokens"], g["draft_q_tok"], g["uniforms"], w.temperature)
+    rs = B.dssd_device_resample(ev["p_row"], g["draft_q"], ev["accept_len"], g["uniforms_rs"], gamma)
+    host = _host(g, "all")
+    tl = host["target_logits"]
+    host["target_logits"] = torch.empty(tl.numel() + offset, dtype=tl.dtype, pin_memory=True)[offset:].view(tl.shape).copy_(tl)
+    arena = torch.full((B.dssd_round_host_arena_bytes(Bn, gamma, V, B.DSSD_BF16 if dtype == "bf16" else B.DSSD_F32),), 0x5A,
+                       dtype=torch.uint8, device="cuda")
+    out = {"p_row": torch.zeros(Bn, V)}
+    out.update({k: torch.zeros(Bn, dtype=torch.int32) for k in ("accept_len", "token", "edge_flags", "rs_flags")})
+    got = B.dssd_round_host(host, w.temperature, arena, out=out)
+    torch.cuda.synchronize()
+    assert torch.equal(got["accept_len"], ev["accept_len"].cpu()) and torch.equal(got["token"], rs["token"].cpu())
+    assert torch.equal(got["p_row"], ev["p_row"].cpu())
