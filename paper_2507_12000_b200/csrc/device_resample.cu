@@ -1,5 +1,6 @@
 // Device half of the verification round: residual (or bonus) inverse-CDF draw, as two kernels, or as one where
-// the batch is small (resample_cluster_kernel: a cluster of CTAs per sequence holds the row in registers).
+// the batch is small (resample_cluster_kernel: a cluster of CTAs per sequence holds the row in registers) or of middle
+// size (resample_stream_kernel: it goes over the row in turns).
 //
 //   resample_mass_kernel  one CTA per (sequence, one to four tiles of kTile entries): streams its part of
 //                         p_row[b] and of Q_n[b], forms r = max(0, p - q) (or r = p for the bonus draw)
@@ -37,17 +38,33 @@ static_assert(2 * kRows == kWarps && kSub == 2 * 512, "a warp of the mass kernel
 // B = 8 V = 32000 (64) 7.9 / 8.7 / 10.2.
 constexpr unsigned long long kTwoTiles = 1200, kFourTiles = 4800;
 constexpr int kClusterThreads = 512;     // most threads per CTA of the cluster kernel
-constexpr int kClusterMax = 8;           // most CTAs per sequence (the portable cluster size)
-// Most CTAs of a launch of the cluster kernel, about one wave (two CTAs of 256 threads fit an SM).  Measured (us a round, cluster
-// kernel / two kernels): B = 8 V = 32000 (64 CTAs) 10.7 / 12.1, B = 32 (256) 15.6 / 15.5, B = 64 (512) 21.3 / 20.5,
-// B = 100 V = 3001 (100) 12.4 / 15.1. CTAs of 512 threads, for vocabularies beyond 32768, pay off in smaller
-// batches only: B = 1 V = 50272 (8) 10.5 / 11.4, B = 16 V = 50257 (128) 17.7 / 16.2.
-constexpr int kClusterWave = 200;
-// One CTA per sequence, vocabularies up to 4096, has no cluster to wait for and pays off up to about two waves of (at 128
-// registers) 512 threads per SM: B = 1000 V = 1024 4.7 / 12.4, B = 1000 V = 2000 7.9 / 12.6, B = 600 V = 4001 10.7 / 11.9; beyond,
-// B = 1000 V = 4001 16.1 / 15.1 (the draw alone).
-constexpr long long kSingleThreads = 153600;
+constexpr int kClusterMax = 8;           // most CTAs per cluster: the portable size,
+constexpr int kClusterWide = 16;         // and where the device has them
 constexpr int kClusterSums = kClusterMax * kClusterThreads / 32;
+// Small draws: one launch whose warps hold the row, 512 entries each (resample_cluster_kernel), while about one wave of the CTAs holds
+// the batch; at 128 registers that is 2368 warps, less for large clusters, which do not pack the GPU's processing
+// clusters completely.  The smallest CTAs that fit one cluster of sixteen leave the fewest warps idle and start soonest.
+// Measured (us per call, this / the two kernels):
+//   a CTA per sequence:  B = 1000 V = 1024 4.7 / 12.4, B = 1000 V = 2000 7.9 / 12.6, B = 600 V = 4001 10.7 / 11.9; beyond, B = 1000
+//              V = 4001 16.1 / 15.1
+//   clusters of 128 threads:  B = 168 V = 5460 (3 CTAs) 4.1 / 6.3, B = 59 V = 13786 (7) 4.2 / 6.7, B = 46 V = 16436 (9) 4.2 / 5.9;
+//              beyond, B = 46 V = 28992 (15, 690 CTAs) 6.7 / 6.1, B = 175 V = 11384 (6) 7.8 / 6.1
+//   of 256:  B = 7 V = 57700 (15) 4.3 / 6.1, of 512:  B = 2 V = 96209 (12) 4.3 / 5.9, B = 6 V = 105317 (13) 4.5 / 6.1, B = 4
+//              V = 129300 (16) 4.6 / 5.1; beyond, B = 21 V = 82900 (11) 12.5 / 7.2.
+constexpr long long kSingleThreads = 153600;
+// More than eight CTAs of 128 threads only for a few sequences: many of them do not find room before the kernel before has drained (a round
+// of B = 23 gamma = 7 V = 23912 bf16, twelve CTAs 13.0 us, six of 256 threads 12.5; B = 8 gamma = 4 V = 32000 bf16, sixteen 9.3, eight 9.5).
+constexpr long long kHeldWideCtas = 148;
+constexpr long long kHeldWarps = 2250, kHeldWideWarps = 1650, kHeldWidestWarps = 1250;  // up to eight CTAs, more, more of 512 threads
+// Batches of middle size: the same in turns (resample_stream_kernel), in which a CTA's or cluster's start, its barrier and the walk are
+// paid for once while the other CTAs on the SM stream.  For rows of up to kStreamSegs segments, at most kStreamTurns of them per warp:
+// as many warps as there are segments while kStreamOne of them suffice, else as many as a wave has (four or five
+// CTAs of 256 threads per SM, seven tenths of that in clusters).  Measured (us per call, this / the two kernels): B = 164 V = 9856
+// 5.6 / 6.5, B = 331 V = 4384 binary16 6.7 / 10.6, B = 425 V = 5800 7.5 / 9.3, B = 714 V = 3728 6.4 / 9.1, B = 567 V = 11886 11.7 / 15.3,
+// B = 665 V = 12640 12.8 / 15.6, B = 305 V = 15760 binary16 9.8 / 12.5, B = 143 V = 19400 7.8 / 9.4; beyond, B = 67 V = 32592 7.0 / 6.6,
+// B = 100 V = 43015 13.3 / 12.2, B = 55 V = 124034 14.4 / 10.5.
+constexpr int kStreamSegs = 45, kStreamTurns = 5;
+constexpr long long kStreamOne = 3600;
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
 constexpr int kDrawWarps = kDrawThreads / 32;
 constexpr int kRun = kSub / kDrawThreads;  // entries of a chunk per thread
@@ -267,12 +284,12 @@ __global__ void __launch_bounds__(kDrawThreads) resample_draw_kernel(const __gri
     }
 }
 
-// Small launches: one cluster of up to eight CTAs per sequence does the whole draw and reads every entry
+// Small launches: one cluster of up to sixteen CTAs per sequence does the whole draw and reads every entry
 // once (draw_held).
 template <bool kShift, typename RV>
 __global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const __grid_constant__ ResampleParams P)
 {
-    __shared__ double s_sum[2 * kClusterSums];
+    __shared__ double s_sum[2 * kClusterWide * kClusterThreads / 32];
     __shared__ Pick s_pick;
     const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const unsigned csize = (unsigned)P.n_ctas, rank = csize > 1 ? cluster_rank() : 0u;
@@ -300,6 +317,41 @@ __global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const
     if (!RV::kFixed) a.load(row.row, P.V, 512ll * g, RV::kFill);
     const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
     draw_held<kShift>(row, a, q, P.V, g, (int)csize * warps, csize, rank, u, s_sum, s_pick, P.token + b, P.flags ? P.flags + b : nullptr);
+}
+
+// Batches of middle size (draw_streamed).  Bound by the chain of loads, sums, barrier and walk of each CTA, under which the others on
+// the SM stream: 48 registers, so five CTAs of 256 threads share one.
+template <bool kShift, typename RV>
+__global__ void __launch_bounds__(kThreads, kShift ? 4 : 5) resample_stream_kernel(const __grid_constant__ ResampleParams P)
+{
+    __shared__ DrawShared sh;
+    const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const unsigned csize = (unsigned)P.n_ctas, rank = csize > 1 ? cluster_rank() : 0u;
+    const int64_t b = blockIdx.x / csize;
+    const int g = warp * (int)csize + (int)rank;
+    if (csize > 1) {  // the first CTA's shared memory may be written once it is known to run
+        cluster_arrive();
+        cluster_wait();
+    }
+    pdl_wait();
+    pdl_trigger();
+    const int n = ld_after(P.accept_len + b);
+    const float u = warp == 0 ? ld_after(P.uniforms + b) : 0.f;
+    WarpQuads<typename RV::Q, 4, kShift> a;
+    const bool early = RV::kFixed && P.select == 0;  // the row is on its way before n is back
+    if (early) a.load(RV::make(P, b, 0).row, P.V, 512ll * g, RV::kFill);
+    const bool invalid = n < 0 || n > P.gamma;
+    if (invalid || !selected(P, n)) {
+        if (rank == 0 && threadIdx.x == 0 && (invalid || P.select == 1)) {  // (the bonus token drawn at the edge: the others get their token later)
+            P.token[b] = -1;
+            if (P.flags) P.flags[b] = invalid ? DSSD_RS_FLAG_INVALID : 0u;
+        }
+        return;
+    }
+    const RV row = RV::make(P, b, n);
+    if (!early) a.load(row.row, P.V, 512ll * g, RV::kFill);
+    const float *q = n < P.gamma ? P.draft_q + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
+    draw_streamed<kShift>(row, a, q, P.V, g, (int)csize * warps, csize, rank, u, sh, P.token + b, P.flags ? P.flags + b : nullptr);
 }
 
 // ---- one shard of the vocabulary ---------------------------------------------------------------
@@ -360,6 +412,7 @@ __global__ void __launch_bounds__(kThreads, 4) shard_mass_kernel(const __grid_co
 // added up in the first CTA's shared memory, which saves the second launch.  For one wave of CTAs (a round of
 // B = 8 V = 32000 in two shards 15.3 us against 15.8); in large launches the warps that stand idle beyond the
 // slice's end and the barrier cost more (B = 256 V = 151936 in eight shards 39.4 against 36.4).
+constexpr int kShardClusterWave = 200;  // CTAs
 template <bool kShift>
 __global__ void __launch_bounds__(kClusterThreads, 2) shard_mass_cluster_kernel(const __grid_constant__ ShardResampleParams P)
 {
@@ -554,18 +607,78 @@ template <typename RV, bool kShift>
 cudaError_t launch_resample_as(const ResampleParams &P, unsigned grid, cudaStream_t stream)
 {
     if (P.cluster_threads)
-        return launch_pdl(resample_cluster_kernel<kShift, RV>, (unsigned)(P.B * P.n_ctas), (unsigned)P.cluster_threads, stream, P,
-                          0, (unsigned)P.n_ctas);
+        return launch_pdl(P.streamed ? resample_stream_kernel<kShift, RV> : resample_cluster_kernel<kShift, RV>, (unsigned)(P.B * P.n_ctas),
+                          (unsigned)P.cluster_threads, stream, P, 0, (unsigned)P.n_ctas);
     const cudaError_t e = launch_pdl(resample_mass_kernel<kShift, RV>, grid, kThreads, stream, P);
     if (e != cudaSuccess) return e;
     return P.n_sub > kLongSums ? launch_pdl(resample_draw_kernel<true, kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P)
                                 : launch_pdl(resample_draw_kernel<false, kShift, RV>, (unsigned)P.B, kDrawThreads, stream, P);
 }
+
 template <typename RV>
-cudaError_t launch_resample(const ResampleParams &P, unsigned grid, cudaStream_t stream)
+bool wide_clusters()
+{
+    return allow_cluster(resample_cluster_kernel<false, RV>, kClusterWide, kClusterThreads) &&
+           allow_cluster(resample_cluster_kernel<true, RV>, kClusterWide, kClusterThreads);
+}
+int most_cluster_ctas()
+{
+    static PerContext most;
+    return most.get([] {
+        const bool wide = wide_clusters<RowF32>() && wide_clusters<RowF16>() && wide_clusters<RowLogits<DSSD_F32>>() &&
+                          wide_clusters<RowLogits<DSSD_BF16>>();
+        if (!wide) cudaGetLastError();
+        return wide ? kClusterWide : kClusterMax;
+    });
+}
+
+// Threads and CTAs per sequence of the kernels that draw in one launch; false where the two kernels are the better ones.
+bool one_launch(ResampleParams &P, bool aligned)
+{
+    const int segs = (P.V + 511) / 512;
+    const long long B = P.B;
+    auto is = [&](int threads, long long ctas, bool streamed) {
+        P.cluster_threads = threads;
+        P.n_ctas = (int)ctas;
+        P.streamed = streamed;
+        return true;
+    };
+    if (segs <= 8) {
+        if (B * 32 * segs <= kSingleThreads) return is(32 * segs, 1, false);
+    } else if (segs <= kClusterWide * kClusterThreads / 32 && B * segs <= kHeldWarps) {
+        for (int warps = 4; warps <= kClusterThreads / 32; warps *= 2) {
+            const long long ctas = (segs + warps - 1) / warps;
+            if (ctas > kClusterWide || (ctas > kClusterMax && (most_cluster_ctas() < kClusterWide || (warps == 4 && B * ctas > kHeldWideCtas)))) continue;
+            if (B * ctas * warps <= (ctas <= kClusterMax ? kHeldWarps : warps < 16 ? kHeldWideWarps : kHeldWidestWarps)) return is(32 * warps, ctas, false);
+            break;
+        }
+    }
+    if (segs > kStreamSegs) return false;
+    const long long wave = 148 * (aligned ? 5 : 4) * kWarps;
+    long long warps = segs;
+    if (B * segs <= kStreamOne) {
+        if (segs <= 2 * kWarps && B >= 250) warps = kWarps;
+    } else if (B * 10 > wave) {
+        warps = wave / B;
+        if (warps < 4) return false;
+        if (warps > kWarps) warps = kWarps;
+    } else {
+        warps = wave * 7 / 10 / B;
+        const long long turns = (segs + warps - 1) / warps;
+        warps = (segs + turns - 1) / turns;
+    }
+    if (warps > segs) warps = segs;
+    if (segs > kStreamTurns * warps) return false;
+    if (warps <= kWarps) return is(32 * (int)warps, 1, true);
+    return warps <= 4 * kClusterMax ? is(128, (warps + 3) / 4, true) : is(kThreads, (warps + kWarps - 1) / kWarps, true);
+}
+
+template <typename RV>
+cudaError_t launch_resample(ResampleParams &P, unsigned grid, cudaStream_t stream)
 {
     const bool aligned = (P.logits ? quads_aligned(P.logits, P.row_stride, RV::Q::kBytes) : quads_aligned(P.p_row, P.V, RV::Q::kBytes)) &&
                          (!P.draft_q || quads_aligned(P.draft_q, P.V, 4));
+    if (!P.test_drop_seq_plus1) one_launch(P, aligned);
     return aligned ? launch_resample_as<RV, false>(P, grid, stream) : launch_resample_as<RV, true>(P, grid, stream);
 }
 
@@ -580,18 +693,7 @@ cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t str
     P.n_ctas = (int)((n_tiles + P.tiles - 1) / P.tiles);
     const unsigned long long grid = (unsigned long long)P.B * (unsigned long long)P.n_ctas;
     if (grid > 0x7fffffffull) return cudaErrorInvalidConfiguration;
-    // small launches: a cluster of CTAs per sequence, while one wave of them holds the batch
-    const long long warps = ((long long)P.V + 511) / 512;  // 512 entries each
-    const int per_cta = warps <= 8 * kClusterMax ? 8 : 16;
-    const long long ctas = (warps + per_cta - 1) / per_cta;
     P.cluster_threads = 0;
-    const int threads = 32 * (int)(warps < per_cta ? warps : per_cta);
-    const bool small = ctas == 1 ? (long long)P.B * threads <= kSingleThreads
-                                 : ctas <= kClusterMax && P.B * ctas <= (per_cta == 8 ? kClusterWave : kClusterWave / 4);
-    if (small && !P.test_drop_seq_plus1) {
-        P.n_ctas = (int)ctas;
-        P.cluster_threads = threads;
-    }
     if (P.logits) {
         return P.logits_dtype == DSSD_BF16 ? launch_resample<RowLogits<DSSD_BF16>>(P, (unsigned)grid, stream)
                                            : launch_resample<RowLogits<DSSD_F32>>(P, (unsigned)grid, stream);
@@ -617,7 +719,7 @@ cudaError_t shard_mass_launch(ShardResampleParams &P, void *workspace, cudaStrea
     const long long warps = ((long long)P.V + 511) / 512;
     const int per_cta = warps <= 8 * kClusterMax ? 8 : 16;
     const long long ctas = (warps + per_cta - 1) / per_cta;
-    if (ctas <= kClusterMax && P.B * ctas <= kClusterWave) {
+    if (ctas <= kClusterMax && P.B * ctas <= kShardClusterWave) {
         P.cluster = (int)ctas;
         const unsigned block = 32u * (unsigned)per_cta, cgrid = (unsigned)(P.B * ctas);
         return shard_aligned(P) ? launch_pdl(shard_mass_cluster_kernel<false>, cgrid, block, stream, P, 0, (unsigned)ctas)

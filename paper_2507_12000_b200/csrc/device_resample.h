@@ -32,7 +32,8 @@ struct ResampleParams {
     uint32_t *flags;
     int tiles;         // tiles per CTA of the mass kernel
     int n_ctas;        // such CTAs per sequence
-    int cluster_threads;  // threads per CTA of the cluster kernel (n_ctas per sequence), 0: mass kernel and draw kernel
+    int cluster_threads;  // threads per CTA where one kernel draws (n_ctas per sequence), 0: mass kernel and draw kernel
+    bool streamed;        // that kernel: in turns (resample_stream_kernel), or the row in registers (resample_cluster_kernel)
     int rows_per_sum;  // chunks per stored sum: 1, or 2 or 4 (a whole tile) in the largest batches
     int n_sub;         // stored sums per sequence
     double *chunk_sum;   // scratch [B, n_sub]

@@ -110,11 +110,10 @@ struct RowLogits {  // row n of the target logits, turned into probabilities on 
 // 4 lane .. + 3.  All loads are requested before the first is used.  q is not read without kHasQ (then
 // r = p); with kPlain the sum of p goes to `plain`.
 template <bool kHasQ, bool kPlain, bool kShift, typename RV>
-__device__ __forceinline__ double share_mass(const RV &row, const float *q, int V, long long base, double &plain)
+__device__ __forceinline__ double share_mass(const RV &row, const WarpQuads<typename RV::Q, 4, kShift> &a, const float *q, int V, long long base,
+                                             double &plain)
 {
-    WarpQuads<typename RV::Q, 4, kShift> a;
     WarpQuads<Quads32, 4, kShift> b;
-    a.load(row.row, V, base, RV::kFill);
     if (kHasQ) b.load(reinterpret_cast<const char *>(q), V, base, 0u);
     double acc = 0.0;
     plain = 0.0;
@@ -132,6 +131,13 @@ __device__ __forceinline__ double share_mass(const RV &row, const float *q, int 
         }
     }
     return acc;
+}
+template <bool kHasQ, bool kPlain, bool kShift, typename RV>
+__device__ __forceinline__ double share_mass(const RV &row, const float *q, int V, long long base, double &plain)
+{
+    WarpQuads<typename RV::Q, 4, kShift> a;
+    a.load(row.row, V, base, RV::kFill);
+    return share_mass<kHasQ, kPlain, kShift>(row, a, q, V, base, plain);
 }
 
 // r for the segment of 512 entries from `base` on: r[4 u + j] is entry base + 128 u + 4 lane + j.  `a` holds the row's quads.
@@ -400,6 +406,76 @@ __device__ __forceinline__ void draw_held(const RV &row, const WarpQuads<typenam
     }
     if (g != pk.chunk) return;
     const int tok = walk_segment(pk, r, g);
+    if (lane == 0) {
+        *token = tok;
+        if (flags) *flags = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u);
+    }
+}
+
+// The same where the warps take segments in turns: warp g of the n_warps the segments g, g + n_warps, ..  The sums go to the first
+// CTA's shared memory, and after a cluster barrier its first warp picks the segment that holds the target, fetches it
+// again and walks it.  `a` is the row's part of the warp's first segment.
+constexpr int kDrawSegs = 1024;  // most segments of such a row (8 KB)
+struct DrawShared {
+    double sum[kDrawSegs];
+    Pick pick;
+    int again;
+};
+template <bool kShift, typename RV>
+__device__ __forceinline__ void draw_streamed(const RV &row, WarpQuads<typename RV::Q, 4, kShift> &a, const float *q, int V, int g, int n_warps,
+                                              unsigned csize, unsigned rank, float u, DrawShared &sh, int32_t *token, uint32_t *flags)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, segs = (V + 511) / 512;
+    unsigned fl = q ? 0u : DSSD_RS_FLAG_BONUS;
+    for (int i = g; i < segs; i += n_warps) {
+        double none, t;
+        if (i != g) a.load(row.row, V, 512ll * i, RV::kFill);
+        if (q) t = share_mass<true, false, kShift>(row, a, q, V, 512ll * i, none);
+        else t = share_mass<false, false, kShift>(row, a, q, V, 512ll * i, none);
+        t = warp_sum(t);
+        if (lane == 0) {
+            if (csize > 1) cluster_store(&sh.sum[i], 0u, t);
+            else sh.sum[i] = t;
+        }
+    }
+    if (csize > 1) {
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+    if (rank) return;
+    Pick pk;
+    auto pick = [&]() {
+        LaneSums L;
+        auto sum = [&](int c) { return sh.sum[c]; };
+        load_sums(L, segs, sum);
+        pk = pick_chunk(L, sum, false, [&](double Z) { return (double)u * Z; });
+    };
+    if (warp == 0) {
+        pick();
+        if (lane == 0) sh.again = !pk.ok && q;
+    }
+    __syncthreads();
+    if (sh.again) {  // the residual has no mass (p == q): draw from p instead; rare, so by this CTA alone
+        q = nullptr;
+        fl |= DSSD_RS_FLAG_FALLBACK;
+        for (int i = warp; i < segs; i += (int)(blockDim.x >> 5)) {
+            double none;
+            const double t = warp_sum(share_mass<false, false, kShift>(row, q, V, 512ll * i, none));
+            if (lane == 0) sh.sum[i] = t;
+        }
+        __syncthreads();
+        if (warp == 0) pick();
+    }
+    if (warp) return;
+    int tok = -1;
+    if (pk.ok) {
+        double r[16];
+        a.load(row.row, V, 512ll * pk.chunk, RV::kFill);
+        segment_residuals<kShift>(row, a, q, V, 512ll * pk.chunk, r);
+        tok = walk_segment(pk, r, pk.chunk);
+    }
     if (lane == 0) {
         *token = tok;
         if (flags) *flags = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u);

@@ -20,9 +20,6 @@
 // before it drains (launch.h).
 #include "edge_verify.h"
 
-#include <atomic>
-
-#include <cuda.h>
 #include <math.h>
 
 #include "draw.cuh"
@@ -370,21 +367,14 @@ __device__ __forceinline__ void emit_pieces(const char *rowp, OUT *outp, int V, 
 }
 
 // The draw from row n of sequence b, by the cluster that has folded it: where its warps can hold the row (draw_held) as
-// the kernel of small draws does it; else the sums of segments of 512 entries go to the first CTA's shared memory,
-// and after a cluster barrier its first warp picks the segment, fetches it again and walks it.
-struct DrawShared {
-    double sum[kEdgeDrawSegs];
-    Pick pick;
-    int again;
-};
-static_assert(kEdgeDrawSegs >= 2 * kEdgeClusterWide * kWarps, "draw_held keeps two sets of sums");
+// the kernel of small draws does it, else in turns (draw_streamed).
+static_assert(kDrawSegs >= 2 * kEdgeClusterWide * kWarps, "draw_held keeps two sets of sums");
 template <int DT, bool kShift, bool kHeld>
 __device__ __forceinline__ void draw_here(const EdgeParams &P, long long b, const char *rowp, int n, float ref2, float invS, unsigned csize,
                                           unsigned rank, DrawShared &sh)
 {
-    [[maybe_unused]] const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, segs = (P.V + 511) / 512;
+    const int warp = threadIdx.x >> 5, n_warps = kWarps * (int)csize, g = warp * (int)csize + (int)rank;
     const float *q = n < P.gamma ? P.draft_q_rows + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
-    [[maybe_unused]] unsigned fl = q ? 0u : DSSD_RS_FLAG_BONUS;
     RowLogits<DT> row;
     row.row = rowp;
     row.c1 = P.c1;
@@ -392,65 +382,10 @@ __device__ __forceinline__ void draw_here(const EdgeParams &P, long long b, cons
     row.invS = invS;
     const float u = warp == 0 ? ld_after(P.draw_uniforms + b) : 0.f;
     WarpQuads<typename RowLogits<DT>::Q, 4, kShift> a;
-    if constexpr (kHeld) {
-        const int g = warp * (int)csize + (int)rank;
-        a.load(rowp, P.V, 512ll * g, RowLogits<DT>::kFill);
-        draw_held<kShift>(row, a, q, P.V, g, kWarps * (int)csize, csize, rank, u, sh.sum, sh.pick, P.draw_token + b,
-                          P.draw_flags ? P.draw_flags + b : nullptr);
-    } else {
-        for (int g = warp * (int)csize + (int)rank; g < segs; g += kWarps * (int)csize) {
-            double none, t;
-            if (q) t = share_mass<true, false, kShift>(row, q, P.V, 512ll * g, none);
-            else t = share_mass<false, false, kShift>(row, q, P.V, 512ll * g, none);
-            t = warp_sum(t);
-            if (lane == 0) {
-                if (csize > 1) cluster_store(&sh.sum[g], 0u, t);
-                else sh.sum[g] = t;
-            }
-        }
-        if (csize > 1) {
-            cluster_arrive();
-            cluster_wait();
-        } else {
-            __syncthreads();
-        }
-        if (rank) return;
-        Pick pk;
-        auto pick = [&]() {
-            LaneSums L;
-            auto sum = [&](int c) { return sh.sum[c]; };
-            load_sums(L, segs, sum);
-            pk = pick_chunk(L, sum, false, [&](double Z) { return (double)u * Z; });
-        };
-        if (warp == 0) {
-            pick();
-            if (lane == 0) sh.again = !pk.ok && q;
-        }
-        __syncthreads();
-        if (sh.again) {  // the residual has no mass (p == q): draw from p instead; rare, so by this CTA alone
-            q = nullptr;
-            fl |= DSSD_RS_FLAG_FALLBACK;
-            for (int g = warp; g < segs; g += kWarps) {
-                double none;
-                const double t = warp_sum(share_mass<false, false, kShift>(row, q, P.V, 512ll * g, none));
-                if (lane == 0) sh.sum[g] = t;
-            }
-            __syncthreads();
-            if (warp == 0) pick();
-        }
-        if (warp) return;
-        int tok = -1;
-        if (pk.ok) {
-            double r[16];
-            a.load(rowp, P.V, 512ll * pk.chunk, RowLogits<DT>::kFill);
-            segment_residuals<kShift>(row, a, q, P.V, 512ll * pk.chunk, r);
-            tok = walk_segment(pk, r, pk.chunk);
-        }
-        if (lane == 0) {
-            P.draw_token[b] = tok;
-            if (P.draw_flags) P.draw_flags[b] = fl | (tok < 0 ? DSSD_RS_FLAG_INVALID : 0u);
-        }
-    }
+    a.load(rowp, P.V, 512ll * g, RowLogits<DT>::kFill);
+    uint32_t *flags = P.draw_flags ? P.draw_flags + b : nullptr;
+    if constexpr (kHeld) draw_held<kShift>(row, a, q, P.V, g, n_warps, csize, rank, u, sh.sum, sh.pick, P.draw_token + b, flags);
+    else draw_streamed<kShift>(row, a, q, P.V, g, n_warps, csize, rank, u, sh, P.draw_token + b, flags);
 }
 
 // One cluster of up to sixteen CTAs per sequence does the whole of it.  Warp g of the cluster's takes the segments
@@ -664,52 +599,26 @@ cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
     return held ? launch_cluster<DT, 2>(P, stream) : launch_cluster<DT, 1>(P, stream);
 }
 
-// Clusters beyond the portable size have to be allowed for each kernel, and a device (or the part of one that the
-// process was given) may not have a processing cluster of that many SMs: asked once per context, which holds the
-// permission.  A device that was reset, or a second context on it, is asked again.
-bool wide_clusters(void (*kernel)(EdgeParams))
-{
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = kEdgeClusterWide;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kEdgeClusterWide);
-    cfg.blockDim = dim3(kThreads);
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
-}
 template <int DT, int kDraw>
 bool wide_clusters()
 {
-    return wide_clusters(edge_cluster_kernel<DT, false, kDraw>) && wide_clusters(edge_cluster_kernel<DT, true, kDraw>);
+    return allow_cluster(edge_cluster_kernel<DT, false, kDraw>, kEdgeClusterWide, kThreads) &&
+           allow_cluster(edge_cluster_kernel<DT, true, kDraw>, kEdgeClusterWide, kThreads);
 }
 template <int DT>
 bool wide_clusters()
 {
-    return wide_clusters<DT, 0>() && wide_clusters<DT, 1>() && wide_clusters<DT, 2>() && wide_clusters(edge_partial_cluster_kernel<DT>);
+    return wide_clusters<DT, 0>() && wide_clusters<DT, 1>() && wide_clusters<DT, 2>() &&
+           allow_cluster(edge_partial_cluster_kernel<DT>, kEdgeClusterWide, kThreads);
 }
 int most_cluster_ctas()
 {
-    typedef CUresult (*ContextId)(CUcontext, unsigned long long *);
-    static const ContextId context_id = driver_call<ContextId>("cuCtxGetId");
-    static std::atomic<unsigned long long> known[16];  // (id + 1) * 32 + the answer; 0: empty
-    static std::atomic<unsigned> turn;
-    unsigned long long id = 0;  // (an id is never given twice)
-    const bool has_id = context_id && context_id(nullptr, &id) == CUDA_SUCCESS;
-    if (has_id)
-        for (const auto &k : known) {
-            const unsigned long long w = k.load(std::memory_order_acquire);
-            if (w / 32 == id + 1) return (int)(w % 32);
-        }
-    const bool wide = wide_clusters<DSSD_F32>() && wide_clusters<DSSD_BF16>();
-    if (!wide) cudaGetLastError();
-    const int most = wide ? kEdgeClusterWide : kEdgeCluster;
-    if (has_id) known[turn.fetch_add(1, std::memory_order_relaxed) % 16].store((id + 1) * 32 + (unsigned long long)most, std::memory_order_release);
-    return most;
+    static PerContext most;
+    return most.get([] {
+        const bool wide = wide_clusters<DSSD_F32>() && wide_clusters<DSSD_BF16>();
+        if (!wide) cudaGetLastError();
+        return wide ? kEdgeClusterWide : kEdgeCluster;
+    });
 }
 
 // at most c CTAs per sequence, no more than `wave` in all, at least one
@@ -723,7 +632,7 @@ long long fit(long long c, long long wave, int B)
 int cluster_ctas(const EdgeParams &P, int esz, long long segs)
 {
     const long long parts = segs * (P.gamma + 1);
-    if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kEdgeDrawSegs)) return 0;
+    if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kDrawSegs)) return 0;
     long long c = (parts + kWarps - 1) / kWarps;
     c = fit(c, kEdgeWave, P.B);
     if (c > 2) c = fit(c, kEdgeClusterWave, P.B);

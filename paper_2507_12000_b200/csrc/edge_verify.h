@@ -44,7 +44,6 @@ constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster
 constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, more
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
-constexpr int kEdgeDrawSegs = 1024;                      // segments of 512 entries of a row that the cluster kernel draws from (8 KB)
 constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory; the limits on the work allow 900)
 
 // What the draw needs to know about a folded sequence when no row is written.

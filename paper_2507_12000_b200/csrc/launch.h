@@ -8,6 +8,9 @@
 // the one before it has.
 #pragma once
 
+#include <atomic>
+
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 namespace dssd {
@@ -41,6 +44,51 @@ Fn driver_call(const char *name)
     const cudaError_t e = cudaGetDriverEntryPoint(name, &fn, cudaEnableDefault, &found);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(fn) : nullptr;
+}
+
+// One small answer (0 .. 31) per context, asked for on the first call made in it.  A device that was reset, or a second
+// context on it, is asked again.
+class PerContext {
+public:
+    template <class Ask>
+    int get(Ask ask)
+    {
+        typedef CUresult (*ContextId)(CUcontext, unsigned long long *);
+        static const ContextId context_id = driver_call<ContextId>("cuCtxGetId");
+        unsigned long long id = 0;  // (an id is never given twice)
+        const bool has_id = context_id && context_id(nullptr, &id) == CUDA_SUCCESS;
+        if (has_id)
+            for (const auto &k : known) {
+                const unsigned long long w = k.load(std::memory_order_acquire);
+                if (w / 32 == id + 1) return (int)(w % 32);
+            }
+        const int answer = ask();
+        if (has_id) known[turn.fetch_add(1, std::memory_order_relaxed) % 16].store((id + 1) * 32 + (unsigned long long)answer, std::memory_order_release);
+        return answer;
+    }
+
+private:
+    std::atomic<unsigned long long> known[16]{};  // (id + 1) * 32 + the answer; 0: empty
+    std::atomic<unsigned> turn{0};
+};
+
+// Clusters beyond the portable size of eight have to be allowed for each kernel in each context, and a device (or the part of one
+// that the process was given) may not have a processing cluster of that many SMs.
+template <class Params>
+bool allow_cluster(void (*kernel)(Params), unsigned ctas, unsigned threads)
+{
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = ctas;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
 }
 
 }  // namespace dssd

@@ -23,6 +23,12 @@ def B():
     (7, 1, 65536, False), (4, 2, 65537, False), (200, 1, 900, False), (201, 1, 900, True), (5, 1, 50257, True), (1199, 1, 4096, False), (1200, 1, 4096, False), (150, 1, 32768, True), (4801, 1, 4000, False),
     (600, 1, 4096, False), (601, 1, 4096, True), (1200, 1, 2047, True), (1201, 1, 2047, False), (2400, 1, 1024, False), (2401, 1, 1024, False),
     (6, 2, 9001, False), (6, 3, 9002, True), (7, 2, 9003, True), (6, 2, 9003, False), (600, 1, 36864, False), (2, 1, 262144, False), (2, 1, 266241, False), (1200, 1, 114700, True), (32768, 1, 4097, False), (32769, 1, 8193, True),
+    # clusters of 128, 256 and 512 threads that hold a row: at and beyond eight and sixteen CTAs and the waves they are chosen for
+    (40, 1, 16384, False), (40, 1, 16385, True), (45, 1, 16896, False), (46, 1, 16896, True), (187, 2, 6144, False), (188, 2, 6144, False),
+    (12, 1, 65536, False), (13, 1, 65533, False), (4, 1, 131072, True), (4, 1, 131073, False), (5, 2, 131072, False),
+    # rows in turns: as many warps as segments, one CTA per sequence in one to five turns, clusters, and beyond
+    (100, 1, 18432, False), (101, 1, 18432, True), (330, 2, 4500, False), (719, 1, 12001, False), (740, 1, 20480, False), (740, 1, 20481, True),
+    (1180, 1, 9001, True), (1201, 1, 2044, False), (150, 2, 23040, False), (150, 2, 23041, False),
     (3, 1, 1 << 19, False), (3, 1, (1 << 19) + 1, False), (4, 1, 1 << 20, False), (4, 1, (1 << 20) + 1, True), (3, 1, (1 << 21) + 3, False), (3, 1, 5000001, False),
 ])
 def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
@@ -54,10 +60,10 @@ def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
     assert (out["flags"].cpu().numpy().astype(np.uint32) == ref["flags"]).all()
 
 
-@pytest.mark.parametrize("Bn,V", [(5, 3000), (3, 20011), (40, 70001), (4, 300001), (4, 1100001)])
+@pytest.mark.parametrize("Bn,V", [(5, 3000), (3, 20011), (40, 70001), (4, 300001), (4, 1100001), (120, 15001), (700, 4200), (4, 100003)])
 def test_fallback_and_invalid_lengths(B, oracle_mod, Bn, V):
     """No residual mass (p == q): drawn from p; lengths outside [0, gamma] and rows without mass: token -1; one
-    cluster per sequence and the two-kernel path."""
+    cluster per sequence, in turns, and the two-kernel path."""
     gamma = 2
     gen = torch.Generator(device="cuda").manual_seed(V)
     p = torch.softmax(2.0 * torch.randn(Bn, V, generator=gen, device="cuda"), dim=-1)
@@ -72,3 +78,41 @@ def test_fallback_and_invalid_lengths(B, oracle_mod, Bn, V):
     near = ref["margin_cdf"] < V * 2.0 ** -52  # V float64 additions in another order
     assert ((out["token"].cpu().numpy() == ref["token"]) | near).all()
     assert (out["flags"].cpu().numpy().astype(np.uint32) == ref["flags"]).all()
+
+
+@pytest.mark.parametrize("Bn,V", [(130, 15000), (500, 9001)])
+def test_rejected_sequences_only_in_turns(B, Bn, V):
+    gamma = 2
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    p = torch.softmax(2.0 * torch.randn(Bn, V, generator=gen, device="cuda"), dim=-1)
+    q = torch.softmax(2.0 * torch.randn(Bn, gamma, V, generator=gen, device="cuda"), dim=-1)
+    n = (torch.arange(Bn, device="cuda") % (gamma + 1)).to(torch.int32)
+    u = torch.rand(Bn, generator=gen, device="cuda").clamp_(max=1.0 - 2.0 ** -24)
+    full = B.dssd_device_resample(p, q, n, u, gamma)
+    some = {"token": torch.full_like(n, 77), "flags": torch.full_like(n, 88)}
+    B.dssd_device_resample_rejected(p, q, n, u, gamma, out=some)
+    torch.cuda.synchronize()
+    bonus = n == gamma
+    assert (some["token"][bonus] == 77).all() and (some["flags"][bonus] == 88).all()
+    assert torch.equal(some["token"][~bonus], full["token"][~bonus]) and torch.equal(some["flags"][~bonus], full["flags"][~bonus])
+
+
+@pytest.mark.parametrize("V", [20000, 20001])
+def test_fused_draw_in_turns(B, V):
+    """The draw straight from the logits, in turns, against the draw from the row that the edge writes (the same float32
+    values and the same float64 sums)."""
+    Bn, gamma, T = 150, 16, 0.9
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    tl = (3.0 * torch.randn(Bn, gamma + 1, V, generator=gen, device="cuda")).to(torch.bfloat16)
+    q = torch.softmax(tl[:, :gamma].float() / T + 0.1 * torch.randn(Bn, gamma, V, generator=gen, device="cuda"), dim=-1)
+    x = torch.multinomial(q.view(-1, V), 1, generator=gen).view(Bn, gamma)
+    q_tok = torch.gather(q, 2, x.unsqueeze(2)).squeeze(2).contiguous()
+    x = x.to(torch.int32)
+    u = torch.rand(Bn, gamma, generator=gen, device="cuda")
+    u_rs = torch.rand(Bn, generator=gen, device="cuda").clamp_(max=1.0 - 2.0 ** -24)
+    ev = B.dssd_edge_verify(tl, x, q_tok, u, T)
+    rs = B.dssd_device_resample(ev["p_row"], q, ev["accept_len"], u_rs, gamma)
+    got = B.dssd_dsd_verify(tl, q, x, u, u_rs, T)
+    torch.cuda.synchronize()
+    assert torch.equal(got["accept_len"], ev["accept_len"]) and torch.equal(got["token"], rs["token"])
+    assert torch.equal(got["rs_flags"], rs["flags"])
