@@ -103,10 +103,11 @@ struct Drafted {
     float z, q, u;  // its logit in the row, its draft probability, the position's uniform
 };
 
-// Run by all kThreads threads of a CTA; the results are in `sh` (n, ref2, invS) when it returns.
+// Run by all threads of a CTA, kCta of them (0: as many as were launched, 128 or at least kThreads); the results are in `sh` (n, ref2, invS)
+// when it returns.
 // `writer`: this CTA writes the sequence's accept_len, flags, lse, p_tok and `ready`.
 // part(i, k) gives the partial sum of run k of row i of the sequence, drafted(i) what belongs to position i.
-template <bool kWide, class Part, class Draft>
+template <bool kWide, int kCta, class Part, class Draft>
 __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh, Part part, Draft drafted)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -132,16 +133,20 @@ __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, 
                 }
             }
         } else {
-            const int r = base + tid / kFoldLanes;
-            float R;
-            double S;
-            bool missing;
-            row_total([&](int k) { return part(r, k); }, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, missing);
-            if (tid % kFoldLanes == 0) {
-                sh.R[tid / kFoldLanes] = R;
-                sh.S[tid / kFoldLanes] = S;
-                sh.missing[tid / kFoldLanes] = missing;
-            }
+            auto total = [&](int w) {
+                const int r = base + w;
+                float R;
+                double S;
+                bool missing;
+                row_total([&](int k) { return part(r, k); }, P.runs, tid % kFoldLanes, r <= P.gamma, R, S, missing);
+                if (tid % kFoldLanes == 0) {
+                    sh.R[w] = R;
+                    sh.S[w] = S;
+                    sh.missing[w] = missing;
+                }
+            };
+            if (kCta || tid < kThreads) total(tid / kFoldLanes);
+            if (!kCta && blockDim.x < kThreads && base + kFoldRows / 2 <= P.gamma) total(tid / kFoldLanes + kFoldRows / 2);  // 128 threads: half of the rows at a time
         }
         __syncthreads();
         if (warp == 0) {
@@ -186,7 +191,7 @@ template <bool kWide>
 __device__ __forceinline__ void fold_sequence(const EdgeParams &P, long long b, bool writer, FoldShared &sh)
 {
     const long long row0 = b * (P.gamma + 1);
-    fold_sequence<kWide>(P, b, writer, sh, [&](int i, int k) { return ld_after(P.part + (size_t)(row0 + i) * P.runs + k); },
+    fold_sequence<kWide, kThreads>(P, b, writer, sh, [&](int i, int k) { return ld_after(P.part + (size_t)(row0 + i) * P.runs + k); },
                   [&](int i) {
                       const size_t di = (size_t)b * P.gamma + i;
                       Drafted d;

@@ -370,10 +370,10 @@ __device__ __forceinline__ void emit_pieces(const char *rowp, OUT *outp, int V, 
 // the kernel of small draws does it, else in turns (draw_streamed).
 static_assert(kDrawSegs >= 2 * kEdgeClusterWide * kWarps, "draw_held keeps two sets of sums");
 template <int DT, bool kShift, bool kHeld>
-__device__ __forceinline__ void draw_here(const EdgeParams &P, long long b, const char *rowp, int n, float ref2, float invS, unsigned csize,
-                                          unsigned rank, DrawShared &sh)
+__device__ __forceinline__ void draw_here(const EdgeParams &P, long long b, const char *rowp, int n, float ref2, float invS, int n_warps,
+                                          unsigned csize, unsigned rank, DrawShared &sh)
 {
-    const int warp = threadIdx.x >> 5, n_warps = kWarps * (int)csize, g = warp * (int)csize + (int)rank;
+    const int warp = threadIdx.x >> 5, g = warp * (int)csize + (int)rank;
     const float *q = n < P.gamma ? P.draft_q_rows + ((size_t)b * P.gamma + n) * (size_t)P.V : nullptr;
     RowLogits<DT> row;
     row.row = rowp;
@@ -393,16 +393,17 @@ __device__ __forceinline__ void draw_here(const EdgeParams &P, long long b, cons
 // one cluster barrier every CTA folds the sequence for itself and emits its part of row n.  kDraw = 1, 2: the call wants
 // tokens too (of every sequence, or of the fully accepted ones); 2 holds the row in registers meanwhile, which
 // saves fetching a segment again (B = 8 V = 32000 fused 7.9 us against 8.6) but costs half of the CTAs per SM.
-template <int DT, bool kShift, int kDraw>
-__global__ void __launch_bounds__(kThreads, kDraw == 2 ? 2 : 4) edge_cluster_kernel(const __grid_constant__ EdgeParams P)
+// kCta: threads of a CTA, 0: as many as were launched (where they are known the shortest calls are 0.2 us shorter).
+template <int DT, bool kShift, int kDraw, int kCta>
+__global__ void __launch_bounds__(kCta ? kCta : kEdgeMostThreads, kDraw == 2 || !kCta ? 2 : 4) edge_cluster_kernel(const __grid_constant__ EdgeParams P)
 {
     __shared__ unsigned long long s_part[kEdgeClusterParts];
     __shared__ Drafted s_draft[kFoldRows];
     __shared__ FoldShared sh;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cta_warps = kCta ? kCta / 32 : (int)(blockDim.x >> 5);
     const unsigned csize = (unsigned)P.cluster, rank = csize > 1 ? cluster_rank() : 0u;
     const long long b = blockIdx.x / csize, row0 = b * (P.gamma + 1);
-    const int g = warp * (int)csize + (int)rank, n_warps = (int)csize * kWarps;
+    const int g = warp * (int)csize + (int)rank, n_warps = (int)csize * cta_warps;
     if (csize > 1) {  // a CTA's shared memory may be written once it is known to run
         cluster_arrive();
         cluster_wait();
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(kThreads, kDraw == 2 ? 2 : 4) edge_cluster_ker
     pdl_wait();
     pdl_trigger();
     // the last warp has the fewest segments: it looks the drafted tokens up
-    if (warp == kWarps - 1 && lane < P.gamma) {
+    if (warp == cta_warps - 1 && lane < P.gamma) {
         const size_t di = (size_t)b * P.gamma + lane;
         Drafted d;
         d.x = ld_after(P.draft_tokens + di);
@@ -437,12 +438,12 @@ __global__ void __launch_bounds__(kThreads, kDraw == 2 ? 2 : 4) edge_cluster_ker
     } else {
         __syncthreads();
     }
-    fold_sequence<false>(P, b, rank == 0, sh, [&](int i, int k) { return s_part[i * P.runs + k]; }, [&](int i) { return s_draft[i]; });
+    fold_sequence<false, kCta>(P, b, rank == 0, sh, [&](int i, int k) { return s_part[i * P.runs + k]; }, [&](int i) { return s_draft[i]; });
     const int n = sh.n;
     if (kDraw) {
         __shared__ DrawShared sd;
         if (n == P.gamma || (n >= 0 && P.draw_rejected)) {
-            draw_here<DT, kShift, kDraw == 2>(P, b, row_ptr<DT>(P, row0 + n), n, sh.ref2, sh.invS, csize, rank, sd);
+            draw_here<DT, kShift, kDraw == 2>(P, b, row_ptr<DT>(P, row0 + n), n, sh.ref2, sh.invS, n_warps, csize, rank, sd);
             return;
         }
         if (rank == 0 && threadIdx.x == 0) {  // no verdict, or a token that the device half draws
@@ -489,11 +490,11 @@ __global__ void __launch_bounds__(kThreads) edge_partial_kernel(const __grid_con
 }
 
 // The same in one launch, chosen as the cluster kernel is: the partial sums go to the first CTA's shared memory.
-template <int DT>
-__global__ void __launch_bounds__(kThreads, 4) edge_partial_cluster_kernel(const __grid_constant__ EdgeParams P)
+template <int DT, int kCta>
+__global__ void __launch_bounds__(kCta ? kCta : kEdgeMostThreads, kCta ? 4 : 2) edge_partial_cluster_kernel(const __grid_constant__ EdgeParams P)
 {
     __shared__ unsigned long long s_part[kEdgeClusterParts];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta_warps = kCta ? kCta / 32 : (int)(blockDim.x >> 5);
     const unsigned csize = (unsigned)P.cluster, rank = csize > 1 ? cluster_rank() : 0u;
     const long long b = blockIdx.x / csize, row0 = b * (P.gamma + 1);
     if (csize > 1) {  // the first CTA's shared memory may be written once it is known to run
@@ -502,12 +503,12 @@ __global__ void __launch_bounds__(kThreads, 4) edge_partial_cluster_kernel(const
     }
     pdl_wait();
     pdl_trigger();
-    if (rank == 0 && warp == kWarps - 1 && lane < P.gamma) {
+    if (rank == 0 && warp == cta_warps - 1 && lane < P.gamma) {
         const size_t di = (size_t)b * P.gamma + lane;
         const long long x = (long long)ld_after(P.draft_tokens + di) - (long long)P.v_begin;
         P.shard_tok_logit[di] = x >= 0 && x < (long long)P.V ? Elem<DT>::load(row_ptr<DT>(P, row0 + lane), x) : __int_as_float(0x7fc00000);
     }
-    for (int t = warp * (int)csize + (int)rank; t < P.runs * (P.gamma + 1); t += kWarps * (int)csize) {
+    for (int t = warp * (int)csize + (int)rank; t < P.runs * (P.gamma + 1); t += cta_warps * (int)csize) {
         const int i = t / P.runs;
         float R, s;
         warp_lse<DT>(row_ptr<DT>(P, row0 + i), P.V, t - i * P.runs, P.runs, P.c1, R, s);
@@ -524,15 +525,18 @@ __global__ void __launch_bounds__(kThreads, 4) edge_partial_cluster_kernel(const
         __syncthreads();
     }
     if (rank) return;
-    const int i = tid / kFoldLanes, sub = tid % kFoldLanes;
-    float R;
-    double S;
-    bool missing;
-    row_total([&](int k) { return s_part[i * P.runs + k]; }, P.runs, sub, i <= P.gamma, R, S, missing);
-    if (i <= P.gamma && sub == 0) {
-        P.shard_ref[row0 + i] = R == DSSD_NEG_INF ? 0.f : R;
-        P.shard_sum[row0 + i] = missing || S != S ? (double)__int_as_float(0x7fc00000) : S;
-    }
+    auto total = [&](int i) {
+        float R;
+        double S;
+        bool missing;
+        row_total([&](int k) { return s_part[i * P.runs + k]; }, P.runs, tid % kFoldLanes, i <= P.gamma, R, S, missing);
+        if (i <= P.gamma && tid % kFoldLanes == 0) {
+            P.shard_ref[row0 + i] = R == DSSD_NEG_INF ? 0.f : R;
+            P.shard_sum[row0 + i] = missing || S != S ? (double)__int_as_float(0x7fc00000) : S;
+        }
+    };
+    if (kCta || tid < kThreads) total(tid / kFoldLanes);
+    if (!kCta && blockDim.x < kThreads && kFoldRows / 2 <= P.gamma) total(tid / kFoldLanes + kFoldRows / 2);  // 128 threads: half of the rows at a time
 }
 
 }  // namespace
@@ -580,36 +584,45 @@ bool outputs_aligned(const EdgeParams &P)
     return emit_aligned(P.logits, P.row_stride, Elem<DT>::kBytes, P.p_row16 ? (const void *)P.p_row16 : P.p_row, P.V, P.p_row16 ? 2 : 4);
 }
 
-template <int DT, int kDraw>
+template <int DT, int kDraw, int kCta>
 cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 {
-    const unsigned grid = (unsigned)P.B * (unsigned)P.cluster;
+    const unsigned grid = (unsigned)P.B * (unsigned)P.cluster, threads = (unsigned)P.cta, cluster = (unsigned)P.cluster;
     const bool aligned = outputs_aligned<DT>(P) && (!P.draw_rejected || reinterpret_cast<uintptr_t>(P.draft_q_rows) % 16 == 0);
-    return aligned ? launch_pdl(edge_cluster_kernel<DT, false, kDraw>, grid, kThreads, stream, P, 0, (unsigned)P.cluster)
-                   : launch_pdl(edge_cluster_kernel<DT, true, kDraw>, grid, kThreads, stream, P, 0, (unsigned)P.cluster);
+    return launch_pdl(aligned ? edge_cluster_kernel<DT, false, kDraw, kCta> : edge_cluster_kernel<DT, true, kDraw, kCta>, grid, threads, stream, P, 0, cluster);
+}
+
+// does a launch of this shape that draws hold the row in registers?
+bool draws_held(const EdgeParams &P, int cta, long long cluster)
+{
+    return P.draw_token && cta == kThreads && P.B * cluster <= kEdgeHeldWave && P.V <= 512 * kWarps * cluster;
 }
 
 template <int DT>
 cudaError_t launch_cluster(const EdgeParams &P, cudaStream_t stream)
 {
+    const bool usual = P.cta == kThreads;
     if (P.shard_sum)
-        return launch_pdl(edge_partial_cluster_kernel<DT>, (unsigned)P.B * (unsigned)P.cluster, kThreads, stream, P, 0, (unsigned)P.cluster);
-    if (!P.draw_token) return launch_cluster<DT, 0>(P, stream);
-    const bool held = P.B * P.cluster <= kEdgeHeldWave && P.V <= 512 * kWarps * P.cluster;
-    return held ? launch_cluster<DT, 2>(P, stream) : launch_cluster<DT, 1>(P, stream);
+        return launch_pdl(usual ? edge_partial_cluster_kernel<DT, kThreads> : edge_partial_cluster_kernel<DT, 0>, (unsigned)P.B * (unsigned)P.cluster,
+                          (unsigned)P.cta, stream, P, 0, (unsigned)P.cluster);
+    if (!P.draw_token) return usual ? launch_cluster<DT, 0, kThreads>(P, stream) : launch_cluster<DT, 0, 0>(P, stream);
+    if (draws_held(P, P.cta, P.cluster)) return launch_cluster<DT, 2, kThreads>(P, stream);
+    return usual ? launch_cluster<DT, 1, kThreads>(P, stream) : launch_cluster<DT, 1, 0>(P, stream);
 }
 
-template <int DT, int kDraw>
+template <int DT, int kDraw, int kCta>
 bool wide_clusters()
 {
-    return allow_cluster(edge_cluster_kernel<DT, false, kDraw>, kEdgeClusterWide, kThreads) &&
-           allow_cluster(edge_cluster_kernel<DT, true, kDraw>, kEdgeClusterWide, kThreads);
+    const unsigned threads = kCta ? kCta : kEdgeMostThreads;
+    return allow_cluster(edge_cluster_kernel<DT, false, kDraw, kCta>, kEdgeClusterWide, threads) &&
+           allow_cluster(edge_cluster_kernel<DT, true, kDraw, kCta>, kEdgeClusterWide, threads);
 }
 template <int DT>
 bool wide_clusters()
 {
-    return wide_clusters<DT, 0>() && wide_clusters<DT, 1>() && wide_clusters<DT, 2>() &&
-           allow_cluster(edge_partial_cluster_kernel<DT>, kEdgeClusterWide, kThreads);
+    return wide_clusters<DT, 0, kThreads>() && wide_clusters<DT, 0, 0>() && wide_clusters<DT, 1, kThreads>() && wide_clusters<DT, 1, 0>() &&
+           wide_clusters<DT, 2, kThreads>() && allow_cluster(edge_partial_cluster_kernel<DT, kThreads>, kEdgeClusterWide, kThreads) &&
+           allow_cluster(edge_partial_cluster_kernel<DT, 0>, kEdgeClusterWide, kEdgeMostThreads);
 }
 int most_cluster_ctas()
 {
@@ -628,27 +641,55 @@ long long fit(long long c, long long wave, int B)
     return c < most ? c : most > 1 ? most : 1;
 }
 
-// CTAs per sequence of the cluster kernel, or 0 where the separate kernels are the better ones (edge_verify.h).
-int cluster_ctas(const EdgeParams &P, int esz, long long segs)
+// Threads per CTA and CTAs per sequence of the cluster kernel; false where the separate kernels are the better ones (edge_verify.h).
+bool cluster_shape(EdgeParams &P, int esz, long long segs)
 {
-    const long long parts = segs * (P.gamma + 1);
-    if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kDrawSegs)) return 0;
-    long long c = (parts + kWarps - 1) / kWarps;
-    c = fit(c, kEdgeWave, P.B);
+    const long long parts = segs * (P.gamma + 1), B = P.B;
+    if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kDrawSegs)) return false;
+    const long long pieces = P.p_row || P.p_row16 || P.draw_token ? ((long long)P.V + 511) / 512 : 0, units = parts > pieces ? parts : pieces;
+    const double work = (double)(parts * (esz == 2 ? 2 : 1) + pieces), draw = P.p_row && P.draw_token ? kEdgeDrawFactor : 1.0;
+    auto is = [&](int cta, long long cluster) {
+        P.cta = cta;
+        P.cluster = (int)cluster;
+        return true;
+    };
+    long long c = fit((units + kWarps - 1) / kWarps, kEdgeWave, P.B);
     if (c > 2) c = fit(c, kEdgeClusterWave, P.B);
+    if (c == 3 && B * c > kEdgeThreesWave) c = 2;
     if (c > kEdgeCluster) {
         const long long wide = fit(c, kEdgeWideWave, P.B);
         c = wide > kEdgeCluster ? wide : kEdgeCluster;
         if (c > kEdgeCluster && c > most_cluster_ctas()) c = most_cluster_ctas();
     }
-    const double work = (double)(parts * (esz == 2 ? 2 : 1)) + (P.p_row || P.p_row16 || P.draw_token ? (double)P.V / (128 * kPieceQuads) : 0.0);
+    if (c > 1 && 2 * c * B <= kEdgeSpread) {
+        const long long most = most_cluster_ctas() < kEdgeSpreadCtas ? most_cluster_ctas() : kEdgeSpreadCtas, twice = 2 * c < most ? 2 * c : most;
+        if (twice > c) c = twice;
+    }
+    if (units > kEdgeBigUnits && kWarps * c < units && !draws_held(P, kThreads, c)) {  // CTAs of 512 threads
+        for (const auto &big : kEdgeBig) {
+            if (B > big.most || (big.ctas > kEdgeCluster && most_cluster_ctas() < big.ctas)) continue;
+            const double fill = (double)(B * big.ctas) / 296.0;
+            if (2 * big.ctas > c && work <= (fill >= 0.8 ? 14.0 : fill >= 0.65 ? 7.0 : fill >= 0.5 ? 3.0 : 2.05) * draw * (double)(16 * big.ctas))
+                return is(kEdgeMostThreads, big.ctas);
+            break;
+        }
+    }
     if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
-    if (c > kEdgeCluster) return (int)c;
-    const long long ctas = P.B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
+    if (c > kEdgeCluster) return is(kThreads, c);
+    const bool held = draws_held(P, kThreads, c);
+    long long small = kEdgeSmallWave / B;  // CTAs of 128 threads
+    if (!held && units >= kEdgeSmallUnits && small >= 3 && small <= 6) {
+        if (small > (units + 3) / 4) small = (units + 3) / 4;
+        const double fill = (double)(B * small) / (double)(2 * kEdgeWave);
+        if (4 * small > kWarps * c)
+            return work <= (P.shard_sum ? 8.0 : draw * (fill >= 0.8 ? 25.0 : fill >= 0.65 ? 14.0 : 10.0)) * (double)(4 * small) ? is(128, small) : false;
+    }
+    const long long ctas = B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
     const double fill = (double)ctas / (double)(waves * kEdgeWave);
-    if (P.shard_sum) return work <= (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0) * (double)(kWarps * c) ? (int)c : 0;
-    const double limit = fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0;
-    return work <= limit * (double)(kWarps * c) ? (int)c : 0;
+    const double limit = P.shard_sum ? (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0)
+                                     : draw * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
+    if (work > limit * (double)(kWarps * c)) return false;
+    return c % 2 == 0 && ctas >= kEdgeEvenCtas && !P.draw_token ? is(kEdgeMostThreads, c / 2) : is(kThreads, c);
 }
 
 template <int DT>
@@ -684,8 +725,8 @@ cudaError_t edge_verify_launch(EdgeParams &P, int dtype, void *workspace, cudaSt
     P.c1 = (float)(1.4426950408889634 / (double)P.temperature);
     const long long nvec = (long long)P.V * esz / 16;
     const long long segs = nvec > kSegVecs ? (nvec + kSegVecs - 1) / kSegVecs : 1;
-    P.cluster = cluster_ctas(P, esz, segs);
-    if (P.cluster) {
+    P.cluster = 0;
+    if (cluster_shape(P, esz, segs)) {
         edge_workspace_layout(P.B, P.gamma, 1, &P, static_cast<char *>(workspace));  // (the partial sums stay on the chip)
         P.runs = (int)segs;
         return dtype == DSSD_BF16 ? launch_cluster<DSSD_BF16>(P, stream) : launch_cluster<DSSD_F32>(P, stream);

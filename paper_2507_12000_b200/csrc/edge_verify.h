@@ -23,26 +23,44 @@ constexpr unsigned long long kLseTwoTiles = 3000, kLseFourTiles = 19000;
 // more than a kernel that folds every sequence once (B = 256 V = 151936: emission 49.9 us against 3.1 + 36.5).
 constexpr unsigned long long kEmitFoldCtas = 592;
 
-// The cluster kernel does the log-sum-exps, the fold and the emission in one launch.  It takes as many CTAs per sequence as
-// have a segment (4 KB of logits) for each of their warps, as a cluster can have - eight, or sixteen while a warp's work
-// stays below kEdgeWideRounds - and as fit a wave: four CTAs per SM, somewhat less for clusters of three and more, which
-// do not pack the GPU's processing clusters completely (B = 113 V = 51071 float32, five each, 565 CTAs: 40.1 against 31.3
-// in separate kernels; B = 31 V = 33584, sixteen each, 496 CTAs: 11.1 against 9.3).  The unit of work is 1024 entries
-// summed or 512 emitted by a warp; how much of it per warp still pays depends on how full the wave is, since a
+// The cluster kernel does the log-sum-exps, the fold and the emission in one launch.  A unit of its work is a segment (4 KB) of
+// logits summed or a piece (512 entries) of the row emitted or drawn from by a warp.  It takes CTAs of 256 threads, as many per
+// sequence as give every warp one segment and one piece, as a cluster can have - eight, or sixteen while a warp's work stays
+// below kEdgeWideRounds - and as fit a wave: four CTAs per SM, somewhat less for clusters of three and more, which
+// do not pack the GPU's processing clusters completely and find no room while the kernel before drains.  From there:
+//   * Launches that leave most SMs idle spread over twice the CTAs, so that fewer warps share an SM (us per call, default / spread):
+//     B = 13 gamma = 7 V = 42256 / 8 bf16 3.07 / 2.63, B = 3 gamma = 15 V = 4160 bf16 4.50 / 4.23, B = 23 gamma = 8 V = 3200 4.49 / 4.21.
+//   * Sequences of more units than such a cluster has warps, few at a time: CTAs of 512 threads, as many as a wave has room for
+//     (kEdgeBig).  B = 3 gamma = 6 V = 37623 float32 7.0 / 7.3, B = 5 gamma = 11 V = 14300 float32 4.8 / 5.2, B = 45 gamma = 6 V = 127696
+//     bf16 25.3 / 29.4, with a draw B = 19 gamma = 7 V = 64337 float32 15.4 / 20.0, a round of B = 3 gamma = 1 V = 129584 float32 12.0 /
+//     12.5; beyond, B = 8 gamma = 5 V = 88369 float32 11.1 / 10.2, a round of B = 1 gamma = 8 V = 50272 float32 11.0 / 10.4.
+//     Not where CTAs of 256 hold the row that is drawn from: fused B = 1 gamma = 12 V = 13930 float32 8.4, of 512 9.9.
+//   * A batch that leaves each sequence one CTA and half of the SM's room idle: three to six of 128 threads (kEdgeSmallWave).  B = 332
+//     gamma = 13 V = 5816 float32 22.1 / 27.0, B = 303 gamma = 2 V = 24064 float32 22.5 / 25.6, B = 203 gamma = 10 V = 7680 float32 15.3 / 16.7.
+//   * Otherwise pairs of CTAs of a full launch are one of 512 threads, whose barrier is cheaper: B = 168 gamma = 7 V = 2048 float32 (a
+//     shard) 4.0 / 4.6, B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, B = 259 gamma = 3 V = 14848 float32 16.3 / 16.5.
+// How much work per warp still pays depends on how full the wave is, since a
 // warp's loads wait for one another from segment to segment and only other CTAs on the SM fill the gaps.  Measured (us per
 // call, cluster kernel / separate kernels):
-//   few CTAs:  B = 1 gamma = 8 V = 2176 bf16 4.2 / 6.1, B = 8 gamma = 4 V = 32000 bf16 4.8 / 6.5, B = 16 5.4 / 7.0;
-//              beyond the limits B = 1 gamma = 8 V = 50272 float32 7.9 / 5.7, B = 2 gamma = 9 V = 36496 float32 6.9 / 6.3
+//   few CTAs:  B = 1 gamma = 8 V = 2176 bf16 4.2 / 6.1, B = 8 gamma = 4 V = 32000 bf16 4.8 / 6.5, B = 16 5.4 / 7.0
 //   one CTA per sequence:  B = 520 gamma = 1 V = 1172 bf16 5.0 / 11.6, B = 979 gamma = 1 V = 4880 bf16 11.8 / 17.5,
 //              B = 318 gamma = 4 V = 9792 bf16 16.3 / 20.2; beyond B = 661 gamma = 1 V = 72431 bf16 110 / 86
 //   full wave:  B = 89 gamma = 4 V = 18896 float32 9.6 / 13.0, B = 64 gamma = 4 V = 128256 bf16 26.5 / 29.7,
 //              B = 128 gamma = 4 V = 50272 float32 30.7 / 32.3; beyond B = 166 gamma = 11 V = 53648 bf16 52.8 / 48.8.
 // A shard's partial sums have no emission to share a launch with and pay off up to less work per warp: B = 256 gamma = 4 V = 18992
 // bf16 13.5 / 14.2, B = 503 gamma = 3 V = 5936 float32 8.5 / 11.1, B = 620 gamma = 15 V = 792 bf16 9.7 / 28.4; beyond B = 173 gamma = 3
-// V = 67023 float32 40.5 / 30.5, B = 2 gamma = 2 V = 79648 float32 5.4 / 4.6.
+// V = 67023 float32 40.5 / 30.5, B = 2 gamma = 2 V = 79648 float32 5.4 / 4.6.  Where the edge draws bonus tokens the separate kernels are
+// five and the cluster kernel pays for longer (B = 33 gamma = 10 V = 32480 bf16 11.7 / 16.5).
 constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
-constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, more
-constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6;
+constexpr int kEdgeMostThreads = 512;                    // per CTA
+constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, three, more
+constexpr long long kEdgeSpread = 140, kEdgeSpreadCtas = 12;  // CTAs, in all and per sequence
+constexpr long long kEdgeBigUnits = 64;
+struct EdgeBig { long long most; int ctas; };             // up to so many sequences, so many CTAs of 512 threads each
+constexpr EdgeBig kEdgeBig[] = {{14, 16}, {19, 12}, {30, 8}, {45, 6}, {52, 5}};
+constexpr long long kEdgeSmallWave = 1110, kEdgeSmallUnits = 24;  // CTAs of 128 threads; units of a sequence
+constexpr long long kEdgeEvenCtas = 150;
+constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
 constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory; the limits on the work allow 900)
 
@@ -91,6 +109,7 @@ struct EdgeParams {
     int runs;                 // runs per row (one CTA of the log-sum-exp kernel each), segments in the cluster kernel
     int run_vecs;             // 16-byte vectors per run
     int cluster;              // CTAs per sequence of the cluster kernel (0: separate kernels)
+    int cta;                  // threads of each
     int emit_tiles;           // tiles (emission CTAs) per sequence
     // test hook (0: off): the partial sums of row test_drop_row_plus1 - 1 are formed but never stored
     long long test_drop_row_plus1;

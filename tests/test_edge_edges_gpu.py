@@ -86,6 +86,23 @@ def test_draws_in_the_same_launch(B, oracle_mod, dtype, Bn, gamma, V):
     compare_dsd(B, oracle_mod, d, w.temperature, threads=16)
 
 
+# Other CTAs than those of 256 threads: of 512 for sequences of many segments (at the batches where their number per sequence
+# changes) and for pairs in full launches, of 128 for batches that would leave a sequence one CTA; and launches that
+# spread over twice the CTAs; with and without a draw.
+@pytest.mark.parametrize("dtype,Bn,gamma,V", [
+    ("f32", 14, 6, 37623), ("bf16", 15, 8, 52000), ("f32", 19, 7, 20000), ("f32", 20, 7, 20001), ("f32", 30, 7, 17000), ("f32", 31, 7, 17003),
+    ("bf16", 45, 7, 40000), ("bf16", 46, 7, 40000), ("f32", 52, 8, 13000), ("f32", 53, 8, 13000), ("bf16", 1, 3, 80000),
+    ("bf16", 300, 4, 9792), ("f32", 332, 13, 5816), ("f32", 203, 10, 7681), ("bf16", 185, 7, 8193), ("f32", 371, 5, 4100),
+    ("bf16", 117, 2, 6656), ("bf16", 61, 11, 7500), ("f32", 259, 3, 14848), ("bf16", 3, 15, 4160), ("f32", 23, 7, 2286), ("bf16", 35, 1, 8200),
+])
+def test_other_cta_sizes(B, oracle_mod, dtype, Bn, gamma, V):
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.4, zipf=True, seed=V + Bn)
+    d = di.generate(w, threads=16)
+    compare_round(B, oracle_mod, d, w.temperature, threads=16)
+    compare_bonus(B, oracle_mod, d, w.temperature, threads=16)
+    compare_dsd(B, oracle_mod, d, w.temperature, threads=16)
+
+
 @pytest.mark.parametrize("dtype,V,stride", [("bf16", 4096, 1), ("bf16", 40000, 97), ("f32", 4096, 1)])
 def test_every_entry_of_a_vector_counts(B, dtype, V, stride):
     """Some terms of a row's sum are formed by a polynomial, the others by the special-function unit: a NaN is seen in
