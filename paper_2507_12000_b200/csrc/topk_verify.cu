@@ -620,7 +620,11 @@ __device__ __forceinline__ unsigned long long merge_many(const unsigned long lon
 // The same where the keys fit a warp's registers and k is small: the largest of the lists' last keys is bound enough (7 runs,
 // k = 5, B = 32 gamma = 4 V = 50257 bf16: the edge call 10.2 us, with merge_many 11.9; k = 32: 19.1 and 14.4).
 // Up to kMergeSmall keys at any k: 4 runs, k = 20, a round of B = 112 gamma = 7 V = 25792 bf16 23.5 us, with merge_many 25.4.
+// kFewRegs, where a kernel has 64 registers: the lists' ends are fetched one turn after the other (there is more than one turn from
+// 33 runs on only); four turns at once cost it 52 bytes of spills (B = 1024 gamma = 4 V = 8192 k = 20: the edge call 37.5 us, now 36.3;
+// B = 1000 gamma = 4 V = 16384 k = 4 59.4 and 58.1), but leave the kernels of 128 registers a shorter chain.
 constexpr int kMergeFew = 256, kMergeSmall = 96;
+template <bool kFewRegs>
 __device__ __forceinline__ unsigned long long merge_few(const unsigned long long *src, int runs, int k, MergeShared &sh)
 {
     const int lane = threadIdx.x & 31, m = runs * k;
@@ -630,7 +634,12 @@ __device__ __forceinline__ unsigned long long merge_few(const unsigned long long
     for (int u = 0; u < 8; ++u) x[u] = 32 * u + lane < m ? ld_after(src + 32 * u + lane) : 0ull;
     // the logit of the largest last key is bound enough, and one instruction finds it (an empty slot has none)
     uint32_t top = 0u;
-    for (int r = lane; r < runs; r += 32) top = max(top, (uint32_t)(ld_after(src + (size_t)r * k + k - 1) >> 32));
+    if constexpr (kFewRegs) {
+#pragma unroll 1
+        for (int r = lane; r < runs; r += 32) top = max(top, (uint32_t)(ld_after(src + (size_t)r * k + k - 1) >> 32));
+    } else {
+        for (int r = lane; r < runs; r += 32) top = max(top, (uint32_t)(ld_after(src + (size_t)r * k + k - 1) >> 32));
+    }
     top = __reduce_max_sync(kFullMask, top);
     if (top == (uint32_t)(kBadList >> 32)) return lane == 0 ? kBadList : 0ull;
     // no list is full: every key counts, empty slots do not
@@ -670,7 +679,7 @@ __device__ __forceinline__ bool judge(const TopkParams &P, const RowDist &d, int
 
 // One row, by a warp: its support's distribution from the lists of its runs (their merged keys in `key`), the acceptance test if
 // a token was drafted for it.  Bit 0 of the result: accepted, flag bits from bit 8 on.
-template <bool kMany>
+template <bool kMany, bool kFewRegs>
 __device__ __forceinline__ unsigned fold_row(const TopkParams &P, int b, int j, MergeShared &sh, RowDist &d, unsigned long long &key)
 {
     const int lane = threadIdx.x & 31, k = P.k;
@@ -683,7 +692,7 @@ __device__ __forceinline__ unsigned fold_row(const TopkParams &P, int b, int j, 
         q = ld_after(P.draft_q_tok + o);
     }
     const unsigned long long *lists = P.lists + ((size_t)b * (P.gamma + 1) + j) * P.runs * k;
-    key = P.runs == 1 ? (lane < k ? ld_after(lists + lane) : 0ull) : kMany ? merge_many(lists, P.runs, k, sh) : merge_few(lists, P.runs, k, sh);
+    key = P.runs == 1 ? (lane < k ? ld_after(lists + lane) : 0ull) : kMany ? merge_many(lists, P.runs, k, sh) : merge_few<kFewRegs>(lists, P.runs, k, sh);
     d = dist_from_keys(P, key);
     unsigned fl = d.bad ? DSSD_EDGE_FLAG_NONFINITE : 0u;
     bool accept = true;
@@ -728,7 +737,7 @@ __global__ void __launch_bounds__(32 * kFoldWarps, kCtas) topk_fold_kernel(const
         unsigned mine = 1u;
         if (j < rows) {
             unsigned long long key;
-            mine = fold_row<kMany>(P, b, j, merge[warp], d, key);
+            mine = fold_row<kMany, (kCtas > 1)>(P, b, j, merge[warp], d, key);
         }
         if (lane == 0) s_verdict[warp] = mine;
         __syncthreads();
@@ -762,7 +771,7 @@ __global__ void __launch_bounds__(32 * kFoldWarps, 1) topk_rows_kernel(const __g
     const int b = (int)(row / (P.gamma + 1)), j = (int)(row - (long long)b * (P.gamma + 1));
     RowDist d;
     unsigned long long key;
-    const unsigned verdict = fold_row<kMany>(P, b, j, merge[warp], d, key);
+    const unsigned verdict = fold_row<kMany, false>(P, b, j, merge[warp], d, key);
     if (lane < P.k) P.lists[(size_t)row * P.runs * P.k + lane] = key;
     if (lane == 0) P.verdict[row] = verdict;
 }
