@@ -18,8 +18,8 @@
 // one entry per thread and step, cutting the buffer back to its k best whenever it fills: slow, never wrong.
 // The end of a kernel is the only synchronisation; nothing in the workspace has to be cleared.
 //
-// Device kernel: one warp per sequence, everything in registers and shuffles, float64 sums in a fixed order, so that the
-// draw is reproducible bit for bit.
+// Device kernel: one warp per sequence, everything in registers and shuffles, sums strictly
+// sequential in float64 so that the draw is reproducible bit for bit.
 #include "topk_verify.h"
 
 #include <math.h>
@@ -432,8 +432,8 @@ __global__ void __launch_bounds__(kSelThreads, 10) topk_select_kernel(const __gr
     }
 }
 
-// Sums over k lanes: up to this k one after the other, beyond by halves, a chain of five additions with two shuffles each (with the other
-// changes of chains below, a round of B = 1 gamma = 8 V = 50272 float32 k = 10 10.5 us, one after the other 11.04).
+// The sum of a row's weights: up to this k one after the other, beyond by halves, a chain of five additions with two shuffles each (the
+// edge call at B = 1 gamma = 8 V = 50272 float32 k = 10 7.8 us; 8.1 with this sum one after the other and with the other chains below as they were).
 constexpr int kChain = 8;
 
 struct RowDist {   // per lane r < k: entry r of the row's support, best first
@@ -806,30 +806,25 @@ __global__ void __launch_bounds__(kThreads) topk_first_kernel(const __grid_const
 __device__ __forceinline__ double shfl_f64(double v, int src) { return __shfl_sync(kFullMask, v, src); }
 
 // inverse CDF over the warp's k entries (lane e holds r_e, entries in increasing index);
-// returns the position, or -1 when the mass is not positive and finite
+// returns the position, or -1 when the mass is not positive and finite.  The sums are those of a loop over the entries, as dssd.h
+// says; the shuffles of eight entries are on their way at a time (the draw at k = 10 2.00 us, four at a time 2.13; at k = 32 2.30.
+// Sums by halves, 2.16 and 2.17, are other sums: entries of far smaller weight than the one before them count there).
 __device__ __forceinline__ int warp_inverse_cdf(double r, int k, double u)
 {
     const int lane = threadIdx.x & 31;
     double C = 0.0, mine = 0.0;  // the running mass in index order (lanes beyond k hold 0); this lane's
-    if (k > kChain) {
-        mine = r;
+    for (int e0 = 0; e0 < k; e0 += 8) {
+        double v[8];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double up = __shfl_up_sync(kFullMask, mine, o);
-            if (lane >= o) mine += up;
-        }
-        C = shfl_f64(mine, 31);
-    } else {
-        for (int e0 = 0; e0 < k; e0 += 4) {
+        for (int j = 0; j < 8; ++j) v[j] = shfl_f64(r, e0 + j);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                C += shfl_f64(r, e0 + j);
-                if (lane == e0 + j) mine = C;
-            }
+        for (int j = 0; j < 8; ++j) {
+            C += v[j];
+            if (lane == e0 + j) mine = C;
         }
     }
     if (!(C > 0.0) || !(C < INFINITY)) return -1;
-    const unsigned hit = __ballot_sync(kFullMask, r > 0.0 && mine > u * C);  // (not an entry without mass whose sum was rounded up)
+    const unsigned hit = __ballot_sync(kFullMask, lane < k && mine > u * C);
     const unsigned positive = __ballot_sync(kFullMask, r > 0.0);
     return hit ? __ffs(hit) - 1 : 31 - __clz(positive);
 }

@@ -101,3 +101,36 @@ def test_many_positions(B, oracle_mod, Bn, gamma, V, k):
     d["target_logits"][0, gamma // 2, 7] = np.nan
     d["draft_tokens"][-1, -1] = V
     compare_topk(B, oracle_mod, d, w.temperature, k)
+
+
+@pytest.mark.parametrize("k", [4, 8, 9, 10, 17, 31, 32])
+def test_draw_sums_in_index_order(B, oracle_mod, k):
+    """The draw's sums are those of a loop over the entries in index order, bit for bit, bonus and residual: entries so much smaller than
+    the sum before them that sums in another order end elsewhere, and uniforms on the steps of the distribution."""
+    import torch
+
+    Bn, gamma = 512, 1
+    rng = np.random.default_rng(k)
+    p = np.ldexp(rng.uniform(0.5, 1.0, (Bn, k)), -rng.integers(0, 64, (Bn, k))).astype(np.float32)
+    p[0], p[1] = 2.0 ** -55, 2.0 ** -54
+    p[:2, 0] = p[:2, k - 1] = 0.5  # (sum 1; the entries between weigh nothing one by one)
+    idx = np.sort(np.stack([rng.choice(100000, k, replace=False) for _ in range(Bn)]), axis=1).astype(np.int32)
+    n = (np.arange(Bn) % 3 != 2).astype(np.int32) * gamma  # a third of them residual draws, from q = 0 but for one entry
+    q_idx, q_val = np.full((Bn, gamma, k), 200000, np.int32), np.zeros((Bn, gamma, k), np.float32)
+    q_idx[:, 0, 0], q_val[:, 0, 0] = idx[:, k // 2], 0.25 * p[:, k // 2]
+    r = np.where((n[:, None] < gamma) & (np.arange(k) == k // 2), 0.75, 1.0) * p.astype(np.float64)
+    C = np.zeros((Bn, k))
+    s = np.zeros(Bn)
+    for e in range(k):
+        s = s + r[:, e]
+        C[:, e] = s
+    u = np.minimum(C[np.arange(Bn), rng.integers(0, k, Bn)] / s, 1 - 2.0 ** -24).astype(np.float32)
+    u[:2] = 0.5
+    over = C > (u.astype(np.float64) * s)[:, None]
+    want = np.where(over.any(axis=1), idx[np.arange(Bn), over.argmax(axis=1)], idx[:, k - 1])
+    ref = oracle_mod.device_resample_topk(idx, p, q_idx, q_val, n, u, gamma)
+    assert (ref["token"] == want).all()
+    up = lambda a: torch.from_numpy(a).cuda()
+    got = B.dssd_device_resample_topk(up(idx), up(p), up(q_idx), up(q_val), up(n), up(u), gamma)
+    torch.cuda.synchronize()
+    assert (got["token"].cpu().numpy() == want).all()
