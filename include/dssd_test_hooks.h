@@ -1,12 +1,13 @@
 /*
  * dssd_test_hooks.h - entry points for the library's own tests.  NOT part of the product API:
  * they exist so that a sum that a kernel hands on can be made to go missing on purpose, in
- * a way that cannot hang or fault a GPU, and the outcome be checked.  (The paper has no
+ * a way that cannot hang or fault a GPU, and the outcome be checked, and so that the choice of a
+ * kernel by size can be looked at.  (The paper has no
  * counterpart: its link model of Section 2.2 has no loss or failure term.)
  *
  * The dense kernels hand sums on from one launch to the next; a sum that has not arrived is reported
  * per sequence (DSSD_EDGE_FLAG_TIMEOUT with accept_len = -1, DSSD_RS_FLAG_TIMEOUT |
- * DSSD_RS_FLAG_INVALID with token = -1) and the kernel ends normally.  The two calls below provoke
+ * DSSD_RS_FLAG_INVALID with token = -1) and the kernel ends normally.  The first two calls below provoke
  * exactly that by withholding ONE store; nothing else about the launch changes, no address is wrong
  * and nothing waits without a bound.
  */
@@ -49,6 +50,15 @@ dssd_status dssd_test_device_resample_wait_runs_out(const float *p_row, const fl
                                                     void *workspace, size_t workspace_bytes,
                                                     int drop_seq, unsigned poll_limit,
                                                     void *cuda_stream);
+
+/*
+ * Which kernels a call of these sizes takes on a device that has clusters of sixteen CTAs: threads per CTA and CTAs per
+ * sequence of the kernel that does it in one launch, 0 and 0 where several do it.  They need no GPU.
+ *   edge: form 0 dssd_edge_verify, 1 dssd_edge_verify_bonus, 2 dssd_dsd_verify, 3 dssd_edge_partial of a slice of V entries
+ *   draw: dssd_device_resample of float32 rows on 16-byte boundaries; *turns = 1 where the kernel goes over the row in turns
+ */
+void dssd_test_edge_shape(dssd_dtype dtype, int form, int B, int gamma, int V, int *threads, int *ctas);
+void dssd_test_draw_shape(int B, int V, int *threads, int *ctas, int *turns);
 
 #ifdef __cplusplus
 }

@@ -129,6 +129,35 @@ dssd_status dssd_test_edge_verify_wait_runs_out(const void *target_logits, dssd_
                            drop_row + 1);
 }
 
+void dssd_test_edge_shape(dssd_dtype dtype, int form, int B, int gamma, int V, int *threads, int *ctas)
+{
+    static float word;  // (only whether a pointer is set matters)
+    static double sum;
+    static int32_t token;
+    dssd::EdgeParams P{};
+    P.B = B;
+    P.gamma = gamma;
+    P.V = V;
+    if (form == 3) P.shard_sum = &sum;
+    if (form <= 1) P.p_row = &word;
+    if (form == 1 || form == 2) P.draw_token = &token;
+    if (form == 2) P.draw_rejected = 1, P.draft_q_rows = &word;
+    dssd::edge_shape_chosen(P, (int)dtype);
+    *threads = P.cta;
+    *ctas = P.cluster;
+}
+
+void dssd_test_draw_shape(int B, int V, int *threads, int *ctas, int *turns)
+{
+    dssd::ResampleParams P{};
+    P.B = B;
+    P.V = V;
+    dssd::resample_shape_chosen(P, V % 4 == 0);
+    *threads = P.cluster_threads;
+    *ctas = P.n_ctas;
+    *turns = P.streamed;
+}
+
 dssd_status dssd_edge_verify(const void *target_logits, dssd_dtype dtype, int64_t row_stride,
                              const int32_t *draft_tokens, const float *draft_q_tok,
                              const float *uniforms, float temperature, int B, int gamma, int V,

@@ -633,7 +633,8 @@ int most_cluster_ctas()
 }
 
 // Threads and CTAs per sequence of the kernels that draw in one launch; false where the two kernels are the better ones.
-bool one_launch(ResampleParams &P, bool aligned)
+template <class Most>
+bool one_launch(ResampleParams &P, bool aligned, Most most_cluster_ctas)
 {
     const int segs = (P.V + 511) / 512;
     const long long B = P.B;
@@ -678,11 +679,18 @@ cudaError_t launch_resample(ResampleParams &P, unsigned grid, cudaStream_t strea
 {
     const bool aligned = (P.logits ? quads_aligned(P.logits, P.row_stride, RV::Q::kBytes) : quads_aligned(P.p_row, P.V, RV::Q::kBytes)) &&
                          (!P.draft_q || quads_aligned(P.draft_q, P.V, 4));
-    if (!P.test_drop_seq_plus1) one_launch(P, aligned);
+    if (!P.test_drop_seq_plus1) one_launch(P, aligned, most_cluster_ctas);
     return aligned ? launch_resample_as<RV, false>(P, grid, stream) : launch_resample_as<RV, true>(P, grid, stream);
 }
 
 }  // namespace
+
+void resample_shape_chosen(ResampleParams &P, bool aligned)
+{
+    P.cluster_threads = P.n_ctas = 0;
+    P.streamed = false;
+    one_launch(P, aligned, [] { return kClusterWide; });
+}
 
 cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t stream)
 {

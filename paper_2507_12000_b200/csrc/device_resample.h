@@ -46,6 +46,10 @@ size_t resample_workspace_layout(int B, int V, ResampleParams *P, char *base);
 
 cudaError_t resample_launch(ResampleParams &P, void *workspace, cudaStream_t stream);
 
+// The shape (cluster_threads, n_ctas, streamed) of the kernel that draws in one launch where clusters of sixteen CTAs are to be had; 0
+// threads: two kernels.  For the tests.
+void resample_shape_chosen(ResampleParams &P, bool aligned);
+
 // ---- one shard of the vocabulary (entries v_begin .. v_begin + V - 1 of every row) ----
 struct ShardResampleParams {
     const float *p_row;     // [B, V] this shard's slice of row P_n, p_stride elements between rows

@@ -642,7 +642,8 @@ long long fit(long long c, long long wave, int B)
 }
 
 // Threads per CTA and CTAs per sequence of the cluster kernel; false where the separate kernels are the better ones (edge_verify.h).
-bool cluster_shape(EdgeParams &P, int esz, long long segs)
+template <class Most>
+bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_ctas)
 {
     const long long parts = segs * (P.gamma + 1), B = P.B;
     if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kDrawSegs)) return false;
@@ -669,7 +670,7 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs)
         for (const auto &big : kEdgeBig) {
             if (B > big.most || (big.ctas > kEdgeCluster && most_cluster_ctas() < big.ctas)) continue;
             const double fill = (double)(B * big.ctas) / 296.0;
-            if (2 * big.ctas > c && work <= (fill >= 0.8 ? 14.0 : fill >= 0.65 ? 7.0 : fill >= 0.5 ? 3.0 : 2.05) * draw * (double)(16 * big.ctas))
+            if (P.shard_sum ? 2 * big.ctas > c && work <= big.shard * (double)(16 * big.ctas) : 2 * big.ctas > c && work <= (fill >= 0.8 ? 14.0 : fill >= 0.65 ? 7.0 : fill >= 0.5 ? 3.0 : 2.05) * draw * (double)(16 * big.ctas))
                 return is(kEdgeMostThreads, big.ctas);
             break;
         }
@@ -690,6 +691,12 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs)
                                      : draw * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
     if (work > limit * (double)(kWarps * c)) return false;
     return c % 2 == 0 && ctas >= kEdgeEvenCtas && !P.draw_token ? is(kEdgeMostThreads, c / 2) : is(kThreads, c);
+}
+
+long long row_segments(int V, int esz)
+{
+    const long long nvec = (long long)V * esz / 16;
+    return nvec > kSegVecs ? (nvec + kSegVecs - 1) / kSegVecs : 1;
 }
 
 template <int DT>
@@ -718,15 +725,22 @@ cudaError_t launch_edge(EdgeParams &P, unsigned lse_ctas, cudaStream_t stream)
 
 }  // namespace
 
+void edge_shape_chosen(EdgeParams &P, int dtype)
+{
+    const int esz = dtype == DSSD_BF16 ? 2 : 4;
+    P.cta = P.cluster = 0;
+    if (!cluster_shape(P, esz, row_segments(P.V, esz), [] { return kEdgeClusterWide; })) P.cta = P.cluster = 0;
+}
+
 cudaError_t edge_verify_launch(EdgeParams &P, int dtype, void *workspace, cudaStream_t stream)
 {
     const int esz = dtype == DSSD_BF16 ? 2 : 4;
     const unsigned long long rows = (unsigned long long)P.B * (unsigned long long)(P.gamma + 1);
     P.c1 = (float)(1.4426950408889634 / (double)P.temperature);
     const long long nvec = (long long)P.V * esz / 16;
-    const long long segs = nvec > kSegVecs ? (nvec + kSegVecs - 1) / kSegVecs : 1;
+    const long long segs = row_segments(P.V, esz);
     P.cluster = 0;
-    if (cluster_shape(P, esz, segs)) {
+    if (cluster_shape(P, esz, segs, most_cluster_ctas)) {
         edge_workspace_layout(P.B, P.gamma, 1, &P, static_cast<char *>(workspace));  // (the partial sums stay on the chip)
         P.runs = (int)segs;
         return dtype == DSSD_BF16 ? launch_cluster<DSSD_BF16>(P, stream) : launch_cluster<DSSD_F32>(P, stream);

@@ -47,7 +47,10 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //              B = 318 gamma = 4 V = 9792 bf16 16.3 / 20.2; beyond B = 661 gamma = 1 V = 72431 bf16 110 / 86
 //   full wave:  B = 89 gamma = 4 V = 18896 float32 9.6 / 13.0, B = 64 gamma = 4 V = 128256 bf16 26.5 / 29.7,
 //              B = 128 gamma = 4 V = 50272 float32 30.7 / 32.3; beyond B = 166 gamma = 11 V = 53648 bf16 52.8 / 48.8.
-// A shard's partial sums have no emission to share a launch with and pay off up to less work per warp: B = 256 gamma = 4 V = 18992
+// A shard's partial sums have no emission to share a launch with and pay off up to less work per warp, in clusters of up to sixteen CTAs of
+// 512 threads about a segment each (the call, in one launch / separate kernels: B = 5 gamma = 6 V = 18928 float32 3.5 / 3.9, B = 48 gamma = 4 V = 26416
+// bf16 5.1 / 5.8; beyond, B = 1 gamma = 8 V = 50272 float32 5.2 / 3.7, B = 19 gamma = 8 V = 50272 11.5 / 9.5, B = 40 gamma = 16 V = 76000 bf16 25.0 / 22.6),
+// in smaller ones more: B = 256 gamma = 4 V = 18992
 // bf16 13.5 / 14.2, B = 503 gamma = 3 V = 5936 float32 8.5 / 11.1, B = 620 gamma = 15 V = 792 bf16 9.7 / 28.4; beyond B = 173 gamma = 3
 // V = 67023 float32 40.5 / 30.5, B = 2 gamma = 2 V = 79648 float32 5.4 / 4.6.  Where the edge draws bonus tokens the separate kernels are
 // five and the cluster kernel pays for longer (B = 33 gamma = 10 V = 32480 bf16 11.7 / 16.5).
@@ -56,8 +59,8 @@ constexpr int kEdgeMostThreads = 512;                    // per CTA
 constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, three, more
 constexpr long long kEdgeSpread = 140, kEdgeSpreadCtas = 12;  // CTAs, in all and per sequence
 constexpr long long kEdgeBigUnits = 64;
-struct EdgeBig { long long most; int ctas; };             // up to so many sequences, so many CTAs of 512 threads each
-constexpr EdgeBig kEdgeBig[] = {{14, 16}, {19, 12}, {30, 8}, {45, 6}, {52, 5}};
+struct EdgeBig { long long most; int ctas; double shard; };  // up to so many sequences, so many CTAs of 512 threads each; work per warp of a shard
+constexpr EdgeBig kEdgeBig[] = {{14, 16, 1.05}, {19, 12, 1.05}, {30, 8, 1.05}, {45, 6, 3.0}, {52, 5, 3.0}};
 constexpr long long kEdgeSmallWave = 1110, kEdgeSmallUnits = 24;  // CTAs of 128 threads; units of a sequence
 constexpr long long kEdgeEvenCtas = 150;
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;
@@ -122,6 +125,10 @@ struct EdgeParams {
 
 // Most runs a row can have for a vocabulary of V entries (any dtype, any launch size).
 int edge_max_runs_per_row(int V);
+
+// Threads per CTA and CTAs per sequence (P.cta, P.cluster) of the kernel that a call takes where clusters of sixteen CTAs are to be had;
+// 0, 0: the separate kernels.  For the tests.
+void edge_shape_chosen(EdgeParams &P, int dtype);
 
 // Carves the workspace for `runs_per_row` partial slots per row; returns the bytes needed.
 // With P == nullptr only computes the size.
