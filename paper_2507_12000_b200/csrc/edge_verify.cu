@@ -648,7 +648,8 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
     const long long parts = segs * (P.gamma + 1), B = P.B;
     if (P.gamma >= kFoldRows || parts > kEdgeClusterParts || (P.draw_token && P.V > 512 * kDrawSegs)) return false;
     const long long pieces = P.p_row || P.p_row16 || P.draw_token ? ((long long)P.V + 511) / 512 : 0, units = parts > pieces ? parts : pieces;
-    const double work = (double)(parts * (esz == 2 ? 2 : 1) + pieces), draw = P.p_row && P.draw_token ? kEdgeDrawFactor : 1.0;
+    const bool both = P.p_row && P.draw_token;
+    const double work = (double)(parts * (esz == 2 ? 2 : 1)) + (pieces ? (double)P.V / 512.0 : 0.0), draw = both ? kEdgeDrawFactor : 1.0;
     auto is = [&](int cta, long long cluster) {
         P.cta = cta;
         P.cluster = (int)cluster;
@@ -666,18 +667,18 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
         const long long most = most_cluster_ctas() < kEdgeSpreadCtas ? most_cluster_ctas() : kEdgeSpreadCtas, twice = 2 * c < most ? 2 * c : most;
         if (twice > c) c = twice;
     }
-    if (units > kEdgeBigUnits && kWarps * c < units && !draws_held(P, kThreads, c)) {  // CTAs of 512 threads
+    if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
+    const bool held = draws_held(P, kThreads, c), draw_only = P.draw_token && !P.p_row;
+    if (units > kEdgeBigUnits && kWarps * c < units && !held && (c <= kEdgeCluster || !draw_only)) {  // CTAs of 512 threads
         for (const auto &big : kEdgeBig) {
-            if (B > big.most || (big.ctas > kEdgeCluster && most_cluster_ctas() < big.ctas)) continue;
-            const double fill = (double)(B * big.ctas) / 296.0;
-            if (P.shard_sum ? 2 * big.ctas > c && work <= big.shard * (double)(16 * big.ctas) : 2 * big.ctas > c && work <= (fill >= 0.8 ? 14.0 : fill >= 0.65 ? 7.0 : fill >= 0.5 ? 3.0 : 2.05) * draw * (double)(16 * big.ctas))
+            if (B > (P.draw_token ? big.most_draw : big.most) || (big.ctas > kEdgeCluster && most_cluster_ctas() < big.ctas)) continue;
+            const double warps = (double)(16 * big.ctas), limit = P.shard_sum ? big.shard : both ? big.both : draw_only ? big.draw : big.row;
+            if (2 * big.ctas > c && work <= limit * warps && (B > kEdgeBigAlone || (double)parts <= (both ? 1.25 : 1.0) * warps))
                 return is(kEdgeMostThreads, big.ctas);
             break;
         }
     }
-    if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
     if (c > kEdgeCluster) return is(kThreads, c);
-    const bool held = draws_held(P, kThreads, c);
     long long small = kEdgeSmallWave / B;  // CTAs of 128 threads
     if (!held && units >= kEdgeSmallUnits && small >= 3 && small <= 6) {
         if (small > (units + 3) / 4) small = (units + 3) / 4;

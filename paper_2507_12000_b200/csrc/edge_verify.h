@@ -30,10 +30,15 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 // do not pack the GPU's processing clusters completely and find no room while the kernel before drains.  From there:
 //   * Launches that leave most SMs idle spread over twice the CTAs, so that fewer warps share an SM (us per call, default / spread):
 //     B = 13 gamma = 7 V = 42256 / 8 bf16 3.07 / 2.63, B = 3 gamma = 15 V = 4160 bf16 4.50 / 4.23, B = 23 gamma = 8 V = 3200 4.49 / 4.21.
-//   * Sequences of more units than such a cluster has warps, few at a time: CTAs of 512 threads, as many as a wave has room for
-//     (kEdgeBig).  B = 3 gamma = 6 V = 37623 float32 7.0 / 7.3, B = 5 gamma = 11 V = 14300 float32 4.8 / 5.2, B = 45 gamma = 6 V = 127696
-//     bf16 25.3 / 29.4, with a draw B = 19 gamma = 7 V = 64337 float32 15.4 / 20.0, a round of B = 3 gamma = 1 V = 129584 float32 12.0 /
-//     12.5; beyond, B = 8 gamma = 5 V = 88369 float32 11.1 / 10.2, a round of B = 1 gamma = 8 V = 50272 float32 11.0 / 10.4.
+//   * Sequences of more units than such a cluster has warps, few at a time: CTAs of 512 threads, as many as a wave has room for, while
+//     a warp's work stays below kEdgeBig's.  Up to eight sequences leave SMs idle that the separate kernels use, and pay
+//     only up to a segment per warp: B = 2 gamma = 11 V = 25408 bf16 5.4 / 6.4, B = 6 gamma = 2 V = 53913 float32 6.5 / 7.6; beyond, B = 1 gamma = 7
+//     V = 50272 float32 6.7 / 5.6, B = 8 gamma = 7 V = 50272 8.3 / 7.5, a round of B = 1 gamma = 8 V = 50272 11.1 / 10.35.  More sequences, 16 CTAs: B = 14
+//     gamma = 2 V = 83517 float32 8.5 / 10.2; beyond, B = 12 gamma = 5 V = 90108 bf16 9.7 / 8.7; 12 CTAs: B = 18 gamma = 11 V = 34312 float32 10.6 / 11.4;
+//     beyond, B = 19 gamma = 8 V = 100000 bf16 15.2 / 14.0; 8: B = 29 gamma = 3 V = 63728 float32 10.4 / 11.5; beyond, B = 30 gamma = 11 V = 100000 bf16
+//     23.3 / 21.1; 6: B = 45 gamma = 6 V = 127696 bf16 25.4 / 29.8, B = 41 gamma = 6 V = 75163 17.1 / 17.9; 5: B = 48 gamma = 6 V = 115296 float32 34.4 / 35.3.  With
+//     a draw as well (five separate kernels): B = 7 gamma = 1 V = 128512 float32 10.0 / 13.7, B = 27 gamma = 2 V = 64064 bf16 10.0 / 14.0; beyond, B = 1 gamma = 4
+//     V = 121880 float32 9.3 / 7.9.  A draw alone: B = 17 gamma = 6 V = 54992 float32 13.7 / 16.3; beyond, B = 44 gamma = 14 V = 57719 float32 41.8 / 38.3.
 //     Not where CTAs of 256 hold the row that is drawn from: fused B = 1 gamma = 12 V = 13930 float32 8.4, of 512 9.9.
 //   * A batch that leaves each sequence one CTA and half of the SM's room idle: three to six of 128 threads (kEdgeSmallWave).  B = 332
 //     gamma = 13 V = 5816 float32 22.1 / 27.0, B = 303 gamma = 2 V = 24064 float32 22.5 / 25.6, B = 203 gamma = 10 V = 7680 float32 15.3 / 16.7.
@@ -59,8 +64,14 @@ constexpr int kEdgeMostThreads = 512;                    // per CTA
 constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, three, more
 constexpr long long kEdgeSpread = 140, kEdgeSpreadCtas = 12;  // CTAs, in all and per sequence
 constexpr long long kEdgeBigUnits = 64;
-struct EdgeBig { long long most; int ctas; double shard; };  // up to so many sequences, so many CTAs of 512 threads each; work per warp of a shard
-constexpr EdgeBig kEdgeBig[] = {{14, 16, 1.05}, {19, 12, 1.05}, {30, 8, 1.05}, {45, 6, 3.0}, {52, 5, 3.0}};
+struct EdgeBig {  // up to so many sequences (with a draw) so many CTAs of 512 threads each; most work per warp: a row, a draw, both, a shard
+    long long most, most_draw;
+    int ctas;
+    double row, draw, both, shard;
+};
+constexpr EdgeBig kEdgeBig[] = {{8, 8, 16, 2.0, 2.0, 2.6, 1.05},  {14, 14, 16, 2.0, 3.0, 6.5, 1.05},   {19, 19, 12, 3.0, 2.7, 5.4, 1.05},
+                                {30, 30, 8, 5.0, 5.0, 8.0, 1.05}, {45, 42, 6, 12.0, 10.0, 14.5, 3.0}, {52, 50, 5, 13.0, 4.0, 14.5, 3.0}};
+constexpr long long kEdgeBigAlone = 8;  // sequences that leave SMs to spare: no more than a segment per warp
 constexpr long long kEdgeSmallWave = 1110, kEdgeSmallUnits = 24;  // CTAs of 128 threads; units of a sequence
 constexpr long long kEdgeEvenCtas = 150;
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;

@@ -38,3 +38,28 @@ def edge(L, dtype, form, B, gamma, V):
 ])
 def test_shard_sums(L, dtype, B, gamma, V, shape):
     assert edge(L, dtype, SHARD, B, gamma, V) == shape
+
+
+# Few sequences of many segments by CTAs of 512 threads, or not
+@pytest.mark.parametrize("dtype,form,B,gamma,V,shape", [
+    (F32, ROW, 1, 7, 50272, SEPARATE),       # 5.6 / 6.7
+    (F32, ROW, 8, 7, 50272, SEPARATE),       # 7.5 / 8.3
+    (BF16, ROW, 12, 5, 90108, SEPARATE),     # 8.7 / 9.7
+    (BF16, ROW, 19, 8, 100000, SEPARATE),    # 14.0 / 15.2
+    (BF16, ROW, 30, 11, 100000, SEPARATE),   # 21.1 / 23.3
+    (F32, BONUS, 1, 4, 121880, SEPARATE),    # 7.9 / 9.3
+    (F32, FUSED, 44, 14, 57719, SEPARATE),   # 38.3 / 41.8
+    (BF16, ROW, 2, 11, 25408, (512, 16)),    # 5.4 / 6.4
+    (F32, ROW, 6, 2, 53913, (512, 16)),      # 6.5 / 7.6
+    (F32, ROW, 14, 2, 83517, (512, 16)),     # 8.5 / 10.2
+    (F32, ROW, 18, 11, 34312, (512, 12)),    # 10.6 / 11.4
+    (F32, ROW, 29, 3, 63728, (512, 8)),      # 10.4 / 11.5
+    (BF16, ROW, 45, 6, 127696, (512, 6)),    # 25.4 / 29.8
+    (F32, ROW, 48, 6, 115296, (512, 5)),     # 34.4 / 35.3
+    (F32, BONUS, 7, 1, 128512, (512, 16)),   # 10.0 / 13.7
+    (BF16, BONUS, 27, 2, 64064, (512, 8)),   # 10.0 / 14.0
+    (F32, FUSED, 17, 6, 54992, (512, 12)),   # 13.7 / 16.3
+    (F32, FUSED, 1, 12, 13930, (256, 16)),   # 8.4 / 9.9 (512 threads do not hold the row)
+])
+def test_few_sequences(L, dtype, form, B, gamma, V, shape):
+    assert edge(L, dtype, form, B, gamma, V) == shape
