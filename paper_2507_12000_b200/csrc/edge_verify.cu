@@ -679,12 +679,12 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
         }
     }
     if (c > kEdgeCluster) return is(kThreads, c);
-    long long small = kEdgeSmallWave / B;  // CTAs of 128 threads
-    if (!held && units >= kEdgeSmallUnits && small >= 3 && small <= 6) {
-        if (small > (units + 3) / 4) small = (units + 3) / 4;
-        const double fill = (double)(B * small) / (double)(2 * kEdgeWave);
-        if (4 * small > kWarps * c)
-            return work <= (P.shard_sum ? 8.0 : draw * (fill >= 0.8 ? 25.0 : fill >= 0.65 ? 14.0 : 10.0)) * (double)(4 * small) ? is(128, small) : false;
+    if (!held && units >= (draw_only ? kEdgeSmallDrawUnits : kEdgeSmallUnits)) {  // CTAs of 128 threads
+        for (const auto &small : kEdgeSmall) {
+            if (B > small.most) continue;
+            if (4 * small.ctas <= kWarps * c) break;
+            return work <= (P.shard_sum ? kEdgeSmallShard : draw_only ? kEdgeSmallDraw : draw * kEdgeSmallRow) * (double)(4 * small.ctas) && is(128, small.ctas);
+        }
     }
     const long long ctas = B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
     const double fill = (double)ctas / (double)(waves * kEdgeWave);

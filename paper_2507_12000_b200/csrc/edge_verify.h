@@ -40,8 +40,13 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //     a draw as well (five separate kernels): B = 7 gamma = 1 V = 128512 float32 10.0 / 13.7, B = 27 gamma = 2 V = 64064 bf16 10.0 / 14.0; beyond, B = 1 gamma = 4
 //     V = 121880 float32 9.3 / 7.9.  A draw alone: B = 17 gamma = 6 V = 54992 float32 13.7 / 16.3; beyond, B = 44 gamma = 14 V = 57719 float32 41.8 / 38.3.
 //     Not where CTAs of 256 hold the row that is drawn from: fused B = 1 gamma = 12 V = 13930 float32 8.4, of 512 9.9.
-//   * A batch that leaves each sequence one CTA and half of the SM's room idle: three to six of 128 threads (kEdgeSmallWave).  B = 332
-//     gamma = 13 V = 5816 float32 22.1 / 27.0, B = 303 gamma = 2 V = 24064 float32 22.5 / 25.6, B = 203 gamma = 10 V = 7680 float32 15.3 / 16.7.
+//   * A batch that leaves each sequence one or two CTAs and half of the SM's room idle: three to six of 128 threads (kEdgeSmall), which find
+//     room in one wave while they are nine tenths of the clusters that the GPU holds.  B = 332 gamma = 13 V = 5816 float32 22.1 / 27.0, B = 303 gamma = 2 V = 24064
+//     float32 22.5 / 25.6, B = 190 gamma = 1 V = 34288 bf16 14.5 / 16.7, fused B = 178 gamma = 3 V = 25552 float32 23.7 / 27.5; beyond, the round of B = 213 gamma = 5
+//     V = 7568 float32 23.2 / 18.8, of B = 220 gamma = 2 V = 90976 106.7 / 87.1, of B = 333 gamma = 10 V = 12288 54.9 / 46.0 with work at the limit, B = 364 gamma = 7 V = 23515 fused
+//     60.6 / 49.2.  From 17 units on (B = 177 gamma = 2 V = 11376 binary16 7.0 against 8.7 with two CTAs of 256, B = 300 gamma = 3 V = 4096 float32, 16 units, 8.5 against
+//     8.3); a draw alone from 30 on (B = 332 gamma = 13 V = 1360, 28 units, 20.2 against 14.9).  More work per warp: fused B = 187 gamma = 2 V = 72378 bf16 (18 per
+//     warp) 45.1 against 40.9 in separate kernels, a shard of B = 190 gamma = 5 V = 49424 bf16 (15) 26.9 / 23.7, B = 370 gamma = 12 V = 20480 float32 (25) 91.2 / 76.1.
 //   * Otherwise pairs of CTAs of a full launch are one of 512 threads, whose barrier is cheaper: B = 168 gamma = 7 V = 2048 float32 (a
 //     shard) 4.0 / 4.6, B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, B = 259 gamma = 3 V = 14848 float32 16.3 / 16.5.
 // How much work per warp still pays depends on how full the wave is, since a
@@ -72,7 +77,10 @@ struct EdgeBig {  // up to so many sequences (with a draw) so many CTAs of 512 t
 constexpr EdgeBig kEdgeBig[] = {{8, 8, 16, 2.0, 2.0, 2.6, 1.05},  {14, 14, 16, 2.0, 3.0, 6.5, 1.05},   {19, 19, 12, 3.0, 2.7, 5.4, 1.05},
                                 {30, 30, 8, 5.0, 5.0, 8.0, 1.05}, {45, 42, 6, 12.0, 10.0, 14.5, 3.0}, {52, 50, 5, 13.0, 4.0, 14.5, 3.0}};
 constexpr long long kEdgeBigAlone = 8;  // sequences that leave SMs to spare: no more than a segment per warp
-constexpr long long kEdgeSmallWave = 1110, kEdgeSmallUnits = 24;  // CTAs of 128 threads; units of a sequence
+struct EdgeSmall { long long most; int ctas; };           // up to so many sequences, so many CTAs of 128 threads each
+constexpr EdgeSmall kEdgeSmall[] = {{181, 6}, {204, 5}, {346, 3}};
+constexpr long long kEdgeSmallUnits = 17, kEdgeSmallDrawUnits = 30;  // units of a sequence; where it is only drawn from
+constexpr double kEdgeSmallRow = 18.0, kEdgeSmallDraw = 13.0, kEdgeSmallShard = 8.0;  // work per warp
 constexpr long long kEdgeEvenCtas = 150;
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)

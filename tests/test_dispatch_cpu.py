@@ -63,3 +63,20 @@ def test_shard_sums(L, dtype, B, gamma, V, shape):
 ])
 def test_few_sequences(L, dtype, form, B, gamma, V, shape):
     assert edge(L, dtype, form, B, gamma, V) == shape
+
+
+# CTAs of 128 threads, or not (a round where the call itself does not tell)
+@pytest.mark.parametrize("dtype,form,B,gamma,V,shape", [
+    (F32, ROW, 370, 12, 20480, SEPARATE),    # 76.1 / 91.2
+    (F32, ROW, 220, 2, 90976, SEPARATE),     # 66.9 / 87.2 (5 CTAs)
+    (F32, BONUS, 185, 9, 68224, SEPARATE),   # a round 122.5 / 143.4 (6)
+    (BF16, FUSED, 364, 7, 23515, SEPARATE),  # 49.2 / 60.6 (3)
+    (F32, FUSED, 332, 13, 1360, (256, 1)),   # 14.9 / 20.2 (3)
+    (F32, FUSED, 208, 5, 6119, (256, 2)),    # 16.6 / 20.6 (5)
+    (F32, ROW, 332, 13, 5816, (128, 3)),     # 22.1 / 27.0
+    (F32, ROW, 199, 9, 7840, (128, 5)),      # 14.9 / 15.9 (256 x 2)
+    (F32, FUSED, 178, 3, 25552, (128, 6)),   # 23.7 / 27.5 (256 x 2)
+    (BF16, ROW, 177, 2, 11376, (128, 6)),    # 7.0 / 8.7 (256 x 2)
+])
+def test_batches_of_one_or_two_ctas(L, dtype, form, B, gamma, V, shape):
+    assert edge(L, dtype, form, B, gamma, V) == shape
