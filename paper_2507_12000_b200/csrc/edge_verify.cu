@@ -668,6 +668,7 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
         if (twice > c) c = twice;
     }
     if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
+    if (c == kEdgeCluster && B * c > kEdgeEightsWave) c = kEdgeCluster - 1;
     const bool held = draws_held(P, kThreads, c), draw_only = P.draw_token && !P.p_row;
     if (units > kEdgeBigUnits && kWarps * c < units && !held && (c <= kEdgeCluster || !draw_only)) {  // CTAs of 512 threads
         for (const auto &big : kEdgeBig) {
@@ -691,7 +692,7 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
     const double limit = P.shard_sum ? (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0)
                                      : draw * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
     if (work > limit * (double)(kWarps * c)) return false;
-    return c % 2 == 0 && ctas >= kEdgeEvenCtas && !P.draw_token ? is(kEdgeMostThreads, c / 2) : is(kThreads, c);
+    return c == 2 && ctas >= kEdgePairCtas && !P.draw_token ? is(kEdgeMostThreads, 1) : is(kThreads, c);
 }
 
 long long row_segments(int V, int esz)

@@ -47,8 +47,13 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //     60.6 / 49.2.  From 17 units on (B = 177 gamma = 2 V = 11376 binary16 7.0 against 8.7 with two CTAs of 256, B = 300 gamma = 3 V = 4096 float32, 16 units, 8.5 against
 //     8.3); a draw alone from 30 on (B = 332 gamma = 13 V = 1360, 28 units, 20.2 against 14.9).  More work per warp: fused B = 187 gamma = 2 V = 72378 bf16 (18 per
 //     warp) 45.1 against 40.9 in separate kernels, a shard of B = 190 gamma = 5 V = 49424 bf16 (15) 26.9 / 23.7, B = 370 gamma = 12 V = 20480 float32 (25) 91.2 / 76.1.
-//   * Otherwise pairs of CTAs of a full launch are one of 512 threads, whose barrier is cheaper: B = 168 gamma = 7 V = 2048 float32 (a
-//     shard) 4.0 / 4.6, B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, B = 259 gamma = 3 V = 14848 float32 16.3 / 16.5.
+//   * Otherwise a sequence's two CTAs are one of 512 threads, which needs no cluster, where they are many: B = 168 gamma = 7 V = 2048 float32 (a
+//     shard) 4.0 / 4.6, B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, B = 259 gamma = 3 V = 14848 float32 16.3 / 16.5.  Not four, six or eight, which as two to four
+//     of 512 threads find less room: a round of B = 92 gamma = 14 V = 10400 float32 20.4 us with six of 256, 28.7 with three of 512; B = 49 gamma = 9 V = 5242
+//     bf16 10.9 and 12.2 with two, B = 67 gamma = 7 V = 7744 9.8 and 11.2.
+// Near the last cluster that the GPU holds, a launch in a pipeline waits for the one before it to drain: eight CTAs each up to 65 sequences (a
+// round of B = 69 gamma = 1 V = 95104 float32 35.2 us, with seven 28.2), three up to 166 (a round of B = 174 gamma = 2 V = 8608 float32 17.8, with six of 128
+// threads 14.2; fused B = 169 gamma = 2 V = 6224 13.2, with two of 256 10.9).
 // How much work per warp still pays depends on how full the wave is, since a
 // warp's loads wait for one another from segment to segment and only other CTAs on the SM fill the gaps.  Measured (us per
 // call, cluster kernel / separate kernels):
@@ -66,7 +71,8 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 // five and the cluster kernel pays for longer (B = 33 gamma = 10 V = 32480 bf16 11.7 / 16.5).
 constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
 constexpr int kEdgeMostThreads = 512;                    // per CTA
-constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, three, more
+constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeEightsWave = 520,
+                    kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, three, eight, more
 constexpr long long kEdgeSpread = 140, kEdgeSpreadCtas = 12;  // CTAs, in all and per sequence
 constexpr long long kEdgeBigUnits = 64;
 struct EdgeBig {  // up to so many sequences (with a draw) so many CTAs of 512 threads each; most work per warp: a row, a draw, both, a shard
@@ -81,7 +87,7 @@ struct EdgeSmall { long long most; int ctas; };           // up to so many seque
 constexpr EdgeSmall kEdgeSmall[] = {{181, 6}, {204, 5}, {346, 3}};
 constexpr long long kEdgeSmallUnits = 17, kEdgeSmallDrawUnits = 30;  // units of a sequence; where it is only drawn from
 constexpr double kEdgeSmallRow = 18.0, kEdgeSmallDraw = 13.0, kEdgeSmallShard = 8.0;  // work per warp
-constexpr long long kEdgeEvenCtas = 150;
+constexpr long long kEdgePairCtas = 150;
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
 constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory; the limits on the work allow 900)

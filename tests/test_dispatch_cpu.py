@@ -80,3 +80,16 @@ def test_few_sequences(L, dtype, form, B, gamma, V, shape):
 ])
 def test_batches_of_one_or_two_ctas(L, dtype, form, B, gamma, V, shape):
     assert edge(L, dtype, form, B, gamma, V) == shape
+
+
+# Pairs of CTAs as one of 512 threads, and clusters near the last that the GPU holds (a round, taken / not taken)
+@pytest.mark.parametrize("dtype,form,B,gamma,V,shape", [
+    (F32, ROW, 92, 14, 10400, (256, 6)),     # 20.4 / 28.7 (512 x 3)
+    (BF16, ROW, 49, 9, 5242, (256, 4)),      # 10.9 / 12.2 (512 x 2)
+    (BF16, ROW, 67, 7, 7744, (256, 4)),      # 9.8 / 11.2
+    (F32, SHARD, 57, 13, 1088, (256, 4)),    # the call 3.1 / 3.3
+    (F32, SHARD, 168, 7, 2048, (512, 1)),    # the call 4.0 / 4.6 (256 x 2)
+    (F32, ROW, 69, 1, 95104, (256, 7)),      # 28.2 / 35.2 (256 x 8)
+])
+def test_pairs_and_full_waves(L, dtype, form, B, gamma, V, shape):
+    assert edge(L, dtype, form, B, gamma, V) == shape
