@@ -690,7 +690,7 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
     const long long ctas = B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
     const double fill = (double)ctas / (double)(waves * kEdgeWave);
     const double limit = P.shard_sum ? (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0)
-                                     : draw * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
+                                     : (held || fill >= 0.65 ? draw : 1.0) * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
     if (work > limit * (double)(kWarps * c)) return false;
     return c == 2 && ctas >= kEdgePairCtas && !P.draw_token ? is(kEdgeMostThreads, 1) : is(kThreads, c);
 }

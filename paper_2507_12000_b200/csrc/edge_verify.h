@@ -68,7 +68,8 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 // in smaller ones more: B = 256 gamma = 4 V = 18992
 // bf16 13.5 / 14.2, B = 503 gamma = 3 V = 5936 float32 8.5 / 11.1, B = 620 gamma = 15 V = 792 bf16 9.7 / 28.4; beyond B = 173 gamma = 3
 // V = 67023 float32 40.5 / 30.5, B = 2 gamma = 2 V = 79648 float32 5.4 / 4.6.  Where the edge draws bonus tokens the separate kernels are
-// five and the cluster kernel pays for longer (B = 33 gamma = 10 V = 32480 bf16 11.7 / 16.5).
+// five and the cluster kernel pays for longer (kEdgeDrawFactor; B = 33 gamma = 10 V = 32480 bf16 11.7 / 16.5), unless it leaves SMs idle and does not hold
+// the row (B = 1 gamma = 5 V = 57440 float32 11.4 / 7.5, B = 9 gamma = 4 V = 64935 13.3 / 12.8; held, B = 2 gamma = 10 V = 31702 bf16 9.3 / 10.4).
 constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
 constexpr int kEdgeMostThreads = 512;                    // per CTA
 constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeEightsWave = 520,

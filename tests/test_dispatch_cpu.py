@@ -93,3 +93,14 @@ def test_batches_of_one_or_two_ctas(L, dtype, form, B, gamma, V, shape):
 ])
 def test_pairs_and_full_waves(L, dtype, form, B, gamma, V, shape):
     assert edge(L, dtype, form, B, gamma, V) == shape
+
+
+# The edge's draw of bonus tokens in the same launch, or not
+@pytest.mark.parametrize("dtype,B,gamma,V,shape", [
+    (F32, 1, 5, 57440, SEPARATE),     # 7.5 / 11.4 (256 x 8)
+    (F32, 1, 8, 42042, SEPARATE),     # 7.6 / 11.2
+    (F32, 3, 5, 58288, SEPARATE),     # 9.2 / 11.4
+    (BF16, 2, 10, 31702, (256, 8)),   # 9.3 / 10.4 (the row is held)
+])
+def test_bonus_draws(L, dtype, B, gamma, V, shape):
+    assert edge(L, dtype, BONUS, B, gamma, V) == shape
