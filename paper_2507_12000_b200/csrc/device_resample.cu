@@ -58,8 +58,8 @@ constexpr long long kHeldWideCtas = 148;
 constexpr long long kHeldWarps = 2250, kHeldWideWarps = 1650, kHeldWidestWarps = 1250;  // up to eight CTAs, more, more of 512 threads
 // Batches of middle size: the same in turns (resample_stream_kernel), in which a CTA's or cluster's start, its barrier and the walk are
 // paid for once while the other CTAs on the SM stream.  For rows of up to kStreamSegs segments, at most kStreamTurns of them per warp:
-// as many warps as there are segments while kStreamOne of them suffice, else as many as a wave has (four or five
-// CTAs of 256 threads per SM, seven tenths of that in clusters).  Measured (us per call, this / the two kernels): B = 164 V = 9856
+// as many warps as there are segments while kStreamOne of them suffice, else as many as a wave of whole CTAs has (32 or 40 warps per
+// SM: six CTAs of six warps, not seven: B = 915 V = 12480 in five turns by five warps, by six 20.8 us, two kernels 18.2), seven tenths of that in clusters.  Measured (us per call, this / the two kernels): B = 164 V = 9856
 // 5.6 / 6.5, B = 331 V = 4384 binary16 6.7 / 10.6, B = 425 V = 5800 7.5 / 9.3, B = 714 V = 3728 6.4 / 9.1, B = 567 V = 11886 11.7 / 15.3,
 // B = 665 V = 12640 12.8 / 15.6, B = 305 V = 15760 binary16 9.8 / 12.5, B = 143 V = 19400 7.8 / 9.4; beyond, B = 67 V = 32592 7.0 / 6.6,
 // B = 100 V = 43015 13.3 / 12.2, B = 55 V = 124034 14.4 / 10.5.
@@ -655,14 +655,14 @@ bool one_launch(ResampleParams &P, bool aligned, Most most_cluster_ctas)
         }
     }
     if (segs > kStreamSegs) return false;
-    const long long wave = 148 * (aligned ? 5 : 4) * kWarps;
+    const long long sm_warps = aligned ? 40 : 32;  // that the registers of an SM hold, a quarter of them in each of its parts
+    const long long wave = 148 * sm_warps;
     long long warps = segs;
     if (B * segs <= kStreamOne) {
         if (segs <= 2 * kWarps && B >= 250) warps = kWarps;
     } else if (B * 10 > wave) {
-        warps = wave / B;
+        for (warps = kWarps; warps >= 4 && B > 148 * (sm_warps / warps);) --warps;
         if (warps < 4) return false;
-        if (warps > kWarps) warps = kWarps;
     } else {
         warps = wave * 7 / 10 / B;
         const long long turns = (segs + warps - 1) / warps;

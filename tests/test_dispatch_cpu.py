@@ -104,3 +104,25 @@ def test_pairs_and_full_waves(L, dtype, form, B, gamma, V, shape):
 ])
 def test_bonus_draws(L, dtype, B, gamma, V, shape):
     assert edge(L, dtype, BONUS, B, gamma, V) == shape
+
+
+def draw(L, B, V):
+    t, c, turns = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+    L.dssd_test_draw_shape(B, V, ctypes.byref(t), ctypes.byref(c), ctypes.byref(turns))
+    return t.value, c.value, turns.value
+
+
+# Draws in turns by one CTA per sequence: all CTAs resident, forty warps of an SM in whole CTAs
+@pytest.mark.parametrize("B,V,shape", [
+    (740, 20480, (256, 1, 1)),    # 17.2 / 19.0 (two kernels)
+    (741, 12800, (192, 1, 1)),    # five CTAs of seven warps are 740
+    (914, 14080, (0, 0, 0)),      # 18.2 / 20.9 (192 x 1: six CTAs of six warps are 888)
+    (795, 16068, (0, 0, 0)),      # 15.0 / 17.2 (224 x 1)
+    (915, 12480, (160, 1, 1)),    # (192 x 1 20.8, two kernels 18.2)
+    (1000, 12288, (160, 1, 1)),   # 15.6 / 17.4
+    (1400, 10240, (128, 1, 1)),   # 16.8 / 20.5
+    (1480, 4609, (128, 1, 1)),    # ten CTAs of four warps are 1480
+    (1481, 4609, (0, 0, 0)),
+])
+def test_draws_by_one_cta(L, B, V, shape):
+    assert draw(L, B, V) == shape
