@@ -121,8 +121,8 @@ def draw(L, B, V):
     (915, 12480, (160, 1, 1)),    # (192 x 1 20.8, two kernels 18.2)
     (1000, 12288, (160, 1, 1)),   # 15.6 / 17.4
     (1400, 10240, (128, 1, 1)),   # 16.8 / 20.5
-    (1480, 4609, (128, 1, 1)),    # ten CTAs of four warps are 1480
-    (1481, 4609, (0, 0, 0)),
+    (1480, 4612, (128, 1, 1)),    # ten CTAs of four warps are 1480
+    (1481, 4612, (0, 0, 0)),
 ])
 def test_draws_by_one_cta(L, B, V, shape):
     assert draw(L, B, V) == shape
