@@ -62,9 +62,19 @@ constexpr long long kHeldWarps = 2250, kHeldWideWarps = 1650, kHeldWidestWarps =
 // SM: six CTAs of six warps, not seven: B = 915 V = 12480 in five turns by five warps, by six 20.8 us, two kernels 18.2), seven tenths of that in clusters.  Measured (us per call, this / the two kernels): B = 164 V = 9856
 // 5.6 / 6.5, B = 331 V = 4384 binary16 6.7 / 10.6, B = 425 V = 5800 7.5 / 9.3, B = 714 V = 3728 6.4 / 9.1, B = 567 V = 11886 11.7 / 15.3,
 // B = 665 V = 12640 12.8 / 15.6, B = 305 V = 15760 binary16 9.8 / 12.5, B = 143 V = 19400 7.8 / 9.4; beyond, B = 67 V = 32592 7.0 / 6.6,
-// B = 100 V = 43015 13.3 / 12.2, B = 55 V = 124034 14.4 / 10.5.
-constexpr int kStreamSegs = 45, kStreamTurns = 5;
-constexpr long long kStreamOne = 3600;
+// B = 100 V = 43015 13.3 / 12.2, B = 55 V = 124034 14.4 / 10.5.  The two kernels are the better ones for
+//   clusters of more warps than kStreamClusters in all (B = 383 V = 23016 15.2 / 13.5, B = 290 V = 19376 by four CTAs 10.6 / 9.6, B = 195 V = 10576 by six 8.3 /
+//   6.5; with fewer CTAs B = 330 V = 23040 11.9 / 13.1),
+//   rows of more than kStreamTurnsFew turns by one CTA each that leave a third of the wave empty (B = 400 V = 18218 16.2 / 14.3, B = 352 V = 19047 17.3 / 13.6; in four
+//   turns B = 416 V = 12881 12.4 / 14.2, B = 385 V = 15189 12.6 / 13.1, B = 421 V = 15520 11.7 / 10.5),
+//   few long rows that need more than a segment per warp (B = 92 V = 20030 8.3 / 7.1 and B = 133 V = 15897 8.8 / 7.4 off the 16-byte boundaries, B = 107 V = 22920
+//   7.2 / 6.4 on them), and most rows of more than 32 segments with one each (B = 105 V = 17034 9.0 / 7.5; B = 90 V = 18316 6.1 / 6.3).
+// Up to sixteen segments by eight warps in two turns, not by as many warps as segments, from kStreamHalf sequences on: B = 340 V = 4608 6.5 / 8.0, B = 300 V =
+// 6144 6.4 / 6.1, B = 251 V = 4608 6.4 / 5.7.
+constexpr int kStreamSegs = 45, kStreamTurns = 5, kStreamTurnsFew = 4;
+constexpr long long kStreamOne = 3600, kStreamOneLong = 3300, kStreamHalf = 320, kStreamClusters = 4200;
+constexpr long long kStreamFew = 150;                              // sequences, of at most
+constexpr int kStreamFewSegs = 41, kStreamFewSegsShifted = 29;     // segments, on and off the boundaries of 16 bytes
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
 constexpr int kDrawWarps = kDrawThreads / 32;
 constexpr int kRun = kSub / kDrawThreads;  // entries of a chunk per thread
@@ -657,19 +667,26 @@ bool one_launch(ResampleParams &P, bool aligned, Most most_cluster_ctas)
     if (segs > kStreamSegs) return false;
     const long long sm_warps = aligned ? 40 : 32;  // that the registers of an SM hold, a quarter of them in each of its parts
     const long long wave = 148 * sm_warps;
-    long long warps = segs;
-    if (B * segs <= kStreamOne) {
-        if (segs <= 2 * kWarps && B >= 250) warps = kWarps;
+    long long warps = segs, most_turns = kStreamTurns;
+    auto even = [&](long long w) {  // no more than w warps, with even shares
+        const long long turns = (segs + w - 1) / w;
+        return (segs + turns - 1) / turns;
+    };
+    if (B * segs <= (segs <= 32 ? kStreamOne : kStreamOneLong)) {
+        if (segs <= 2 * kWarps && B >= kStreamHalf) warps = kWarps;
     } else if (B * 10 > wave) {
         for (warps = kWarps; warps >= 4 && B > 148 * (sm_warps / warps);) --warps;
         if (warps < 4) return false;
     } else {
-        warps = wave * 7 / 10 / B;
-        const long long turns = (segs + warps - 1) / warps;
-        warps = (segs + turns - 1) / turns;
+        if (B < kStreamFew && segs > (aligned ? kStreamFewSegs : kStreamFewSegsShifted)) return false;
+        warps = even(wave * 7 / 10 / B);
+        long long most = kStreamClusters / B / 4 * 4;  // whole CTAs of four warps
+        if (most < kWarps) most = kWarps;
+        if (warps > kWarps && (warps + 3) / 4 * 4 > most) warps = even(most);
     }
+    if (warps <= kWarps && 10 * kWarps * B < 7 * wave) most_turns = kStreamTurnsFew;
     if (warps > segs) warps = segs;
-    if (segs > kStreamTurns * warps) return false;
+    if (segs > most_turns * warps) return false;
     if (warps <= kWarps) return is(32 * (int)warps, 1, true);
     return warps <= 4 * kClusterMax ? is(128, (warps + 3) / 4, true) : is(kThreads, (warps + kWarps - 1) / kWarps, true);
 }

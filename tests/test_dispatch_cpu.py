@@ -126,3 +126,23 @@ def draw(L, B, V):
 ])
 def test_draws_by_one_cta(L, B, V, shape):
     assert draw(L, B, V) == shape
+
+
+# Draws in turns by clusters, by one CTA while the wave is not full, and of few long rows
+@pytest.mark.parametrize("B,V,shape", [
+    (383, 23016, (0, 0, 0)),      # 13.5 / 15.2 (128 x 3)
+    (406, 18672, (0, 0, 0)),      # 12.2 / 14.2 (128 x 3)
+    (330, 23040, (128, 3, 1)),    # 11.9 / 13.1
+    (290, 19376, (128, 3, 1)),    # 9.6 / 10.6 (128 x 4; two kernels 9.6)
+    (352, 19047, (0, 0, 0)),      # 13.6 / 17.3 (256 x 1)
+    (400, 18218, (0, 0, 0)),      # 14.3 / 16.2
+    (92, 20030, (0, 0, 0)),       # 7.1 / 8.3 (128 x 5)
+    (133, 15897, (0, 0, 0)),      # 7.4 / 8.8 (128 x 4)
+    (105, 17034, (0, 0, 0)),      # 7.5 / 9.0 (256 x 5)
+    (107, 22920, (0, 0, 0)),      # 6.4 / 7.2 (128 x 6)
+    (141, 17020, (128, 5, 1)),    # 7.0 / 9.6 (two kernels)
+    (251, 4608, (128, 3, 1)),     # 5.7 / 6.4 (256 x 1)
+    (340, 4608, (256, 1, 1)),     # 6.5 / 8.0 (128 x 3)
+])
+def test_draws_in_turns(L, B, V, shape):
+    assert draw(L, B, V) == shape
