@@ -46,7 +46,7 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //     V = 7568 float32 23.2 / 18.8, of B = 220 gamma = 2 V = 90976 106.7 / 87.1, of B = 333 gamma = 10 V = 12288 54.9 / 46.0 with work at the limit, B = 364 gamma = 7 V = 23515 fused
 //     60.6 / 49.2.  From 17 units on (B = 177 gamma = 2 V = 11376 binary16 7.0 against 8.7 with two CTAs of 256, B = 300 gamma = 3 V = 4096 float32, 16 units, 8.5 against
 //     8.3); a draw alone from 30 on (B = 332 gamma = 13 V = 1360, 28 units, 20.2 against 14.9).  More work per warp: fused B = 187 gamma = 2 V = 72378 bf16 (18 per
-//     warp) 45.1 against 40.9 in separate kernels, a shard of B = 190 gamma = 5 V = 49424 bf16 (15) 26.9 / 23.7, B = 370 gamma = 12 V = 20480 float32 (25) 91.2 / 76.1.
+//     warp) 45.1 against 40.9 in separate kernels, a shard of B = 190 gamma = 5 V = 49424 bf16 (15) 26.9 / 23.7, B = 370 gamma = 12 V = 20480 float32 (25) 91.2 / 76.1, a round of B = 300 gamma = 4 V = 30011 bf16 (17.4) 49.8 / 49.5.
 //   * Otherwise a sequence's two CTAs are one of 512 threads, which needs no cluster, where they are many: B = 168 gamma = 7 V = 2048 float32 (a
 //     shard) 4.0 / 4.6, B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, B = 259 gamma = 3 V = 14848 float32 16.3 / 16.5.  Not four, six or eight, which as two to four
 //     of 512 threads find less room: a round of B = 92 gamma = 14 V = 10400 float32 20.4 us with six of 256, 28.7 with three of 512; B = 49 gamma = 9 V = 5242
@@ -87,11 +87,11 @@ constexpr long long kEdgeBigAlone = 8;  // sequences that leave SMs to spare: no
 struct EdgeSmall { long long most; int ctas; };           // up to so many sequences, so many CTAs of 128 threads each
 constexpr EdgeSmall kEdgeSmall[] = {{181, 6}, {204, 5}, {346, 3}};
 constexpr long long kEdgeSmallUnits = 17, kEdgeSmallDrawUnits = 30;  // units of a sequence; where it is only drawn from
-constexpr double kEdgeSmallRow = 18.0, kEdgeSmallDraw = 13.0, kEdgeSmallShard = 8.0;  // work per warp
+constexpr double kEdgeSmallRow = 15.0, kEdgeSmallDraw = 13.0, kEdgeSmallShard = 8.0;  // work per warp
 constexpr long long kEdgePairCtas = 150;
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
-constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory; the limits on the work allow 900)
+constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory).  It ends the calls by CTAs of 512 threads; the other limits allow 900
 
 // What the draw needs to know about a folded sequence when no row is written.
 struct ReadySlot {

@@ -69,6 +69,7 @@ def test_few_sequences(L, dtype, form, B, gamma, V, shape):
 @pytest.mark.parametrize("dtype,form,B,gamma,V,shape", [
     (F32, ROW, 370, 12, 20480, SEPARATE),    # 76.1 / 91.2
     (F32, ROW, 220, 2, 90976, SEPARATE),     # 66.9 / 87.2 (5 CTAs)
+    (BF16, ROW, 300, 4, 30011, SEPARATE),    # a round 49.5 / 49.8 (3)
     (F32, BONUS, 185, 9, 68224, SEPARATE),   # a round 122.5 / 143.4 (6)
     (BF16, FUSED, 364, 7, 23515, SEPARATE),  # 49.2 / 60.6 (3)
     (F32, FUSED, 332, 13, 1360, (256, 1)),   # 14.9 / 20.2 (3)
