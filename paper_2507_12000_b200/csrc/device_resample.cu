@@ -50,7 +50,11 @@ constexpr int kClusterSums = kClusterMax * kClusterThreads / 32;
 //   clusters of 128 threads:  B = 168 V = 5460 (3 CTAs) 4.1 / 6.3, B = 59 V = 13786 (7) 4.2 / 6.7, B = 46 V = 16436 (9) 4.2 / 5.9;
 //              beyond, B = 46 V = 28992 (15, 690 CTAs) 6.7 / 6.1, B = 175 V = 11384 (6) 7.8 / 6.1
 //   of 256:  B = 7 V = 57700 (15) 4.3 / 6.1, of 512:  B = 2 V = 96209 (12) 4.3 / 5.9, B = 6 V = 105317 (13) 4.5 / 6.1, B = 4
-//              V = 129300 (16) 4.6 / 5.1; beyond, B = 21 V = 82900 (11) 12.5 / 7.2.
+//              V = 129300 (16) 4.6 / 5.1; beyond, B = 21 V = 82900 (11) 12.5 / 7.2.  In rounds too (a CTA of 512 threads has its SM to itself, so that a
+//              cluster starts when up to sixteen SMs of one processing cluster are free): gamma = 4, B = 1 V = 96209 float32 11.3 / 13.4, B = 4 V = 128256 bf16
+//              12.7 / 13.7, B = 8 V = 66000 12.4 / 14.5.  While another stream keeps the GPU busy a launch waits for its CTAs' room, one for
+//              more of it, two twice (the latency of a round, B = 1 V = 96209, B = 2 V = 128256 and B = 4 V = 128256: beside products of 4096 x 4096 bf16 62 / 31, 67 / 41,
+//              67 / 68 us, beside products of 2048 x 1024 19 / 22, 19 / 20, 21 / 22, beside copies of a GB 295 / 617, 297 / 618, 298 / 617).
 constexpr long long kSingleThreads = 153600;
 // More than eight CTAs of 128 threads only for a few sequences: many of them do not find room before the kernel before has drained (a round
 // of B = 23 gamma = 7 V = 23912 bf16, twelve CTAs 13.0 us, six of 256 threads 12.5; B = 8 gamma = 4 V = 32000 bf16, sixteen 9.3, eight 9.5).
@@ -69,10 +73,10 @@ constexpr long long kHeldWarps = 2250, kHeldWideWarps = 1650, kHeldWidestWarps =
 //   turns B = 416 V = 12881 12.4 / 14.2, B = 385 V = 15189 12.6 / 13.1, B = 421 V = 15520 11.7 / 10.5),
 //   few long rows that need more than a segment per warp (B = 92 V = 20030 8.3 / 7.1 and B = 133 V = 15897 8.8 / 7.4 off the 16-byte boundaries, B = 107 V = 22920
 //   7.2 / 6.4 on them), and most rows of more than 32 segments with one each (B = 105 V = 17034 9.0 / 7.5; B = 90 V = 18316 6.1 / 6.3).
-// Up to sixteen segments by eight warps in two turns, not by as many warps as segments, from kStreamHalf sequences on: B = 340 V = 4608 6.5 / 8.0, B = 300 V =
-// 6144 6.4 / 6.1, B = 251 V = 4608 6.4 / 5.7.
+// Up to sixteen segments by eight warps in two turns, not by as many warps as segments, from kStreamHalf sequences on: B = 340 V = 4608 6.5 / 8.0, B = 318 V =
+// 4880 6.9 / 8.3; below, B = 290 V = 5120 6.3 / 5.9, B = 251 V = 4608 6.4 / 5.7.
 constexpr int kStreamSegs = 45, kStreamTurns = 5, kStreamTurnsFew = 4;
-constexpr long long kStreamOne = 3600, kStreamOneLong = 3300, kStreamHalf = 320, kStreamClusters = 4200;
+constexpr long long kStreamOne = 3600, kStreamOneLong = 3300, kStreamHalf = 300, kStreamClusters = 4200;
 constexpr long long kStreamFew = 150;                              // sequences, of at most
 constexpr int kStreamFewSegs = 41, kStreamFewSegsShifted = 29;     // segments, on and off the boundaries of 16 bytes
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
@@ -330,7 +334,8 @@ __global__ void __launch_bounds__(kClusterThreads) resample_cluster_kernel(const
 }
 
 // Batches of middle size (draw_streamed).  Bound by the chain of loads, sums, barrier and walk of each CTA, under which the others on
-// the SM stream: 48 registers, so five CTAs of 256 threads share one.
+// the SM stream: 48 registers, so five CTAs of 256 threads share one, for 24 to 48 bytes per thread in local memory (64 and 8 to 48 off the 16-byte
+// boundaries).
 template <bool kShift, typename RV>
 __global__ void __launch_bounds__(kThreads, kShift ? 4 : 5) resample_stream_kernel(const __grid_constant__ ResampleParams P)
 {

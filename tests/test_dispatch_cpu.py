@@ -143,7 +143,9 @@ def test_draws_by_one_cta(L, B, V, shape):
     (107, 22920, (0, 0, 0)),      # 6.4 / 7.2 (128 x 6)
     (141, 17020, (128, 5, 1)),    # 7.0 / 9.6 (two kernels)
     (251, 4608, (128, 3, 1)),     # 5.7 / 6.4 (256 x 1)
-    (340, 4608, (256, 1, 1)),     # 6.5 / 8.0 (128 x 3)
+    (290, 5120, (128, 3, 1)),     # 5.9 / 6.3 (256 x 1)
+    (318, 4880, (256, 1, 1)),     # 6.9 / 8.3 (128 x 3)
+    (340, 4608, (256, 1, 1)),     # 6.5 / 8.0
 ])
 def test_draws_in_turns(L, B, V, shape):
     assert draw(L, B, V) == shape
