@@ -103,6 +103,50 @@ def test_other_cta_sizes(B, oracle_mod, dtype, Bn, gamma, V):
     compare_dsd(B, oracle_mod, d, w.temperature, threads=16)
 
 
+def _shape(B, dtype, form, Bn, gamma, V):
+    import ctypes
+
+    t, c = ctypes.c_int(), ctypes.c_int()
+    B.lib.dssd_test_edge_shape(int(dtype == "bf16"), form, Bn, gamma, V, ctypes.byref(t), ctypes.byref(c))
+    return t.value, c.value
+
+
+# The last batch of each row of the tables of other CTA sizes and the first beyond it, and as many partial sums as a CTA's shared
+# memory holds (1024: sixteen positions of 64 segments, eight of 128) and one segment more per row.
+@pytest.mark.parametrize("dtype,Bn,gamma,V,shape", [
+    ("f32", 8, 2, 53913, (512, 16)), ("f32", 9, 2, 53913, (512, 16)), ("f32", 14, 2, 83517, (512, 16)), ("f32", 15, 2, 53913, (512, 12)),
+    ("f32", 19, 11, 17000, (512, 12)), ("f32", 20, 3, 63728, (512, 8)), ("f32", 30, 3, 63728, (512, 8)), ("f32", 31, 9, 26000, (512, 6)),
+    ("f32", 45, 7, 20000, (512, 6)), ("f32", 46, 7, 20000, (512, 5)), ("f32", 52, 7, 20000, (512, 5)), ("f32", 53, 7, 20000, (256, 8)),
+    ("f32", 181, 4, 4200, (128, 6)), ("f32", 182, 4, 4200, (128, 5)), ("f32", 204, 4, 4200, (128, 5)), ("f32", 205, 4, 4200, (512, 1)),
+    ("f32", 346, 4, 4200, (128, 3)), ("f32", 347, 4, 4200, (256, 1)), ("bf16", 177, 2, 11376, (128, 6)), ("f32", 65, 7, 8200, (256, 8)), ("f32", 66, 7, 8200, (256, 7)),
+    ("f32", 45, 15, 65536, (512, 6)), ("f32", 45, 15, 65540, (0, 0)),
+])
+def test_edges_of_the_tables(B, oracle_mod, dtype, Bn, gamma, V, shape):
+    assert _shape(B, dtype, 0, Bn, gamma, V) == shape
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.4, zipf=True, seed=V + Bn)
+    compare_round(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
+
+
+@pytest.mark.parametrize("V,shape", [(131072, (512, 16)), (131076, (0, 0))])
+def test_as_many_partial_sums_as_fit_with_a_draw(B, oracle_mod, V, shape):
+    assert _shape(B, "f32", 1, 14, 7, V) == shape
+    w = di.custom(B=14, gamma=7, V=V, dtype="f32", temperature=0.9, sigma_d=0.1, zipf=True, seed=V)
+    compare_bonus(B, oracle_mod, di.generate(w, threads=16), w.temperature, threads=16)
+
+
+# Residuals without mass, drawn for by CTAs of 128 and of 512 threads
+@pytest.mark.parametrize("dtype,Bn,gamma,V,shape", [
+    ("f32", 178, 3, 9000, (128, 6)), ("bf16", 187, 4, 12384, (128, 5)), ("f32", 320, 3, 8193, (128, 3)), ("f32", 17, 6, 54992, (512, 12)), ("bf16", 2, 3, 75001, (512, 16)),
+])
+def test_fallback_of_other_cta_sizes(B, oracle_mod, dtype, Bn, gamma, V, shape):
+    assert _shape(B, dtype, 2, Bn, gamma, V) == shape
+    w = di.custom(B=Bn, gamma=gamma, V=V, dtype=dtype, temperature=0.9, sigma_d=0.4, zipf=True, seed=V + Bn)
+    d = di.generate(w, threads=16)
+    d["draft_q"][: (Bn + 1) // 2] = 1.0  # rejected nearly always, and max(0, p - q) is 0 everywhere
+    d["draft_q_tok"][: (Bn + 1) // 2] = 1.0
+    compare_dsd(B, oracle_mod, d, w.temperature, threads=16)
+
+
 @pytest.mark.parametrize("dtype,V,stride", [("bf16", 4096, 1), ("bf16", 40000, 97), ("f32", 4096, 1)])
 def test_every_entry_of_a_vector_counts(B, dtype, V, stride):
     """Some terms of a row's sum are formed by a polynomial, the others by the special-function unit: a NaN is seen in

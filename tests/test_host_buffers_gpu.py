@@ -96,7 +96,11 @@ def test_draft_rows_pinned_in_pieces(B, pages):
 @pytest.mark.parametrize("Bn,gamma,V,dtype,offset", [
     (1, 0, 5, "bf16", 0),       # shorter than one vector
     (5, 1, 4096, "bf16", 0),    # whole CTAs of the kernel that reads them over the bus
-    (3, 1, 8193, "bf16", 0),    # a vector and two bytes more than that
+    (3, 1, 8193, "bf16", 0),    # six whole CTAs and twelve bytes
+    (1, 0, 8191, "bf16", 0),    # a vector less than a whole CTA, and fourteen bytes
+    (1, 0, 8201, "bf16", 0),    # a vector more, and two bytes
+    (1, 0, 10595, "bf16", 0),   # 300 vectors more, within a thread's second load, and six bytes
+    (1, 0, 4099, "f32", 0),     # a whole CTA and twelve bytes, of the other type
     (3, 1, 8193, "bf16", 3),    # not on a boundary of 16 bytes: copied
     (2, 1, 262144, "f32", 0),   # the longest logits that are read over the bus ...
     (2, 1, 262145, "f32", 0),   # ... and longer ones

@@ -29,6 +29,8 @@ def B():
     # rows in turns: as many warps as segments, one CTA per sequence in one to five turns, clusters, and beyond
     (100, 1, 18432, False), (101, 1, 18432, True), (330, 2, 4500, False), (719, 1, 12001, False), (740, 1, 20480, False), (740, 1, 20481, True),
     (1180, 1, 9001, True), (1201, 1, 2044, False), (150, 2, 23040, False), (150, 2, 23041, False),
+    (740, 1, 12800, False), (741, 1, 12800, False), (888, 1, 9000, False), (889, 1, 9000, True), (914, 1, 14080, False), (915, 1, 12480, False), (149, 1, 20992, False), (149, 1, 20993, True),
+    (350, 1, 11248, False), (351, 1, 11248, False), (319, 1, 6144, False), (320, 1, 6144, True), (290, 1, 19376, False),
     (3, 1, 1 << 19, False), (3, 1, (1 << 19) + 1, False), (4, 1, 1 << 20, False), (4, 1, (1 << 20) + 1, True), (3, 1, (1 << 21) + 3, False), (3, 1, 5000001, False),
 ])
 def test_draw_at_the_edges(B, oracle_mod, Bn, gamma, V, half):
@@ -97,13 +99,14 @@ def test_rejected_sequences_only_in_turns(B, Bn, V):
     assert torch.equal(some["token"][~bonus], full["token"][~bonus]) and torch.equal(some["flags"][~bonus], full["flags"][~bonus])
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("V", [20000, 20001])
-def test_fused_draw_in_turns(B, V):
+def test_fused_draw_in_turns(B, V, dtype):
     """The draw straight from the logits, in turns, against the draw from the row that the edge writes (the same float32
     values and the same float64 sums)."""
     Bn, gamma, T = 150, 16, 0.9
     gen = torch.Generator(device="cuda").manual_seed(V)
-    tl = (3.0 * torch.randn(Bn, gamma + 1, V, generator=gen, device="cuda")).to(torch.bfloat16)
+    tl = (3.0 * torch.randn(Bn, gamma + 1, V, generator=gen, device="cuda")).to(dtype)
     q = torch.softmax(tl[:, :gamma].float() / T + 0.1 * torch.randn(Bn, gamma, V, generator=gen, device="cuda"), dim=-1)
     x = torch.multinomial(q.view(-1, V), 1, generator=gen).view(Bn, gamma)
     q_tok = torch.gather(q, 2, x.unsqueeze(2)).squeeze(2).contiguous()
@@ -116,3 +119,26 @@ def test_fused_draw_in_turns(B, V):
     torch.cuda.synchronize()
     assert torch.equal(got["accept_len"], ev["accept_len"]) and torch.equal(got["token"], rs["token"])
     assert torch.equal(got["rs_flags"], rs["flags"])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", [20000, 20001])
+def test_bonus_tokens_in_turns(B, V, dtype):
+    """The bonus tokens drawn straight from the logits, in turns (more positions than the edge's one launch takes), against the draw
+    from the rows that the edge writes; the others keep -1."""
+    Bn, gamma, T = 60, 32, 0.9
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    tl = (3.0 * torch.randn(Bn, gamma + 1, V, generator=gen, device="cuda")).to(dtype)
+    x = torch.randint(0, V, (Bn, gamma), generator=gen, device="cuda", dtype=torch.int32)
+    half = torch.full((Bn, gamma), 0.5, device="cuda")
+    u = torch.zeros(Bn, gamma, device="cuda")  # accepted
+    u[::3, 5] = 0.999
+    u_rs = torch.rand(Bn, generator=gen, device="cuda").clamp_(max=1.0 - 2.0 ** -24)
+    ev = B.dssd_edge_verify(tl, x, half, u, T)
+    rs = B.dssd_device_resample(ev["p_row"], torch.zeros(Bn, gamma, V, device="cuda"), ev["accept_len"], u_rs, gamma)
+    got = B.dssd_edge_verify_bonus(tl, x, half, u, u_rs, T)
+    torch.cuda.synchronize()
+    full = ev["accept_len"] == gamma
+    assert torch.equal(got["accept_len"], ev["accept_len"]) and 0 < full.sum() < Bn
+    assert torch.equal(got["token"][full], rs["token"][full]) and (got["token"][~full] == -1).all()
+    assert torch.equal(got["token_flags"][full], rs["flags"][full]) and (got["token_flags"][~full] == 0).all()
