@@ -221,7 +221,8 @@ size_t dssd_round_host_arena_bytes(int B, int gamma, int V, dssd_dtype dtype);
  *
  * Of the draft distributions only the rows the device half reads cross the bus, B * V * 4 bytes at
  * most instead of B * gamma * V * 4: row Q_n of every sequence with a rejection.  Pinned host
- * buffers are mapped, and the kernels read those rows (and the short arrays) and write the results
+ * buffers are mapped, and the kernels read those rows (and the short arrays, and logits of up to 4 MB on a boundary
+ * of 16 bytes) and write the results
  * over the bus themselves; a buffer of which any part is pageable is copied.  The call waits on the host for the accepted
  * lengths (accept_len is final when the call returns) and therefore cannot be made while the stream
  * is being captured (DSSD_ERR_CUDA then).
@@ -319,6 +320,8 @@ size_t dssd_round_host_topk_arena_bytes(int B, int gamma, int V, int k, dssd_dty
  * uploaded and nothing is waited for: unlike dssd_round_host the call returns without
  * synchronising and can be captured).  The host buffers must stay valid until the stream has
  * finished; use pinned memory for the copies to be asynchronous.
+ *
+ * Pinned buffers are mapped as in dssd_round_host, logits of up to 4 MB among them.
  *
  * host inputs:  target_logits [B, gamma+1, V] contiguous, draft_tokens, draft_q_tok, uniforms
  *               [B, gamma], q_idx, q_val [B, gamma, k], uniforms_rs [B]

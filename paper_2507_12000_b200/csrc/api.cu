@@ -736,10 +736,12 @@ T *mapped(T *host, size_t count)
 // arrays over the bus (a copy each costs the host 3 us and the stream 2 to 4; a read by the kernels that use
 // them waits for the bus, about 5 us, once in each of them).  Pageable and long arrays are copied.
 //
-// Bound by the bus: the logits of B = 8 gamma = 4 V = 32000 bf16 (2.6 MB), four 16-byte loads per thread in flight, where a
-// copy took 64 us and the kernel after it started 7 us later: a round 82.6 us against 92; B = 6 gamma = 3 V = 33498 bf16
-// (1.6 MB) 61.5 and 75, B = 6 gamma = 8 V = 8048 float32 (1.7 MB) 55.7 and 63.2, B = 2 gamma = 2 V = 3000 float32 24.7 and 28.5.  The
-// copy engine moves long arrays faster: B = 16 gamma = 4 V = 50272 float32 (16 MB) 378 against 363.
+// Bound by the bus: the logits of B = 8 gamma = 4 V = 32000 bf16 (2.4 MB), four 16-byte loads per thread in flight, where a
+// copy took 64 us and the kernel after it started 7 us later: a round 83.2 us, copied 96.4; B = 6 gamma = 3 V = 33498 bf16
+// (1.5 MB) 60.8 and 72.8, B = 6 gamma = 8 V = 8048 float32 (1.7 MB) 55.7 and 61.7, B = 2 gamma = 2 V = 3000 float32 24.6 and 26.6.  The
+// copy engine moves long arrays faster, which uses the gain up at about 8 MB: gamma = 4 V = 32768 bf16, B = 9 (2.8 MB) 88.5 and 95.8, B = 12 (3.8 MB) 112.8
+// and 119.1, B = 16 (5 MB) 150.8 and 154.5, B = 24 (7.5 MB) 224.8 and 226.7; B = 16 gamma = 4 V = 50272 float32 (15 MB) 369 and 356.  Beyond 4 MB it is within
+// 3 %, for a kernel that holds SMs all the while.
 struct StageParams {
     const uint32_t *src[4];
     uint32_t *dst[4];
