@@ -803,23 +803,29 @@ __global__ void __launch_bounds__(kThreads) topk_first_kernel(const __grid_const
 // ---------------------------------------------------------------------------------------------
 // device half: one warp per sequence
 
-__device__ __forceinline__ double shfl_f64(double v, int src) { return __shfl_sync(kFullMask, v, src); }
-
 // inverse CDF over the warp's k entries (lane e holds r_e, entries in increasing index);
 // returns the position, or -1 when the mass is not positive and finite.  The sums are those of a loop over the entries, as dssd.h
-// says; the shuffles of eight entries are on their way at a time (the draw at k = 10 2.00 us, four at a time 2.13; at k = 32 2.30.
-// Sums by halves, 2.16 and 2.17, are other sums: entries of far smaller weight than the one before them count there).
+// says: a chain of additions, the entries from shared memory, two to a load and eight on their way at a time (the draw at B = 1 k = 10 2.03 us, at k = 32 2.25;
+// by shuffles 2.12 and 2.28, a round of B = 4 gamma = 2 V = 100744 bf16 k = 32 12.9 and 13.4.  Sums by halves, 2.14 and 2.25, are other
+// sums: entries of far smaller weight than the one before them count there).
 __device__ __forceinline__ int warp_inverse_cdf(double r, int k, double u)
 {
+    __shared__ __align__(16) double s_r[kWarps][32];
     const int lane = threadIdx.x & 31;
     double C = 0.0, mine = 0.0;  // the running mass in index order (lanes beyond k hold 0); this lane's
-    for (int e0 = 0; e0 < k; e0 += 8) {
-        double v[8];
+    double *const row = s_r[threadIdx.x >> 5];
+    __syncwarp();
+    row[lane] = r;
+    __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = shfl_f64(r, e0 + j);
+    for (int e0 = 0; e0 < 32; e0 += 8) {
+        if (e0 >= k) break;
+        double2 v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = reinterpret_cast<const double2 *>(row + e0)[j];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            C += v[j];
+            C += j & 1 ? v[j / 2].y : v[j / 2].x;
             if (lane == e0 + j) mine = C;
         }
     }
