@@ -668,23 +668,26 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
         if (twice > c) c = twice;
     }
     if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
-    if (c == kEdgeCluster && B * c > kEdgeEightsWave) c = kEdgeCluster - 1;
+    const bool full_eights = c == kEdgeCluster && B * c > kEdgeEightsWave;
+    if (full_eights && P.draw_token) c = kEdgeCluster - 1;
     const bool held = draws_held(P, kThreads, c), draw_only = P.draw_token && !P.p_row;
-    if (units > kEdgeBigUnits && kWarps * c < units && !held && (c <= kEdgeCluster || !draw_only)) {  // CTAs of 512 threads
+    if (units > kEdgeBigUnits && kWarps * c < units && !held) {  // CTAs of 512 threads
         for (const auto &big : kEdgeBig) {
             if (B > (P.draw_token ? big.most_draw : big.most) || (big.ctas > kEdgeCluster && most_cluster_ctas() < big.ctas)) continue;
             const double warps = (double)(16 * big.ctas), limit = P.shard_sum ? big.shard : both ? big.both : draw_only ? big.draw : big.row;
-            if (2 * big.ctas > c && work <= limit * warps && (B > kEdgeBigAlone || (double)parts <= (both ? 1.25 : 1.0) * warps))
+            if (draw_only && c > kEdgeCluster && big.ctas > kEdgeCluster) break;
+            if (2 * big.ctas > c && work <= limit * warps && (B > 1 || P.shard_sum || (double)parts <= (both ? 1.25 : 1.0) * warps))
                 return is(kEdgeMostThreads, big.ctas);
             break;
         }
     }
     if (c > kEdgeCluster) return is(kThreads, c);
-    if (!held && units >= (draw_only ? kEdgeSmallDrawUnits : kEdgeSmallUnits)) {  // CTAs of 128 threads
+    if (!held && units >= (P.draw_token ? kEdgeSmallDrawUnits : kEdgeSmallUnits)) {  // CTAs of 128 threads
         for (const auto &small : kEdgeSmall) {
             if (B > small.most) continue;
-            if (4 * small.ctas <= kWarps * c) break;
-            return work <= (P.shard_sum ? kEdgeSmallShard : draw_only ? kEdgeSmallDraw : draw * kEdgeSmallRow) * (double)(4 * small.ctas) && is(128, small.ctas);
+            const double limit = P.shard_sum ? small.shard : both ? small.both : draw_only ? small.draw : small.row;
+            if (units >= small.units && 4 * small.ctas > kWarps * c && work <= limit * (double)(4 * small.ctas)) return is(128, small.ctas);
+            break;
         }
     }
     const long long ctas = B * c, waves = (ctas + kEdgeWave - 1) / kEdgeWave;
@@ -692,7 +695,8 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
     const double limit = P.shard_sum ? (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0)
                                      : (held || fill >= 0.65 ? draw : 1.0) * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
     if (work > limit * (double)(kWarps * c)) return false;
-    return c == 2 && ctas >= kEdgePairCtas && !P.draw_token ? is(kEdgeMostThreads, 1) : is(kThreads, c);
+    const bool pairs = P.shard_sum ? c % 2 == 0 : !P.draw_token && (full_eights || (c == 2 && (B < kEdgeNoPairs || B > kEdgeNoPairsTo)));
+    return pairs && ctas >= kEdgePairCtas ? is(kEdgeMostThreads, c / 2) : is(kThreads, c);
 }
 
 long long row_segments(int V, int esz)

@@ -31,29 +31,33 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //   * Launches that leave most SMs idle spread over twice the CTAs, so that fewer warps share an SM (us per call, default / spread):
 //     B = 13 gamma = 7 V = 42256 / 8 bf16 3.07 / 2.63, B = 3 gamma = 15 V = 4160 bf16 4.50 / 4.23, B = 23 gamma = 8 V = 3200 4.49 / 4.21.
 //   * Sequences of more units than such a cluster has warps, few at a time: CTAs of 512 threads, as many as a wave has room for, while
-//     a warp's work stays below kEdgeBig's.  Up to eight sequences leave SMs idle that the separate kernels use, and pay
-//     only up to a segment per warp: B = 2 gamma = 11 V = 25408 bf16 5.4 / 6.4, B = 6 gamma = 2 V = 53913 float32 6.5 / 7.6; beyond, B = 1 gamma = 7
-//     V = 50272 float32 6.7 / 5.6, B = 8 gamma = 7 V = 50272 8.3 / 7.5, a round of B = 1 gamma = 8 V = 50272 11.1 / 10.35.  More sequences, 16 CTAs: B = 14
-//     gamma = 2 V = 83517 float32 8.5 / 10.2; beyond, B = 12 gamma = 5 V = 90108 bf16 9.7 / 8.7; 12 CTAs: B = 18 gamma = 11 V = 34312 float32 10.6 / 11.4;
-//     beyond, B = 19 gamma = 8 V = 100000 bf16 15.2 / 14.0; 8: B = 29 gamma = 3 V = 63728 float32 10.4 / 11.5; beyond, B = 30 gamma = 11 V = 100000 bf16
-//     23.3 / 21.1; 6: B = 45 gamma = 6 V = 127696 bf16 25.4 / 29.8, B = 41 gamma = 6 V = 75163 17.1 / 17.9; 5: B = 48 gamma = 6 V = 115296 float32 34.4 / 35.3.  With
-//     a draw as well (five separate kernels): B = 7 gamma = 1 V = 128512 float32 10.0 / 13.7, B = 27 gamma = 2 V = 64064 bf16 10.0 / 14.0; beyond, B = 1 gamma = 4
-//     V = 121880 float32 9.3 / 7.9.  A draw alone: B = 17 gamma = 6 V = 54992 float32 13.7 / 16.3; beyond, B = 44 gamma = 14 V = 57719 float32 41.8 / 38.3.
-//     Not where CTAs of 256 hold the row that is drawn from: fused B = 1 gamma = 12 V = 13930 float32 8.4, of 512 9.9.
+//     a warp's work stays below kEdgeBig's.  One sequence alone leaves SMs idle that the separate kernels use, and pays up to a segment per warp
+//     (a round, CTAs of 512 / separate: B = 1 gamma = 8 V = 50272 float32 11.1 / 10.35); two to eight up to two units (B = 2 gamma = 5 V = 48272 float32 10.3 /
+//     11.1, B = 4 gamma = 15 V = 29151 12.3 / 13.3, B = 8 gamma = 7 V = 50272 12.5 / 13.0; beyond, B = 5 gamma = 2 V = 133456 15.9 / 15.3, B = 2 gamma = 8 V = 56240 11.6 / 11.2);
+//     more sequences by 16 CTAs: B = 14 gamma = 2 V = 83517 float32, a call, 8.5 / 10.2; beyond, B = 12 gamma = 5 V = 90108 bf16 9.7 / 8.7; 12 CTAs: B = 18
+//     gamma = 11 V = 34312 float32 10.6 / 11.4; beyond, B = 19 gamma = 8 V = 100000 bf16 15.2 / 14.0; 8: B = 29 gamma = 3 V = 63728 float32 10.4 / 11.5; beyond, B = 30
+//     gamma = 11 V = 100000 bf16 23.3 / 21.1; 6: B = 45 gamma = 6 V = 127696 bf16 25.4 / 29.8, B = 35 gamma = 2 V = 140736 float32 19.8 / 20.7; beyond, a round of B = 33 gamma = 11
+//     V = 68752 bf16 30.3 / 27.4; 5: B = 48 gamma = 6 V = 115296 float32 34.4 / 35.3.  With a draw as well (five separate kernels): B = 7 gamma = 1 V = 128512 float32
+//     10.0 / 13.7, B = 27 gamma = 2 V = 64064 bf16 10.0 / 14.0, a round of B = 6 gamma = 2 V = 109056 float32 17.0 / 19.4; beyond, B = 1 gamma = 4 V = 121880 float32 9.3 / 7.9.
+//     A draw alone: B = 17 gamma = 6 V = 54992 float32 13.7 / 16.3, B = 14 gamma = 8 V = 74608 16.4 / 18.9; beyond, B = 44 gamma = 14 V = 57719 float32 41.8 / 38.3.  Not
+//     where CTAs of 256 hold the row that is drawn from (fused B = 1 gamma = 12 V = 13930 float32 8.4, of 512 9.9).
 //   * A batch that leaves each sequence one or two CTAs and half of the SM's room idle: three to six of 128 threads (kEdgeSmall), which find
-//     room in one wave while they are nine tenths of the clusters that the GPU holds.  B = 332 gamma = 13 V = 5816 float32 22.1 / 27.0, B = 303 gamma = 2 V = 24064
-//     float32 22.5 / 25.6, B = 190 gamma = 1 V = 34288 bf16 14.5 / 16.7, fused B = 178 gamma = 3 V = 25552 float32 23.7 / 27.5; beyond, the round of B = 213 gamma = 5
-//     V = 7568 float32 23.2 / 18.8, of B = 220 gamma = 2 V = 90976 106.7 / 87.1, of B = 333 gamma = 10 V = 12288 54.9 / 46.0 with work at the limit, B = 364 gamma = 7 V = 23515 fused
-//     60.6 / 49.2.  From 17 units on (B = 177 gamma = 2 V = 11376 binary16 7.0 against 8.7 with two CTAs of 256, B = 300 gamma = 3 V = 4096 float32, 16 units, 8.5 against
-//     8.3); a draw alone from 30 on (B = 332 gamma = 13 V = 1360, 28 units, 20.2 against 14.9).  More work per warp: fused B = 187 gamma = 2 V = 72378 bf16 (18 per
-//     warp) 45.1 against 40.9 in separate kernels, a shard of B = 190 gamma = 5 V = 49424 bf16 (15) 26.9 / 23.7, B = 370 gamma = 12 V = 20480 float32 (25) 91.2 / 76.1, a round of B = 300 gamma = 4 V = 30011 bf16 (17.4) 49.8 / 49.5.
-//   * Otherwise a sequence's two CTAs are one of 512 threads, which needs no cluster, where they are many: B = 168 gamma = 7 V = 2048 float32 (a
-//     shard) 4.0 / 4.6, B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, B = 259 gamma = 3 V = 14848 float32 16.3 / 16.5.  Not four, six or eight, which as two to four
-//     of 512 threads find less room: a round of B = 92 gamma = 14 V = 10400 float32 20.4 us with six of 256, 28.7 with three of 512; B = 49 gamma = 9 V = 5242
-//     bf16 10.9 and 12.2 with two, B = 67 gamma = 7 V = 7744 9.8 and 11.2.
-// Near the last cluster that the GPU holds, a launch in a pipeline waits for the one before it to drain: eight CTAs each up to 65 sequences (a
-// round of B = 69 gamma = 1 V = 95104 float32 35.2 us, with seven 28.2), three up to 166 (a round of B = 174 gamma = 2 V = 8608 float32 17.8, with six of 128
-// threads 14.2; fused B = 169 gamma = 2 V = 6224 13.2, with two of 256 10.9).
+//     room in one wave while they are about nine tenths of the clusters that the GPU holds.  B = 303 gamma = 2 V = 24064 float32 22.5 / 25.6, B = 190 gamma = 1
+//     V = 34288 bf16 14.5 / 16.7, fused B = 178 gamma = 3 V = 25552 float32 23.7 / 27.5; beyond, the round of B = 213 gamma = 5 V = 7568 float32 23.2 / 18.8, of B = 220 gamma = 2
+//     V = 90976 106.7 / 87.1.  Near the last cluster, from 326 sequences on, only with less work per warp: rounds of B = 359 gamma = 7 V = 4993 float32 25.3 / 26.9, B = 367 gamma = 8
+//     V = 8080 bf16 26.0 / 29.5, with a draw as well B = 350 gamma = 13 V = 11171 45.7 / 54.3; beyond, B = 327 gamma = 9 V = 11968 float32 51.8 / 45.1, B = 333 gamma = 10 V = 12288
+//     54.9 / 46.0, fused B = 349 gamma = 3 V = 12233 32.5 / 27.5.  From 17 units on (five CTAs 24: a round of B = 204 gamma = 6 V = 5721 bf16, 21 units, 18.5 / 17.5), with a draw
+//     from 30 on (fused B = 332 gamma = 13 V = 1360, 28 units, 20.2 / 14.9).  Beyond the limits on the work: fused B = 187 gamma = 2 V = 72378 bf16 (18 per warp) 45.1 / 40.9 in
+//     separate kernels, a shard of B = 190 gamma = 5 V = 49424 bf16 (15) 26.9 / 23.7, B = 370 gamma = 12 V = 20480 float32 (25) 91.2 / 76.1, a round of B = 300 gamma = 4 V = 30011
+//     bf16 (17.4) 49.8 / 49.5.
+//   * Otherwise a sequence's two CTAs are one of 512 threads, which needs no cluster, where they are many: B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, a round of B = 225
+//     gamma = 11 V = 1520 float32 11.3 / 11.7; not from 150 to 203 sequences, where the draw's clusters that follow find less room (a round of B = 175 gamma = 4 V = 5280 bf16
+//     13.2 / 11.6).  Not four or six, which as two or three of 512 threads find less room: a round of B = 92 gamma = 14 V = 10400 float32 20.4 us with six of 256, 28.7 with
+//     three of 512; B = 49 gamma = 9 V = 5242 bf16 10.9 and 12.2 with two.  Eight from 66 sequences on (a round of B = 69 gamma = 1 V = 95104 float32 26.7, with seven of 256
+//     threads 28.2, with eight 35.2), and a shard's, whose next kernel has few CTAs (the calls of B = 61 gamma = 6 V = 10528 17.4 / 19.2, of B = 90 gamma = 7 V = 16752
+//     26.2 / 29.5; of B = 57 gamma = 13 V = 1088 level).
+// Near the last cluster that the GPU holds, a launch in a pipeline waits for the one before it to drain: eight CTAs each up to 65 sequences, three up to 166 (a round of B = 174
+// gamma = 2 V = 8608 float32 17.8, with six of 128 threads 14.2; fused B = 169 gamma = 2 V = 6224 13.2, with two of 256 10.9).
 // How much work per warp still pays depends on how full the wave is, since a
 // warp's loads wait for one another from segment to segment and only other CTAs on the SM fill the gaps.  Measured (us per
 // call, cluster kernel / separate kernels):
@@ -62,9 +66,10 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //              B = 318 gamma = 4 V = 9792 bf16 16.3 / 20.2; beyond B = 661 gamma = 1 V = 72431 bf16 110 / 86
 //   full wave:  B = 89 gamma = 4 V = 18896 float32 9.6 / 13.0, B = 64 gamma = 4 V = 128256 bf16 26.5 / 29.7,
 //              B = 128 gamma = 4 V = 50272 float32 30.7 / 32.3; beyond B = 166 gamma = 11 V = 53648 bf16 52.8 / 48.8.
-// A shard's partial sums have no emission to share a launch with and pay off up to less work per warp, in clusters of up to sixteen CTAs of
-// 512 threads about a segment each (the call, in one launch / separate kernels: B = 5 gamma = 6 V = 18928 float32 3.5 / 3.9, B = 48 gamma = 4 V = 26416
-// bf16 5.1 / 5.8; beyond, B = 1 gamma = 8 V = 50272 float32 5.2 / 3.7, B = 19 gamma = 8 V = 50272 11.5 / 9.5, B = 40 gamma = 16 V = 76000 bf16 25.0 / 22.6),
+// A shard's partial sums have no emission to share a launch with and pay off up to less work per warp.  By up to sixteen CTAs of 512 threads the kernel is slower than the two
+// from about one unit per warp on (B = 5 gamma = 6 V = 18928 float32 3.5 / 3.9; B = 1 gamma = 8 V = 50272 5.2 / 3.7), but a round is seven launches, which the host
+// enqueues in 20 us, and so one less is quicker up to two units, except from a CUDA graph (the calls of B = 1 gamma = 8 V = 50272 17.5 / 20.0, from a graph 15.9 / 14.3; of B = 2 gamma = 7
+// V = 36176 18.1 / 20.6 and 15.2 / 14.4, of B = 2 gamma = 9 V = 55623 bf16 17.7 / 21.5 and 15.6 / 14.3); beyond, B = 19 gamma = 8 V = 50272 11.5 / 9.5, B = 40 gamma = 16 V = 76000 bf16 25.0 / 22.6, a round of B = 7 gamma = 13 V = 58416 1.05 of it;
 // in smaller ones more: B = 256 gamma = 4 V = 18992
 // bf16 13.5 / 14.2, B = 503 gamma = 3 V = 5936 float32 8.5 / 11.1, B = 620 gamma = 15 V = 792 bf16 9.7 / 28.4; beyond B = 173 gamma = 3
 // V = 67023 float32 40.5 / 30.5, B = 2 gamma = 2 V = 79648 float32 5.4 / 4.6.  Where the edge draws bonus tokens the separate kernels are
@@ -81,14 +86,17 @@ struct EdgeBig {  // up to so many sequences (with a draw) so many CTAs of 512 t
     int ctas;
     double row, draw, both, shard;
 };
-constexpr EdgeBig kEdgeBig[] = {{8, 8, 16, 2.0, 2.0, 2.6, 1.05},  {14, 14, 16, 2.0, 3.0, 6.5, 1.05},   {19, 19, 12, 3.0, 2.7, 5.4, 1.05},
-                                {30, 30, 8, 5.0, 5.0, 8.0, 1.05}, {45, 42, 6, 12.0, 10.0, 14.5, 3.0}, {52, 50, 5, 13.0, 4.0, 14.5, 3.0}};
-constexpr long long kEdgeBigAlone = 8;  // sequences that leave SMs to spare: no more than a segment per warp
-struct EdgeSmall { long long most; int ctas; };           // up to so many sequences, so many CTAs of 128 threads each
-constexpr EdgeSmall kEdgeSmall[] = {{181, 6}, {204, 5}, {346, 3}};
-constexpr long long kEdgeSmallUnits = 17, kEdgeSmallDrawUnits = 30;  // units of a sequence; where it is only drawn from
-constexpr double kEdgeSmallRow = 15.0, kEdgeSmallDraw = 13.0, kEdgeSmallShard = 8.0;  // work per warp
-constexpr long long kEdgePairCtas = 150;
+constexpr EdgeBig kEdgeBig[] = {{1, 1, 16, 2.0, 2.0, 2.6, 2.2},     {8, 8, 16, 2.08, 2.05, 3.5, 2.2},  {14, 14, 16, 2.0, 3.3, 6.5, 1.4},   {19, 19, 12, 3.0, 2.7, 5.4, 1.05},
+                                {30, 30, 8, 5.0, 7.6, 8.0, 1.05}, {39, 39, 6, 8.0, 10.0, 14.5, 3.0}, {45, 43, 6, 12.0, 10.0, 25.0, 3.0}, {52, 50, 5, 13.0, 4.0, 14.5, 3.0}};
+struct EdgeSmall {  // up to so many sequences of so many units so many CTAs of 128 threads each; most work per warp as above
+    long long most, units;
+    int ctas;
+    double row, draw, both, shard;
+};
+constexpr EdgeSmall kEdgeSmall[] = {{181, 17, 6, 15.0, 15.0, 35.0, 8.0}, {204, 24, 5, 15.0, 13.0, 35.0, 8.0}, {325, 17, 3, 15.0, 13.0, 35.0, 8.0},
+                                    {335, 17, 3, 9.0, 13.0, 35.0, 8.0},  {350, 17, 3, 9.0, 0.0, 35.0, 8.0},   {370, 17, 3, 9.0, 0.0, 0.0, 0.0}};
+constexpr long long kEdgeSmallUnits = 17, kEdgeSmallDrawUnits = 30;  // units of a sequence; with a draw
+constexpr long long kEdgePairCtas = 150, kEdgeNoPairs = 150, kEdgeNoPairsTo = 203;
 constexpr double kEdgeWideRounds = 2.8, kEdgeWidePartial = 1.6, kEdgeDrawFactor = 1.8;
 constexpr int kEdgeHeldWave = 200;                       // CTAs of a launch that draws with the row in registers (two per SM)
 constexpr int kEdgeClusterParts = 1024;                  // segments of a sequence (8 KB of shared memory).  It ends the calls by CTAs of 512 threads; the other limits allow 900

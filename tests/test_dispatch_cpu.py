@@ -24,12 +24,13 @@ def edge(L, dtype, form, B, gamma, V):
     return t.value, c.value
 
 
-# A shard's partial sums by CTAs of 512 threads: about a segment per warp in clusters of more than eight CTAs, up to three in smaller ones
+# A shard's partial sums by CTAs of 512 threads: a launch less in rounds that the host cannot enqueue as fast as they run, where few sequences
+# have little work per warp (rounds of pipelined calls), or quicker in itself
 @pytest.mark.parametrize("dtype,B,gamma,V,shape", [
-    (F32, 1, 8, 50272, SEPARATE),    # 3.7 / 5.2 (16 CTAs)
-    (F32, 4, 5, 50272, SEPARATE),    # 4.0 / 5.0
-    (BF16, 8, 4, 76000, SEPARATE),   # 4.4 / 5.0
-    (F32, 14, 4, 60000, SEPARATE),   # 5.2 / 6.3
+    (F32, 1, 8, 50272, (512, 16)),   # a round 17.5 / 20.0 (from a graph 15.9 / 14.3)
+    (BF16, 2, 9, 55623, (512, 16)),  # a round 17.7 / 21.5 (15.6 / 14.3)
+    (F32, 7, 13, 58416, SEPARATE),   # a round 5 % less
+    (F32, 10, 7, 51165, SEPARATE),   # a round 3 % less
     (F32, 19, 8, 50272, SEPARATE),   # 9.5 / 11.5 (12 CTAs)
     (BF16, 40, 16, 76000, SEPARATE),  # 22.6 / 25.0 (6 CTAs)
     (F32, 5, 6, 18928, (512, 16)),   # 3.5 / 3.9
@@ -43,7 +44,11 @@ def test_shard_sums(L, dtype, B, gamma, V, shape):
 # Few sequences of many segments by CTAs of 512 threads, or not
 @pytest.mark.parametrize("dtype,form,B,gamma,V,shape", [
     (F32, ROW, 1, 7, 50272, SEPARATE),       # 5.6 / 6.7
-    (F32, ROW, 8, 7, 50272, SEPARATE),       # 7.5 / 8.3
+    (F32, ROW, 5, 2, 133456, SEPARATE),      # a round 15.3 / 15.9
+    (F32, ROW, 2, 5, 48272, (512, 16)),      # a round 10.3 / 11.1
+    (BF16, ROW, 33, 11, 68752, SEPARATE),    # a round 27.4 / 30.3 (6)
+    (F32, FUSED, 38, 3, 24400, (512, 6)),    # 10.2 / 10.7 (256 x 10)
+    (F32, BONUS, 6, 2, 109056, (512, 16)),   # a round 17.0 / 19.4
     (BF16, ROW, 12, 5, 90108, SEPARATE),     # 8.7 / 9.7
     (BF16, ROW, 19, 8, 100000, SEPARATE),    # 14.0 / 15.2
     (BF16, ROW, 30, 11, 100000, SEPARATE),   # 21.1 / 23.3
@@ -74,7 +79,11 @@ def test_few_sequences(L, dtype, form, B, gamma, V, shape):
     (BF16, FUSED, 364, 7, 23515, SEPARATE),  # 49.2 / 60.6 (3)
     (F32, FUSED, 332, 13, 1360, (256, 1)),   # 14.9 / 20.2 (3)
     (F32, FUSED, 208, 5, 6119, (256, 2)),    # 16.6 / 20.6 (5)
-    (F32, ROW, 332, 13, 5816, (128, 3)),     # 22.1 / 27.0
+    (F32, ROW, 303, 2, 24064, (128, 3)),     # 22.5 / 25.6
+    (F32, ROW, 359, 7, 4993, (128, 3)),      # a round 25.3 / 26.9 (256 x 1)
+    (F32, ROW, 333, 10, 12288, SEPARATE),    # a round 46.0 / 54.9
+    (BF16, BONUS, 350, 13, 11171, (128, 3)),  # a round 45.7 / 54.3 (256 x 1)
+    (BF16, ROW, 204, 6, 5721, (512, 1)),     # a round 17.5 / 18.5 (128 x 5)
     (F32, ROW, 199, 9, 7840, (128, 5)),      # 14.9 / 15.9 (256 x 2)
     (F32, FUSED, 178, 3, 25552, (128, 6)),   # 23.7 / 27.5 (256 x 2)
     (BF16, ROW, 177, 2, 11376, (128, 6)),    # 7.0 / 8.7 (256 x 2)
@@ -88,9 +97,10 @@ def test_batches_of_one_or_two_ctas(L, dtype, form, B, gamma, V, shape):
     (F32, ROW, 92, 14, 10400, (256, 6)),     # 20.4 / 28.7 (512 x 3)
     (BF16, ROW, 49, 9, 5242, (256, 4)),      # 10.9 / 12.2 (512 x 2)
     (BF16, ROW, 67, 7, 7744, (256, 4)),      # 9.8 / 11.2
-    (F32, SHARD, 57, 13, 1088, (256, 4)),    # the call 3.1 / 3.3
+    (F32, SHARD, 90, 7, 16752, (512, 3)),    # 26.2 / 29.5 (256 x 6)
+    (BF16, ROW, 175, 4, 5280, (256, 2)),     # 11.6 / 13.2 (512 x 1)
     (F32, SHARD, 168, 7, 2048, (512, 1)),    # the call 4.0 / 4.6 (256 x 2)
-    (F32, ROW, 69, 1, 95104, (256, 7)),      # 28.2 / 35.2 (256 x 8)
+    (F32, ROW, 69, 1, 95104, (512, 4)),      # 26.7 / 35.2 (256 x 8)
 ])
 def test_pairs_and_full_waves(L, dtype, form, B, gamma, V, shape):
     assert edge(L, dtype, form, B, gamma, V) == shape
@@ -100,7 +110,7 @@ def test_pairs_and_full_waves(L, dtype, form, B, gamma, V, shape):
 @pytest.mark.parametrize("dtype,B,gamma,V,shape", [
     (F32, 1, 5, 57440, SEPARATE),     # 7.5 / 11.4 (256 x 8)
     (F32, 1, 8, 42042, SEPARATE),     # 7.6 / 11.2
-    (F32, 3, 5, 58288, SEPARATE),     # 9.2 / 11.4
+    (F32, 3, 5, 58288, (512, 16)),    # a round 12.3 / 15.4
     (BF16, 2, 10, 31702, (256, 8)),   # 9.3 / 10.4 (the row is held)
 ])
 def test_bonus_draws(L, dtype, B, gamma, V, shape):

@@ -118,7 +118,7 @@ def _shape(B, dtype, form, Bn, gamma, V):
     ("f32", 19, 11, 17000, (512, 12)), ("f32", 20, 3, 63728, (512, 8)), ("f32", 30, 3, 63728, (512, 8)), ("f32", 31, 9, 26000, (512, 6)),
     ("f32", 45, 7, 20000, (512, 6)), ("f32", 46, 7, 20000, (512, 5)), ("f32", 52, 7, 20000, (512, 5)), ("f32", 53, 7, 20000, (256, 8)),
     ("f32", 181, 4, 4200, (128, 6)), ("f32", 182, 4, 4200, (128, 5)), ("f32", 204, 4, 4200, (128, 5)), ("f32", 205, 4, 4200, (512, 1)),
-    ("f32", 346, 4, 4200, (128, 3)), ("f32", 347, 4, 4200, (256, 1)), ("bf16", 177, 2, 11376, (128, 6)), ("f32", 65, 7, 8200, (256, 8)), ("f32", 66, 7, 8200, (256, 7)),
+    ("f32", 370, 4, 4200, (128, 3)), ("f32", 371, 4, 4200, (256, 1)), ("bf16", 177, 2, 11376, (128, 6)), ("f32", 65, 7, 8200, (256, 8)), ("f32", 66, 7, 8200, (512, 4)),
     ("f32", 45, 15, 65536, (512, 6)), ("f32", 45, 15, 65540, (0, 0)),
 ])
 def test_edges_of_the_tables(B, oracle_mod, dtype, Bn, gamma, V, shape):
