@@ -68,7 +68,8 @@ constexpr long long kHeldWarps = 2250, kHeldWideWarps = 1650, kHeldWidestWarps =
 // B = 665 V = 12640 12.8 / 15.6, B = 305 V = 15760 binary16 9.8 / 12.5, B = 143 V = 19400 7.8 / 9.4; beyond, B = 67 V = 32592 7.0 / 6.6,
 // B = 100 V = 43015 13.3 / 12.2, B = 55 V = 124034 14.4 / 10.5.  The two kernels are the better ones for
 //   clusters of more warps than kStreamClusters in all (B = 383 V = 23016 15.2 / 13.5, B = 290 V = 19376 by four CTAs 10.6 / 9.6, B = 195 V = 10576 by six 8.3 /
-//   6.5; with fewer CTAs B = 330 V = 23040 11.9 / 13.1),
+//   6.5; with fewer CTAs B = 330 V = 23040 11.9 / 13.1), of three CTAs from kStreamThrees sequences on (a round of B = 340 V = 15924 26.7, by one CTA of 256 threads 24.7, two
+//   kernels 24.5) and of five of 256 threads (a round of B = 105 V = 17084 17.4, by five of 128 15.2, two kernels 14.9),
 //   rows of more than kStreamTurnsFew turns by one CTA each that leave a third of the wave empty (B = 400 V = 18218 16.2 / 14.3, B = 352 V = 19047 17.3 / 13.6; in four
 //   turns B = 416 V = 12881 12.4 / 14.2, B = 385 V = 15189 12.6 / 13.1, B = 421 V = 15520 11.7 / 10.5),
 //   few long rows that need more than a segment per warp (B = 92 V = 20030 8.3 / 7.1 and B = 133 V = 15897 8.8 / 7.4 off the 16-byte boundaries, B = 107 V = 22920
@@ -76,7 +77,7 @@ constexpr long long kHeldWarps = 2250, kHeldWideWarps = 1650, kHeldWidestWarps =
 // Up to sixteen segments by eight warps in two turns, not by as many warps as segments, from kStreamHalf sequences on: B = 340 V = 4608 6.5 / 8.0, B = 318 V =
 // 4880 6.9 / 8.3; below, B = 290 V = 5120 6.3 / 5.9, B = 251 V = 4608 6.4 / 5.7.
 constexpr int kStreamSegs = 45, kStreamTurns = 5, kStreamTurnsFew = 4;
-constexpr long long kStreamOne = 3600, kStreamOneLong = 3300, kStreamHalf = 300, kStreamClusters = 4200;
+constexpr long long kStreamOne = 3600, kStreamOneLong = 3300, kStreamHalf = 300, kStreamClusters = 4200, kStreamThrees = 333;
 constexpr long long kStreamFew = 150;                              // sequences, of at most
 constexpr int kStreamFewSegs = 41, kStreamFewSegsShifted = 29;     // segments, on and off the boundaries of 16 bytes
 constexpr int kDrawThreads = 128;        // threads that draw for a sequence
@@ -686,7 +687,8 @@ bool one_launch(ResampleParams &P, bool aligned, Most most_cluster_ctas)
         if (B < kStreamFew && segs > (aligned ? kStreamFewSegs : kStreamFewSegsShifted)) return false;
         warps = even(wave * 7 / 10 / B);
         long long most = kStreamClusters / B / 4 * 4;  // whole CTAs of four warps
-        if (most < kWarps) most = kWarps;
+        if (most > 4 * kClusterMax) most = 4 * kClusterMax;
+        if (most < kWarps || B > kStreamThrees) most = kWarps;
         if (warps > kWarps && (warps + 3) / 4 * 4 > most) warps = even(most);
     }
     if (warps <= kWarps && 10 * kWarps * B < 7 * wave) most_turns = kStreamTurnsFew;

@@ -145,6 +145,8 @@ def test_draws_by_one_cta(L, B, V, shape):
     (406, 18672, (0, 0, 0)),      # 12.2 / 14.2 (128 x 3)
     (330, 23040, (128, 3, 1)),    # 11.9 / 13.1
     (290, 19376, (128, 3, 1)),    # 9.6 / 10.6 (128 x 4; two kernels 9.6)
+    (340, 15924, (256, 1, 1)),    # a round 24.7 / 26.7 (128 x 3)
+    (105, 17084, (128, 5, 1)),    # a round 15.2 / 17.4 (256 x 5)
     (352, 19047, (0, 0, 0)),      # 13.6 / 17.3 (256 x 1)
     (400, 18218, (0, 0, 0)),      # 14.3 / 16.2
     (92, 20030, (0, 0, 0)),       # 7.1 / 8.3 (128 x 5)
