@@ -656,20 +656,21 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
         return true;
     };
     long long c = fit((units + kWarps - 1) / kWarps, kEdgeWave, P.B);
-    if (c > 2) c = fit(c, kEdgeClusterWave, P.B);
-    if (c == 3 && B * c > kEdgeThreesWave) c = 2;
     if (c > kEdgeCluster) {
         const long long wide = fit(c, kEdgeWideWave, P.B);
         c = wide > kEdgeCluster ? wide : kEdgeCluster;
         if (c > kEdgeCluster && c > most_cluster_ctas()) c = most_cluster_ctas();
+    }
+    bool full = false;  // four or eight that find room as half as many CTAs of 512 threads
+    while (c > 2 && c <= kEdgeCluster && B > kEdgeMostOf[c] && !full) {
+        full = c % 4 == 0 && B * c <= kEdgeClusterWave && !P.draw_token;
+        if (!full) --c;
     }
     if (c > 1 && 2 * c * B <= kEdgeSpread) {
         const long long most = most_cluster_ctas() < kEdgeSpreadCtas ? most_cluster_ctas() : kEdgeSpreadCtas, twice = 2 * c < most ? 2 * c : most;
         if (twice > c) c = twice;
     }
     if (c > kEdgeCluster && work > (P.shard_sum ? kEdgeWidePartial : kEdgeWideRounds) * (double)(kWarps * c)) c = kEdgeCluster;
-    const bool full_eights = c == kEdgeCluster && B * c > kEdgeEightsWave;
-    if (full_eights && P.draw_token) c = kEdgeCluster - 1;
     const bool held = draws_held(P, kThreads, c), draw_only = P.draw_token && !P.p_row;
     if (units > kEdgeBigUnits && kWarps * c < units && !held) {  // CTAs of 512 threads
         for (const auto &big : kEdgeBig) {
@@ -695,7 +696,7 @@ bool cluster_shape(EdgeParams &P, int esz, long long segs, Most most_cluster_cta
     const double limit = P.shard_sum ? (fill >= 0.65 ? 8.0 : fill >= 0.5 ? 5.0 : 2.0)
                                      : (held || fill >= 0.65 ? draw : 1.0) * (fill >= 0.8 && c <= 4 ? 25.0 : fill >= 0.65 ? 14.0 : fill >= 0.5 ? 10.0 : 4.0);
     if (work > limit * (double)(kWarps * c)) return false;
-    const bool pairs = P.shard_sum ? c % 2 == 0 : !P.draw_token && (full_eights || (c == 2 && (B < kEdgeNoPairs || B > kEdgeNoPairsTo)));
+    const bool pairs = P.shard_sum ? c % 2 == 0 : !P.draw_token && (full || (c == 2 && (B < kEdgeNoPairs || B > kEdgeNoPairsTo)));
     return pairs && ctas >= kEdgePairCtas ? is(kEdgeMostThreads, c / 2) : is(kThreads, c);
 }
 

@@ -53,11 +53,12 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 //   * Otherwise a sequence's two CTAs are one of 512 threads, which needs no cluster, where they are many: B = 117 gamma = 2 V = 6656 bf16 5.0 / 5.4, a round of B = 225
 //     gamma = 11 V = 1520 float32 11.3 / 11.7; not from 150 to 203 sequences, where the draw's clusters that follow find less room (a round of B = 175 gamma = 4 V = 5280 bf16
 //     13.2 / 11.6).  Not four or six, which as two or three of 512 threads find less room: a round of B = 92 gamma = 14 V = 10400 float32 20.4 us with six of 256, 28.7 with
-//     three of 512; B = 49 gamma = 9 V = 5242 bf16 10.9 and 12.2 with two.  Eight from 66 sequences on (a round of B = 69 gamma = 1 V = 95104 float32 26.7, with seven of 256
+//     three of 512; B = 49 gamma = 9 V = 5242 bf16 10.9 and 12.2 with two.  Eight from 66 sequences and four from 137 sequences on (a round of B = 137 gamma = 14 V = 44928 bf16 55.5, with four of 256 threads 59.6; of B = 69 gamma = 1 V = 95104 float32 26.7, with seven of 256
 //     threads 28.2, with eight 35.2), and a shard's, whose next kernel has few CTAs (the calls of B = 61 gamma = 6 V = 10528 17.4 / 19.2, of B = 90 gamma = 7 V = 16752
 //     26.2 / 29.5; of B = 57 gamma = 13 V = 1088 level).
-// Near the last cluster that the GPU holds, a launch in a pipeline waits for the one before it to drain: eight CTAs each up to 65 sequences, three up to 166 (a round of B = 174
-// gamma = 2 V = 8608 float32 17.8, with six of 128 threads 14.2; fused B = 169 gamma = 2 V = 6224 13.2, with two of 256 10.9).
+// Near the last cluster that the GPU holds, a launch in a pipeline waits for the one before it to drain (kEdgeMostOf).  Rounds, with one CTA less: B = 70 gamma = 2 V = 42528 float32
+// by eight 28.8, by seven 22.2; B = 75 gamma = 2 V = 84960 by seven 39.1, by six 33.6; B = 91 gamma = 3 V = 17695 by six 18.2, by five 17.7; B = 108 gamma = 3 V = 61178 bf16 by five
+// 40.2, by four 36.0; fused B = 169 gamma = 2 V = 6224 float32 by three 13.2, by two 10.9.
 // How much work per warp still pays depends on how full the wave is, since a
 // warp's loads wait for one another from segment to segment and only other CTAs on the SM fill the gaps.  Measured (us per
 // call, cluster kernel / separate kernels):
@@ -77,8 +78,8 @@ constexpr unsigned long long kEmitFoldCtas = 592;
 // the row (B = 1 gamma = 5 V = 57440 float32 11.4 / 7.5, B = 9 gamma = 4 V = 64935 13.3 / 12.8; held, B = 2 gamma = 10 V = 31702 bf16 9.3 / 10.4).
 constexpr int kEdgeCluster = 8, kEdgeClusterWide = 16;  // most CTAs per cluster: portable, and where the device has them
 constexpr int kEdgeMostThreads = 512;                    // per CTA
-constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeThreesWave = 500, kEdgeEightsWave = 520,
-                    kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, three, eight, more
+constexpr long long kEdgeWave = 592, kEdgeClusterWave = 552, kEdgeWideWave = 400;  // CTAs: up to two per sequence, up to eight, more
+constexpr int kEdgeMostOf[] = {0, 0, 0, 166, 136, 106, 92, 74, 65};  // sequences by so many CTAs each
 constexpr long long kEdgeSpread = 140, kEdgeSpreadCtas = 12;  // CTAs, in all and per sequence
 constexpr long long kEdgeBigUnits = 64;
 struct EdgeBig {  // up to so many sequences (with a draw) so many CTAs of 512 threads each; most work per warp: a row, a draw, both, a shard

@@ -101,6 +101,10 @@ def test_batches_of_one_or_two_ctas(L, dtype, form, B, gamma, V, shape):
     (BF16, ROW, 175, 4, 5280, (256, 2)),     # 11.6 / 13.2 (512 x 1)
     (F32, SHARD, 168, 7, 2048, (512, 1)),    # the call 4.0 / 4.6 (256 x 2)
     (F32, ROW, 69, 1, 95104, (512, 4)),      # 26.7 / 35.2 (256 x 8)
+    (BF16, ROW, 137, 14, 44928, (512, 2)),   # 55.5 / 59.6 (256 x 4)
+    (F32, ROW, 70, 2, 42528, (256, 7)),      # 22.2 / 28.8 (256 x 8)
+    (F32, ROW, 75, 2, 84960, (256, 6)),      # 33.6 / 39.1 (256 x 7)
+    (BF16, ROW, 108, 3, 61178, (256, 4)),    # 36.0 / 40.2 (256 x 5)
 ])
 def test_pairs_and_full_waves(L, dtype, form, B, gamma, V, shape):
     assert edge(L, dtype, form, B, gamma, V) == shape
