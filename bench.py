@@ -41,12 +41,12 @@ FALLBACK_HBM_GBS = 6650.0
 # DRAM traffic of the edge call from ncu (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the kernel
 # sources whose hash is recorded with it.
 NCU_TRAFFIC = {
-    # profiles/edge_call_c4.md: log-sum-exp kernel 389.1 MB read, fold 0.02, emission 70.7 MB read and 141.2 MB written
-    # inside it; the other 14.4 MB of p_row were still in L2 when it ended.  "bytes" counts all of p_row.
-    "c4": {"bytes": 389077504 + 16384 + 70693888 + 155582464, "kernel_hash": "1df65fdbb1f64d66",
-           "note": "dram__bytes_read.sum 459.8 MB + all 155.6 MB of p_row; reads are 1.18x the logits: the second read of "
+    # profiles/edge_call_c4.md: log-sum-exp kernel 389.0 MB read, fold 0.02, emission 70.9 MB read and 140.8 MB written
+    # inside it; the other 14.8 MB of p_row were still in L2 when it ended.  "bytes" counts all of p_row.
+    "c4": {"bytes": 389024512 + 16128 + 70899712 + 155582464, "kernel_hash": "280eb2734f6ca6c1",
+           "note": "dram__bytes_read.sum 459.9 MB + all 155.6 MB of p_row; reads are 1.18x the logits: the second read of "
                    "row n misses L2 for 91 % of its bytes",
-           "counted_inside_kernel": 389077504 + 16384 + 70693888 + 5616128 + 13568 + 141220096},
+           "counted_inside_kernel": 389024512 + 16128 + 70899712 + 5264896 + 12800 + 140778496},
 }
 
 
